@@ -2,21 +2,12 @@
 //
 // The handle carves every device array out of the caller's workspace, keeps
 // the per-replica tables there, and drives the kernels on the caller's stream.
-// md_step() runs as one CUDA graph:
-//
-//   integrate(FIRST) -> IF(rebuild){bin, scan, scatter, permute, nbuild}
-//     -> WHILE(loop){ step x c -> IF(rebuild){...} -> step x c -> IF ... }
-//
-// with kUnroll step kernels per loop iteration and a rebuild check after every
-// c of them (the check interval).  The last block of each kernel sets the
-// conditions on the device (rebuild when the displacement since the last
-// build, plus a bound on the motion until the next check, could exceed
-// skin/2; loop while steps
-// remain), so a whole md_step of n steps is one graph launch with no host
-// round trip.  Conditional nodes cost microseconds each on this hardware,
-// which is why the loop is unrolled and the check is spaced.  With
-// use_graph = 0 the same kernel sequence, with the same check points, is
-// launched from the host (the results are bitwise identical).
+// md_step() is one cooperative launch of the run kernel (md_kernels.cuh): the
+// half kick and drift that open it, the MD steps, and the list rebuilds that
+// the displacements call for, all decided on the device, so a whole md_step of
+// n steps needs no host round trip.  With use_graph = 0 the same kernel is
+// launched once per phase (each step, each rebuild) with its time taken (the
+// results are bitwise identical).
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
@@ -55,16 +46,13 @@ struct ApiRange {
 namespace {
 
 constexpr size_t kAlign = 256;
-constexpr int kIntBlock = 256, kForceBlock = 128, kScanBlock = 1024;
+constexpr int kIntBlock = 256, kForceBlock = 128;
+constexpr int kMaxRunBlocks = 4096;    // bound on the run kernel's blocks (entries of KArgs::slice)
 constexpr int kNbWarpCellsPerSm = 8;                     // warp-per-cell build from this many cells per SM
-constexpr int kNbCells = 4, kNbBlock = 32 * kNbCells;   // neighbour build: one warp per cell ...
-constexpr int kNbBlockB = 256;                          // ... or one block per cell
 constexpr double kCellMargin = 1e-3;   // cell edge exceeds the largest list radius by this
-constexpr int kUnroll = 16;            // step kernels per loop iteration of the graph
+constexpr int kUnroll = 16;            // largest check interval
 constexpr int kCheck = 4;              // automatic check interval below kCheckLargeN particles
-constexpr int64_t kCheckLargeN = 262144;   // from here a check after every step: the conditional
-                                           // node costs little against the step, the earlier
-                                           // rebuilds of a long interval cost more
+constexpr int64_t kCheckLargeN = 262144;   // from here a check after every step
 
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
@@ -73,11 +61,11 @@ struct Geometry {
     int R = 0;
     int64_t n = 0;
     int K = 0, Kmax = 0, tpp = 8, ppb_f = 32;   // starting list capacity, its cap
-    int check = kCheck;                 // MD steps between rebuild checks of the graph
-    bool nb_block = false;              // neighbour build with one block (8 warps) per cell
+    int check = kCheck;                 // MD steps between rebuild checks
+    bool nb_block = false;              // neighbour build with one block per cell
     int nblk_i = 0, nblk_f = 0, ncell = 0;
-    bool sweep = false;                 // step kernel: resident blocks sweeping runs of chunks
-    int nblk_s = 0, cpb = 1;            // step kernel: blocks launched, chunks per block
+    bool sweep = false;                 // step_form as reported: more chunks than resident blocks
+    int nblk_r = 0, nwork = 0, cpb = 1; // run kernel: blocks launched, of them with chunks, chunks per block
     double rl_max = 0.0;
     std::vector<mdk::Rep> rep;
     std::vector<int4> blk_i, blk_f;
@@ -86,12 +74,12 @@ struct Geometry {
 };
 
 struct Layout {
-    size_t off_ctl, off_rep, off_blk_i, off_blk_f, off_blk_s, off_crank, off_cxyz;
+    size_t off_ctl, off_rep, off_blk_i, off_blk_f, off_blk_r, off_crank, off_cxyz;
     size_t off_pa, off_pb, off_va, off_vb, off_pa2, off_pb2, off_va2, off_vb2, off_qa, off_qb, off_force;
     size_t off_rref, off_image, off_image2, off_key, off_tmpidx, off_skey;
     size_t off_ccount, off_ccursor, off_cstart, off_nbr, off_nnbr, off_part_f, off_part_i, off_part_e;
     size_t off_ring, off_totals, off_scale, off_st_pos, off_st_vel, off_st_img, off_st_code;
-    size_t off_epot, off_epot_step;
+    size_t off_epot, off_epot_step, off_rs, off_slice;
     size_t off_st_f, off_st_e, total;
 };
 
@@ -348,7 +336,9 @@ Layout make_layout(const md_params *p, const Geometry &g)
     L.off_rep = take(sizeof(mdk::Rep) * g.R);
     L.off_blk_i = take(sizeof(int4) * g.nblk_i);
     L.off_blk_f = take(sizeof(int4) * g.nblk_f);
-    L.off_blk_s = take(sizeof(int4) * 2 * (size_t)g.nblk_f);   // < nblk_f + resident blocks rows
+    L.off_blk_r = take(sizeof(int4) * 2 * (size_t)g.nblk_f);   // < nblk_f + resident blocks rows
+    L.off_rs = take(sizeof(mdk::RunSync));
+    L.off_slice = take(sizeof(int) * kMaxRunBlocks);
     L.off_crank = take(sizeof(int) * g.ncell);
     L.off_cxyz = take(sizeof(int4) * g.ncell);
     L.off_pa = take(pb * n);
@@ -373,9 +363,9 @@ Layout make_layout(const md_params *p, const Geometry &g)
     L.off_cstart = take(4 * ((size_t)g.ncell + 1));
     L.off_nbr = take(4 * n * (size_t)g.Kmax);       // room for the cap: K grows in place
     L.off_nnbr = take(4 * n);
-    L.off_part_f = take(8 * 12 * (size_t)g.nblk_f);
+    L.off_part_f = take(2 * 8 * 12 * (size_t)g.nblk_f);        // (2 parities)
     L.off_part_i = take(8 * 4 * (size_t)g.nblk_i);
-    L.off_part_e = take(8 * 2 * (size_t)(kForceBlock / 32) * (size_t)g.nblk_f);   // per warp, 2 parities
+    L.off_part_e = take(2 * 8 * (size_t)g.nblk_f);
     L.off_ring = take(sizeof(mdk::Obs) * (size_t)cap * g.R);
     L.off_epot = take(sizeof(double) * (size_t)cap * g.R);
     L.off_epot_step = take(sizeof(long long) * (size_t)cap);
@@ -418,15 +408,13 @@ struct md_handle {
     char *ws = nullptr;
     KArgs a;
     const KernelSet *ks = nullptr;
+    const void *runk = nullptr;      // the run kernel in use: precision, lanes per particle, smoothing
     int cap = 4096;
     // pinned host staging
     char *pin = nullptr;
     size_t pin_bytes = 0;
     cudaEvent_t ev_stage = nullptr;
-    // graph
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t gexec = nullptr;
-    // timing of the force kernel (use_graph = 0)
+    // timing of the run kernel's phases (use_graph = 0)
     cudaEvent_t ev_f0 = nullptr, ev_f1 = nullptr, ev_i1 = nullptr;
     double step_ms = 0.0, rebuild_ms = 0.0;
     int64_t step_launches = 0, rebuild_checks = 0;
@@ -458,13 +446,6 @@ int cuda_fail(md_handle *h, cudaError_t e, const char *what)
             return cuda_fail((h), e_, #expr);         \
     } while (0)
 
-// The step kernel in use: lanes per particle, smoothing, and the block form.
-const void *step_kernel(const md_handle *h)
-{
-    const int sm = h->p.smooth_h > 0.0, li = force_index(h->g.tpp);
-    return h->g.sweep ? h->ks->step_sweep[sm][li] : h->ks->step[sm][li];
-}
-
 int launch(md_handle *h, const void *f, int grid, int block, const KArgs &a)
 {
     if (grid <= 0)
@@ -476,219 +457,26 @@ int launch(md_handle *h, const void *f, int grid, int block, const KArgs &a)
 
 int grid_n(int64_t n, int per) { return (int)((n + per - 1) / per); }
 
-// The rebuild chain: kernel, grid, block.
-struct ChainStep { const void *f; int grid, block; };
-
-// The neighbour build's kernel and launch shape: one warp per cell, kNbCells
-// cells per block, unless the cells are too few to fill the GPU that way
-// (fewer than one per resident warp slot), then one 8-warp block per cell.
-ChainStep nbuild_step(const md_handle *h)
-{
-    if (h->g.nb_block)
-        return {h->ks->nbuild_blk, h->g.ncell, kNbBlockB};
-    return {h->ks->nbuild, (h->g.ncell + kNbCells - 1) / kNbCells, kNbBlock};
-}
-
-int rebuild_chain(const md_handle *h, ChainStep *seq)
-{
-    const KernelSet &k = *h->ks;
-    const int nb = grid_n(h->g.n, kIntBlock);
-    seq[0] = {k.bin, h->g.nblk_i, kIntBlock};
-    seq[1] = {k.scan, 1, kScanBlock};
-    seq[2] = {k.scatter, nb, kIntBlock};
-    seq[3] = {k.permute, nb, kIntBlock};
-    seq[4] = nbuild_step(h);                             // its last block makes
-    return 5;                                            // the permuted buffers current or asks
-}                                                        // for a redo with a larger K
-
-// The redo of the build after its capacity grew: one block per cell as well.
-KArgs retry_args(const md_handle *h)
+// One launch of the run kernel: what it does (mdk::RUN_*), steps and their
+// place in the md_step.
+int launch_run(md_handle *h, int what, int64_t nsteps = 0, int64_t budget = 0, int pos0 = 0, bool last = true)
 {
     KArgs a = h->a;
-    a.nb_retry = 1;
-    return a;
+    a.what = what;
+    a.nsteps = nsteps;
+    a.budget = budget;
+    a.pos0 = pos0;
+    a.last = last ? 1 : 0;
+    void *pp[1] = {(void *)&a};
+    CK(h, cudaLaunchCooperativeKernel(h->runk, dim3((unsigned)h->g.nblk_r), dim3(kForceBlock), pp, 0, h->s));
+    return MD_OK;
 }
 
-// Stream launches of the chain; the redo is launched every time and returns at
-// once unless the first build asked for it.
-int launch_rebuild(md_handle *h)
-{
-    ChainStep seq[8];
-    const int ns = rebuild_chain(h, seq);
-    for (int s = 0; s < ns; ++s) {
-        int rc = launch(h, seq[s].f, seq[s].grid, seq[s].block, h->a);
-        if (rc)
-            return rc;
-    }
-    const ChainStep nb = nbuild_step(h);
-    return launch(h, nb.f, nb.grid, nb.block, retry_args(h));
-}
-
-// Arguments of the step kernel at position `slot` of the unrolled loop.
-KArgs step_args(const md_handle *h, int slot)
-{
-    KArgs a = h->a;
-    a.imode = mdk::IM_LOOP;
-    const int ci = h->g.check;
-    const bool check = (slot % ci) == ci - 1;
-    a.lookahead = check ? ci - 1 : 0;
-    a.set_rebuild = check ? 1 : 0;
-    a.set_loop = slot == kUnroll - 1 ? 1 : 0;
-    return a;
-}
-
-KArgs first_args(const md_handle *h)
-{
-    KArgs a = h->a;
-    a.imode = mdk::IM_FIRST;
-    a.lookahead = h->g.check - 1;
-    a.set_rebuild = 1;
-    return a;
-}
-
-// Energies of a step still awaiting their sum go into the per-step series
-// first: the force kernel reuses the partials' storage.
-int flush_epot(md_handle *h) { return launch(h, h->ks->epot_flush, 1, kForceBlock, h->a); }
-
-int launch_force(md_handle *h, int fsample)
-{
-    KArgs a = h->a;
-    a.fsample = fsample;
-    int rc = flush_epot(h);
-    if (rc)
-        return rc;
-    return launch(h, h->ks->force[h->p.smooth_h > 0.0][force_index(h->g.tpp)], h->g.nblk_f, kForceBlock, a);
-}
-
-int launch_integrate(md_handle *h, int mode)
+int launch_kinetic(md_handle *h, int mode)
 {
     KArgs a = h->a;
     a.imode = mode;
-    a.use_cond = 0;
-    return launch(h, h->ks->integrate, h->g.nblk_i, kIntBlock, a);
-}
-
-// ---- graph construction ----
-int add_kernel(md_handle *h, cudaGraph_t g, cudaGraphNode_t *node, const cudaGraphNode_t *deps, size_t ndeps,
-               const void *f, int grid, int block, const KArgs &a)
-{
-    alignas(cudaGraphNodeParams) unsigned char np_buf[sizeof(cudaGraphNodeParams)] = {};
-    cudaGraphNodeParams &np = *reinterpret_cast<cudaGraphNodeParams *>(np_buf);
-    np.type = cudaGraphNodeTypeKernel;
-    np.kernel.func = (void *)f;
-    np.kernel.gridDim = dim3((unsigned)grid);
-    np.kernel.blockDim = dim3((unsigned)block);
-    np.kernel.sharedMemBytes = 0;
-    void *pp[1] = {(void *)&a};
-    np.kernel.kernelParams = pp;
-    CK(h, cudaGraphAddNode(node, g, deps, nullptr, ndeps, &np));
-    return MD_OK;
-}
-
-int add_conditional(md_handle *h, cudaGraph_t g, cudaGraphNode_t *node, cudaGraphNode_t dep,
-                    cudaGraphConditionalHandle c, cudaGraphConditionalNodeType type, cudaGraph_t *body);
-
-// The rebuild chain as graph nodes, closed by a conditional redo of the build
-// that runs only when the build grew the list capacity.
-int add_rebuild_chain(md_handle *h, cudaGraph_t g)
-{
-    ChainStep seq[8];
-    const int ns = rebuild_chain(h, seq);
-    cudaGraphConditionalHandle c_regrow;
-    CK(h, cudaGraphConditionalHandleCreate(&c_regrow, g, 0, 0));
-    cudaGraphNode_t prev = nullptr;
-    for (int s = 0; s < ns; ++s) {
-        cudaGraphNode_t node;
-        KArgs a = h->a;
-        if (s == ns - 1) {                              // the build
-            a.use_cond = 1;
-            a.set_regrow = 1;
-            a.h_regrow = c_regrow;
-        }
-        int rc = add_kernel(h, g, &node, prev ? &prev : nullptr, prev ? 1 : 0, seq[s].f, seq[s].grid,
-                            seq[s].block, a);
-        if (rc)
-            return rc;
-        prev = node;
-    }
-    cudaGraphNode_t n_if;
-    cudaGraph_t body;
-    int rc = add_conditional(h, g, &n_if, prev, c_regrow, cudaGraphCondTypeIf, &body);
-    if (rc)
-        return rc;
-    cudaGraphNode_t n_retry;
-    const ChainStep nb = nbuild_step(h);
-    return add_kernel(h, body, &n_retry, nullptr, 0, nb.f, nb.grid, nb.block, retry_args(h));
-}
-
-int add_conditional(md_handle *h, cudaGraph_t g, cudaGraphNode_t *node, cudaGraphNode_t dep,
-                    cudaGraphConditionalHandle c, cudaGraphConditionalNodeType type, cudaGraph_t *body)
-{
-    alignas(cudaGraphNodeParams) unsigned char np_buf[sizeof(cudaGraphNodeParams)] = {};
-    cudaGraphNodeParams &np = *reinterpret_cast<cudaGraphNodeParams *>(np_buf);
-    np.type = cudaGraphNodeTypeConditional;
-    np.conditional.handle = c;
-    np.conditional.type = type;
-    np.conditional.size = 1;
-    CK(h, cudaGraphAddNode(node, g, &dep, nullptr, 1, &np));
-    *body = np.conditional.phGraph_out[0];
-    return MD_OK;
-}
-
-int build_graph(md_handle *h)
-{
-    int rc;
-    cudaGraph_t g;
-    CK(h, cudaGraphCreate(&g, 0));
-    h->graph = g;
-    cudaGraphConditionalHandle c_loop, c_reb0;
-    CK(h, cudaGraphConditionalHandleCreate(&c_loop, g, 1, cudaGraphCondAssignDefault));
-    CK(h, cudaGraphConditionalHandleCreate(&c_reb0, g, 0, 0));
-
-    KArgs first = first_args(h);
-    first.use_cond = 1;
-    first.h_rebuild = c_reb0;
-    first.h_loop = c_loop;
-    cudaGraphNode_t n_first, n_if0, n_while;
-    if ((rc = add_kernel(h, g, &n_first, nullptr, 0, h->ks->integrate, h->g.nblk_i, kIntBlock, first)))
-        return rc;
-    cudaGraph_t body0;
-    if ((rc = add_conditional(h, g, &n_if0, n_first, c_reb0, cudaGraphCondTypeIf, &body0)))
-        return rc;
-    if ((rc = add_rebuild_chain(h, body0)))
-        return rc;
-    cudaGraph_t wbody;
-    if ((rc = add_conditional(h, g, &n_while, n_if0, c_loop, cudaGraphCondTypeWhile, &wbody)))
-        return rc;
-    // loop body: kUnroll step kernels, a conditional rebuild after every g.check
-    const void *stepk = step_kernel(h);
-    cudaGraphNode_t prev = nullptr;
-    for (int slot = 0; slot < kUnroll; ++slot) {
-        KArgs sa = step_args(h, slot);
-        sa.use_cond = 1;
-        sa.h_loop = c_loop;
-        cudaGraphConditionalHandle c_reb = 0;
-        if (sa.set_rebuild) {
-            CK(h, cudaGraphConditionalHandleCreate(&c_reb, wbody, 0, 0));
-            sa.h_rebuild = c_reb;
-        }
-        cudaGraphNode_t n_s;
-        if ((rc = add_kernel(h, wbody, &n_s, prev ? &prev : nullptr, prev ? 1 : 0, stepk, h->g.nblk_s,
-                             kForceBlock, sa)))
-            return rc;
-        prev = n_s;
-        if (sa.set_rebuild) {
-            cudaGraphNode_t n_if;
-            cudaGraph_t body;
-            if ((rc = add_conditional(h, wbody, &n_if, n_s, c_reb, cudaGraphCondTypeIf, &body)))
-                return rc;
-            if ((rc = add_rebuild_chain(h, body)))
-                return rc;
-            prev = n_if;
-        }
-    }
-    CK(h, cudaGraphInstantiate(&h->gexec, g, 0));
-    return MD_OK;
+    return launch(h, h->ks->kinetic, h->g.nblk_i, kIntBlock, a);
 }
 
 int stage_wait(md_handle *h)
@@ -727,8 +515,8 @@ int read_ctl(md_handle *h, mdk::Ctl *out)
     return MD_OK;
 }
 
-// Stream-launch mode: launch the rebuild chain if the device flag asks for it
-// (waits for the stream); adds its CUDA-event time to *ms when given.
+// Stream-launch mode: launch the rebuild if the device flag asks for it (waits
+// for the stream); adds its CUDA-event time to *ms when given.
 int rebuild_if_flagged(md_handle *h, float *ms)
 {
     mdk::Ctl c;
@@ -738,7 +526,7 @@ int rebuild_if_flagged(md_handle *h, float *ms)
     if (!c.rebuild || c.status)
         return MD_OK;
     CK(h, cudaEventRecord(h->ev_f1, h->s));
-    if ((rc = launch_rebuild(h)))
+    if ((rc = launch_run(h, mdk::RUN_REBUILD)))
         return rc;
     CK(h, cudaEventRecord(h->ev_i1, h->s));
     CK(h, cudaEventSynchronize(h->ev_i1));
@@ -789,7 +577,7 @@ int check_device(md_handle *h)
 }
 
 // Copy the caller's state into pinned staging, upload it, load it into the
-// working layout, rebuild, evaluate forces.
+// working layout, rebuild, evaluate forces and record them as a sample.
 int upload_state(md_handle *h, const int32_t *species, const double *pos, const double *vel,
                  const int32_t *image)
 {
@@ -818,9 +606,7 @@ int upload_state(md_handle *h, const int32_t *species, const double *pos, const 
     CK(h, cudaEventRecord(h->ev_stage, h->s));
     if ((rc = launch(h, h->ks->load, h->g.nblk_i, kIntBlock, h->a)))
         return rc;
-    if ((rc = launch_rebuild(h)))
-        return rc;
-    return launch_force(h, 1);
+    return launch_run(h, mdk::RUN_REBUILD | mdk::RUN_SAMPLE);
 }
 
 }  // namespace
@@ -942,8 +728,10 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
     a.nnbr = (int *)(w + L.off_nnbr);
     a.blk_i = (const int4 *)(w + L.off_blk_i);
     a.blk_f = (const int4 *)(w + L.off_blk_f);
-    a.blk_s = (const int4 *)(w + L.off_blk_s);
-    a.cpb = g.cpb;
+    a.blk_r = (const int4 *)(w + L.off_blk_r);
+    a.rs = (mdk::RunSync *)(w + L.off_rs);
+    a.slice = (int *)(w + L.off_slice);
+    a.check = g.check;
     a.part_f = (double *)(w + L.off_part_f);
     a.part_i = (double *)(w + L.off_part_i);
     a.part_e = w + L.off_part_e;
@@ -1010,20 +798,16 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
     if (a.hdtm_hi[0] == 0.0f)
         return fail(h, MD_E_INVAL, "dt / (2 m) underflows single precision");
 
-    int dev = 0, nsm = 0, per_sm = 0, per_sm_sw = 0;
+    int dev = 0, nsm = 0, per_sm = 0;
     CK(h, cudaGetDevice(&dev));
     CK(h, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    {
-        // step kernel: the sweeping form when asked for, or (automatic) when one block per chunk
-        // would need more blocks than the GPU holds at once
-        const int sm = h->p.smooth_h > 0.0, li = force_index(g.tpp);
-        const void *sweepk = li < 2 ? h->ks->step_sweep[sm][li] : nullptr;
-        CK(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, h->ks->step[sm][li], kForceBlock, 0));
-        if (sweepk)
-            CK(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_sw, sweepk, kForceBlock, 0));
-        h->g.sweep = sweepk && per_sm_sw > 0 &&
-                     (p->step_form == 2 || (p->step_form == 0 && (int64_t)g.nblk_f > (int64_t)nsm * per_sm_sw));
-    }
+    h->runk = h->ks->run[h->p.smooth_h > 0.0][force_index(g.tpp)];
+    CK(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, h->runk, kForceBlock, 0));
+    if (per_sm < 1 || nsm < 1)
+        return fail(h, MD_E_CUDA, "the run kernel does not fit the device");
+    per_sm = std::min(per_sm, kMaxRunBlocks / nsm);
+    const bool one_each = g.nblk_f <= nsm * per_sm;   // a block for every chunk
+    h->g.sweep = p->step_form == 2 || (p->step_form == 0 && !one_each && p->precision != MD_PREC_FP64 && g.tpp <= 2);
     // the build takes a warp per cell when there are at least kNbWarpCellsPerSm cells per SM
     // and a cell's particles fit one batch of lanes on average; a block per cell otherwise
     // (measured on GB300: LJ at 729 cells or fewer and dense cells of ~40 are faster with a
@@ -1031,6 +815,7 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
     h->g.nb_block = p->build_form == 2 ||
                     (p->build_form == 0 && ((int64_t)g.ncell < (int64_t)kNbWarpCellsPerSm * nsm ||
                                             (double)g.n > 32.0 * (double)g.ncell));
+    h->a.nb_block = h->g.nb_block ? 1 : 0;
     // pinned staging, events
     CK(h, cudaEventCreateWithFlags(&h->ev_stage, cudaEventDisableTiming));
     CK(h, cudaEventCreate(&h->ev_f0));
@@ -1052,13 +837,18 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
             return e == cudaSuccess ? MD_OK : cuda_fail(h, e, "table upload");
         };
         const std::vector<int4> bf = mdt::sm_block_order(g.blk_f, nsm, nsm * per_sm);
-        const std::vector<int4> bs =
-            mdt::step_table(bf, g.blk_f, h->g.sweep, nsm, per_sm_sw, h->g.nblk_s, h->g.cpb);
+        const std::vector<int4> br =
+            mdt::step_table(bf, g.blk_f, !one_each, nsm, per_sm, h->g.nwork, h->g.cpb);
         h->a.cpb = h->g.cpb;
+        h->a.nrow = (int)br.size();
+        h->a.nslot = g.R == 1 ? h->g.nwork : g.nblk_f;
+        // blocks without chunks, where the GPU holds more than there are chunks: they add up
+        // the steps' partial sums, a replica each
+        h->g.nblk_r = std::min(nsm * per_sm, h->g.nwork + std::min(g.R, nsm));
         if ((rc = put(L.off_rep, g.rep.data(), sizeof(mdk::Rep) * g.R)) ||
             (rc = put(L.off_blk_i, g.blk_i.data(), sizeof(int4) * g.nblk_i)) ||
             (rc = put(L.off_blk_f, bf.data(), sizeof(int4) * g.nblk_f)) ||
-            (rc = put(L.off_blk_s, bs.data(), sizeof(int4) * bs.size())) ||
+            (rc = put(L.off_blk_r, br.data(), sizeof(int4) * br.size())) ||
             (rc = put(L.off_crank, g.crank.data(), sizeof(int) * g.ncell)) ||
             (rc = put(L.off_cxyz, g.cxyz.data(), sizeof(int4) * g.ncell)))
             return rc;
@@ -1066,10 +856,13 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
         memset(&c0, 0, sizeof c0);
         c0.K = g.K;
         c0.Kmax = g.Kmax;
-        c0.epot_pending = -1;
         if ((rc = put(L.off_ctl, &c0, sizeof c0)))
             return rc;
         cudaError_t e = cudaMemsetAsync(a.ccount, 0, 4 * (size_t)g.ncell, h->s);
+        if (e == cudaSuccess)
+            e = cudaMemsetAsync(a.slice, 0, sizeof(int) * kMaxRunBlocks, h->s);
+        if (e == cudaSuccess)
+            e = cudaMemsetAsync(a.rs, 0, sizeof(mdk::RunSync), h->s);
         if (e == cudaSuccess)   // every slot of the per-step series empty (step -1)
             e = cudaMemsetAsync(a.epot_step, 0xff, sizeof(long long) * (size_t)h->cap, h->s);
         if (e == cudaSuccess)
@@ -1077,7 +870,7 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
         if (e != cudaSuccess)
             return cuda_fail(h, e, "initialisation");
     }
-    if ((rc = upload_state(h, species, pos, vel, image)) || (rc = launch_integrate(h, mdk::IM_SAMPLE)))
+    if ((rc = upload_state(h, species, pos, vel, image)))
         return rc;
     return check_device(h);
 }
@@ -1113,46 +906,31 @@ int md_step(md_handle *h, int64_t nsteps)
     if (nsteps < 1)
         return fail(h, MD_E_INVAL, "nsteps must be >= 1");
     int rc;
-    KArgs a = h->a;
-    a.nsteps = nsteps;
-    a.budget = h->p.step_budget;
-    if ((rc = launch(h, h->ks->set_steps, 1, 1, a)))
+    // bound on the steps executed (a device loop that could not end would hold the GPU)
+    const int64_t budget = h->p.step_budget > 0 ? h->p.step_budget : nsteps + 64;
+    if (h->p.use_graph)
+        return launch_run(h, mdk::RUN_FIRST | mdk::RUN_STEPS, nsteps, budget);
+    // The same phases as launches of their own, with their times.  At each check
+    // point the host reads the device's rebuild flag and launches the rebuild
+    // when it is set, so exactly the same work runs (results are bitwise equal).
+    if ((rc = launch_run(h, mdk::RUN_FIRST | mdk::RUN_DEFER)) || (rc = rebuild_if_flagged(h, nullptr)))
         return rc;
-    if (h->p.use_graph) {
-        if (!h->gexec && (rc = build_graph(h)))
+    const int ci = h->g.check;
+    for (int64_t k = 0; k < nsteps && k < budget; ++k) {
+        CK(h, cudaEventRecord(h->ev_f0, h->s));
+        if ((rc = launch_run(h, mdk::RUN_STEPS, 1, budget - k, (int)(k % ci), k == nsteps - 1)))
             return rc;
-        CK(h, cudaGraphLaunch(h->gexec, h->s));
-        return MD_OK;
-    }
-    // The graph's kernel sequence, launched from the host with per-kernel
-    // timing.  At each check point the host reads the device's rebuild flag
-    // and launches the rebuild chain only when the graph's IF node would run
-    // it, so exactly the same kernels execute (results are bitwise equal).
-    if ((rc = launch(h, h->ks->integrate, h->g.nblk_i, kIntBlock, first_args(h))) ||
-        (rc = rebuild_if_flagged(h, nullptr)))
-        return rc;
-    const void *stepk = step_kernel(h);
-    const int64_t iters = (nsteps + kUnroll - 1) / kUnroll;
-    for (int64_t it = 0; it < iters; ++it) {
-        for (int slot = 0; slot < kUnroll; ++slot) {
-            const KArgs sa = step_args(h, slot);
-            CK(h, cudaEventRecord(h->ev_f0, h->s));
-            if ((rc = launch(h, stepk, h->g.nblk_s, kForceBlock, sa)))
+        CK(h, cudaEventRecord(h->ev_f1, h->s));
+        CK(h, cudaEventSynchronize(h->ev_f1));
+        float ms = 0.f;
+        CK(h, cudaEventElapsedTime(&ms, h->ev_f0, h->ev_f1));
+        h->step_ms += ms;
+        h->step_launches += 1;
+        if (k % ci == ci - 1 && k < nsteps - 1) {
+            float mr = 0.f;
+            if ((rc = rebuild_if_flagged(h, &mr)))
                 return rc;
-            CK(h, cudaEventRecord(h->ev_f1, h->s));
-            CK(h, cudaEventSynchronize(h->ev_f1));
-            float ms = 0.f;
-            CK(h, cudaEventElapsedTime(&ms, h->ev_f0, h->ev_f1));
-            if (it * kUnroll + slot < nsteps) {
-                h->step_ms += ms;
-                h->step_launches += 1;
-            }
-            if (sa.set_rebuild) {
-                float mr = 0.f;
-                if ((rc = rebuild_if_flagged(h, &mr)))
-                    return rc;
-                h->rebuild_ms += mr;
-            }
+            h->rebuild_ms += mr;
         }
     }
     return MD_OK;
@@ -1172,7 +950,7 @@ int md_rescale_velocities(md_handle *h, const double *T_target)
     memcpy(h->pin, T_target, 8 * (size_t)h->g.R);
     CK(h, cudaMemcpyAsync(h->a.scale, h->pin, 8 * (size_t)h->g.R, cudaMemcpyHostToDevice, h->s));
     CK(h, cudaEventRecord(h->ev_stage, h->s));
-    if ((rc = launch_integrate(h, mdk::IM_KE)))
+    if ((rc = launch_kinetic(h, mdk::IM_KE)))
         return rc;
     return launch(h, h->ks->scale, h->g.nblk_i, kIntBlock, h->a);
 }
@@ -1214,7 +992,7 @@ int md_andersen(md_handle *h, const double *T_target, uint64_t seed, int64_t eve
     a.r48_CN = CN;
     a.r48_base = (long long)(4ull * (unsigned long long)event * n);
     if ((rc = launch(h, h->ks->andersen, h->g.nblk_i, kIntBlock, a)) ||
-        (rc = launch_integrate(h, mdk::IM_TOTALS)))
+        (rc = launch_kinetic(h, mdk::IM_TOTALS)))
         return rc;
     return launch(h, h->ks->andersen_fix, h->g.nblk_i, kIntBlock, h->a);
 }
@@ -1430,8 +1208,7 @@ int md_compute_forces(md_handle *h, double *f, double *e, md_obs *totals)
         return MD_E_INVAL;
     int rc;
     const size_t n = (size_t)h->g.n;
-    if ((rc = launch(h, h->ks->mark_rebuild, 1, 1, h->a)) || (rc = launch_rebuild(h)) ||
-        (rc = launch_force(h, 1)) || (rc = launch_integrate(h, mdk::IM_TOTALS)) ||
+    if ((rc = launch_run(h, mdk::RUN_REBUILD | mdk::RUN_TOTALS)) ||
         (rc = launch(h, h->ks->expforce, grid_n(h->g.n, kIntBlock), kIntBlock, h->a)))
         return rc;
     if ((rc = check_device(h)))
@@ -1496,11 +1273,9 @@ int md_epot_series(md_handle *h, int64_t *steps, double *e_pot, int32_t max_step
     if (!h || !n_steps || (max_steps > 0 && (!steps || !e_pot)))
         return MD_E_INVAL;
     *n_steps = 0;
-    int rc = flush_epot(h);
-    if (rc)
-        return rc;
     mdk::Ctl c;
-    if ((rc = read_ctl(h, &c)))
+    int rc = read_ctl(h, &c);
+    if (rc)
         return rc;
     const size_t cap = (size_t)h->cap, R = (size_t)h->g.R;
     const size_t sb = align_up(sizeof(long long) * cap);
@@ -1577,9 +1352,9 @@ int md_set_state(md_handle *h, const double *pos, const double *vel, const int32
     CK(h, cudaMemcpyAsync(h->a.st_vel, q + 24 * n, 24 * n, cudaMemcpyHostToDevice, h->s));
     CK(h, cudaMemcpyAsync(h->a.st_img, q + 48 * n, 12 * n, cudaMemcpyHostToDevice, h->s));
     CK(h, cudaEventRecord(h->ev_stage, h->s));
-    if ((rc = launch(h, h->ks->load, h->g.nblk_i, kIntBlock, h->a)) || (rc = launch_rebuild(h)))
+    if ((rc = launch(h, h->ks->load, h->g.nblk_i, kIntBlock, h->a)))
         return rc;
-    return launch_force(h, 1);
+    return launch_run(h, mdk::RUN_REBUILD | mdk::RUN_FORCES);
 }
 
 int md_get_neighbours(md_handle *h, int32_t *counts, int32_t *lists, int32_t kmax)
@@ -1637,7 +1412,7 @@ int md_info(md_handle *h, md_info_t *out)
     out->cells_per_edge = h->g.rep[0].nc;
     out->step = c.step;
     out->rebuilds = c.rebuilds;
-    out->kernel_launches = c.n_force + c.n_integrate + c.n_rebuild_k + c.n_other;
+    out->kernel_launches = c.n_kernels;
     out->max_neighbours = c.max_nbr;
     out->status = status_code(c.status);
     out->step_ms = h->step_ms;
@@ -1663,10 +1438,6 @@ int md_destroy(md_handle *h)
         return MD_E_INVAL;
     if (h->ws)
         cudaStreamSynchronize(h->s);
-    if (h->gexec)
-        cudaGraphExecDestroy(h->gexec);
-    if (h->graph)
-        cudaGraphDestroy(h->graph);
     if (h->pin)
         cudaFreeHost(h->pin);
     if (h->ev_stage)

@@ -13,12 +13,20 @@ enum { FP64 = 0, MIXED = 1, FP32 = 2 };
 // device status bits
 enum { ST_OVERFLOW = 1u, ST_NONFINITE = 2u, ST_UNSTABLE = 4u, ST_TIMEOUT = 8u, ST_BOUNDS = 16u };
 
-// integrate-kernel modes
+// what a launch of the run kernel does (KArgs::what)
 enum {
-    IM_FIRST = 0,   // half kick + drift (start of md_step)
-    IM_LOOP = 1,    // half kick, sample, then half kick + drift unless this is the last step
-    IM_SAMPLE = 2,  // kinetic reductions only; record a ring-buffer sample
-    IM_TOTALS = 3,  // kinetic reductions only; write the per-replica totals record
+    RUN_REBUILD = 1,   // rebuild the lists first, whatever the displacements
+    RUN_FIRST = 2,     // half kick and drift that open md_step (and the rebuild they call for)
+    RUN_STEPS = 4,     // KArgs::nsteps MD steps, with the rebuilds they call for
+    RUN_SAMPLE = 8,    // forces and reductions at the current positions into the sample ring ...
+    RUN_TOTALS = 16,   // ... or into the totals record; the state stays as it is
+    RUN_FORCES = 32,   // forces at the current positions, nothing recorded
+    RUN_DEFER = 64     // RUN_FIRST only notes a rebuild in Ctl::rebuild (stream launches)
+};
+
+// modes of the kinetic kernel
+enum {
+    IM_TOTALS = 3,  // kinetic energy and momentum into the per-replica totals record
     IM_KE = 4       // kinetic energy only; turn targets in scale[] into rescale factors
 };
 
@@ -30,33 +38,31 @@ constexpr float kDispMargin = 1e-4f;
 // Control block in device memory, written by the kernels.
 struct Ctl {
     unsigned int status;      // ST_* bits
-    unsigned int rebuild;     // 1: lists must be rebuilt before the next force evaluation
-    unsigned int maxdisp2;    // float bits of the largest squared displacement (this step)
-    unsigned int ticket;      // last-block counter of the step / integrate kernels
-    unsigned int maxv2;       // float bits of the largest squared speed (this step)
-    unsigned int maxa2;       // float bits of the largest squared acceleration (this step)
+    unsigned int rebuild;     // 1: the last check asked for a rebuild that has not run yet
+    unsigned int ticket;      // last-block counter of the kinetic kernel
     int pos_par;              // which of the two position buffers is current
     int state_par;            // which of the two velocity / image buffers is current
     int max_nbr;              // largest list length seen at the last build
     int K;                    // list entries per particle in use; grows on the device when a
                               // build finds a longer list, up to Kmax
     int Kmax;                 // capacity cap: the row stride of nbr (KArgs::Kstride)
-    unsigned int regrow;      // 1: the last build overflowed K; K was raised and the build
-                              // must be redone before the lists are used
     long long step;           // time index of the current positions
-    long long remaining;      // force evaluations left in the running md_step
-    long long budget;         // loop-iteration bound of the running md_step
     long long rebuilds;
     long long obs_count;      // samples written to the ring
-    long long n_force, n_integrate, n_rebuild_k, n_other;   // kernel executions
-    unsigned long long t_first_inv;   // step kernel: ~(earliest block start, %globaltimer ns) of the
-                                      // running launch (0 = none yet; atomicMax of the complement)
-    unsigned long long dev_ns;        // summed device duration of the step-kernel launches
-    long long dev_launches;
+    long long n_kernels;      // kernel executions
+    unsigned long long dev_ns;        // summed device duration of the MD steps of the run kernel
+    long long dev_launches;           // MD steps summed into dev_ns
     float last_maxdisp2;
     float pad1;
     long long regrows;        // builds redone with a larger K since md_create
-    long long epot_pending;   // a step whose warp energy partials still await their sum (-1: none)
+};
+
+// Grid barrier and shared decisions of the run kernel, each on a cache line of its own.
+struct RunSync {
+    unsigned int arrive, pad0[31];   // blocks that have reached the running barrier
+    unsigned int word, pad1[31];     // (barriers passed << 4) | what the last one decided (RunFlag)
+    unsigned int m[2][4], pad2[24];  // float bits of the largest squared displacement, speed and
+                                     // acceleration of a step, by the parity of the step
 };
 
 struct Rep {                  // one independent system
@@ -91,14 +97,15 @@ struct __align__(32) d4 { double x, y, z, w; };
 
 // Every kernel takes this one struct by value.
 struct KArgs {
-    int n, nrep, ncell, tpp, si, obs_cap, epot_cap, imode, use_cond, fsample;
+    int n, nrep, ncell, tpp, si, obs_cap, epot_cap, imode, what;
     int Kstride;                      // list row stride: the capacity cap (Ctl::Kmax); the rows hold
                                       // at most Ctl::K entries, so K can grow without a new layout
     int nblk_i, nblk_f;
-    int lookahead;                    // MD steps until the next rebuild check (after this node)
-    int set_rebuild, set_loop;        // this graph node sets the rebuild / loop condition
-    int nb_retry;                     // neighbour build: 0 = first pass, 1 = the redo after a regrow
-    int set_regrow;                   // this build node sets the regrow condition
+    int check;                        // MD steps between rebuild checks
+    int pos0;                         // position of the first step of this launch in its md_step
+    int last;                         // this launch ends its md_step
+    int nb_block;                     // neighbour build: a block per cell (else a warp per cell)
+    int nslot, nrow;                  // slots of the partial sums (per parity), rows of blk_r
     void *pa, *pb, *va, *vb;          // buffer 0: MIXED pos hi/lo, vel hi/lo (float4);
                                       // FP64 pos, vel (d4); FP32 pos, vel (float4)
     void *pa2, *pb2, *va2, *vb2;      // buffer 1 (positions: Ctl::pos_par, velocities: state_par)
@@ -114,16 +121,18 @@ struct KArgs {
     int *nbr, *nnbr;
     const int4 *blk_i, *blk_f;        // per block: first particle, end, replica (blk_f: + its
                                       // chunk index, the slot of its partial sums)
-    const int4 *blk_s;                // step kernel: rows of blk_f in the order the resident blocks
-                                      // take them, cpb per block (w = -1: padding)
-    int cpb;                          // step kernel: chunks per block
-    double *part_f, *part_i;          // per-block partial sums [nblk_f][12], [nblk_i][4]
-    void *part_e;                     // per-block potential energy [nblk_f]: double (FP64 mode) or
-                                      // float2 double-single (MIXED, FP32)
+    const int4 *blk_r;                // run kernel: rows of blk_f in the order its blocks take them,
+                                      // cpb per block (w = -1: padding)
+    int cpb;                          // run kernel: chunks per block
+    int *slice;                       // run kernel: particles in each block's slice of the cells
+    double *part_f, *part_i;          // partial sums [2][nslot][12], [nblk_i][4]
+    void *part_e;                     // potential energy [2][nslot]: double (FP64 mode) or float2
+                                      // double-single (MIXED, FP32)
     Obs *ring, *totals;
     double *epot;                     // per-step potential energy [epot_cap][nrep], slot = step % cap
     long long *epot_step;             // [epot_cap]: the step held by each slot (-1 = none)
     Ctl *ctl;
+    RunSync *rs;
     const Rep *rep;
     double *st_pos, *st_vel, *st_f, *st_e;   // staging, original order
     int *st_img, *st_code;
@@ -135,11 +144,10 @@ struct KArgs {
     int *snap_species;                //   species, both by original particle index
     PairTab tab;
     double hdtm[2], dt, mass[2];      // dt / (2 m_a), dt, m_a
-    long long nsteps;                 // for k_set_steps
+    long long nsteps;                 // run kernel: MD steps of this launch
     float hdtm_hi[2], hdtm_lo[2], dt_hi, dt_lo, inv_mass[2];
     float disp_thr2, disp_thr;        // (skin/2 - margin)^2 and skin/2 - margin
-    long long budget;                 // for k_set_steps: step-loop bound (0 = nsteps + 64)
-    cudaGraphConditionalHandle h_loop, h_rebuild, h_regrow;
+    long long budget;                 // run kernel: bound on the steps of this launch
 };
 
 // ---------------------------------------------------------------------------
@@ -198,12 +206,9 @@ __device__ __forceinline__ ds ds_from_double(double x)
 
 // table of kernel entry addresses for one precision (one translation unit each)
 struct KernelSet {
-    const void *integrate, *force[2][6], *step[2][6];   // [smoothed][log2 lanes per particle]
-    const void *step_sweep[2][2];     // step kernel, resident blocks sweeping runs of chunks
-                                      // (single-precision pair loops, 1 or 2 lanes; else null)
-    const void *bin, *scan, *scatter, *permute, *nbuild, *nbuild_blk;
-    const void *load, *getstate, *expforce, *scale, *set_steps, *reset, *mark_rebuild;
-    const void *andersen, *andersen_fix, *snapshot, *epot_flush;
+    const void *run[2][6];            // [smoothed][log2 lanes per particle]
+    const void *kinetic, *load, *getstate, *expforce, *scale, *reset;
+    const void *andersen, *andersen_fix, *snapshot;
 };
 
 const KernelSet &kernels_fp64();

@@ -33,11 +33,8 @@ namespace mdk {
 
 constexpr int kIntBlock = 256;   // per-particle kernels: one thread per particle
 constexpr int kForceBlock = 128; // force / step kernels: tpp threads per particle
-constexpr int kNbCells = 4;      // neighbour build, warp per cell: cells per block
-constexpr int kNbBlock = 32 * kNbCells;
-constexpr int kNbBlockB = 256;   // neighbour build, block per cell: threads per block
-constexpr int kScanBlock = 1024;
-constexpr int kScanPer = 8;      // cell counts per thread and tile of the scan
+constexpr int kNbCells = kForceBlock / 32;   // neighbour build, warp per cell: cells per block
+constexpr int kNbBlockB = kForceBlock;   // neighbour build, block per cell: threads per block
 constexpr int kPartF = 12;       // doubles per block partial of the force / step kernels
 constexpr int kUnr = 8;          // list entries per lane and iteration of the FP32 pair loops
                                  // (a multiple of 4, at most 8: lists are padded to 8)
@@ -269,6 +266,33 @@ __device__ __forceinline__ unsigned int fixq(float H, float l, const Rep &rp)
 __device__ __forceinline__ float sep_q(unsigned int qi, unsigned int qj, float unit)
 {
     return __int2float_rn((int)(qi - qj)) * unit;
+}
+
+// two at a time
+__device__ __forceinline__ float2 sep_q2(int qi, int qa, int qb, float unit)
+{
+    return __fmul2_rn(make_float2(__int2float_rn((int)((unsigned int)qi - (unsigned int)qa)),
+                                  __int2float_rn((int)((unsigned int)qi - (unsigned int)qb))),
+                      make_float2(unit, unit));
+}
+
+// minimum-image separations of one coordinate from two others (FP32 mode): the
+// rounding to a whole number of boxes adds and takes away 1.5 2^23
+__device__ __forceinline__ float2 sep_f2(float xi, float2 xj, float L, float invL)
+{
+    const float2 d = __fadd2_rn(make_float2(xi, xi), make_float2(-xj.x, -xj.y));
+    const float2 big = make_float2(12582912.0f, 12582912.0f);
+    const float2 t = __ffma2_rn(d, make_float2(invL, invL), big);
+    const float2 k = __fadd2_rn(t, make_float2(-12582912.0f, -12582912.0f));
+    return __ffma2_rn(k, make_float2(-L, -L), d);
+}
+
+// reciprocal of a normal number by the hardware's approximation (1 ulp)
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
 }
 
 __device__ __forceinline__ int4 *q_of(const KArgs &a, int par) { return par ? a.qb : a.qa; }
@@ -529,47 +553,18 @@ __device__ __forceinline__ float drift(const KArgs &a, const Rep &rp, PState<P> 
 }
 
 // ---------------------------------------------------------------------------
-// reductions finished by the last block of a step / integrate kernel
+// Per-step reductions.  Every block of the run kernel leaves one partial per
+// slot: the potential energy of the step (part_e: double in FP64 mode,
+// double-single elsewhere, so that the every-step sum costs no FP64 arithmetic
+// in the single-precision modes) and, on sample steps, the virial, kinetic and
+// momentum sums (part_f).  A slot is a block for a handle of one replica and a
+// chunk otherwise (a block may hold chunks of several replicas).  Two sets, by
+// the parity of the step, so that one block can add up a step's partials while
+// the others already write the next step's.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void write_record(const KArgs &a, int mode, int r, const double *v, long long step,
-                                             float md2, long long rebuilds, long long slot)
+__device__ __forceinline__ size_t part_index(const KArgs &a, long long step, int slot)
 {
-    Obs o;
-    o.step = step;
-    o.e_pot = v[0];
-    o.virial = v[1];
-    for (int k = 0; k < 6; ++k)
-        o.w[k] = v[2 + k];
-    o.e_kin = v[8];
-    o.p[0] = v[9];
-    o.p[1] = v[10];
-    o.p[2] = v[11];
-    o.max_disp = sqrt((double)md2);
-    o.rebuilds = rebuilds;
-    if (mode == IM_LOOP || mode == IM_SAMPLE)
-        a.epot[(step % a.epot_cap) * a.nrep + r] = v[0];
-    if (mode == IM_TOTALS)
-        a.totals[r] = o;
-    else if (mode == IM_KE) {
-        const Rep &rp = a.rep[r];
-        double dof = 3.0 * (double)rp.n - 3.0;
-        double target = a.scale[r];
-        a.scale[r] = (v[8] > 0.0) ? sqrt(target * dof / (2.0 * v[8])) : 1.0;
-    } else
-        a.ring[slot * a.nrep + r] = o;
-}
-
-// Potential-energy partial sums, one per warp of the force / step kernels
-// (part_e): double in FP64 mode, double-single elsewhere, so that the every-
-// step energy reduction costs no FP64 arithmetic in the single-precision
-// modes.  Two sets, by the parity of the step the energies belong to, so that
-// a step's partials survive the next step until they are added up.
-constexpr int kWarpsF = kForceBlock / 32;
-
-template <int P>
-__device__ __forceinline__ size_t epart_index(const KArgs &a, long long step, int chunk, int warp)
-{
-    return (size_t)(step & 1) * (size_t)a.nblk_f * kWarpsF + (size_t)chunk * kWarpsF + warp;
+    return (size_t)(step & 1) * (size_t)a.nslot + (size_t)slot;
 }
 
 template <int P>
@@ -595,149 +590,65 @@ __device__ __forceinline__ ET<P> get_epart(const KArgs &a, size_t k)
 __device__ __forceinline__ double e_add(double x, double y) { return x + y; }
 __device__ __forceinline__ ds e_add(ds x, ds y) { return ds_add(x, y); }
 
-__device__ __forceinline__ double e_warp_sum(double e) { return warp_sum(e); }
-__device__ __forceinline__ ds e_warp_sum(ds e)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        e = ds_add(e, ds_from(__shfl_xor_sync(0xffffffffu, e.hi, o), __shfl_xor_sync(0xffffffffu, e.lo, o)));
-    return e;
-}
-
-// The warp's energy sum into its partial of step `step`.  Every lane of the
-// warp calls it (the sum is a full-warp shuffle); lane 0 writes if `write`.
+// The reductions of replica r at `step` from its slots' partials, by one whole
+// block, in a fixed order (thread t adds partials t, t + blockDim, ..., then the
+// block's tree): the potential energy into the per-step series and, for a
+// sample, the record into the ring or (totals) into the totals array.
 template <int P>
-__device__ __forceinline__ void store_warp_energy(const KArgs &a, long long step, int chunk, ET<P> e, bool write)
+__device__ void finish_replica(const KArgs &a, int r, long long step, bool sample, bool totals, long long slot,
+                               float md2, long long rebuilds, double *sh, float *shf)
 {
-    e = e_warp_sum(e);
-    if ((threadIdx.x & 31) == 0 && write)
-        put_epart<P>(a, epart_index<P>(a, step, chunk, threadIdx.x >> 5), e);
-}
-
-// Potential energy of one replica at `step` from its warps' partials, by the
-// whole block: thread t adds partials p0 + t, p0 + t + blockDim, ... in that
-// order (eight loads in flight), then the threads' sums are added in a fixed
-// tree.  Valid in thread 0.  Every thread of the block must call it.
-template <int P>
-__device__ double epot_sum_block(const KArgs &a, const Rep &rp, long long step, float *shf, double *sh)
-{
-    ET<P> v = e_zero<P>();
-    const int stride = blockDim.x;
-    const size_t base = epart_index<P>(a, step, 0, 0);
-    int b = rp.bf0 * kWarpsF + threadIdx.x;
-    const int end = rp.bf1 * kWarpsF;
-    for (; b + 7 * stride < end; b += 8 * stride) {
+    const int s0 = a.nrep == 1 ? 0 : a.rep[r].bf0, s1 = a.nrep == 1 ? a.nslot : a.rep[r].bf1;
+    ET<P> e = e_zero<P>();
+    int b = s0 + threadIdx.x;
+    const int st = blockDim.x;
+    for (; b + 7 * st < s1; b += 8 * st) {
         ET<P> x[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-            x[u] = get_epart<P>(a, base + b + u * stride);
+            x[u] = get_epart<P>(a, part_index(a, step, b + u * st));
 #pragma unroll
         for (int u = 0; u < 8; ++u)
-            v = e_add(v, x[u]);
+            e = e_add(e, x[u]);
     }
-    for (; b < end; b += stride)
-        v = e_add(v, get_epart<P>(a, base + b));
+    for (; b < s1; b += st)
+        e = e_add(e, get_epart<P>(a, part_index(a, step, b)));
     float d0 = 0.f, d1 = 0.f, d2 = 0.f;
-    block_max3_sum1(d0, d1, d2, v, shf, sh);
-    return e_value(v);
-}
-
-// The same by one thread, for handles with many replicas (one thread each).
-template <int P>
-__device__ double epot_sum_seq(const KArgs &a, const Rep &rp, long long step)
-{
-    ET<P> v = e_zero<P>();
-    const size_t base = epart_index<P>(a, step, 0, 0);
-    for (int b = rp.bf0 * kWarpsF; b < rp.bf1 * kWarpsF; ++b)
-        v = e_add(v, get_epart<P>(a, base + b));
-    return e_value(v);
-}
-
-// Per-replica sums of the block partials, in a fixed order (deterministic).
-// Potential-side values come from part_f[.][1..7] and the energy sums
-// part_e; kinetic values from part_f[.][8..11] (step kernel, from_f = true)
-// or part_i[.][0..3].
-template <int P>
-__device__ void finish_reductions(const KArgs &a, int mode, bool from_f, long long step, float md2, double *sh,
-                                  float *shf)
-{
-    const Ctl *ctl = a.ctl;
-    const long long slot = ctl->obs_count % (long long)a.obs_cap;
-    const long long rebuilds = ctl->rebuilds;
-    const bool want_f = mode != IM_KE;
-    if (a.nrep <= 8) {
-        for (int r = 0; r < a.nrep; ++r) {
-            const Rep rp = a.rep[r];
-            double v[12];
+    block_max3_sum1(d0, d1, d2, e, shf, sh);
+    const double epot = e_value(e);
+    if (threadIdx.x == 0 && !totals)
+        a.epot[(step % a.epot_cap) * a.nrep + r] = epot;
+    if (!sample)
+        return;
+    double v[kPartF];
 #pragma unroll
-            for (int k = 0; k < 12; ++k)
-                v[k] = 0.0;
-            if (want_f || from_f)
-                for (int b = rp.bf0 + threadIdx.x; b < rp.bf1; b += blockDim.x)
+    for (int k = 0; k < kPartF; ++k)
+        v[k] = 0.0;
+    for (int b2 = s0 + threadIdx.x; b2 < s1; b2 += st) {
+        const double *p = a.part_f + part_index(a, step, b2) * kPartF;
 #pragma unroll
-                    for (int k = 1; k < kPartF; ++k)
-                        v[k] += a.part_f[(size_t)b * kPartF + k];
-            if (!from_f) {
-#pragma unroll
-                for (int k = 8; k < 12; ++k)
-                    v[k] = 0.0;
-                for (int b = rp.bi0 + threadIdx.x; b < rp.bi1; b += blockDim.x)
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        v[8 + k] += a.part_i[(size_t)b * 4 + k];
-            }
-            block_sum<12>(v, sh);
-            const double e = want_f ? epot_sum_block<P>(a, rp, step, shf, sh) : 0.0;
-            if (threadIdx.x == 0) {
-                v[0] = e;
-                write_record(a, mode, r, v, step, md2, rebuilds, slot);
-            }
-        }
-    } else {
-        for (int r = threadIdx.x; r < a.nrep; r += blockDim.x) {
-            const Rep rp = a.rep[r];
-            double v[12];
-            for (int k = 0; k < 12; ++k)
-                v[k] = 0.0;
-            if (want_f || from_f)
-                for (int b = rp.bf0; b < rp.bf1; ++b)
-                    for (int k = 1; k < kPartF; ++k)
-                        v[k] += a.part_f[(size_t)b * kPartF + k];
-            if (!from_f) {
-                for (int k = 8; k < 12; ++k)
-                    v[k] = 0.0;
-                for (int b = rp.bi0; b < rp.bi1; ++b)
-                    for (int k = 0; k < 4; ++k)
-                        v[8 + k] += a.part_i[(size_t)b * 4 + k];
-            }
-            if (want_f)
-                v[0] = epot_sum_seq<P>(a, rp, step);
-            write_record(a, mode, r, v, step, md2, rebuilds, slot);
-        }
-        __syncthreads();
+        for (int k = 1; k < kPartF; ++k)
+            v[k] += p[k];
     }
-}
-
-// The potential energy of every replica at `step` (a step that recorded no
-// sample) into the per-step series: the same sums as finish_reductions takes.
-// Run by one whole block.
-template <int P>
-__device__ void finish_epot(const KArgs &a, long long step, double *sh, float *shf)
-{
-    const long long slot = step % a.epot_cap;
-    if (a.nrep <= 8) {
-        for (int r = 0; r < a.nrep; ++r) {
-            const double e = epot_sum_block<P>(a, a.rep[r], step, shf, sh);
-            if (threadIdx.x == 0)
-                a.epot[slot * a.nrep + r] = e;
-        }
-    } else {
-        for (int r = threadIdx.x; r < a.nrep; r += blockDim.x)
-            a.epot[slot * a.nrep + r] = epot_sum_seq<P>(a, a.rep[r], step);
-        __syncthreads();
+    block_sum<kPartF>(v, sh);
+    if (threadIdx.x == 0) {
+        Obs o;
+        o.step = step;
+        o.e_pot = epot;
+        o.virial = v[1];
+        for (int k = 0; k < 6; ++k)
+            o.w[k] = v[2 + k];
+        o.e_kin = v[8];
+        o.p[0] = v[9];
+        o.p[1] = v[10];
+        o.p[2] = v[11];
+        o.max_disp = sqrt((double)md2);
+        o.rebuilds = rebuilds;
+        if (totals)
+            a.totals[r] = o;
+        else
+            a.ring[slot * a.nrep + r] = o;
     }
-    if (threadIdx.x == 0)
-        a.epot_step[slot] = step;
 }
 
 // Rebuild decision: the list built at the last rebuild holds every pair
@@ -745,12 +656,11 @@ __device__ void finish_epot(const KArgs &a, long long step, double *sh, float *s
 // than skin/2.  The next check comes after `look` further drifts, each at
 // most dt (v + look dt a) per particle: rebuild now if the largest
 // displacement plus that bound could exceed skin/2 (with a rounding margin).
-__device__ __forceinline__ unsigned int need_rebuild(const KArgs &a, float md2, float mv2, float ma2)
+__device__ __forceinline__ bool need_rebuild(const KArgs &a, int lookahead, float md2, float mv2, float ma2)
 {
-    const float ahead = (float)a.lookahead * (float)a.dt * (sqrtf(mv2) + 2.0f * (float)a.lookahead *
-                                                                              (float)a.dt * sqrtf(ma2));
-    const float d = sqrtf(md2) + ahead;
-    return d > a.disp_thr ? 1u : 0u;
+    const float look = (float)lookahead * (float)a.dt;
+    const float d = sqrtf(md2) + look * (sqrtf(mv2) + 2.0f * look * sqrtf(ma2));
+    return d > a.disp_thr;
 }
 
 // ---------------------------------------------------------------------------
@@ -800,7 +710,7 @@ __device__ __forceinline__ void pair_forces(const KArgs &a, const Rep &rp, int p
         }
         double sx = 0, sy = 0, sz = 0, se = 0;          // se: sum of 12 V
         for (int k0 = 4 * lane; k0 < nn; k0 += 4 * TPP) {
-            const int4 q = __ldg((const int4 *)(lst + k0));
+            const int4 q = *(const int4 *)(lst + k0);
             const int jj[4] = {q.x, q.y, q.z, q.w};
             d4 xs[4];
 #pragma unroll
@@ -855,17 +765,13 @@ __device__ __forceinline__ void pair_forces(const KArgs &a, const Rep &rp, int p
             Hi = pos[ii];
             ti = species_of(Hi.w);
         }
-        PairRow<float> pr;
+        float rc2[2], sig2[2], eps48[2], vc[2];
 #pragma unroll
         for (int tj = 0; tj < 2; ++tj) {
-            pr.rc2[tj] = a.tab.rc2[ti * 2 + tj];
-            pr.sig2[tj] = a.tab.sig2[ti * 2 + tj];
-            pr.eps4[tj] = a.tab.eps4[ti * 2 + tj];
-            pr.eps48[tj] = a.tab.eps48[ti * 2 + tj];
-            pr.shift[tj] = a.tab.shift[ti * 2 + tj];
-            pr.rc[tj] = a.tab.rc[ti * 2 + tj];
-            pr.ihs[tj] = a.tab.ihs[ti * 2 + tj];
-            pr.c[tj] = a.tab.vc[ti * 2 + tj];
+            rc2[tj] = a.tab.rc2[ti * 2 + tj];
+            sig2[tj] = a.tab.sig2[ti * 2 + tj];
+            eps48[tj] = a.tab.eps48[ti * 2 + tj];
+            vc[tj] = a.tab.vc[ti * 2 + tj];
         }
         // the energy is accumulated as 12 V = eps48_ab (s6^2 - s6 - c_ab), c_ab = S_ab / (4 eps_ab):
         // eps48, masked by the cutoff test, serves the force and the energy alike
@@ -880,7 +786,7 @@ __device__ __forceinline__ void pair_forces(const KArgs &a, const Rep &rp, int p
 #pragma unroll
             for (int w = 0; w < kUnr / 4; ++w) {
                 const int k = kUnr * lane + d * kStride;
-                pf[d][w] = k < nn ? __ldg((const int4 *)(lst + k + 4 * w)) : make_int4(0, 0, 0, 0);
+                pf[d][w] = k < nn ? *(const int4 *)(lst + k + 4 * w) : make_int4(0, 0, 0, 0);
             }
         for (int k0 = kUnr * lane; k0 < nn; k0 += kStride) {
             int jj[kUnr];
@@ -900,7 +806,7 @@ __device__ __forceinline__ void pair_forces(const KArgs &a, const Rep &rp, int p
             if (k0 + kPfDepth * kStride < nn)
 #pragma unroll
                 for (int w = 0; w < kUnr / 4; ++w)
-                    pf[kPfDepth - 1][w] = __ldg((const int4 *)(lst + k0 + kPfDepth * kStride + 4 * w));
+                    pf[kPfDepth - 1][w] = *(const int4 *)(lst + k0 + kPfDepth * kStride + 4 * w);
             float4 Hs[kUnr];
             int4 Qs[kUnr];
 #pragma unroll
@@ -908,50 +814,63 @@ __device__ __forceinline__ void pair_forces(const KArgs &a, const Rep &rp, int p
                 // rows are padded with the particle itself up to a multiple of kUnr
                 const int j = checked(a, jj[u], a.n, ii);
                 if constexpr (P == MIXED)
-                    Qs[u] = __ldg(qp + j);
+                    Qs[u] = qp[j];
                 else
-                    Hs[u] = __ldg(pos + j);
+                    Hs[u] = pos[j];
             }
+            // two entries at a time: the single-precision arithmetic of a pair of
+            // entries is one packed instruction each
             float gx = 0.f, gy = 0.f, gz = 0.f, gv = 0.f;
 #pragma unroll
-            for (int u = 0; u < kUnr; ++u) {
-                int tj;
-                float dx, dy, dz;
+            for (int u = 0; u < kUnr; u += 2) {
+                float2 dx, dy, dz;
+                bool bj[2];
                 if constexpr (P == MIXED) {
-                    const int4 Qj = Qs[u];
-                    tj = Qj.w;
-                    dx = sep_q(Qi.x, Qj.x, rp.qunit);
-                    dy = sep_q(Qi.y, Qj.y, rp.qunit);
-                    dz = sep_q(Qi.z, Qj.z, rp.qunit);
+                    dx = sep_q2(Qi.x, Qs[u].x, Qs[u + 1].x, rp.qunit);
+                    dy = sep_q2(Qi.y, Qs[u].y, Qs[u + 1].y, rp.qunit);
+                    dz = sep_q2(Qi.z, Qs[u].z, Qs[u + 1].z, rp.qunit);
+                    bj[0] = Qs[u].w != 0;
+                    bj[1] = Qs[u + 1].w != 0;
                 } else {
-                    const float4 Hj = Hs[u];
-                    tj = species_of(Hj.w);
-                    dx = sep_f(Hi.x, Hj.x, rp.Lhi, rp.invLf);
-                    dy = sep_f(Hi.y, Hj.y, rp.Lhi, rp.invLf);
-                    dz = sep_f(Hi.z, Hj.z, rp.Lhi, rp.invLf);
+                    dx = sep_f2(Hi.x, make_float2(Hs[u].x, Hs[u + 1].x), rp.Lhi, rp.invLf);
+                    dy = sep_f2(Hi.y, make_float2(Hs[u].y, Hs[u + 1].y), rp.Lhi, rp.invLf);
+                    dz = sep_f2(Hi.z, make_float2(Hs[u].z, Hs[u + 1].z), rp.Lhi, rp.invLf);
+                    bj[0] = species_of(Hs[u].w) != 0;
+                    bj[1] = species_of(Hs[u + 1].w) != 0;
                 }
-                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+                const float rca = bj[0] ? rc2[1] : rc2[0], rcb = bj[1] ? rc2[1] : rc2[0];
                 // (the particle itself, r2 = 0 exactly, is never inside)
-                const bool in = r2 > 0.0f && r2 < (tj ? pr.rc2[1] : pr.rc2[0]);
-                const float sig2 = tj ? pr.sig2[1] : pr.sig2[0];
-                const float e48 = in ? (tj ? pr.eps48[1] : pr.eps48[0]) : 0.0f;
-                const float ir2 = __fdividef(1.0f, in ? r2 : 1.0f);
-                const float s2 = sig2 * ir2;
-                const float s6 = s2 * s2 * s2;
-                float fr = e48 * ir2 * s6 * (s6 - 0.5f);
+                const bool ina = r2.x > 0.0f && r2.x < rca, inb = r2.y > 0.0f && r2.y < rcb;
+                const float2 sg = make_float2(bj[0] ? sig2[1] : sig2[0], bj[1] ? sig2[1] : sig2[0]);
+                const float2 e48 = make_float2(ina ? (bj[0] ? eps48[1] : eps48[0]) : 0.0f,
+                                               inb ? (bj[1] ? eps48[1] : eps48[0]) : 0.0f);
+                const float2 ir2 = make_float2(rcp_approx(ina ? r2.x : rca), rcp_approx(inb ? r2.y : rcb));
+                const float2 s2 = __fmul2_rn(sg, ir2);
+                const float2 s6 = __fmul2_rn(__fmul2_rn(s2, s2), s2);
+                float2 fr = __fmul2_rn(__fmul2_rn(__fmul2_rn(e48, ir2), s6),
+                                       __fadd2_rn(s6, make_float2(-0.5f, -0.5f)));
                 if (SM) {
-                    const float eps4 = tj ? pr.eps4[1] : pr.eps4[0];
-                    const float shift = tj ? pr.shift[1] : pr.shift[0];
-                    float v = in ? fmaf(eps4, s6 * s6 - s6, -shift) : 0.0f;
-                    smooth_pair(in ? r2 : 1.0f, tj ? pr.rc[1] : pr.rc[0], tj ? pr.ihs[1] : pr.ihs[0], fr, v);
-                    gv = fmaf(12.0f, v, gv);
+                    float fs[2] = {fr.x, fr.y}, vs[2];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const bool in = h ? inb : ina;
+                        const int ab = ti * 2 + (bj[h] ? 1 : 0);
+                        const float q6 = h ? s6.y : s6.x, rr = h ? (inb ? r2.y : rcb) : (ina ? r2.x : rca);
+                        vs[h] = in ? fmaf(a.tab.eps4[ab], q6 * q6 - q6, -a.tab.shift[ab]) : 0.0f;
+                        smooth_pair(rr, a.tab.rc[ab], a.tab.ihs[ab], fs[h], vs[h]);
+                    }
+                    fr = make_float2(fs[0], fs[1]);
+                    gv = fmaf(12.0f, vs[1], fmaf(12.0f, vs[0], gv));
                 } else {
-                    const float c = tj ? pr.c[1] : pr.c[0];
-                    gv = fmaf(e48, fmaf(s6, s6, -(s6 + c)), gv);
+                    const float2 c = make_float2(bj[0] ? vc[1] : vc[0], bj[1] ? vc[1] : vc[0]);
+                    const float2 t = __fadd2_rn(s6, c);
+                    const float2 w = __ffma2_rn(s6, s6, make_float2(-t.x, -t.y));
+                    gv = fmaf(e48.y, w.y, fmaf(e48.x, w.x, gv));
                 }
-                gx = fmaf(fr, dx, gx);
-                gy = fmaf(fr, dy, gy);
-                gz = fmaf(fr, dz, gz);
+                gx = fmaf(fr.y, dx.y, fmaf(fr.x, dx.x, gx));
+                gy = fmaf(fr.y, dy.y, fmaf(fr.x, dy.x, gy));
+                gz = fmaf(fr.y, dz.y, fmaf(fr.x, dz.x, gz));
             }
             if constexpr (P == MIXED) {
                 kahan_add(sx, cx, gx);
@@ -1011,7 +930,7 @@ __device__ __forceinline__ void pair_virial(const KArgs &a, const Rep &rp, int p
         const d4 xi = pos[ii];
         const int ti = species_of(xi.w);
         for (int k = lane; k < nn; k += TPP) {
-            const d4 xj = pos[checked(a, __ldg(lst + k), a.n, ii)];
+            const d4 xj = pos[checked(a, lst[k], a.n, ii)];
             const int ab = ti * 2 + species_of(xj.w);
             const double dx = sep_d(xi.x, xj.x, rp.L, rp.invL);
             const double dy = sep_d(xi.y, xj.y, rp.L, rp.invL);
@@ -1045,17 +964,17 @@ __device__ __forceinline__ void pair_virial(const KArgs &a, const Rep &rp, int p
             ti = species_of(Hi.w);
         }
         for (int k = lane; k < nn; k += TPP) {
-            const int j = checked(a, __ldg(lst + k), a.n, ii);
+            const int j = checked(a, lst[k], a.n, ii);
             float dx, dy, dz;
             int ab;
             if constexpr (P == MIXED) {
-                const int4 Qj = __ldg(qp + j);
+                const int4 Qj = qp[j];
                 ab = ti * 2 + Qj.w;
                 dx = sep_q(Qi.x, Qj.x, rp.qunit);
                 dy = sep_q(Qi.y, Qj.y, rp.qunit);
                 dz = sep_q(Qi.z, Qj.z, rp.qunit);
             } else {
-                const float4 Hj = __ldg(pos + j);
+                const float4 Hj = pos[j];
                 ab = ti * 2 + species_of(Hj.w);
                 dx = sep_f(Hi.x, Hj.x, rp.Lhi, rp.invLf);
                 dy = sep_f(Hi.y, Hj.y, rp.Lhi, rp.invLf);
@@ -1100,70 +1019,11 @@ __device__ __forceinline__ void store_force(const KArgs &a, int i, FT<P> fx, FT<
 }
 
 // ---------------------------------------------------------------------------
-// k_force: forces (and on request the potential-side reductions) at the
-// current positions; used when a handle is created or its state replaced and
-// by md_compute_forces.
-// ---------------------------------------------------------------------------
-template <int P, int TPP, bool SAMPLE, bool SM>
-__device__ __forceinline__ void force_only(const KArgs &a)
-{
-    __shared__ double sh[32 * kPartF];
-    const Ctl *ctl = a.ctl;
-    const int pp = ctl->pos_par;
-    const int4 b = a.blk_f[blockIdx.x];
-    const Rep rp = a.rep[b.z];
-    const int lane = threadIdx.x & (TPP - 1);
-    const int i = b.x + (int)(threadIdx.x / TPP);
-    const bool valid = i < b.y;
-    const int ii = valid ? i : b.x;
-    const int nn = valid ? a.nnbr[ii] : 0;
-    FT<P> fx, fy, fz;
-    ET<P> ep;
-    double acc[kPartF];
-#pragma unroll
-    for (int k = 0; k < kPartF; ++k)
-        acc[k] = 0.0;
-    pair_forces<P, TPP, SM>(a, rp, pp, ii, nn, fx, fy, fz, ep);
-    acc[0] = e_value(ep);
-    if (SAMPLE)
-        pair_virial<P, TPP, SM>(a, rp, pp, ii, nn, acc);
-    if (!(valid && lane == 0)) {
-#pragma unroll
-        for (int k = 0; k < kPartF; ++k)
-            acc[k] = 0.0;
-    }
-    if (valid && lane == 0)
-        store_force<P>(a, i, fx, fy, fz, ep);
-    if (SAMPLE) {
-        store_warp_energy<P>(a, ctl->step, b.w, (valid && lane == 0) ? ep : e_zero<P>(), true);
-        block_sum<kPartF>(acc, sh);
-        if (threadIdx.x == 0)
-#pragma unroll
-            for (int k = 0; k < kPartF; ++k)
-                a.part_f[(size_t)b.w * kPartF + k] = acc[k];
-    }
-}
-
-template <int P, int TPP, bool SM>
-__global__ void __launch_bounds__(kForceBlock) k_force(KArgs a)
-{
-    const Ctl *ctl = a.ctl;
-    if (ctl->status)
-        return;
-    if (blockIdx.x == 0 && threadIdx.x == 0)
-        atomicAdd((unsigned long long *)&a.ctl->n_force, 1ull);
-    if (a.fsample || (ctl->step % a.si) == 0)
-        force_only<P, TPP, true, SM>(a);
-    else
-        force_only<P, TPP, false, SM>(a);
-}
-
-// ---------------------------------------------------------------------------
-// k_step: one whole MD step.  Positions r(t) (current buffer), forces f(t)
-// from the list, then per particle: v(t) = v(t-1/2) + dt/2m f(t) [sample],
+// One MD step of a chunk of particles.  Positions r(t) (current buffer), forces
+// f(t) from the list, then per particle: v(t) = v(t-1/2) + dt/2m f(t) [sample],
 // and unless this is the last step of md_step: v(t+1/2) = v(t) + dt/2m f(t),
-// r(t+1) = r(t) + dt v(t+1/2) into the other buffer.  Last block: step
-// counter, buffer flip, sample record, rebuild decision, graph conditions.
+// r(t+1) = r(t) + dt v(t+1/2) into the other buffer.  Without `kick` the forces
+// and reductions alone, the state left as it is.
 // ---------------------------------------------------------------------------
 // One Cartesian component of the velocity-Verlet update, done by lane c of
 // the particle's group: half kick(s), drift, re-anchor / wrap, displacement
@@ -1171,14 +1031,16 @@ __global__ void __launch_bounds__(kForceBlock) k_force(KArgs a)
 // alone otherwise); returns the squared displacement component.
 template <int P>
 __device__ __forceinline__ void component_update(const KArgs &a, const Rep &rp, int pp, int spar, int i, int c,
-                                                 int sp, float f_c, double f_cd, bool sample, bool last,
+                                                 int sp, float f_c, double f_cd, bool sample, bool kick, bool last,
                                                  float &vh, float &vl, double &vd, float rr,
                                                  double &ke, double &pc, float &dd, float &vv, unsigned int &bad)
 {
     const size_t e = 4 * (size_t)i + c;
     if constexpr (P == MIXED) {
         const ds hk = ds_from(a.hdtm_hi[sp], a.hdtm_lo[sp]);
-        ds v = ds_add(ds_from(vh, vl), ds_mul_f(hk, f_c));
+        ds v = ds_from(vh, vl);
+        if (kick)
+            v = ds_add(v, ds_mul_f(hk, f_c));
         if (sample) {
             const double x = ds_to_double(v);
             ke = 0.5 * a.mass[sp] * x * x;
@@ -1207,7 +1069,9 @@ __device__ __forceinline__ void component_update(const KArgs &a, const Rep &rp, 
         vl = v.lo;
     } else if constexpr (P == FP64) {
         const double hk = a.hdtm[sp];            // (roundings spelled out, as in half_kick / drift)
-        double v = fma(hk, f_cd, vd);
+        double v = vd;
+        if (kick)
+            v = fma(hk, f_cd, v);
         if (sample) {
             ke = 0.5 * a.mass[sp] * v * v;
             pc = a.mass[sp] * v;
@@ -1232,7 +1096,9 @@ __device__ __forceinline__ void component_update(const KArgs &a, const Rep &rp, 
         vd = v;
     } else {
         const float hk = a.hdtm_hi[sp];
-        float v = fmaf(hk, f_c, vh);
+        float v = vh;
+        if (kick)
+            v = fmaf(hk, f_c, v);
         if (sample) {
             ke = 0.5 * a.mass[sp] * (double)v * (double)v;
             pc = a.mass[sp] * (double)v;
@@ -1267,17 +1133,16 @@ __device__ __forceinline__ void component_update(const KArgs &a, const Rep &rp, 
 // position buffer.  The operands of the update are loaded before the
 // neighbour loop so that their latency is hidden.
 template <int P, int TPP, bool SAMPLE, bool SM>
-__device__ __forceinline__ void step_body_split(const KArgs &a, const int4 *tab, int row, bool active, bool last,
+__device__ __forceinline__ void step_body_split(const KArgs &a, const int4 b, bool kick, bool last,
                                                 int pp, int spar, double *part, ET<P> &eo, float &d2, float &v2, float &a2,
                                                 unsigned int &bad)
 {
     constexpr int NC = TPP >= 4 ? 1 : 4 / TPP;
-    const int4 b = tab[row];
     const Rep rp = a.rep[b.z];
     const int lane = threadIdx.x & (TPP - 1);
     const int i = b.x + (int)(threadIdx.x / TPP);
-    const bool valid = active && i < b.y;
-    const int ii = (i < b.y) ? i : b.x;
+    const bool valid = i < b.y;
+    const int ii = valid ? i : b.x;
     const int nn = valid ? a.nnbr[ii] : 0;
     float vh[NC], vl[NC], rr[NC];
     double vd[NC];
@@ -1330,7 +1195,7 @@ __device__ __forceinline__ void step_body_split(const KArgs &a, const int4 *tab,
             const FT<P> f_c = c == 0 ? fx : (c == 1 ? fy : fz);
             double kc = 0.0, pc = 0.0;
             float dc = 0.f, wc = 0.f;
-            component_update<P>(a, rp, pp, spar, i, c, sp, (float)f_c, (double)f_c, SAMPLE, last, vh[u], vl[u],
+            component_update<P>(a, rp, pp, spar, i, c, sp, (float)f_c, (double)f_c, SAMPLE, kick, last, vh[u], vl[u],
                                 vd[u], rr[u], kc, pc, dc, wc, bad);
             ke += kc;
             dd += dc;
@@ -1389,20 +1254,19 @@ __device__ __forceinline__ void step_body_split(const KArgs &a, const int4 *tab,
 }
 
 template <int P, int TPP, bool SAMPLE, bool SM>
-__device__ __forceinline__ void step_body(const KArgs &a, const int4 *tab, int row, bool active, bool last,
+__device__ __forceinline__ void step_body(const KArgs &a, const int4 b, bool kick, bool last,
                                           int pp, int spar, double *part, ET<P> &eo, float &d2, float &v2, float &a2,
                                           unsigned int &bad)
 {
     if constexpr (kSplitUpdate || TPP >= 4) {
-        step_body_split<P, TPP, SAMPLE, SM>(a, tab, row, active, last, pp, spar, part, eo, d2, v2, a2, bad);
+        step_body_split<P, TPP, SAMPLE, SM>(a, b, kick, last, pp, spar, part, eo, d2, v2, a2, bad);
         return;
     }
-    const int4 b = tab[row];
     const Rep rp = a.rep[b.z];
     const int lane = threadIdx.x & (TPP - 1);
     const int i = b.x + (int)(threadIdx.x / TPP);
-    const bool valid = active && i < b.y;
-    const int ii = (i < b.y) ? i : b.x;
+    const bool valid = i < b.y;
+    const int ii = valid ? i : b.x;
     const int nn = valid ? a.nnbr[ii] : 0;
     FT<P> fx = 0, fy = 0, fz = 0;
     ET<P> ep = e_zero<P>();
@@ -1424,7 +1288,8 @@ __device__ __forceinline__ void step_body(const KArgs &a, const int4 *tab, int r
     PState<P> s;
     load_pos<P>(a, pp, i, s);
     load_vel<P>(a, spar, i, s);
-    half_kick<P>(a, s, fx, fy, fz);                 // completes v(t)
+    if (kick)
+        half_kick<P>(a, s, fx, fy, fz);             // completes v(t)
     if (SAMPLE)
         kinetic<P>(a, s, part + 8);
     if (!last) {
@@ -1437,312 +1302,15 @@ __device__ __forceinline__ void step_body(const KArgs &a, const int4 *tab, int r
     store_vel<P>(a, spar, i, s);
 }
 
-// Blocks per SM the unsmoothed single-precision step kernels are compiled for:
-// 7 x 128 threads at <= 72 registers, so that a 1024-block launch (KA N=65536
-// at 2 lanes per particle) is a single wave on 152 SMs.  FP64 and the smoothed
-// kernels keep the compiler's own register choice (they would spill).
-template <int P, bool SM> constexpr int step_min_blocks() { return (P != FP64 && !SM) ? 7 : 0; }
-
-template <int P, int TPP, bool SM, bool SWEEP>
-__global__ void __launch_bounds__(kForceBlock, step_min_blocks<P, SM>()) k_step(KArgs a)
-{
-    __shared__ double sh[32 * kPartF];
-    __shared__ float shf[160];
-    __shared__ int s_last, s_first;
-    __shared__ float s_m[4];
-    Ctl *ctl = a.ctl;
-    const unsigned int st0 = ctl->status;
-    const long long step = ctl->step;
-    const long long remaining = ctl->remaining;
-    const long long pend = ctl->epot_pending;   // an earlier step whose energies await their sum
-    const int pp = ctl->pos_par, spar = ctl->state_par;
-    // The status word can change while the launch runs (another block's atomicOr),
-    // so threads of one block may read different values: it gates only per-particle
-    // work.  Everything that shapes the block's barriers and the lanes' shuffles
-    // (sample) depends on fields that change only in the last block.
-    const bool active = st0 == 0u && remaining > 0;
-    const bool last = remaining == 1;
-    const bool sample = remaining > 0 && (step % a.si) == 0;
-    if (threadIdx.x == 0)                       // device timing of this launch: earliest start
-        atomicMax(&ctl->t_first_inv, ~global_ns());
-
-    if constexpr (SWEEP) {
-        // The block sweeps its run of chunks: rows blockIdx.x * cpb ... of the
-        // step table.  Per chunk: this step's potential energy, one partial per
-        // warp (written only by active launches, so that an idle one never
-        // overwrites partials that still await their sum; the shuffles run in
-        // every lane regardless); block maxima into the launch's maxima every
-        // step; the chunk's other reductions on sample steps (component 0 stays
-        // unused).
-        for (int q = 0; q < a.cpb; ++q) {
-            const int row = blockIdx.x * a.cpb + q;
-            const int chunk = a.blk_s[row].w;
-            if (chunk < 0)                       // (padding rows: the same for the whole block)
-                break;
-            double part[kPartF];
-            ET<P> eo;
-            float d2 = 0.f, v2 = 0.f, a2 = 0.f;
-            unsigned int bad = 0u;
-            if (sample)
-                step_body<P, TPP, true, SM>(a, a.blk_s, row, active, last, pp, spar, part, eo, d2, v2, a2,
-                                            bad);
-            else
-                step_body<P, TPP, false, SM>(a, a.blk_s, row, active, last, pp, spar, part, eo, d2, v2, a2,
-                                             bad);
-            if (bad)
-                atomicOr(&ctl->status, bad);
-            store_warp_energy<P>(a, step, chunk, eo, active);
-            block_max3(d2, v2, a2, shf);
-            if (sample)
-                block_sum<kPartF>(part, sh);
-            if (threadIdx.x == 0) {
-                if (sample) {
-                    const size_t pb = (size_t)chunk * kPartF;
-#pragma unroll
-                    for (int k = 1; k < kPartF; ++k)
-                        a.part_f[pb + k] = part[k];
-                }
-                if (d2 > 0.f)
-                    atomicMax(&ctl->maxdisp2, __float_as_uint(d2));
-                if (v2 > 0.f)
-                    atomicMax(&ctl->maxv2, __float_as_uint(v2));
-                if (a2 > 0.f)
-                    atomicMax(&ctl->maxa2, __float_as_uint(a2));
-            }
-            __syncthreads();                     // (shf and sh serve the next chunk)
-        }
-    } else {
-        // One chunk per block: the block's row of the force kernel's table.
-        // This step's potential energy, every step: one partial per warp
-        // (written only by active launches, so that an idle one never
-        // overwrites partials that still await their sum; the shuffles run in
-        // every lane regardless).  Block sums of the maxima every step, of the
-        // other reductions on sample steps (their component 0 stays unused).
-        double part[kPartF];
-        ET<P> eo;
-        float d2 = 0.f, v2 = 0.f, a2 = 0.f;
-        unsigned int bad = 0u;
-        if (sample)
-            step_body<P, TPP, true, SM>(a, a.blk_f, blockIdx.x, active, last, pp, spar, part, eo, d2, v2, a2,
-                                        bad);
-        else
-            step_body<P, TPP, false, SM>(a, a.blk_f, blockIdx.x, active, last, pp, spar, part, eo, d2, v2, a2,
-                                         bad);
-        if (bad)
-            atomicOr(&ctl->status, bad);
-        store_warp_energy<P>(a, step, a.blk_f[blockIdx.x].w, eo, active);
-        block_max3(d2, v2, a2, shf);
-        if (sample)
-            block_sum<kPartF>(part, sh);
-        if (threadIdx.x == 0) {
-            const size_t pb = (size_t)a.blk_f[blockIdx.x].w * kPartF;
-            if (sample) {
-#pragma unroll
-                for (int k = 1; k < kPartF; ++k)
-                    a.part_f[pb + k] = part[k];
-            }
-            if (d2 > 0.f)
-                atomicMax(&ctl->maxdisp2, __float_as_uint(d2));
-            if (v2 > 0.f)
-                atomicMax(&ctl->maxv2, __float_as_uint(v2));
-            if (a2 > 0.f)
-                atomicMax(&ctl->maxa2, __float_as_uint(a2));
-        }
-    }
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const unsigned int t = atomicAdd(&ctl->ticket, 1u);
-        s_first = (t == 0);
-        s_last = (t == gridDim.x - 1);
-    }
-    __syncthreads();
-    // The first block to finish adds up the energies of the earlier step that
-    // still awaits its sum (the previous step, written by the previous launch):
-    // the other blocks are still working, so this is off the critical path.
-    if (s_first && pend >= 0)
-        finish_epot<P>(a, pend, sh, shf);
-    if (!s_last)
-        return;
-
-    // ---- last block ----
-    __threadfence();
-    if (threadIdx.x == 0) {
-        s_m[0] = __uint_as_float(atomicExch(&ctl->maxdisp2, 0u));
-        s_m[1] = __uint_as_float(atomicExch(&ctl->maxv2, 0u));
-        s_m[2] = __uint_as_float(atomicExch(&ctl->maxa2, 0u));
-        s_m[3] = ctl->last_maxdisp2;    // displacement of r(step), the positions of this sample
-    }
-    __syncthreads();
-    const unsigned int st = atomicOr(&ctl->status, 0u);
-    if (sample && st == 0u)
-        finish_reductions<P>(a, IM_LOOP, true, step, s_m[3], sh, shf);   // (its E_pot enters the series)
-    if (threadIdx.x == 0) {
-        if (sample && st == 0u)
-            a.epot_step[step % a.epot_cap] = step;
-        // this step's energies: summed into the series here (sample) or by the
-        // first block to finish the next launch (or by k_epot_flush)
-        ctl->epot_pending = (remaining > 0 && st == 0u && !sample) ? step : -1ll;
-        const bool drifted = active && !last;
-        unsigned int reb = 0u;
-        if (drifted && st == 0u) {
-            reb = need_rebuild(a, s_m[0], s_m[1], s_m[2]);
-            ctl->step = step + 1;
-            ctl->pos_par = pp ^ 1;
-            ctl->last_maxdisp2 = s_m[0];
-        }
-        ctl->rebuild = reb;
-        if (sample && st == 0u)
-            ctl->obs_count += 1;
-        long long rem = remaining;
-        if (active)
-            rem -= 1;
-        ctl->remaining = rem;
-        const long long bud = ctl->budget - 1;
-        ctl->budget = bud;
-        unsigned int s2 = st;
-        if (bud <= 0 && rem > 0) {
-            atomicOr(&ctl->status, ST_TIMEOUT);
-            s2 |= ST_TIMEOUT;
-        }
-        ctl->ticket = 0u;
-        ctl->n_integrate += 1;
-        if (a.use_cond) {
-            if (a.set_rebuild)
-                cudaGraphSetConditional(a.h_rebuild, reb);
-            if (a.set_loop)
-                cudaGraphSetConditional(a.h_loop, (s2 == 0u && rem > 0) ? 1u : 0u);
-        }
-        // duration of this launch (one that advanced a step): earliest block start
-        // to the end of the last block
-        const unsigned long long t0 = ~ctl->t_first_inv;
-        const unsigned long long t1 = global_ns();
-        if (active) {
-            ctl->dev_ns += t1 > t0 ? t1 - t0 : 0ull;
-            ctl->dev_launches += 1;
-        }
-        ctl->t_first_inv = 0ull;
-    }
-}
-
-// ---------------------------------------------------------------------------
-// k_integrate: the per-particle half kick + drift that opens md_step
-// (IM_FIRST), and the kinetic reductions alone (IM_SAMPLE, IM_TOTALS, IM_KE).
-// ---------------------------------------------------------------------------
-template <int P>
-__global__ void __launch_bounds__(kIntBlock) k_integrate(KArgs a)
-{
-    __shared__ double sh[32 * 12];
-    __shared__ float shf[160];
-    __shared__ int s_last;
-    __shared__ float s_m[3];
-    Ctl *ctl = a.ctl;
-    const unsigned int st0 = ctl->status;
-    const bool halted = st0 != 0u;
-    const long long step = ctl->step;
-    const int pp = ctl->pos_par, spar = ctl->state_par;
-    const int mode = a.imode;
-    const bool first = mode == IM_FIRST;
-    const bool rec = !first;
-
-    const int4 b = a.blk_i[blockIdx.x];
-    const Rep rp = a.rep[b.z];
-    const int i = b.x + threadIdx.x;
-    const bool valid = (i < b.y) && !halted;
-    float d2 = 0.f, v2 = 0.f, a2 = 0.f;
-    double kin[4] = {0.0, 0.0, 0.0, 0.0};
-    unsigned int bad = 0u;
-    if (valid) {
-        PState<P> s;
-        load_pos<P>(a, pp, i, s);
-        load_vel<P>(a, spar, i, s);
-        if (rec)
-            kinetic<P>(a, s, kin);
-        if (first) {
-            FT<P> f[3];
-            if constexpr (P == FP64) {
-                const d4 q = ((const d4 *)a.force)[i];
-                f[0] = q.x; f[1] = q.y; f[2] = q.z;
-            } else {
-                const float4 q = ((const float4 *)a.force)[i];
-                f[0] = q.x; f[1] = q.y; f[2] = q.z;
-            }
-            half_kick<P>(a, s, f[0], f[1], f[2]);
-            d2 = drift<P>(a, rp, s, pp ^ 1, spar, i, bad);
-            v2 = speed2(s);
-            const float im = a.inv_mass[s.sp];
-            a2 = __fmul_rn(__fmul_rn(norm2(f[0], f[1], f[2]), im), im);
-            store_vel<P>(a, spar, i, s);
-        }
-    }
-    if (bad)
-        atomicOr(&ctl->status, bad);
-    block_max3(d2, v2, a2, shf);
-    if (rec)
-        block_sum<4>(kin, sh);
-    if (threadIdx.x == 0) {
-        if (rec)
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-                a.part_i[(size_t)blockIdx.x * 4 + k] = kin[k];
-        if (d2 > 0.f)
-            atomicMax(&ctl->maxdisp2, __float_as_uint(d2));
-        if (v2 > 0.f)
-            atomicMax(&ctl->maxv2, __float_as_uint(v2));
-        if (a2 > 0.f)
-            atomicMax(&ctl->maxa2, __float_as_uint(a2));
-        __threadfence();
-        const unsigned int t = atomicAdd(&ctl->ticket, 1u);
-        s_last = (t == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!s_last)
-        return;
-    __threadfence();
-    if (threadIdx.x == 0) {
-        s_m[0] = __uint_as_float(atomicExch(&ctl->maxdisp2, 0u));
-        s_m[1] = __uint_as_float(atomicExch(&ctl->maxv2, 0u));
-        s_m[2] = __uint_as_float(atomicExch(&ctl->maxa2, 0u));
-    }
-    __syncthreads();
-    const unsigned int st = atomicOr(&ctl->status, 0u);
-    if (rec && st == 0u)
-        finish_reductions<P>(a, mode, false, step, s_m[0], sh, shf);
-    if (threadIdx.x == 0) {
-        unsigned int reb = 0u;
-        if (first && !halted && st == 0u) {
-            reb = need_rebuild(a, s_m[0], s_m[1], s_m[2]);
-            ctl->step = step + 1;
-            ctl->pos_par = pp ^ 1;
-            ctl->last_maxdisp2 = s_m[0];
-        }
-        if (first)
-            ctl->rebuild = reb;
-        if (mode == IM_SAMPLE && st == 0u) {
-            ctl->obs_count += 1;
-            a.epot_step[step % a.epot_cap] = step;
-        }
-        ctl->ticket = 0u;
-        ctl->n_integrate += 1;
-        if (a.use_cond && a.set_rebuild)
-            cudaGraphSetConditional(a.h_rebuild, reb);
-    }
-}
-
 // ---------------------------------------------------------------------------
 // Cell binning by counting sort (Sec. 2.2: integer cell index per particle,
 // particles sorted by cell, start index of each cell) with the cells ordered
-// along a space-filling curve (the periodic reorder of Sec. 2.2).
-// Kernels: k_bin (cell key + histogram) -> k_scan -> k_scatter ->
-// k_permute (deterministic order inside a cell; gather of the state into the
-// other buffers) -> k_nbuild (lists from the permuted positions; its last
-// block makes the permuted buffers current).  Each returns at once unless a
-// rebuild is pending; k_scan clears the histogram for the next binning.
+// along a space-filling curve (the periodic reorder of Sec. 2.2).  Phases of a
+// rebuild, each ending at a grid barrier of the run kernel: bin (cell key,
+// histogram) -> scan (cell starts) -> scatter -> permute (deterministic order
+// inside a cell; gather of the state into the other buffers) -> neighbour build
+// (lists from the permuted positions).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ bool rebuild_pending(const Ctl *ctl)
-{
-    return ctl->status == 0u && ctl->rebuild != 0u;
-}
-
 __device__ __forceinline__ int cell_coord(double x, double cscale, int nc)
 {
     int c = (int)floor(x * cscale);
@@ -1778,23 +1346,11 @@ __device__ __forceinline__ int morton6(unsigned int x, unsigned int y, unsigned 
                  ((z & 2u) << 4));
 }
 
+// Cell key and sub-cell code of particle i from the positions in buffer pp.
 template <int P>
-__global__ void __launch_bounds__(kIntBlock) k_bin(KArgs a)
+__device__ __forceinline__ int cell_of(const KArgs &a, const Rep &rp, int pp, int i, int &sub)
 {
-    Ctl *ctl = a.ctl;
-    if (!rebuild_pending(ctl))
-        return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        ctl->max_nbr = 0;
-        atomicAdd((unsigned long long *)&ctl->n_rebuild_k, 1ull);
-    }
-    const int4 b = a.blk_i[blockIdx.x];
-    const int i = b.x + threadIdx.x;
-    if (i >= b.y)
-        return;
-    const Rep rp = a.rep[b.z];
-    const int pp = ctl->pos_par;
-    int cx, cy, cz, sub;
+    int cx, cy, cz;
     if constexpr (P == FP64) {
         const d4 x = ((const d4 *)pos_a(a, pp))[i];
         cx = cell_coord(x.x, rp.cscale, rp.nc);
@@ -1808,154 +1364,129 @@ __global__ void __launch_bounds__(kIntBlock) k_bin(KArgs a)
         cz = cell_coord_f(x.z, rp.cscalef, rp.nc);
         sub = morton6(sub2f(x.x, rp.cscalef, cx), sub2f(x.y, rp.cscalef, cy), sub2f(x.z, rp.cscalef, cz));
     }
-    const int key = checked(a, a.crank[rp.cell0 + (cz * rp.nc + cy) * rp.nc + cx], a.ncell, 0);
-    a.key[i] = key;
-    a.skey[i] = sub;
-    atomicAdd(&a.ccount[key], 1);
+    return checked(a, a.crank[rp.cell0 + (cz * rp.nc + cy) * rp.nc + cx], a.ncell, 0);
 }
 
-// exclusive scan of the cell histogram by one block; also clears the cursors
+// Phase 1: cell keys, histogram, and the particles in each block's slice of
+// slice_cells consecutive cells.
 template <int P>
-__global__ void __launch_bounds__(kScanBlock) k_scan(KArgs a)
+__device__ __forceinline__ void rebuild_bin(const KArgs &a, int pp, int slice_cells)
 {
-    // Exclusive prefix sum of the cell counts (one block), in tiles of
-    // kScanBlock x kScanPer cells: each tile is read and written with coalesced
-    // accesses through shared memory, each thread scans kScanPer consecutive
-    // counts, and the per-thread sums are scanned across the block.  The
-    // counts are cleared for the next binning.
-    constexpr int T = kScanBlock, R = kScanPer;
-    __shared__ int tile[T * R + T * R / 32];      // padded: one word every 32
-    __shared__ int wsum[32];
-    __shared__ int s_carry;
-    Ctl *ctl = a.ctl;
-    if (!rebuild_pending(ctl))
-        return;
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    if (t == 0) {
-        atomicAdd((unsigned long long *)&ctl->n_rebuild_k, 1ull);
-        s_carry = 0;
+    for (int row = blockIdx.x; row < a.nblk_i; row += gridDim.x) {
+        const int4 b = a.blk_i[row];
+        const Rep &rp = a.rep[b.z];
+        for (int i = b.x + threadIdx.x; i < b.y; i += blockDim.x) {
+            int sub;
+            const int key = cell_of<P>(a, rp, pp, i, sub);
+            a.key[i] = key;
+            a.skey[i] = sub;
+            atomicAdd(&a.ccount[key], 1);
+            atomicAdd(&a.slice[key / slice_cells], 1);
+        }
     }
-    const int n = a.ncell;
-    auto at = [](int i) { return i + (i >> 5); };
-    for (int base = 0; base < n; base += T * R) {
-#pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const int i = base + k * T + t;
-            tile[at(k * T + t)] = i < n ? a.ccount[i] : 0;
-        }
-        __syncthreads();
-        int v[R], sum = 0;
-#pragma unroll
-        for (int k = 0; k < R; ++k) {
-            v[k] = tile[at(t * R + k)];
-            sum += v[k];
-        }
-        int incl = sum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o)
-                incl += y;
-        }
-        if (lane == 31)
-            wsum[w] = incl;
-        __syncthreads();
-        if (w == 0) {
-            int x = lane < T / 32 ? wsum[lane] : 0;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, x, o);
-                if (lane >= o)
-                    x += y;
-            }
-            wsum[lane] = x;                       // inclusive sums of the warps
-        }
-        __syncthreads();
-        const int carry = s_carry;
-        int run = carry + (w > 0 ? wsum[w - 1] : 0) + incl - sum;
-#pragma unroll
-        for (int k = 0; k < R; ++k) {
-            tile[at(t * R + k)] = run;
-            run += v[k];
-        }
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const int i = base + k * T + t;
-            if (i < n) {
-                a.cstart[i] = tile[at(k * T + t)];
-                a.ccount[i] = 0;          // ready for the next binning
-                a.ccursor[i] = 0;
-            }
-        }
-        if (t == 0)
-            s_carry = carry + wsum[T / 32 - 1];
-        __syncthreads();
-    }
-    if (t == 0)
-        a.cstart[n] = s_carry;
 }
 
-template <int P>
-__global__ void __launch_bounds__(kIntBlock) k_scatter(KArgs a)
+// Exclusive prefix sum of one value per thread over the block; `total` gets the
+// sum.  sh: one int per warp.
+__device__ __forceinline__ int block_scan(int v, int &total, int *sh)
 {
-    Ctl *ctl = a.ctl;
-    if (!rebuild_pending(ctl))
-        return;
-    if (blockIdx.x == 0 && threadIdx.x == 0)
-        atomicAdd((unsigned long long *)&ctl->n_rebuild_k, 1ull);
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.n)
-        return;
-    const int k = checked(a, a.key[i], a.ncell, 0);
-    const int slot = checked(a, a.cstart[k] + atomicAdd(&a.ccursor[k], 1), a.n, 0);
-    a.tmpidx[slot] = i;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    int incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o)
+            incl += y;
+    }
+    if (lane == 31)
+        sh[w] = incl;
+    __syncthreads();
+    int before = 0, sum = 0;
+    for (int k = 0; k < nw; ++k) {
+        before += k < w ? sh[k] : 0;
+        sum += sh[k];
+    }
+    __syncthreads();
+    total = sum;
+    return before + incl - v;
 }
 
-// Final slot of each particle: its cell's start plus the number of particles
-// of the same cell that come before it in (sub-cell code, current index)
-// order (deterministic), then gather of the whole state into the other
+// Phase 2: first particle of every cell.  Each block adds up the slices before
+// its own, then scans its slice; the counts are cleared for the next binning.
+__device__ __forceinline__ void rebuild_scan(const KArgs &a, int slice_cells, int *sh)
+{
+    const int c0 = blockIdx.x * slice_cells, c1 = min(c0 + slice_cells, a.ncell);
+    if (c0 >= a.ncell)
+        return;
+    int before = 0, carry;
+    for (int b = threadIdx.x; b < (int)blockIdx.x; b += blockDim.x)
+        before += a.slice[b];
+    block_scan(before, carry, sh);
+    for (int base = c0; base < c1; base += blockDim.x) {
+        const int c = base + threadIdx.x;
+        const int v = c < c1 ? a.ccount[c] : 0;
+        int sum;
+        const int at = carry + block_scan(v, sum, sh);
+        if (c < c1) {
+            a.cstart[c] = at;
+            a.ccount[c] = 0;
+            a.ccursor[c] = 0;
+        }
+        carry += sum;
+    }
+    if (threadIdx.x == 0 && c1 == a.ncell)
+        a.cstart[a.ncell] = carry;
+}
+
+// Phase 3: particles into their cells, in any order.
+__device__ __forceinline__ void rebuild_scatter(const KArgs &a)
+{
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += gridDim.x * blockDim.x) {
+        const int k = checked(a, a.key[i], a.ncell, 0);
+        const int slot = checked(a, a.cstart[k] + atomicAdd(&a.ccursor[k], 1), a.n, 0);
+        a.tmpidx[slot] = i;
+    }
+    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < (int)gridDim.x; b += gridDim.x * blockDim.x)
+        a.slice[b] = 0;                                  // ready for the next binning
+}
+
+// Phase 4: final slot of each particle: its cell's start plus the number of
+// particles of the same cell that come before it in (sub-cell code, current
+// index) order (deterministic), then gather of the whole state into the other
 // buffers.
 template <int P>
-__global__ void __launch_bounds__(kIntBlock) k_permute(KArgs a)
+__device__ __forceinline__ void rebuild_permute(const KArgs &a, int pp, int spar)
 {
-    Ctl *ctl = a.ctl;
-    if (!rebuild_pending(ctl))
-        return;
-    if (blockIdx.x == 0 && threadIdx.x == 0)
-        atomicAdd((unsigned long long *)&ctl->n_rebuild_k, 1ull);
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= a.n)
-        return;
-    const int pp = ctl->pos_par, spar = ctl->state_par;
-    const int i = checked(a, a.tmpidx[s], a.n, 0);
-    const int k = checked(a, a.key[i], a.ncell, 0);
-    const int b0 = a.cstart[k], b1 = a.cstart[k + 1];
-    const int si = a.skey[i];
-    int rank = 0;
-    for (int t = b0; t < b1; ++t) {
-        const int j = checked(a, a.tmpidx[t], a.n, 0);
-        const int sj = a.skey[j];
-        rank += (sj < si || (sj == si && j < i)) ? 1 : 0;
-    }
-    const int d = checked(a, b0 + rank, a.n, 0);
-    if constexpr (P == FP64) {
-        const d4 x = ((const d4 *)pos_a(a, pp))[i];
-        ((d4 *)pos_a(a, pp ^ 1))[d] = x;
-        ((d4 *)vel_a(a, spar ^ 1))[d] = ((const d4 *)vel_a(a, spar))[i];
-        a.rref[d] = make_float4(__double2float_rn(x.x), __double2float_rn(x.y), __double2float_rn(x.z), 0.f);
-    } else {
-        const float4 x = ((const float4 *)pos_a(a, pp))[i];
-        ((float4 *)pos_a(a, pp ^ 1))[d] = x;
-        ((float4 *)vel_a(a, spar ^ 1))[d] = ((const float4 *)vel_a(a, spar))[i];
-        if constexpr (P == MIXED) {
-            ((float4 *)pos_b(a, pp ^ 1))[d] = ((const float4 *)pos_b(a, pp))[i];
-            q_of(a, pp ^ 1)[d] = q_of(a, pp)[i];
-            ((float4 *)vel_b(a, spar ^ 1))[d] = ((const float4 *)vel_b(a, spar))[i];
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < a.n; s += gridDim.x * blockDim.x) {
+        const int i = checked(a, a.tmpidx[s], a.n, 0);
+        const int k = checked(a, a.key[i], a.ncell, 0);
+        const int b0 = a.cstart[k], b1 = a.cstart[k + 1];
+        const int si = a.skey[i];
+        int rank = 0;
+        for (int t = b0; t < b1; ++t) {
+            const int j = checked(a, a.tmpidx[t], a.n, 0);
+            const int sj = a.skey[j];
+            rank += (sj < si || (sj == si && j < i)) ? 1 : 0;
         }
-        a.rref[d] = make_float4(x.x, x.y, x.z, 0.f);
+        const int d = checked(a, b0 + rank, a.n, 0);
+        if constexpr (P == FP64) {
+            const d4 x = ((const d4 *)pos_a(a, pp))[i];
+            ((d4 *)pos_a(a, pp ^ 1))[d] = x;
+            ((d4 *)vel_a(a, spar ^ 1))[d] = ((const d4 *)vel_a(a, spar))[i];
+            a.rref[d] = make_float4(__double2float_rn(x.x), __double2float_rn(x.y), __double2float_rn(x.z), 0.f);
+        } else {
+            const float4 x = ((const float4 *)pos_a(a, pp))[i];
+            ((float4 *)pos_a(a, pp ^ 1))[d] = x;
+            ((float4 *)vel_a(a, spar ^ 1))[d] = ((const float4 *)vel_a(a, spar))[i];
+            if constexpr (P == MIXED) {
+                ((float4 *)pos_b(a, pp ^ 1))[d] = ((const float4 *)pos_b(a, pp))[i];
+                q_of(a, pp ^ 1)[d] = q_of(a, pp)[i];
+                ((float4 *)vel_b(a, spar ^ 1))[d] = ((const float4 *)vel_b(a, spar))[i];
+            }
+            a.rref[d] = make_float4(x.x, x.y, x.z, 0.f);
+        }
+        img_of(a, spar ^ 1)[d] = img_of(a, spar)[i];
     }
-    img_of(a, spar ^ 1)[d] = img_of(a, spar)[i];
 }
 
 // ---------------------------------------------------------------------------
@@ -1977,7 +1508,7 @@ __global__ void __launch_bounds__(kIntBlock) k_permute(KArgs a)
 // more particles in the cell than 32, are processed in rounds, so no cell
 // size is too large.
 // ---------------------------------------------------------------------------
-constexpr int kNbStage = 256;    // staged candidates per round and warp
+constexpr int kNbStage = 128;    // staged candidates per round and warp
 
 struct NbWarp {
     float4 pos[kNbStage];
@@ -2166,20 +1697,22 @@ __device__ __forceinline__ void nbuild_cell_warp(const KArgs &a, int pn, int c, 
 // order and filter as above), and each of its warps takes kNbPass particles
 // of the cell at a time, testing 32 staged candidates per ballot; the list
 // rows come out the same as with a warp per cell.
-constexpr int kNbCap = 1024;     // staged candidates per round
+constexpr int kNbCap = 512;      // staged candidates per round
 constexpr int kNbOwn = 256;      // own-cell particles per batch
 constexpr int kNbPass = 2;       // own-cell particles tested per warp pass over the candidates
 
-template <int P>
-__device__ __forceinline__ void nbuild_cell_block(const KArgs &a, int pn, int c, int K)
-{
-    __shared__ float4 s_pos[kNbCap];
-    __shared__ int s_idx[kNbCap];
-    __shared__ int s_cnt[kNbOwn];
-    __shared__ int s_pref[28];
-    __shared__ int s_cell[27];
-    __shared__ int s_wsum[kNbBlockB / 32];
+struct NbBlock {
+    float4 pos[kNbCap];
+    int idx[kNbCap];
+    int cnt[kNbOwn];
+    int pref[28];
+    int cell[27];
+    int wsum[kNbBlockB / 32];
+};
 
+template <int P>
+__device__ __forceinline__ void nbuild_cell_block(const KArgs &a, int pn, int c, int K, NbBlock &S)
+{
     Ctl *ctl = a.ctl;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int NW = kNbBlockB / 32;
@@ -2198,19 +1731,19 @@ __device__ __forceinline__ void nbuild_cell_block(const KArgs &a, int pn, int c,
             y = (y + (tid / 3) % 3 - 1 + nc) % nc;
             z = (z + tid / 9 - 1 + nc) % nc;
         }
-        s_cell[tid] = a.crank[rp.cell0 + (z * nc + y) * nc + x];
+        S.cell[tid] = a.crank[rp.cell0 + (z * nc + y) * nc + x];
     }
     __syncthreads();
     if (tid == 0) {
         int s = 0;
         for (int k = 0; k < nst; ++k) {
-            s_pref[k] = s;
-            s += a.cstart[s_cell[k] + 1] - a.cstart[s_cell[k]];
+            S.pref[k] = s;
+            s += a.cstart[S.cell[k] + 1] - a.cstart[S.cell[k]];
         }
-        s_pref[nst] = s;
+        S.pref[nst] = s;
     }
     __syncthreads();
-    const int total = s_pref[nst];
+    const int total = S.pref[nst];
 
     // own cell box (centre, half edge) for the candidate filter
     const float edge = rp.Lhi / (float)nc;
@@ -2225,7 +1758,7 @@ __device__ __forceinline__ void nbuild_cell_block(const KArgs &a, int pn, int c,
     for (int ob = c0; ob < c1; ob += kNbOwn) {
         const int nown = min(kNbOwn, c1 - ob);
         for (int t = tid; t < nown; t += kNbBlockB)
-            s_cnt[t] = 0;
+            S.cnt[t] = 0;
         int staged = 0;
         for (int base = 0; base < total; base += kNbBlockB) {
             // stage candidates base .. base + kNbBlockB - 1, order-preserving compaction
@@ -2235,9 +1768,9 @@ __device__ __forceinline__ void nbuild_cell_block(const KArgs &a, int pn, int c,
             int j = 0;
             if (t < total) {
                 int k = 0;
-                while (k + 1 < nst && s_pref[k + 1] <= t)
+                while (k + 1 < nst && S.pref[k + 1] <= t)
                     ++k;
-                j = checked(a, a.cstart[s_cell[k]] + (t - s_pref[k]), a.n, 0);
+                j = checked(a, a.cstart[S.cell[k]] + (t - S.pref[k]), a.n, 0);
                 q = nb_word<P>(a, pn, j);
                 keep = true;
                 if (nst == 27) {
@@ -2250,18 +1783,18 @@ __device__ __forceinline__ void nbuild_cell_block(const KArgs &a, int pn, int c,
             }
             const unsigned m = __ballot_sync(0xffffffffu, keep);
             if (lane == 0)
-                s_wsum[warp] = __popc(m);
+                S.wsum[warp] = __popc(m);
             __syncthreads();
             int off = staged, add = 0;
 #pragma unroll
             for (int w = 0; w < NW; ++w) {
-                off += (w < warp) ? s_wsum[w] : 0;
-                add += s_wsum[w];
+                off += (w < warp) ? S.wsum[w] : 0;
+                add += S.wsum[w];
             }
             if (keep) {
                 const int s = off + __popc(m & lt_mask);
-                s_pos[s] = q;
-                s_idx[s] = j;
+                S.pos[s] = q;
+                S.idx[s] = j;
             }
             staged += add;
             __syncthreads();
@@ -2281,13 +1814,13 @@ __device__ __forceinline__ void nbuild_cell_block(const KArgs &a, int pn, int c,
                     const int ti = nb_species<P>(H[p]);
                     rl0[p] = ok ? a.tab.rl2[ti * 2] * r2unit : -1.0f;       // -1: nothing passes
                     rl1[p] = ok ? a.tab.rl2[ti * 2 + 1] * r2unit : -1.0f;
-                    cnt[p] = ok ? s_cnt[o0 + p] : 0;
+                    cnt[p] = ok ? S.cnt[o0 + p] : 0;
                 }
                 for (int s0 = 0; s0 < staged; s0 += 32) {
                     const int s = s0 + lane;
                     const bool sv = s < staged;
-                    const float4 y = sv ? s_pos[s] : make_float4(0.f, 0.f, 0.f, 0.f);
-                    const int jj = sv ? s_idx[s] : -1;
+                    const float4 y = sv ? S.pos[s] : make_float4(0.f, 0.f, 0.f, 0.f);
+                    const int jj = sv ? S.idx[s] : -1;
                     const bool tj = nb_species<P>(y) != 0;
 #pragma unroll
                     for (int p = 0; p < kNbPass; ++p) {
@@ -2305,13 +1838,13 @@ __device__ __forceinline__ void nbuild_cell_block(const KArgs &a, int pn, int c,
 #pragma unroll
                     for (int p = 0; p < kNbPass; ++p)
                         if (o0 + p < nown)
-                            s_cnt[o0 + p] = cnt[p];
+                            S.cnt[o0 + p] = cnt[p];
             }
             staged = 0;
             __syncthreads();
         }
         for (int o = tid; o < nown; o += kNbBlockB) {
-            const int cnt = s_cnt[o];
+            const int cnt = S.cnt[o];
             a.nnbr[ob + o] = cnt < K ? cnt : K;
             // pad the row with the particle itself to a multiple of kUnr entries, so the
             // pair loop reads whole groups without masking (K is a multiple of 8)
@@ -2333,111 +1866,556 @@ __device__ __forceinline__ int grown_capacity(int mx, int Kmax)
     return want < Kmax ? want : Kmax;
 }
 
-// The neighbour build closes the rebuild chain.  The last block to finish
-// (ticket pattern) reads the longest list of the build and
-//   - makes the permuted buffers current if every list fitted its K entries;
-//   - otherwise, if the longest list fits the cap, raises K (grown_capacity)
-//     and asks for the build to be redone (Ctl::regrow, and the graph's regrow
-//     condition): the redo (nb_retry = 1, same positions, so the same counts)
-//     then fits, and its last block makes the buffers current;
-//   - otherwise reports ST_OVERFLOW, leaving the buffers of the last completed
-//     step current.
-// The pending check is read once per block (the status can change during the
-// launch) and every block takes a ticket.  k_nbuild: warp w of block b takes
-// cells kNbCells b + w, then kNbCells gridDim.x further on, ...; k_nbuild_blk:
-// block b takes cells b, b + gridDim.x, ...
+// ---------------------------------------------------------------------------
+// k_run: md_step and force evaluations as one cooperative launch.  Its blocks
+// are all resident; each MD step is one sweep over the block's chunks of
+// particles and one barrier of the grid, whose last arriver decides, with a
+// bound on how far particles can move before the next check, whether the lists
+// must be rebuilt (the displacement criterion of Sec. 2.2); the rebuild runs in
+// the same launch, a grid barrier after each of its phases.
+//
+// What bounds a step of a small system is latency: the launches, conditional
+// nodes and idle steps of a graph of one kernel per step cost more than the
+// forces.  The barrier (one atomic per block, then polling one word) replaces
+// all of them.
+//
+// What every block must know alike (step, buffer parities, list capacity, what
+// to do next) is kept per block in shared memory and follows from the flags
+// that a barrier returns, so no block reads control words that another one may
+// be changing.
+// ---------------------------------------------------------------------------
+enum RunFlag : unsigned int {
+    RF_REBUILD = 1u,   // step: the lists must be rebuilt; build: redo it with the raised capacity
+    RF_STOP = 2u,      // nothing follows
+    RF_BAD = 4u,       // the phase failed (Ctl::status): its results are not made current
+    RF_ABORT = 8u      // a barrier gave up waiting: leave at once
+};
 
-// First thread of every block of the build: is a build (or its redo) pending,
-// and the capacity in use; counts the launch.
-__device__ __forceinline__ void nbuild_begin(const KArgs &a, int &s_go, int &s_K)
-{
-    Ctl *ctl = a.ctl;
-    if (threadIdx.x == 0) {
-        s_go = (rebuild_pending(ctl) && (a.nb_retry == 0 || ctl->regrow != 0u)) ? 1 : 0;
-        s_K = ctl->K;
-        if (s_go && blockIdx.x == 0) {
-            atomicAdd((unsigned long long *)&ctl->n_rebuild_k, 1ull);
-            if (a.nb_retry)
-                atomicAdd((unsigned long long *)&ctl->regrows, 1ull);
-            else
-                atomicAdd((unsigned long long *)&ctl->rebuilds, 1ull);
-        }
-    }
-}
+// Polls before a barrier gives up (about ten seconds of polling; the count does
+// not advance while the kernel is preempted).
+constexpr unsigned int kSpinMax = 1u << 24;
 
-// Every block's ticket; the last block swaps in the permuted buffers, grows the
-// capacity and asks for the redo, or reports the overflow (see above).
-__device__ __forceinline__ void nbuild_end(const KArgs &a, int s_go, int s_K)
+struct RunState {
+    long long step, left, obs, rebuilds, regrows, budget;
+    long long pend;                // step whose partial sums await their sum (-1: none)
+    long long pend_obs, pend_rebuilds;
+    unsigned long long t0, ns;
+    int pp, spar, K, pos;
+    float md2, pend_md2;           // largest squared displacement since the build: now, of `pend`
+    int pend_sample;
+    int last, sample;              // of the running step
+    long long done;
+    unsigned int count, flags;     // barriers passed (thread 0), flags of the last one
+};
+
+// shared scratch of the phases, one at a time
+union RunScratch {
+    NbWarp warp[kNbCells];
+    NbBlock block;
+    int scan[32];
+};
+
+// ... and of a step: block reductions, and what a thread keeps between its
+// chunks (registers are scarce in the pair loop)
+struct RunSums {
+    double sh[32 * kPartF];
+    double tot[kPartF];                              // sums of a one-replica sample
+    double e[kForceBlock];                           // energy (ET) and maxima so far, per thread
+    float d2[kForceBlock], v2[kForceBlock], a2[kForceBlock];
+};
+
+// Every block arrives; `decide` runs in thread 0 of the last one, sees the
+// writes of all blocks and returns the flags that every block gets.
+template <class F>
+__device__ __forceinline__ unsigned int grid_barrier(const KArgs &a, RunState &S, F &&decide)
 {
-    Ctl *ctl = a.ctl;
+    __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();                    // this block's list counts before its ticket
-        const unsigned int t = atomicAdd(&ctl->ticket, 1u);
+        RunSync *rs = a.rs;
+        __threadfence();
+        const unsigned int t = atomicAdd(&rs->arrive, 1u);
+        const unsigned int next = (S.count + 1u) & 0x0fffffffu;
+        unsigned int w;
         if (t == gridDim.x - 1) {
             __threadfence();
-            unsigned int regrow = 0u;
-            if (s_go && atomicOr(&ctl->status, 0u) == 0u) {
-                const int mx = atomicMax(&ctl->max_nbr, 0);
-                if (mx <= s_K) {
-                    ctl->pos_par ^= 1;
-                    ctl->state_par ^= 1;
-                    ctl->last_maxdisp2 = 0.f;   // the lists start from these positions
-                } else if (mx <= ctl->Kmax && a.nb_retry == 0) {
-                    ctl->K = grown_capacity(mx, ctl->Kmax);
-                    regrow = 1u;
-                } else {
-                    atomicOr(&ctl->status, ST_OVERFLOW);
-                }
+            rs->arrive = 0u;
+            w = (next << 4) | decide();
+            __threadfence();
+            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&rs->word), "r"(w) : "memory");
+        } else {
+            unsigned int n = 0;
+            do {
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(w) : "l"(&rs->word) : "memory");
+            } while ((w >> 4) != next && ++n < kSpinMax);
+            if ((w >> 4) != next) {
+                atomicOr(&a.ctl->status, ST_TIMEOUT);
+                w = RF_STOP | RF_BAD | RF_ABORT;
             }
-            if (s_go || a.nb_retry == 0)
-                ctl->regrow = regrow;
-            ctl->ticket = 0u;
-            if (a.use_cond && a.set_regrow)
-                cudaGraphSetConditional(a.h_regrow, regrow);
+        }
+        S.count = next;
+        S.flags = w & 15u;
+    }
+    __syncthreads();
+    return S.flags;
+}
+
+// Maxima of this block's displacements, speeds and accelerations into the
+// step's, thread 0.
+__device__ __forceinline__ void put_maxima(const KArgs &a, long long step, float d2, float v2, float a2)
+{
+    unsigned int *m = a.rs->m[step & 1];
+    if (d2 > 0.f)
+        atomicMax(&m[0], __float_as_uint(d2));
+    if (v2 > 0.f)
+        atomicMax(&m[1], __float_as_uint(v2));
+    if (a2 > 0.f)
+        atomicMax(&m[2], __float_as_uint(a2));
+}
+
+// The whole grid's maxima (cleared for the step after the next): does a drift
+// call for a rebuild?  md2 gets the largest squared displacement.
+__device__ __forceinline__ bool take_maxima(const KArgs &a, long long step, int lookahead, float &md2)
+{
+    unsigned int *m = a.rs->m[step & 1];
+    md2 = __uint_as_float(atomicExch(&m[0], 0u));
+    const float mv2 = __uint_as_float(atomicExch(&m[1], 0u));
+    const float ma2 = __uint_as_float(atomicExch(&m[2], 0u));
+    return need_rebuild(a, lookahead, md2, mv2, ma2);
+}
+
+// Rebuild of the lists; returns the flags of its last barrier (the state's
+// parities and capacity are those of the new lists unless RF_BAD).
+template <int P>
+__device__ __forceinline__ unsigned int run_rebuild(const KArgs &a, RunState &S, RunScratch &X)
+{
+    Ctl *ctl = a.ctl;
+    const auto nothing = []() -> unsigned int { return 0u; };
+    const int slice_cells = (a.ncell + (int)gridDim.x - 1) / (int)gridDim.x;
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        ctl->max_nbr = 0;
+    rebuild_bin<P>(a, S.pp, slice_cells);
+    if (grid_barrier(a, S, nothing) & RF_ABORT)
+        return S.flags;
+    rebuild_scan(a, slice_cells, X.scan);
+    if (grid_barrier(a, S, nothing) & RF_ABORT)
+        return S.flags;
+    rebuild_scatter(a);
+    if (grid_barrier(a, S, nothing) & RF_ABORT)
+        return S.flags;
+    rebuild_permute<P>(a, S.pp, S.spar);
+    if (grid_barrier(a, S, nothing) & RF_ABORT)
+        return S.flags;
+    for (int retry = 0;; ++retry) {
+        // the lists: at most K entries a row; the longest list decides
+        const int pn = S.pp ^ 1, K = S.K;
+        if (a.nb_block) {
+            for (int c = blockIdx.x; c < a.ncell; c += gridDim.x)
+                nbuild_cell_block<P>(a, pn, c, K, X.block);
+        } else {
+            const int w = threadIdx.x >> 5;
+            for (int c = blockIdx.x * kNbCells + w; c < a.ncell; c += gridDim.x * kNbCells)
+                nbuild_cell_warp<P>(a, pn, c, K, X.warp[w]);
+        }
+        const unsigned int f = grid_barrier(a, S, [&]() -> unsigned int {
+            if (atomicOr(&ctl->status, 0u))
+                return RF_STOP | RF_BAD;
+            const int mx = atomicMax(&ctl->max_nbr, 0);
+            if (mx <= K)
+                return 0u;
+            if (mx <= ctl->Kmax && retry == 0) {
+                // grow the capacity and redo the build: same positions, so the
+                // same counts, and they fit
+                ctl->K = grown_capacity(mx, ctl->Kmax);
+                return RF_REBUILD;
+            }
+            atomicOr(&ctl->status, ST_OVERFLOW);
+            return RF_STOP | RF_BAD;
+        });
+        if (threadIdx.x == 0) {
+            if (retry == 0)
+                S.rebuilds += 1;
+            if (f & RF_REBUILD) {
+                S.K = ctl->K;
+                S.regrows += 1;
+            } else if (!(f & RF_BAD)) {
+                S.pp ^= 1;
+                S.spar ^= 1;
+                S.md2 = 0.f;                         // the lists start from these positions
+            }
+        }
+        __syncthreads();
+        if (!(f & RF_REBUILD))
+            return f;
+    }
+}
+
+// The half kick and drift that open md_step.
+template <int P>
+__device__ __forceinline__ void run_first(const KArgs &a, RunState &S, float *shf)
+{
+    const int pp = S.pp, spar = S.spar;
+    float d2 = 0.f, v2 = 0.f, a2 = 0.f;
+    unsigned int bad = 0u;
+    for (int row = blockIdx.x; row < a.nblk_i; row += gridDim.x) {
+        const int4 b = a.blk_i[row];
+        const Rep rp = a.rep[b.z];
+        for (int i = b.x + threadIdx.x; i < b.y; i += blockDim.x) {
+            PState<P> s;
+            load_pos<P>(a, pp, i, s);
+            load_vel<P>(a, spar, i, s);
+            FT<P> f[3];
+            if constexpr (P == FP64) {
+                const d4 q = ((const d4 *)a.force)[i];
+                f[0] = q.x; f[1] = q.y; f[2] = q.z;
+            } else {
+                const float4 q = ((const float4 *)a.force)[i];
+                f[0] = q.x; f[1] = q.y; f[2] = q.z;
+            }
+            half_kick<P>(a, s, f[0], f[1], f[2]);
+            d2 = fmaxf(d2, drift<P>(a, rp, s, pp ^ 1, spar, i, bad));
+            v2 = fmaxf(v2, speed2(s));
+            const float im = a.inv_mass[s.sp];
+            a2 = fmaxf(a2, __fmul_rn(__fmul_rn(norm2(f[0], f[1], f[2]), im), im));
+            store_vel<P>(a, spar, i, s);
+        }
+    }
+    if (bad)
+        atomicOr(&a.ctl->status, bad);
+    block_max3(d2, v2, a2, shf);
+    if (threadIdx.x == 0)
+        put_maxima(a, S.step, d2, v2, a2);
+}
+
+// One sweep over the block's chunks: forces, the particles' update, and the
+// partial sums and maxima.
+template <int P, int TPP, bool SM, bool SAMPLE>
+__device__ __forceinline__ void run_chunks(const KArgs &a, RunState &S, RunSums &X, float *shf)
+{
+    X.d2[threadIdx.x] = X.v2[threadIdx.x] = X.a2[threadIdx.x] = 0.f;
+    ET<P> *xe = reinterpret_cast<ET<P> *>(X.e);
+    xe[threadIdx.x] = e_zero<P>();
+    if (SAMPLE && threadIdx.x < kPartF)
+        X.tot[threadIdx.x] = 0.0;
+    if ((int)blockIdx.x * a.cpb >= a.nrow)
+        return;                                      // (a block without chunks)
+    for (int q = 0; q < a.cpb; ++q) {
+        const int4 b = a.blk_r[blockIdx.x * a.cpb + q];
+        if (b.w < 0)                                 // (padding rows: the same for the whole block)
+            break;
+        double part[kPartF];
+        ET<P> eo;
+        float d2 = 0.f, v2 = 0.f, a2 = 0.f;
+        unsigned int bad = 0u;
+        step_body<P, TPP, SAMPLE, SM>(a, b, (a.what & RUN_STEPS) != 0, S.last != 0, S.pp, S.spar, part, eo, d2, v2, a2,
+                                      bad);
+        if (bad)
+            atomicOr(&a.ctl->status, bad);
+        X.d2[threadIdx.x] = fmaxf(X.d2[threadIdx.x], d2);
+        X.v2[threadIdx.x] = fmaxf(X.v2[threadIdx.x], v2);
+        X.a2[threadIdx.x] = fmaxf(X.a2[threadIdx.x], a2);
+        if (SAMPLE) {
+            block_sum<kPartF>(part, X.sh);
+            if (threadIdx.x == 0) {
+                double *p = a.nrep == 1 ? X.tot : a.part_f + part_index(a, S.step, b.w) * kPartF;
+#pragma unroll
+                for (int k = 1; k < kPartF; ++k)
+                    p[k] = a.nrep == 1 ? p[k] + part[k] : part[k];
+            }
+        }
+        if (a.nrep == 1) {
+            xe[threadIdx.x] = e_add(xe[threadIdx.x], eo);
+        } else {
+            float z0 = 0.f, z1 = 0.f, z2 = 0.f;
+            block_max3_sum1(z0, z1, z2, eo, shf, X.sh);
+            if (threadIdx.x == 0)
+                put_epart<P>(a, part_index(a, S.step, b.w), eo);
+        }
+    }
+    float d2 = X.d2[threadIdx.x], v2 = X.v2[threadIdx.x], a2 = X.a2[threadIdx.x];
+    ET<P> e = xe[threadIdx.x];
+    block_max3_sum1(d2, v2, a2, e, shf, X.sh);
+    if (threadIdx.x == 0) {
+        put_maxima(a, S.step, d2, v2, a2);
+        if (a.nrep == 1) {
+            put_epart<P>(a, part_index(a, S.step, blockIdx.x), e);
+            if (SAMPLE) {
+                double *p = a.part_f + part_index(a, S.step, blockIdx.x) * kPartF;
+#pragma unroll
+                for (int k = 1; k < kPartF; ++k)
+                    p[k] = X.tot[k];
+            }
         }
     }
 }
 
+// Sums of the step that awaits them, one block per replica, the last blocks of
+// the grid first: they have the fewest chunks (none, where blocks are to spare).
 template <int P>
-__global__ void __launch_bounds__(kNbBlock) k_nbuild(KArgs a)
+__device__ __forceinline__ void run_service(const KArgs &a, RunState &S, bool totals, double *sh, float *shf)
 {
-    __shared__ NbWarp s_nb[kNbCells];
-    __shared__ int s_go, s_K;
-    nbuild_begin(a, s_go, s_K);
-    __syncthreads();
-    if (s_go) {
-        const int pn = a.ctl->pos_par ^ 1;
-        const int w = threadIdx.x >> 5;
-        for (int c = blockIdx.x * kNbCells + w; c < a.ncell; c += gridDim.x * kNbCells)
-            nbuild_cell_warp<P>(a, pn, c, s_K, s_nb[w]);
+    if (S.pend < 0)
+        return;
+    for (int r = (int)gridDim.x - 1 - (int)blockIdx.x; r < a.nrep; r += gridDim.x) {
+        finish_replica<P>(a, r, S.pend, S.pend_sample != 0, totals, S.pend_obs % (long long)a.obs_cap, S.pend_md2,
+                          S.pend_rebuilds, sh, shf);
+        if (r == 0 && threadIdx.x == 0 && !totals)
+            a.epot_step[S.pend % a.epot_cap] = S.pend;
+    }
+}
+
+// Blocks of 128 threads per SM the unsmoothed single-precision kernels are
+// compiled for: 7 at <= 72 registers, so that 1024 chunks (KA N=65536 at 2 lanes
+// per particle) are one per block on 152 SMs.  FP64 and the smoothed kernels
+// keep the compiler's own register choice (they would spill).
+template <int P, bool SM> constexpr int run_min_blocks() { return P == FP64 ? 0 : SM ? 5 : 7; }
+
+template <int P, int TPP, bool SM>
+__global__ void __launch_bounds__(kForceBlock, run_min_blocks<P, SM>()) k_run(KArgs a)
+{
+    __shared__ union {
+        RunScratch nb;
+        RunSums step;
+    } X;
+    __shared__ float shf[160];
+    __shared__ RunState S;
+    double *sh = X.step.sh;
+    Ctl *ctl = a.ctl;
+    if (threadIdx.x == 0) {
+        S.step = ctl->step;
+        S.left = a.nsteps;
+        S.budget = a.budget;
+        S.obs = ctl->obs_count;
+        S.rebuilds = ctl->rebuilds;
+        S.regrows = ctl->regrows;
+        S.pend = -1;
+        S.pp = ctl->pos_par;
+        S.spar = ctl->state_par;
+        S.K = ctl->K;
+        S.pos = a.pos0;
+        S.md2 = ctl->last_maxdisp2;
+        S.count = a.rs->word >> 4;
+        S.ns = 0ull;
+        S.done = 0;
+        S.flags = ctl->status ? RF_STOP | RF_BAD : 0u;
     }
     __syncthreads();
-    nbuild_end(a, s_go, s_K);
+    // A status pending from before: no phase does work, but every block goes to
+    // the first barrier, which ends the launch.  (A block that comes late may see
+    // a status set by another one's first phase: that phase has failed, so its
+    // own share of it is not wanted either.)
+    const bool halted = S.flags != 0u;
+    unsigned int f = 0u;
+    if (a.what & RUN_REBUILD)
+        f = run_rebuild<P>(a, S, X.nb);
+    if (!(f & RF_STOP) && (a.what & RUN_FIRST)) {
+        if (!halted)
+            run_first<P>(a, S, shf);
+        f = grid_barrier(a, S, [&]() -> unsigned int {
+            float md2;
+            const bool reb = take_maxima(a, S.step, a.check - 1, md2);
+            if (atomicOr(&ctl->status, 0u))
+                return RF_STOP | RF_BAD;
+            ctl->last_maxdisp2 = md2;
+            return reb ? RF_REBUILD : 0u;
+        });
+        if (!(f & RF_BAD)) {
+            if (threadIdx.x == 0) {
+                S.step += 1;
+                S.pp ^= 1;
+                S.md2 = ctl->last_maxdisp2;
+            }
+            __syncthreads();
+            if ((f & RF_REBUILD) && !(a.what & RUN_DEFER))
+                f = run_rebuild<P>(a, S, X.nb);
+        }
+    }
+    const bool steps = (a.what & RUN_STEPS) != 0, record = (a.what & (RUN_STEPS | RUN_SAMPLE | RUN_TOTALS)) != 0;
+    if (!(f & RF_STOP) && (a.what & (RUN_STEPS | RUN_SAMPLE | RUN_TOTALS | RUN_FORCES))) {
+        for (;;) {
+            if (threadIdx.x == 0) {
+                S.last = !steps || (S.left == 1 && a.last);
+                S.sample = steps ? S.step % a.si == 0 : record;
+                if (blockIdx.x == 0)
+                    S.t0 = global_ns();
+            }
+            __syncthreads();
+            // the previous step's sums (its partials were complete at the last barrier)
+            run_service<P>(a, S, false, sh, shf);
+            if (halted) {
+                // (only the launch's first phase: its barrier ends the launch)
+            } else if (S.sample) {
+                run_chunks<P, TPP, SM, true>(a, S, X.step, shf);
+            } else {
+                run_chunks<P, TPP, SM, false>(a, S, X.step, shf);
+            }
+            f = grid_barrier(a, S, [&]() -> unsigned int {
+                float md2;
+                const int ci = a.check;
+                const bool check = steps && S.pos == ci - 1;
+                const bool reb = take_maxima(a, S.step, ci - 1, md2) && check && !S.last;
+                if (atomicOr(&ctl->status, 0u))
+                    return RF_STOP | RF_BAD;
+                if (!S.last)
+                    ctl->last_maxdisp2 = md2;
+                unsigned int g = reb ? RF_REBUILD : 0u;
+                if (!S.last && S.budget == 1) {
+                    atomicOr(&ctl->status, ST_TIMEOUT);
+                    g |= RF_STOP;
+                }
+                if (!steps || S.left == 1)
+                    g |= RF_STOP;
+                return g;
+            });
+            if (f & RF_ABORT)
+                return;
+            if (threadIdx.x == 0) {
+                S.pend = -1;
+                if (!(f & RF_BAD)) {
+                    // this step's sums: by the service blocks during the next one
+                    S.pend = record ? S.step : -1;
+                    S.pend_sample = S.sample;
+                    S.pend_obs = S.obs;
+                    S.pend_rebuilds = S.rebuilds;
+                    S.pend_md2 = S.md2;
+                    if (S.sample && !(a.what & RUN_TOTALS))
+                        S.obs += 1;
+                    if (!S.last) {
+                        S.step += 1;
+                        S.pp ^= 1;
+                        S.md2 = ctl->last_maxdisp2;
+                    }
+                    S.left -= 1;
+                    S.budget -= 1;
+                    S.pos = S.pos == a.check - 1 ? 0 : S.pos + 1;
+                }
+                if (blockIdx.x == 0) {
+                    const unsigned long long t = global_ns();
+                    S.ns += t > S.t0 ? t - S.t0 : 0ull;
+                }
+                S.done += 1;
+            }
+            __syncthreads();
+            if (f & RF_STOP) {
+                run_service<P>(a, S, (a.what & RUN_TOTALS) != 0, sh, shf);
+                break;
+            }
+            if (f & RF_REBUILD) {
+                f = run_rebuild<P>(a, S, X.nb);
+                if (f & RF_ABORT)
+                    return;
+                if (f & RF_STOP) {
+                    run_service<P>(a, S, false, sh, shf);
+                    break;
+                }
+            }
+        }
+    }
+    if (f & RF_ABORT)
+        return;
+    // the state of the handle, by one thread: the other blocks have passed their last barrier
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        ctl->step = S.step;
+        ctl->obs_count = S.obs;
+        ctl->rebuilds = S.rebuilds;
+        ctl->regrows = S.regrows;
+        ctl->pos_par = S.pp;
+        ctl->state_par = S.spar;
+        ctl->last_maxdisp2 = S.md2;
+        ctl->rebuild = (f & (RF_REBUILD | RF_BAD)) == RF_REBUILD;
+        ctl->n_kernels += 1;
+        if (steps) {
+            ctl->dev_ns += S.ns;
+            ctl->dev_launches += S.done;
+        }
+    }
+}
+
+// Kinetic energy and momentum of the current velocities per replica: into the
+// totals record (IM_TOTALS), or as rescale factors (IM_KE) in scale[], which
+// holds the target temperatures.  The last block adds up the blocks' sums, a
+// block per replica up to 8 replicas, a warp per replica beyond.
+__device__ __forceinline__ void put_kinetic(const KArgs &a, int r, const double *v)
+{
+    if (a.imode == IM_TOTALS) {
+        Obs o;
+        o.step = a.ctl->step;
+        o.e_pot = o.virial = 0.0;
+        for (int k = 0; k < 6; ++k)
+            o.w[k] = 0.0;
+        o.e_kin = v[0];
+        o.p[0] = v[1];
+        o.p[1] = v[2];
+        o.p[2] = v[3];
+        o.max_disp = 0.0;
+        o.rebuilds = a.ctl->rebuilds;
+        a.totals[r] = o;
+    } else {
+        const double dof = 3.0 * (double)a.rep[r].n - 3.0;
+        const double target = a.scale[r];
+        a.scale[r] = (v[0] > 0.0) ? sqrt(target * dof / (2.0 * v[0])) : 1.0;
+    }
 }
 
 template <int P>
-__global__ void __launch_bounds__(kNbBlockB) k_nbuild_blk(KArgs a)
+__global__ void __launch_bounds__(kIntBlock) k_kinetic(KArgs a)
 {
-    __shared__ int s_go, s_K;
-    nbuild_begin(a, s_go, s_K);
-    __syncthreads();
-    if (s_go) {
-        const int pn = a.ctl->pos_par ^ 1;
-        for (int c = blockIdx.x; c < a.ncell; c += gridDim.x)
-            nbuild_cell_block<P>(a, pn, c, s_K);
+    __shared__ double sh[32 * 4];
+    __shared__ int s_last;
+    Ctl *ctl = a.ctl;
+    const bool halted = ctl->status != 0u;
+    const int4 b = a.blk_i[blockIdx.x];
+    const int i = b.x + threadIdx.x;
+    double kin[4] = {0.0, 0.0, 0.0, 0.0};
+    if (i < b.y && !halted) {
+        PState<P> s;
+        load_pos<P>(a, ctl->pos_par, i, s);
+        load_vel<P>(a, ctl->state_par, i, s);
+        kinetic<P>(a, s, kin);
+    }
+    block_sum<4>(kin, sh);
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            a.part_i[(size_t)blockIdx.x * 4 + k] = kin[k];
+        __threadfence();
+        s_last = atomicAdd(&ctl->ticket, 1u) == gridDim.x - 1;
     }
     __syncthreads();
-    nbuild_end(a, s_go, s_K);
+    if (!s_last)
+        return;
+    __threadfence();
+    const bool block_each = a.nrep <= 8;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if (!halted)
+        for (int r = block_each ? 0 : w; r < a.nrep; r += block_each ? 1 : nw) {
+            const int b0 = a.rep[r].bi0, b1 = a.rep[r].bi1;
+            double v[4] = {0.0, 0.0, 0.0, 0.0};
+            for (int q = b0 + (block_each ? (int)threadIdx.x : lane); q < b1; q += block_each ? (int)blockDim.x : 32)
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    v[k] += a.part_i[(size_t)q * 4 + k];
+            if (block_each) {
+                block_sum<4>(v, sh);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    v[k] = warp_sum(v[k]);
+            }
+            if (block_each ? threadIdx.x == 0 : lane == 0)
+                put_kinetic(a, r, v);
+        }
+    if (threadIdx.x == 0) {
+        ctl->ticket = 0u;
+        ctl->n_kernels += 1;
+    }
 }
 
 template <int P>
 __global__ void __launch_bounds__(kIntBlock) k_load(KArgs a)
 {
     Ctl *ctl = a.ctl;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        ctl->rebuild = 1u;
-        atomicAdd((unsigned long long *)&ctl->n_other, 1ull);
-    }
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        atomicAdd((unsigned long long *)&ctl->n_kernels, 1ull);
     const int4 b = a.blk_i[blockIdx.x];
     const int i = b.x + threadIdx.x;
     if (i >= b.y)
@@ -2499,7 +2477,7 @@ __global__ void __launch_bounds__(kIntBlock) k_getstate(KArgs a)
     const Ctl *ctl = a.ctl;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (blockIdx.x == 0 && threadIdx.x == 0)
-        atomicAdd((unsigned long long *)&a.ctl->n_other, 1ull);
+        atomicAdd((unsigned long long *)&a.ctl->n_kernels, 1ull);
     if (s >= a.n)
         return;
     const int pp = ctl->pos_par, spar = ctl->state_par;
@@ -2535,7 +2513,7 @@ __global__ void __launch_bounds__(kIntBlock) k_expforce(KArgs a)
     const Ctl *ctl = a.ctl;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (blockIdx.x == 0 && threadIdx.x == 0)
-        atomicAdd((unsigned long long *)&a.ctl->n_other, 1ull);
+        atomicAdd((unsigned long long *)&a.ctl->n_kernels, 1ull);
     if (s >= a.n)
         return;
     const size_t t = (size_t)img_of(a, ctl->state_par)[s].w;
@@ -2561,7 +2539,7 @@ __global__ void __launch_bounds__(kIntBlock) k_scale(KArgs a)
     if (ctl->status)
         return;
     if (blockIdx.x == 0 && threadIdx.x == 0)
-        atomicAdd((unsigned long long *)&a.ctl->n_other, 1ull);
+        atomicAdd((unsigned long long *)&a.ctl->n_kernels, 1ull);
     const int4 b = a.blk_i[blockIdx.x];
     const int i = b.x + threadIdx.x;
     if (i >= b.y)
@@ -2587,25 +2565,16 @@ __global__ void __launch_bounds__(kIntBlock) k_scale(KArgs a)
     }
 }
 
-template <int P>
-__global__ void k_set_steps(KArgs a)
-{
-    a.ctl->remaining = a.nsteps;
-    a.ctl->budget = a.budget > 0 ? a.budget : a.nsteps + 64;
-    a.ctl->n_other += 1;
-}
-
 // clear a reported status so that the handle can be inspected and reused
 template <int P>
 __global__ void k_reset(KArgs a)
 {
     a.ctl->status = 0u;
     a.ctl->ticket = 0u;
-    a.ctl->maxdisp2 = 0u;
-    a.ctl->maxv2 = 0u;
-    a.ctl->maxa2 = 0u;
-    a.ctl->remaining = 0;
-    a.ctl->n_other += 1;
+    a.rs->arrive = 0u;
+    for (int k = 0; k < 8; ++k)
+        a.rs->m[k >> 2][k & 3] = 0u;
+    a.ctl->n_kernels += 1;
 }
 
 // ---------------------------------------------------------------------------
@@ -2688,7 +2657,7 @@ __global__ void __launch_bounds__(kIntBlock) k_andersen_fix(KArgs a)
     if (ctl->status)
         return;
     if (blockIdx.x == 0 && threadIdx.x == 0)
-        atomicAdd((unsigned long long *)&a.ctl->n_other, 1ull);
+        atomicAdd((unsigned long long *)&a.ctl->n_kernels, 1ull);
     const int4 b = a.blk_i[blockIdx.x];
     const int i = b.x + threadIdx.x;
     if (i >= b.y)
@@ -2726,7 +2695,7 @@ __global__ void __launch_bounds__(kIntBlock) k_snapshot(KArgs a)
 {
     const Ctl *ctl = a.ctl;
     if (blockIdx.x == 0 && threadIdx.x == 0)
-        atomicAdd((unsigned long long *)&a.ctl->n_other, 1ull);
+        atomicAdd((unsigned long long *)&a.ctl->n_kernels, 1ull);
     const int4 b = a.blk_i[blockIdx.x];
     const int i = b.x + threadIdx.x;
     if (i >= b.y)
@@ -2756,87 +2725,29 @@ __global__ void __launch_bounds__(kIntBlock) k_snapshot(KArgs a)
     a.snap_species[t] = sp;
 }
 
-// Sum the energies of a step that still awaits it into the per-step series
-// (before the host reads the series, and before a force evaluation outside
-// the step loop reuses the partials).  One block.
-template <int P>
-__global__ void __launch_bounds__(kForceBlock) k_epot_flush(KArgs a)
-{
-    __shared__ double sh[32 * kPartF];
-    __shared__ float shf[160];
-    const long long pend = a.ctl->epot_pending;
-    if (pend >= 0)
-        finish_epot<P>(a, pend, sh, shf);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        a.ctl->epot_pending = -1;
-        a.ctl->n_other += 1;
-    }
-}
-
-// request a list rebuild before the next force evaluation
-template <int P>
-__global__ void k_mark_rebuild(KArgs a)
-{
-    a.ctl->rebuild = 1u;
-    a.ctl->n_other += 1;
-}
-
 template <int P>
 KernelSet make_kernel_set()
 {
     KernelSet k;
-    k.integrate = (const void *)k_integrate<P>;
-    k.force[0][0] = (const void *)k_force<P, 1, false>;
-    k.force[0][1] = (const void *)k_force<P, 2, false>;
-    k.force[0][2] = (const void *)k_force<P, 4, false>;
-    k.force[0][3] = (const void *)k_force<P, 8, false>;
-    k.force[0][4] = (const void *)k_force<P, 16, false>;
-    k.force[0][5] = (const void *)k_force<P, 32, false>;
-    k.step[0][0] = (const void *)k_step<P, 1, false, false>;
-    k.step[0][1] = (const void *)k_step<P, 2, false, false>;
-    k.step[0][2] = (const void *)k_step<P, 4, false, false>;
-    k.step[0][3] = (const void *)k_step<P, 8, false, false>;
-    k.step[0][4] = (const void *)k_step<P, 16, false, false>;
-    k.step[0][5] = (const void *)k_step<P, 32, false, false>;
+    k.kinetic = (const void *)k_kinetic<P>;
+    k.run[0][0] = (const void *)k_run<P, 1, false>;
+    k.run[0][1] = (const void *)k_run<P, 2, false>;
+    k.run[0][2] = (const void *)k_run<P, 4, false>;
+    k.run[0][3] = (const void *)k_run<P, 8, false>;
+    k.run[0][4] = (const void *)k_run<P, 16, false>;
+    k.run[0][5] = (const void *)k_run<P, 32, false>;
     // smoothed potential (Sec. 4): the common lane counts only
-    k.force[1][0] = (const void *)k_force<P, 1, true>;
-    k.force[1][1] = (const void *)k_force<P, 2, true>;
-    k.force[1][2] = (const void *)k_force<P, 4, true>;
-    k.force[1][3] = (const void *)k_force<P, 8, true>;
-    k.force[1][4] = nullptr;
-    k.force[1][5] = nullptr;
-    k.step[1][0] = (const void *)k_step<P, 1, true, false>;
-    k.step[1][1] = (const void *)k_step<P, 2, true, false>;
-    k.step[1][2] = (const void *)k_step<P, 4, true, false>;
-    k.step[1][3] = (const void *)k_step<P, 8, true, false>;
-    k.step[1][4] = nullptr;
-    k.step[1][5] = nullptr;
-    // resident blocks sweeping runs of chunks: single-precision pair loops at 1 and 2 lanes
-    // (at 4 lanes the chunk loop costs registers and was measured slower)
-    for (int m = 0; m < 2; ++m)
-        for (int l = 0; l < 2; ++l)
-            k.step_sweep[m][l] = nullptr;
-    if constexpr (P != FP64) {
-        k.step_sweep[0][0] = (const void *)k_step<P, 1, false, true>;
-        k.step_sweep[0][1] = (const void *)k_step<P, 2, false, true>;
-        k.step_sweep[1][0] = (const void *)k_step<P, 1, true, true>;
-        k.step_sweep[1][1] = (const void *)k_step<P, 2, true, true>;
-    }
-    k.bin = (const void *)k_bin<P>;
-    k.scan = (const void *)k_scan<P>;
-    k.scatter = (const void *)k_scatter<P>;
-    k.permute = (const void *)k_permute<P>;
-    k.nbuild = (const void *)k_nbuild<P>;
-    k.nbuild_blk = (const void *)k_nbuild_blk<P>;
+    k.run[1][0] = (const void *)k_run<P, 1, true>;
+    k.run[1][1] = (const void *)k_run<P, 2, true>;
+    k.run[1][2] = (const void *)k_run<P, 4, true>;
+    k.run[1][3] = (const void *)k_run<P, 8, true>;
+    k.run[1][4] = nullptr;
+    k.run[1][5] = nullptr;
     k.load = (const void *)k_load<P>;
     k.getstate = (const void *)k_getstate<P>;
     k.expforce = (const void *)k_expforce<P>;
     k.scale = (const void *)k_scale<P>;
-    k.set_steps = (const void *)k_set_steps<P>;
     k.reset = (const void *)k_reset<P>;
-    k.mark_rebuild = (const void *)k_mark_rebuild<P>;
-    k.epot_flush = (const void *)k_epot_flush<P>;
     k.andersen = (const void *)k_andersen<P>;
     k.andersen_fix = (const void *)k_andersen_fix<P>;
     k.snapshot = (const void *)k_snapshot<P>;
