@@ -99,40 +99,43 @@ typedef struct {
     int32_t threads_per_particle; /* force-kernel lanes per particle: 0 = automatic (2 for MIXED
                                      and FP32, 4 for FP64), else a power of two in 1..32 (1..8
                                      with smooth_h > 0)                                          */
-    int32_t use_graph;        /* 1 = md_step runs as one CUDA graph with the rebuild branch and
-                                 the step loop decided on the device (default); 0 = plain
-                                 stream launches, for debugging and per-kernel timing          */
+    int32_t use_graph;        /* 1 = md_step is one launch with the rebuild branch and the step
+                                 loop decided on the device (default); 0 = a launch for every
+                                 step and rebuild, for debugging and per-phase timing; the
+                                 results are the same, bit for bit                             */
     int32_t reorder;          /* cell order in memory: 1 = Morton curve (default), 2 = Hilbert
                                  curve (the paper's reorder, Sec. 2.2), 0 = x-fastest           */
-    int32_t step_form;        /* blocks of the step kernel: 0 = automatic (form 2 when MIXED or
-                                 FP32 at 1 or 2 lanes per particle needs more blocks than the
-                                 GPU holds at once, else form 1), 1 = one block per chunk of
-                                 particles, 2 = only the resident blocks, each sweeping a run of
-                                 neighbouring chunks (MIXED or FP32 at 1 or 2 lanes only);
-                                 the results are the same either way, bit for bit            */
+    int32_t step_form;        /* how the chunks of particles are shared out: 0 = automatic (2 when
+                                 MIXED or FP32 at 1 or 2 lanes per particle has more chunks than
+                                 the GPU holds at once, else 1), 1 = a chunk at a time, 2 = runs
+                                 of neighbouring chunks (MIXED or FP32 at 1 or 2 lanes only).
+                                 Reported by md_info; the resident groups of threads sweep runs
+                                 of chunks wherever there are more chunks than groups, so the
+                                 results and the speed are the same either way                 */
     double  smooth_h;         /* h >= 0 of the smoothing of Sec. 4: every pair potential is
                                  multiplied by g(x) = x^4 / (1 + x^4), x = (r - r_c,ab) /
                                  (h sigma_ab), which makes it and its first two derivatives
                                  vanish at r_c; 0 = no smoothing (the paper uses h = 0.005).
                                  Not supported by md_forces_noalloc.                           */
-    int32_t check_interval;   /* MD steps between the rebuild checks of md_step's CUDA graph:
+    int32_t check_interval;   /* MD steps between the rebuild checks of md_step:
                                  1, 2, 4, 8 or 16; 0 = automatic (4 below 262,144 particles, 1
                                  from there).  Between checks the rebuild decision adds a bound
                                  on how far particles can still move (speed and acceleration
                                  over the unchecked steps), so a longer interval rebuilds
-                                 earlier; a check costs one conditional graph node           */
+                                 earlier; steps without a check need no maxima               */
     int32_t neigh_capacity_max; /* cap on the list entries per particle (rounded up to 8): the
                                  workspace holds this many; 0 = twice the starting capacity.
                                  Only a list longer than the cap is an error (MD_E_CAPACITY);
                                  neigh_capacity_max = neigh_capacity keeps the size fixed     */
     int32_t step_budget;      /* 0 = automatic.  > 0: md_step's device loop stops with
-                                 MD_E_TIMEOUT after this many step-kernel executions (its
+                                 MD_E_TIMEOUT after this many MD steps (its
                                  iteration bound; automatic = nsteps + 64), so the bounded-
                                  loop path can be exercised                                     */
     int32_t build_form;       /* neighbour build: 0 = automatic (one warp per cell when there
                                  are at least 8 cells per SM and at most 32 particles per cell
-                                 on average, else one block per cell), 1 = one warp per cell,
-                                 2 = one block per cell; the lists are the same either way     */
+                                 on average, else a group of 128 threads or several per cell),
+                                 1 = one warp per cell, 2 = groups; the lists are the same
+                                 either way                                                    */
 } md_params;
 
 /* one sample of the reductions of Sec. 2.2, per replica */
@@ -159,22 +162,21 @@ typedef struct {
     int64_t kernel_launches;  /* library kernels executed on the device since md_create         */
     int32_t max_neighbours;   /* largest list length at the last build                          */
     int32_t status;           /* pending device status (MD_OK if none)                          */
-    double  step_ms;          /* with use_graph = 0: summed CUDA-event time of the step kernel
-                                 (pair forces + velocity-Verlet update, one launch per step)   */
-    int64_t step_launches;    /* with use_graph = 0: step-kernel launches timed                 */
-    double  rebuild_ms;       /* with use_graph = 0: summed time of the rebuild chains (sort,
-                                 list build) launched when a check point asked for one         */
-    int64_t rebuild_checks;   /* with use_graph = 0: rebuild chains launched                    */
-    double  step_device_ms;   /* any mode: summed device duration of the step-kernel launches
-                                 that advanced a step (first block start to last block end,
-                                 read from the GPU's global timer)                              */
-    int64_t step_device_launches; /* launches summed into step_device_ms (one per MD step)      */
+    double  step_ms;          /* with use_graph = 0: summed CUDA-event time of the launches of
+                                 one MD step each (pair forces + velocity-Verlet update)       */
+    int64_t step_launches;    /* with use_graph = 0: step launches timed                        */
+    double  rebuild_ms;       /* with use_graph = 0: summed time of the rebuilds (sort, list
+                                 build) launched when a check point asked for one              */
+    int64_t rebuild_checks;   /* with use_graph = 0: rebuilds launched                          */
+    double  step_device_ms;   /* any mode: summed device duration of the MD steps, rebuilds
+                                 excluded (from one grid barrier to the next, read from the
+                                 GPU's global timer)                                            */
+    int64_t step_device_launches; /* MD steps summed into step_device_ms                        */
     int32_t check_interval;   /* MD steps between rebuild checks, as resolved                   */
     int32_t neigh_capacity_max; /* the cap on neigh_capacity, as resolved                       */
     int64_t regrows;          /* list builds redone with a larger capacity since md_create      */
-    int32_t build_form;       /* neighbour build in use: 1 = one warp per cell, 2 = one block   */
-    int32_t step_form;        /* step-kernel blocks in use: 1 = one per chunk, 2 = resident
-                                 blocks sweeping runs of chunks                                 */
+    int32_t build_form;       /* neighbour build in use: 1 = one warp per cell, 2 = groups      */
+    int32_t step_form;        /* sharing of chunks, as resolved                                 */
 } md_info_t;
 
 typedef struct md_handle md_handle;

@@ -47,7 +47,7 @@ namespace {
 
 constexpr size_t kAlign = 256;
 constexpr int kIntBlock = 256, kForceBlock = 128;
-constexpr int kMaxRunBlocks = 4096;    // bound on the run kernel's blocks (entries of KArgs::slice)
+constexpr int kMaxRunGroups = 4096;    // bound on the run kernel's groups (entries of KArgs::slice)
 constexpr int kNbWarpCellsPerSm = 8;                     // warp-per-cell build from this many cells per SM
 constexpr double kCellMargin = 1e-3;   // cell edge exceeds the largest list radius by this
 constexpr int kUnroll = 16;            // largest check interval
@@ -65,7 +65,7 @@ struct Geometry {
     bool nb_block = false;              // neighbour build with one block per cell
     int nblk_i = 0, nblk_f = 0, ncell = 0;
     bool sweep = false;                 // step_form as reported: more chunks than resident blocks
-    int nblk_r = 0, nwork = 0, cpb = 1; // run kernel: blocks launched, of them with chunks, chunks per block
+    int groups = 1, nwork = 0, cpb = 1; // run kernel: groups per block, groups with chunks, chunks per group
     double rl_max = 0.0;
     std::vector<mdk::Rep> rep;
     std::vector<int4> blk_i, blk_f;
@@ -76,7 +76,7 @@ struct Geometry {
 struct Layout {
     size_t off_ctl, off_rep, off_blk_i, off_blk_f, off_blk_r, off_crank, off_cxyz;
     size_t off_pa, off_pb, off_va, off_vb, off_pa2, off_pb2, off_va2, off_vb2, off_qa, off_qb, off_force;
-    size_t off_rref, off_image, off_image2, off_key, off_tmpidx, off_skey;
+    size_t off_rref, off_image, off_image2, off_key, off_tmpidx;
     size_t off_ccount, off_ccursor, off_cstart, off_nbr, off_nnbr, off_part_f, off_part_i, off_part_e;
     size_t off_ring, off_totals, off_scale, off_st_pos, off_st_vel, off_st_img, off_st_code;
     size_t off_epot, off_epot_step, off_rs, off_slice;
@@ -338,7 +338,7 @@ Layout make_layout(const md_params *p, const Geometry &g)
     L.off_blk_f = take(sizeof(int4) * g.nblk_f);
     L.off_blk_r = take(sizeof(int4) * 2 * (size_t)g.nblk_f);   // < nblk_f + resident blocks rows
     L.off_rs = take(sizeof(mdk::RunSync));
-    L.off_slice = take(sizeof(int) * kMaxRunBlocks);
+    L.off_slice = take(sizeof(int) * kMaxRunGroups);
     L.off_crank = take(sizeof(int) * g.ncell);
     L.off_cxyz = take(sizeof(int4) * g.ncell);
     L.off_pa = take(pb * n);
@@ -355,9 +355,8 @@ Layout make_layout(const md_params *p, const Geometry &g)
     L.off_rref = take(16 * n);
     L.off_image = take(16 * n);
     L.off_image2 = take(16 * n);
-    L.off_key = take(4 * n);
-    L.off_tmpidx = take(4 * n);
-    L.off_skey = take(4 * n);
+    L.off_key = take(8 * n);
+    L.off_tmpidx = take(8 * n);
     L.off_ccount = take(4 * (size_t)g.ncell);
     L.off_ccursor = take(4 * (size_t)g.ncell);
     L.off_cstart = take(4 * ((size_t)g.ncell + 1));
@@ -408,6 +407,7 @@ struct md_handle {
     char *ws = nullptr;
     KArgs a;
     const KernelSet *ks = nullptr;
+    int nsm = 0;                     // blocks of the run kernel: one per SM
     const void *runk = nullptr;      // the run kernel in use: precision, lanes per particle, smoothing
     int cap = 4096;
     // pinned host staging
@@ -468,7 +468,8 @@ int launch_run(md_handle *h, int what, int64_t nsteps = 0, int64_t budget = 0, i
     a.pos0 = pos0;
     a.last = last ? 1 : 0;
     void *pp[1] = {(void *)&a};
-    CK(h, cudaLaunchCooperativeKernel(h->runk, dim3((unsigned)h->g.nblk_r), dim3(kForceBlock), pp, 0, h->s));
+    CK(h, cudaLaunchCooperativeKernel(h->runk, dim3((unsigned)h->nsm), dim3((unsigned)(kForceBlock * h->g.groups)), pp,
+                                      (size_t)h->g.groups * (size_t)h->ks->group_smem, h->s));
     return MD_OK;
 }
 
@@ -716,9 +717,8 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
     a.rref = (float4 *)(w + L.off_rref);
     a.image = (int4 *)(w + L.off_image);
     a.image2 = (int4 *)(w + L.off_image2);
-    a.key = (int *)(w + L.off_key);
-    a.tmpidx = (int *)(w + L.off_tmpidx);
-    a.skey = (int *)(w + L.off_skey);
+    a.key = (int2 *)(w + L.off_key);
+    a.tmpidx = (int2 *)(w + L.off_tmpidx);
     a.ccount = (int *)(w + L.off_ccount);
     a.ccursor = (int *)(w + L.off_ccursor);
     a.cstart = (int *)(w + L.off_cstart);
@@ -798,14 +798,20 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
     if (a.hdtm_hi[0] == 0.0f)
         return fail(h, MD_E_INVAL, "dt / (2 m) underflows single precision");
 
-    int dev = 0, nsm = 0, per_sm = 0;
+    int dev = 0, nsm = 0, per_sm = 0, resident = 0;
     CK(h, cudaGetDevice(&dev));
     CK(h, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     h->runk = h->ks->run[h->p.smooth_h > 0.0][force_index(g.tpp)];
-    CK(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, h->runk, kForceBlock, 0));
-    if (per_sm < 1 || nsm < 1)
+    const int most = std::min(h->ks->groups[h->p.smooth_h > 0.0], kMaxRunGroups / std::max(nsm, 1));
+    if (most < 1)
         return fail(h, MD_E_CUDA, "the run kernel does not fit the device");
-    per_sm = std::min(per_sm, kMaxRunBlocks / nsm);
+    CK(h, cudaFuncSetAttribute(h->runk, cudaFuncAttributeMaxDynamicSharedMemorySize, most * h->ks->group_smem));
+    CK(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, h->runk, kForceBlock * most,
+                                                        (size_t)most * (size_t)h->ks->group_smem));
+    if (resident < 1)
+        return fail(h, MD_E_CUDA, "the run kernel does not fit the device");
+    per_sm = most;
+    h->nsm = nsm;
     const bool one_each = g.nblk_f <= nsm * per_sm;   // a block for every chunk
     h->g.sweep = p->step_form == 2 || (p->step_form == 0 && !one_each && p->precision != MD_PREC_FP64 && g.tpp <= 2);
     // the build takes a warp per cell when there are at least kNbWarpCellsPerSm cells per SM
@@ -815,7 +821,7 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
     h->g.nb_block = p->build_form == 2 ||
                     (p->build_form == 0 && ((int64_t)g.ncell < (int64_t)kNbWarpCellsPerSm * nsm ||
                                             (double)g.n > 32.0 * (double)g.ncell));
-    h->a.nb_block = h->g.nb_block ? 1 : 0;
+    h->a.nb_warp = h->g.nb_block ? 0 : 1;
     // pinned staging, events
     CK(h, cudaEventCreateWithFlags(&h->ev_stage, cudaEventDisableTiming));
     CK(h, cudaEventCreate(&h->ev_f0));
@@ -842,9 +848,13 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
         h->a.cpb = h->g.cpb;
         h->a.nrow = (int)br.size();
         h->a.nslot = g.R == 1 ? h->g.nwork : g.nblk_f;
-        // blocks without chunks, where the GPU holds more than there are chunks: they add up
-        // the steps' partial sums, a replica each
-        h->g.nblk_r = std::min(nsm * per_sm, h->g.nwork + std::min(g.R, nsm));
+        // groups without chunks, where the GPU holds more than there are chunks, add up the
+        // steps' partial sums, a replica each; in a rebuild a group takes a cell (or a share of
+        // one where cells are few)
+        const int parts = std::max(1, std::min(8, 4 * nsm / g.ncell));
+        const int want = std::max(h->g.nwork + std::min(g.R, nsm), g.ncell < kMaxRunGroups ? g.ncell * parts : kMaxRunGroups);
+        h->g.groups = std::min(per_sm, (want + nsm - 1) / nsm);
+        h->a.nb_parts = std::max(1, std::min(8, nsm * h->g.groups / g.ncell));
         if ((rc = put(L.off_rep, g.rep.data(), sizeof(mdk::Rep) * g.R)) ||
             (rc = put(L.off_blk_i, g.blk_i.data(), sizeof(int4) * g.nblk_i)) ||
             (rc = put(L.off_blk_f, bf.data(), sizeof(int4) * g.nblk_f)) ||
@@ -860,7 +870,7 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
             return rc;
         cudaError_t e = cudaMemsetAsync(a.ccount, 0, 4 * (size_t)g.ncell, h->s);
         if (e == cudaSuccess)
-            e = cudaMemsetAsync(a.slice, 0, sizeof(int) * kMaxRunBlocks, h->s);
+            e = cudaMemsetAsync(a.slice, 0, sizeof(int) * kMaxRunGroups, h->s);
         if (e == cudaSuccess)
             e = cudaMemsetAsync(a.rs, 0, sizeof(mdk::RunSync), h->s);
         if (e == cudaSuccess)   // every slot of the per-step series empty (step -1)

@@ -52,8 +52,6 @@ struct Ctl {
     long long n_kernels;      // kernel executions
     unsigned long long dev_ns;        // summed device duration of the MD steps of the run kernel
     long long dev_launches;           // MD steps summed into dev_ns
-    float last_maxdisp2;
-    float pad1;
     long long regrows;        // builds redone with a larger K since md_create
 };
 
@@ -62,7 +60,9 @@ struct RunSync {
     unsigned int arrive, pad0[31];   // blocks that have reached the running barrier
     unsigned int word, pad1[31];     // (barriers passed << 4) | what the last one decided (RunFlag)
     unsigned int m[2][4], pad2[24];  // float bits of the largest squared displacement, speed and
-                                     // acceleration of a step, by the parity of the step
+                                     // acceleration of a step, and its ST_* bits, by the parity of the step
+    float md2[2];                    // largest squared displacement since the build, by the parity of
+    unsigned int unit, pad3[29];     //   the positions' step; next unit of the build
 };
 
 struct Rep {                  // one independent system
@@ -104,7 +104,7 @@ struct KArgs {
     int check;                        // MD steps between rebuild checks
     int pos0;                         // position of the first step of this launch in its md_step
     int last;                         // this launch ends its md_step
-    int nb_block;                     // neighbour build: a block per cell (else a warp per cell)
+    int nb_warp, nb_parts;            // neighbour build: a warp per cell, or nb_parts groups per cell
     int nslot, nrow;                  // slots of the partial sums (per parity), rows of blk_r
     void *pa, *pb, *va, *vb;          // buffer 0: MIXED pos hi/lo, vel hi/lo (float4);
                                       // FP64 pos, vel (d4); FP32 pos, vel (float4)
@@ -114,8 +114,8 @@ struct KArgs {
     void *force;                      // float4 (MIXED, FP32) or d4 (FP64): f.xyz, e_i in w
     float4 *rref;                     // positions at the last list build
     int4 *image, *image2;             // image counters (w = original index), by state_par
-    int *key, *ccount, *cstart, *ccursor, *tmpidx;
-    int *skey;                        // sub-cell code of each particle (order inside its cell)
+    int2 *key, *tmpidx;               // (cell, sub-cell code) by particle; (particle, sub-cell code) by slot
+    int *ccount, *cstart, *ccursor;
     const int *crank;                 // [global linear cell] -> global sorted cell id
     const int4 *cxyz;                 // [global sorted cell id] -> cx, cy, cz, replica
     int *nbr, *nnbr;
@@ -207,6 +207,7 @@ __device__ __forceinline__ ds ds_from_double(double x)
 // table of kernel entry addresses for one precision (one translation unit each)
 struct KernelSet {
     const void *run[2][6];            // [smoothed][log2 lanes per particle]
+    int groups[2], group_smem;        // run kernel: most groups of a block, shared memory of one
     const void *kinetic, *load, *getstate, *expforce, *scale, *reset;
     const void *andersen, *andersen_fix, *snapshot;
 };

@@ -17,12 +17,13 @@
 // other one.  Velocities and images are double-buffered by Ctl::state_par,
 // which changes only when a rebuild permutes the particles.
 //
-// One MD step = one launch of k_step: pair forces over the neighbour list,
-// then, per particle, the velocity-Verlet half kick that completes v(t), the
-// kinetic sample, the half kick that starts the next step and the drift
-// (Sec. 2.2).  Its last block finishes the reductions and decides, with a
-// bound on how far particles can move before the next check, whether the
-// lists must be rebuilt (the displacement criterion of Sec. 2.2).
+// One kernel, k_run, does all of md_step in one cooperative launch (one block
+// per SM): the opening half kick and drift, the MD steps -- pair forces over
+// the neighbour list, then, per particle, the velocity-Verlet half kick that
+// completes v(t), the kinetic sample, the half kick that starts the next step
+// and the drift (Sec. 2.2) --, and the list rebuilds that the displacement
+// criterion of Sec. 2.2 calls for.  Force evaluations outside md_step are
+// launches of the same kernel.
 #pragma once
 
 #include <type_traits>
@@ -32,9 +33,7 @@
 namespace mdk {
 
 constexpr int kIntBlock = 256;   // per-particle kernels: one thread per particle
-constexpr int kForceBlock = 128; // force / step kernels: tpp threads per particle
-constexpr int kNbCells = kForceBlock / 32;   // neighbour build, warp per cell: cells per block
-constexpr int kNbBlockB = kForceBlock;   // neighbour build, block per cell: threads per block
+constexpr int kForceBlock = 128; // run kernel: threads of a group (tpp threads per particle)
 constexpr int kPartF = 12;       // doubles per block partial of the force / step kernels
 constexpr int kUnr = 8;          // list entries per lane and iteration of the FP32 pair loops
                                  // (a multiple of 4, at most 8: lists are padded to 8)
@@ -63,6 +62,21 @@ __device__ __forceinline__ int checked(const KArgs &a, int i, int n, int safe)
 }
 
 // ---------------------------------------------------------------------------
+// Groups of kForceBlock threads.  The run kernel launches one block per SM and
+// splits it into groups that work like blocks of their own (a chunk of particles
+// or a cell each), synchronised by a named barrier each; only the grid barrier
+// joins them, so it has one arrival and one poller per SM.
+// ---------------------------------------------------------------------------
+struct Grp {
+    int id, vb, nvb;                   // group of the block, of the grid, groups in the grid
+    __device__ __forceinline__ static int tid() { return threadIdx.x & (kForceBlock - 1); }
+    __device__ __forceinline__ void sync() const
+    {
+        asm volatile("bar.sync %0, %1;" ::"r"(id + 1), "n"(kForceBlock) : "memory");
+    }
+};
+
+// ---------------------------------------------------------------------------
 // small helpers
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ unsigned long long global_ns()
@@ -72,12 +86,10 @@ __device__ __forceinline__ unsigned long long global_ns()
     return t;
 }
 
+// maximum of non-negative floats (NaN counts as 0): their bits order like them
 __device__ __forceinline__ float warp_max(float v)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(v, 0.f))));
 }
 
 __device__ __forceinline__ double warp_sum(double v)
@@ -113,10 +125,40 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double *sh)
     __syncthreads();
 }
 
-// Maxima of three non-negative floats over the block; valid in thread 0.
-__device__ __forceinline__ void block_max3(float &a, float &b, float &c, float *sh)
+// Sum of NV doubles over a group in a fixed order; valid in its thread 0.
+// sh: kGrpWarps*NV doubles.  Every thread of the group must call it.
+constexpr int kGrpWarps = kForceBlock / 32;
+
+template <int NV>
+__device__ __forceinline__ void grp_sum(const Grp &g, double (&v)[NV], double *sh)
 {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, w = g.tid() >> 5;
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+        v[k] = warp_sum(v[k]);
+    if (lane == 0) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k)
+            sh[w * NV + k] = v[k];
+    }
+    g.sync();
+    if (g.tid() == 0) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            double x = sh[k];
+#pragma unroll
+            for (int u = 1; u < kGrpWarps; ++u)
+                x += sh[u * NV + k];
+            v[k] = x;
+        }
+    }
+    g.sync();
+}
+
+// Maxima of three non-negative floats over a group; valid in its thread 0.
+__device__ __forceinline__ void grp_max3(const Grp &g, float &a, float &b, float &c, float *sh)
+{
+    const int lane = threadIdx.x & 31, w = g.tid() >> 5;
     a = warp_max(a);
     b = warp_max(b);
     c = warp_max(c);
@@ -125,72 +167,44 @@ __device__ __forceinline__ void block_max3(float &a, float &b, float &c, float *
         sh[3 * w + 1] = b;
         sh[3 * w + 2] = c;
     }
-    __syncthreads();
-    if (w == 0) {
-        a = warp_max(lane < nw ? sh[3 * lane] : 0.f);
-        b = warp_max(lane < nw ? sh[3 * lane + 1] : 0.f);
-        c = warp_max(lane < nw ? sh[3 * lane + 2] : 0.f);
+    g.sync();
+    if (g.tid() == 0) {
+#pragma unroll
+        for (int u = 1; u < kGrpWarps; ++u) {
+            a = fmaxf(a, sh[3 * u]);
+            b = fmaxf(b, sh[3 * u + 1]);
+            c = fmaxf(c, sh[3 * u + 2]);
+        }
     }
-    __syncthreads();
 }
 
-// Maxima of three non-negative floats and the sum of one double over the
-// block, valid in thread 0, with one pair of barriers.  The sum takes the
-// same steps as component 0 of block_sum (so a per-step potential energy
-// equals the one of a sample record bit for bit).
-__device__ __forceinline__ void block_max3_sum1(float &a, float &b, float &c, double &e, float *shf, double *sh)
+// Sum of the energies over a group, in double or double-single (FP32
+// arithmetic): warps by shuffles in a fixed butterfly order, then the warps'
+// sums in order; valid in thread 0.  shf: 2 floats per warp (8-byte aligned).
+__device__ __forceinline__ double e_warp(double e) { return warp_sum(e); }
+__device__ __forceinline__ ds e_warp(ds e)
 {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    a = warp_max(a);
-    b = warp_max(b);
-    c = warp_max(c);
-    e = warp_sum(e);
-    if (lane == 0) {
-        shf[3 * w] = a;
-        shf[3 * w + 1] = b;
-        shf[3 * w + 2] = c;
-        sh[w] = e;
-    }
-    __syncthreads();
-    if (w == 0) {
-        a = warp_max(lane < nw ? shf[3 * lane] : 0.f);
-        b = warp_max(lane < nw ? shf[3 * lane + 1] : 0.f);
-        c = warp_max(lane < nw ? shf[3 * lane + 2] : 0.f);
-        e = warp_sum(lane < nw ? sh[lane] : 0.0);
-    }
-    __syncthreads();
-}
-
-// The same with the energy sum in double-single (FP32 arithmetic): warps add
-// by shuffles in a fixed butterfly order, then warp 0 adds the warps' sums.
-// shf: 3 * 32 + 2 * 32 floats.
-__device__ __forceinline__ void block_max3_sum1(float &a, float &b, float &c, ds &e, float *shf, double *)
-{
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    a = warp_max(a);
-    b = warp_max(b);
-    c = warp_max(c);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1)
         e = ds_add(e, ds_from(__shfl_xor_sync(0xffffffffu, e.hi, o), __shfl_xor_sync(0xffffffffu, e.lo, o)));
-    if (lane == 0) {
-        shf[3 * w] = a;
-        shf[3 * w + 1] = b;
-        shf[3 * w + 2] = c;
-        shf[96 + 2 * w] = e.hi;
-        shf[97 + 2 * w] = e.lo;
-    }
-    __syncthreads();
-    if (w == 0) {
-        a = warp_max(lane < nw ? shf[3 * lane] : 0.f);
-        b = warp_max(lane < nw ? shf[3 * lane + 1] : 0.f);
-        c = warp_max(lane < nw ? shf[3 * lane + 2] : 0.f);
-        e = lane < nw ? ds_from(shf[96 + 2 * lane], shf[97 + 2 * lane]) : ds_from(0.f, 0.f);
+    return e;
+}
+__device__ __forceinline__ double e_add(double x, double y) { return x + y; }
+__device__ __forceinline__ ds e_add(ds x, ds y) { return ds_add(x, y); }
+
+template <class E>
+__device__ __forceinline__ void grp_esum(const Grp &g, E &e, float *shf)
+{
+    E *sh = reinterpret_cast<E *>(shf);
+    e = e_warp(e);
+    if ((threadIdx.x & 31) == 0)
+        sh[g.tid() >> 5] = e;
+    g.sync();
+    if (g.tid() == 0) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-            e = ds_add(e, ds_from(__shfl_xor_sync(0xffffffffu, e.hi, o), __shfl_xor_sync(0xffffffffu, e.lo, o)));
+        for (int u = 1; u < kGrpWarps; ++u)
+            e = e_add(e, sh[u]);
     }
-    __syncthreads();
 }
 
 __device__ __forceinline__ int species_of(float w) { return __float_as_int(w) & 15; }
@@ -466,13 +480,13 @@ __device__ __forceinline__ float speed2(const PState<FP32> &s) { return norm2f(s
 
 // r += dt v, wrapped into [0, L) with image counting; writes the new position
 // into buffer `dst`, updates the image counter in the state buffers `spar`,
-// returns the squared displacement since the last list build.
+// returns the squared displacement since the last list build (if wanted: `track`).
 template <int P>
-__device__ __forceinline__ float drift(const KArgs &a, const Rep &rp, PState<P> &s, int dst, int spar, int i,
+__device__ __forceinline__ float drift(const KArgs &a, const Rep &rp, PState<P> &s, int dst, int spar, int i, bool track,
                                        unsigned int &bad)
 {
     int ix, iy, iz;
-    float dd;
+    float dd = 0.f;
     if constexpr (P == MIXED) {
         const ds dt = ds_from(a.dt_hi, a.dt_lo);
         const ds sx = ds_mul(dt, s.vx), sy = ds_mul(dt, s.vy), sz = ds_mul(dt, s.vz);
@@ -491,11 +505,13 @@ __device__ __forceinline__ float drift(const KArgs &a, const Rep &rp, PState<P> 
         ((float4 *)pos_b(a, dst))[i] = s.l;
         q_of(a, dst)[i] = make_int4((int)fixq(s.H.x, s.l.x, rp), (int)fixq(s.H.y, s.l.y, rp),
                                     (int)fixq(s.H.z, s.l.z, rp), s.sp);
-        const float4 rr = a.rref[i];
-        const float ex = __fadd_rn(sep_f(s.H.x, rr.x, rp.Lhi, rp.invLf), s.l.x);
-        const float ey = __fadd_rn(sep_f(s.H.y, rr.y, rp.Lhi, rp.invLf), s.l.y);
-        const float ez = __fadd_rn(sep_f(s.H.z, rr.z, rp.Lhi, rp.invLf), s.l.z);
-        dd = norm2f(ex, ey, ez);
+        if (track) {
+            const float4 rr = a.rref[i];
+            const float ex = __fadd_rn(sep_f(s.H.x, rr.x, rp.Lhi, rp.invLf), s.l.x);
+            const float ey = __fadd_rn(sep_f(s.H.y, rr.y, rp.Lhi, rp.invLf), s.l.y);
+            const float ez = __fadd_rn(sep_f(s.H.z, rr.z, rp.Lhi, rp.invLf), s.l.z);
+            dd = norm2f(ex, ey, ez);
+        }
     } else if constexpr (P == FP64) {
         const double sx = __dmul_rn(a.dt, s.vx), sy = __dmul_rn(a.dt, s.vy), sz = __dmul_rn(a.dt, s.vz);
         const double lim = 0.25 * rp.L;
@@ -510,11 +526,13 @@ __device__ __forceinline__ float drift(const KArgs &a, const Rep &rp, PState<P> 
             bad |= ST_NONFINITE;
         s.x.x = x; s.x.y = y; s.x.z = z;
         ((d4 *)pos_a(a, dst))[i] = s.x;
-        const float4 rr = a.rref[i];
-        const float ex = sep_f(__double2float_rn(x), rr.x, rp.Lhi, rp.invLf);
-        const float ey = sep_f(__double2float_rn(y), rr.y, rp.Lhi, rp.invLf);
-        const float ez = sep_f(__double2float_rn(z), rr.z, rp.Lhi, rp.invLf);
-        dd = norm2f(ex, ey, ez);
+        if (track) {
+            const float4 rr = a.rref[i];
+            const float ex = sep_f(__double2float_rn(x), rr.x, rp.Lhi, rp.invLf);
+            const float ey = sep_f(__double2float_rn(y), rr.y, rp.Lhi, rp.invLf);
+            const float ez = sep_f(__double2float_rn(z), rr.z, rp.Lhi, rp.invLf);
+            dd = norm2f(ex, ey, ez);
+        }
     } else {
         const float dt = a.dt_hi;
         const float sx = __fmul_rn(dt, s.vx), sy = __fmul_rn(dt, s.vy), sz = __fmul_rn(dt, s.vz);
@@ -535,11 +553,13 @@ __device__ __forceinline__ float drift(const KArgs &a, const Rep &rp, PState<P> 
             bad |= ST_NONFINITE;
         s.x.x = x; s.x.y = y; s.x.z = z;
         ((float4 *)pos_a(a, dst))[i] = s.x;
-        const float4 rr = a.rref[i];
-        const float ex = sep_f(x, rr.x, L, rp.invLf);
-        const float ey = sep_f(y, rr.y, L, rp.invLf);
-        const float ez = sep_f(z, rr.z, L, rp.invLf);
-        dd = norm2f(ex, ey, ez);
+        if (track) {
+            const float4 rr = a.rref[i];
+            const float ex = sep_f(x, rr.x, L, rp.invLf);
+            const float ey = sep_f(y, rr.y, L, rp.invLf);
+            const float ez = sep_f(z, rr.z, L, rp.invLf);
+            dd = norm2f(ex, ey, ez);
+        }
     }
     if (ix | iy | iz) {
         int4 *im = img_of(a, spar);
@@ -587,21 +607,18 @@ __device__ __forceinline__ ET<P> get_epart(const KArgs &a, size_t k)
     }
 }
 
-__device__ __forceinline__ double e_add(double x, double y) { return x + y; }
-__device__ __forceinline__ ds e_add(ds x, ds y) { return ds_add(x, y); }
-
-// The reductions of replica r at `step` from its slots' partials, by one whole
-// block, in a fixed order (thread t adds partials t, t + blockDim, ..., then the
-// block's tree): the potential energy into the per-step series and, for a
+// The reductions of replica r at `step` from its slots' partials, by one
+// group, in a fixed order (thread t adds partials t, t + 128, ..., then the
+// group's tree): the potential energy into the per-step series and, for a
 // sample, the record into the ring or (totals) into the totals array.
 template <int P>
-__device__ void finish_replica(const KArgs &a, int r, long long step, bool sample, bool totals, long long slot,
+__device__ void finish_replica(const KArgs &a, const Grp &g, int r, long long step, bool sample, bool totals, long long slot,
                                float md2, long long rebuilds, double *sh, float *shf)
 {
     const int s0 = a.nrep == 1 ? 0 : a.rep[r].bf0, s1 = a.nrep == 1 ? a.nslot : a.rep[r].bf1;
     ET<P> e = e_zero<P>();
-    int b = s0 + threadIdx.x;
-    const int st = blockDim.x;
+    int b = s0 + g.tid();
+    const int st = kForceBlock;
     for (; b + 7 * st < s1; b += 8 * st) {
         ET<P> x[8];
 #pragma unroll
@@ -613,25 +630,26 @@ __device__ void finish_replica(const KArgs &a, int r, long long step, bool sampl
     }
     for (; b < s1; b += st)
         e = e_add(e, get_epart<P>(a, part_index(a, step, b)));
-    float d0 = 0.f, d1 = 0.f, d2 = 0.f;
-    block_max3_sum1(d0, d1, d2, e, shf, sh);
+    grp_esum(g, e, shf);
     const double epot = e_value(e);
-    if (threadIdx.x == 0 && !totals)
+    if (g.tid() == 0 && !totals)
         a.epot[(step % a.epot_cap) * a.nrep + r] = epot;
-    if (!sample)
+    if (!sample) {
+        g.sync();                                    // (shf is written again)
         return;
+    }
     double v[kPartF];
 #pragma unroll
     for (int k = 0; k < kPartF; ++k)
         v[k] = 0.0;
-    for (int b2 = s0 + threadIdx.x; b2 < s1; b2 += st) {
+    for (int b2 = s0 + g.tid(); b2 < s1; b2 += st) {
         const double *p = a.part_f + part_index(a, step, b2) * kPartF;
 #pragma unroll
         for (int k = 1; k < kPartF; ++k)
             v[k] += p[k];
     }
-    block_sum<kPartF>(v, sh);
-    if (threadIdx.x == 0) {
+    grp_sum<kPartF>(g, v, sh);
+    if (g.tid() == 0) {
         Obs o;
         o.step = step;
         o.e_pot = epot;
@@ -786,7 +804,8 @@ __device__ __forceinline__ void pair_forces(const KArgs &a, const Rep &rp, int p
 #pragma unroll
             for (int w = 0; w < kUnr / 4; ++w) {
                 const int k = kUnr * lane + d * kStride;
-                pf[d][w] = k < nn ? *(const int4 *)(lst + k + 4 * w) : make_int4(0, 0, 0, 0);
+                // (the first ones without waiting for the row's length)
+                pf[d][w] = k < (d == 0 ? a.Kstride : nn) ? *(const int4 *)(lst + k + 4 * w) : make_int4(0, 0, 0, 0);
             }
         for (int k0 = kUnr * lane; k0 < nn; k0 += kStride) {
             int jj[kUnr];
@@ -1133,14 +1152,14 @@ __device__ __forceinline__ void component_update(const KArgs &a, const Rep &rp, 
 // position buffer.  The operands of the update are loaded before the
 // neighbour loop so that their latency is hidden.
 template <int P, int TPP, bool SAMPLE, bool SM>
-__device__ __forceinline__ void step_body_split(const KArgs &a, const int4 b, bool kick, bool last,
+__device__ __forceinline__ void step_body_split(const KArgs &a, const Rep &rep, const int4 b, bool kick, bool last, bool track,
                                                 int pp, int spar, double *part, ET<P> &eo, float &d2, float &v2, float &a2,
                                                 unsigned int &bad)
 {
     constexpr int NC = TPP >= 4 ? 1 : 4 / TPP;
-    const Rep rp = a.rep[b.z];
+    const Rep rp = rep;
     const int lane = threadIdx.x & (TPP - 1);
-    const int i = b.x + (int)(threadIdx.x / TPP);
+    const int i = b.x + Grp::tid() / TPP;
     const bool valid = i < b.y;
     const int ii = valid ? i : b.x;
     const int nn = valid ? a.nnbr[ii] : 0;
@@ -1254,17 +1273,17 @@ __device__ __forceinline__ void step_body_split(const KArgs &a, const int4 b, bo
 }
 
 template <int P, int TPP, bool SAMPLE, bool SM>
-__device__ __forceinline__ void step_body(const KArgs &a, const int4 b, bool kick, bool last,
+__device__ __forceinline__ void step_body(const KArgs &a, const Rep &rep, const int4 b, bool kick, bool last, bool track,
                                           int pp, int spar, double *part, ET<P> &eo, float &d2, float &v2, float &a2,
                                           unsigned int &bad)
 {
     if constexpr (kSplitUpdate || TPP >= 4) {
-        step_body_split<P, TPP, SAMPLE, SM>(a, b, kick, last, pp, spar, part, eo, d2, v2, a2, bad);
+        step_body_split<P, TPP, SAMPLE, SM>(a, rep, b, kick, last, track, pp, spar, part, eo, d2, v2, a2, bad);
         return;
     }
-    const Rep rp = a.rep[b.z];
+    const Rep rp = rep;
     const int lane = threadIdx.x & (TPP - 1);
-    const int i = b.x + (int)(threadIdx.x / TPP);
+    const int i = b.x + Grp::tid() / TPP;
     const bool valid = i < b.y;
     const int ii = valid ? i : b.x;
     const int nn = valid ? a.nnbr[ii] : 0;
@@ -1294,7 +1313,7 @@ __device__ __forceinline__ void step_body(const KArgs &a, const int4 b, bool kic
         kinetic<P>(a, s, part + 8);
     if (!last) {
         half_kick<P>(a, s, fx, fy, fz);             // v(t + 1/2)
-        d2 = drift<P>(a, rp, s, pp ^ 1, spar, i, bad);
+        d2 = drift<P>(a, rp, s, pp ^ 1, spar, i, track, bad);
         v2 = speed2(s);
         const float im = a.inv_mass[s.sp];
         a2 = __fmul_rn(__fmul_rn(norm2(fx, fy, fz), im), im);
@@ -1367,30 +1386,27 @@ __device__ __forceinline__ int cell_of(const KArgs &a, const Rep &rp, int pp, in
     return checked(a, a.crank[rp.cell0 + (cz * rp.nc + cy) * rp.nc + cx], a.ncell, 0);
 }
 
-// Phase 1: cell keys, histogram, and the particles in each block's slice of
-// slice_cells consecutive cells.
+// Phase 1: cell keys and histogram.
 template <int P>
-__device__ __forceinline__ void rebuild_bin(const KArgs &a, int pp, int slice_cells)
+__device__ __forceinline__ void rebuild_bin(const KArgs &a, const Grp &g, int pp)
 {
-    for (int row = blockIdx.x; row < a.nblk_i; row += gridDim.x) {
+    for (int row = g.vb; row < a.nblk_i; row += g.nvb) {
         const int4 b = a.blk_i[row];
         const Rep &rp = a.rep[b.z];
-        for (int i = b.x + threadIdx.x; i < b.y; i += blockDim.x) {
+        for (int i = b.x + g.tid(); i < b.y; i += kForceBlock) {
             int sub;
             const int key = cell_of<P>(a, rp, pp, i, sub);
-            a.key[i] = key;
-            a.skey[i] = sub;
+            a.key[i] = make_int2(key, sub);
             atomicAdd(&a.ccount[key], 1);
-            atomicAdd(&a.slice[key / slice_cells], 1);
         }
     }
 }
 
-// Exclusive prefix sum of one value per thread over the block; `total` gets the
+// Exclusive prefix sum of one value per thread over the group; `total` gets the
 // sum.  sh: one int per warp.
-__device__ __forceinline__ int block_scan(int v, int &total, int *sh)
+__device__ __forceinline__ int grp_scan(const Grp &g, int v, int &total, int *sh)
 {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, w = g.tid() >> 5, nw = kGrpWarps;
     int incl = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -1400,54 +1416,73 @@ __device__ __forceinline__ int block_scan(int v, int &total, int *sh)
     }
     if (lane == 31)
         sh[w] = incl;
-    __syncthreads();
+    g.sync();
     int before = 0, sum = 0;
     for (int k = 0; k < nw; ++k) {
         before += k < w ? sh[k] : 0;
         sum += sh[k];
     }
-    __syncthreads();
+    g.sync();
     total = sum;
     return before + incl - v;
 }
 
-// Phase 2: first particle of every cell.  Each block adds up the slices before
-// its own, then scans its slice; the counts are cleared for the next binning.
-__device__ __forceinline__ void rebuild_scan(const KArgs &a, int slice_cells, int *sh)
+// Phase 2: first particle of every cell.  Each group scans a slice of
+// slice_cells consecutive cells, after the particles of the cells before it,
+// added up from the counts themselves, or beyond kScanDirect cells from the
+// slices' sums (a barrier more); the counts are
+// cleared for the next binning in the phase after.
+constexpr int kScanDirect = 8192;
+
+__device__ __forceinline__ void rebuild_slices(const KArgs &a, const Grp &g, int slice_cells, int *sh)
 {
-    const int c0 = blockIdx.x * slice_cells, c1 = min(c0 + slice_cells, a.ncell);
+    const int c0 = g.vb * slice_cells, c1 = min(c0 + slice_cells, a.ncell);
+    int v = 0, sum;
+    for (int c = c0 + g.tid(); c < c1; c += kForceBlock)
+        v += a.ccount[c];
+    grp_scan(g, v, sum, sh);
+    if (g.tid() == 0)
+        a.slice[g.vb] = sum;
+}
+
+__device__ __forceinline__ void rebuild_scan(const KArgs &a, const Grp &g, int slice_cells, int *sh)
+{
+    const int c0 = g.vb * slice_cells, c1 = min(c0 + slice_cells, a.ncell);
     if (c0 >= a.ncell)
         return;
     int before = 0, carry;
-    for (int b = threadIdx.x; b < (int)blockIdx.x; b += blockDim.x)
-        before += a.slice[b];
-    block_scan(before, carry, sh);
-    for (int base = c0; base < c1; base += blockDim.x) {
-        const int c = base + threadIdx.x;
+    const int *from = a.ncell > kScanDirect ? a.slice : a.ccount;
+    const int upto = a.ncell > kScanDirect ? g.vb : c0;
+#pragma unroll 8
+    for (int b = g.tid(); b < upto; b += kForceBlock)
+        before += from[b];
+    grp_scan(g, before, carry, sh);
+    for (int base = c0; base < c1; base += kForceBlock) {
+        const int c = base + g.tid();
         const int v = c < c1 ? a.ccount[c] : 0;
         int sum;
-        const int at = carry + block_scan(v, sum, sh);
+        const int at = carry + grp_scan(g, v, sum, sh);
         if (c < c1) {
             a.cstart[c] = at;
-            a.ccount[c] = 0;
             a.ccursor[c] = 0;
         }
         carry += sum;
     }
-    if (threadIdx.x == 0 && c1 == a.ncell)
+    if (g.tid() == 0 && c1 == a.ncell)
         a.cstart[a.ncell] = carry;
 }
 
 // Phase 3: particles into their cells, in any order.
-__device__ __forceinline__ void rebuild_scatter(const KArgs &a)
+__device__ __forceinline__ void rebuild_scatter(const KArgs &a, const Grp &g)
 {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += gridDim.x * blockDim.x) {
-        const int k = checked(a, a.key[i], a.ncell, 0);
+    for (int i = g.vb * kForceBlock + g.tid(); i < a.n; i += g.nvb * kForceBlock) {
+        const int2 key = a.key[i];
+        const int k = checked(a, key.x, a.ncell, 0);
         const int slot = checked(a, a.cstart[k] + atomicAdd(&a.ccursor[k], 1), a.n, 0);
-        a.tmpidx[slot] = i;
+        a.tmpidx[slot] = make_int2(i, key.y);
     }
-    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < (int)gridDim.x; b += gridDim.x * blockDim.x)
-        a.slice[b] = 0;                                  // ready for the next binning
+    for (int c = g.vb * kForceBlock + g.tid(); c < a.ncell; c += g.nvb * kForceBlock)
+        a.ccount[c] = 0;                                 // ready for the next binning
 }
 
 // Phase 4: final slot of each particle: its cell's start plus the number of
@@ -1455,18 +1490,18 @@ __device__ __forceinline__ void rebuild_scatter(const KArgs &a)
 // index) order (deterministic), then gather of the whole state into the other
 // buffers.
 template <int P>
-__device__ __forceinline__ void rebuild_permute(const KArgs &a, int pp, int spar)
+__device__ __forceinline__ void rebuild_permute(const KArgs &a, const Grp &g, int pp, int spar)
 {
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < a.n; s += gridDim.x * blockDim.x) {
-        const int i = checked(a, a.tmpidx[s], a.n, 0);
-        const int k = checked(a, a.key[i], a.ncell, 0);
+    for (int s = g.vb * kForceBlock + g.tid(); s < a.n; s += g.nvb * kForceBlock) {
+        const int2 me = a.tmpidx[s];
+        const int i = checked(a, me.x, a.n, 0);
+        const int k = checked(a, a.key[i].x, a.ncell, 0);
         const int b0 = a.cstart[k], b1 = a.cstart[k + 1];
-        const int si = a.skey[i];
         int rank = 0;
+#pragma unroll 8
         for (int t = b0; t < b1; ++t) {
-            const int j = checked(a, a.tmpidx[t], a.n, 0);
-            const int sj = a.skey[j];
-            rank += (sj < si || (sj == si && j < i)) ? 1 : 0;
+            const int2 other = a.tmpidx[t];
+            rank += (other.y < me.y || (other.y == me.y && other.x < i)) ? 1 : 0;
         }
         const int d = checked(a, b0 + rank, a.n, 0);
         if constexpr (P == FP64) {
@@ -1490,191 +1525,498 @@ __device__ __forceinline__ void rebuild_permute(const KArgs &a, int pp, int spar
 }
 
 // ---------------------------------------------------------------------------
-// Neighbour-list build (Sec. 2.2), one warp per cell, one lane per particle
-// of the cell (batches of 32).  The warp stages the particles of the 27
-// surrounding cells (all cells of the replica when fewer than three fit along
-// its edge) in shared memory, in a fixed order (stencil order, then slot order
-// inside a cell), dropping those farther than the largest list radius from
-// the cell's own box; then every lane tests the staged candidates one after
-// the other (each read is a broadcast) against its own particle and appends
-// those closer than r_c,ab + skin (plus a rounding margin) to its row of the
-// particle-major list nbr[i*Kstride + k], in that order, one store per entry
-// kept (the L2 merges the row's words).  No block
-// barrier: the cells of a block never wait for one another.  Distances are
-// single precision: from the fixed-point copy in MIXED mode, from the
-// (rounded) positions otherwise; the list only has to contain every pair
-// within r_c + skin, and the margin covers the rounding.  Reads the permuted
-// positions (other buffer).  More candidates than fit in shared memory, or
-// more particles in the cell than 32, are processed in rounds, so no cell
-// size is too large.
+// Neighbour-list build (Sec. 2.2), one group of threads per cell (or several, each
+// taking a share of the cell's particles, where cells are few).  The group
+// stages the particles of the 27 surrounding cells (all cells of the replica
+// when fewer than three fit along its edge) in shared memory, in a fixed order
+// (stencil order, then slot order inside a cell), as single-precision
+// coordinates relative to the cell's centre, dropping those farther than the
+// largest list radius from the cell's own box.  Each warp then takes its
+// particles two at a time, its lanes the candidates, two per lane and
+// iteration: the distance test of two candidates is six packed instructions,
+// and one ballot per 32 candidates places the entries kept in the row, in
+// candidate order, with stores that run along the row.  Rows are particle-major,
+// nbr[i*Kstride + k], and hold every partner closer than r_c,ab + skin (plus a
+// rounding margin: the list only has to contain every pair within r_c + skin,
+// and the margin covers the rounding).  Reads the permuted positions (other
+// buffer).  More candidates or own particles than fit are processed in rounds.
+//
+// Measured against a warp per cell with the particles as lanes (every lane
+// testing the same candidate, a scattered store per entry kept): the test loop
+// takes half the instructions per particle, and the stores are coalesced.
 // ---------------------------------------------------------------------------
-constexpr int kNbStage = 128;    // staged candidates per round and warp
+constexpr int kNbCap = 896;      // staged candidates per round (a multiple of 64)
+constexpr int kNbGrp = 7;        // groups of up to 32 candidates a warp stages at once
+constexpr int kNbOwn = 256;      // own-cell particles per batch
+constexpr int kNbPass = 2;       // own-cell particles tested per warp pass over the candidates
+constexpr int kNbChunks = 256;   // groups of up to 32 particles of one stencil cell per round of staging
 
-struct NbWarp {
-    float4 pos[kNbStage];
-    int idx[kNbStage];
-    int cell[27];
+struct NbBlock {
+    float2 x[kNbCap / 2], y[kNbCap / 2], z[kNbCap / 2];   // candidates c, c + 32 side by side
+    int2 w[kNbCap / 2];                                   // index | species << 31
+    int cnt[kNbOwn];
+    int c0[kNbChunks], c1[kNbChunks];
+    int nchunk, max_nbr;
+    int wsum[kForceBlock / 32];
 };
 
-// Position word staged by the neighbour build: MIXED stages the fixed-point copy
-// (bits of X, Y, Z, species), whose wrapped differences give the exact minimum
-// image; the other modes the single-precision position and species bits.
-constexpr bool kNbFixed = true;
+// Word of particle j for the build: coordinates relative to `ctr` (nearest
+// image) and index with the species in the sign bit.
+struct NbCentre { float x, y, z; unsigned int qx, qy, qz; };
 
 template <int P>
-__device__ __forceinline__ float4 nb_word(const KArgs &a, int pn, int j)
+__device__ __forceinline__ NbCentre nb_centre(const Rep &rp, const int4 &cc)
 {
-    if constexpr (P == MIXED && kNbFixed) {
+    NbCentre c;
+    const float edge = rp.Lhi / (float)rp.nc;
+    c.x = ((float)cc.x + 0.5f) * edge;
+    c.y = ((float)cc.y + 0.5f) * edge;
+    c.z = ((float)cc.z + 0.5f) * edge;
+    // the same on the fixed-point circle
+    c.qx = (unsigned int)((((unsigned long long)(2 * cc.x + 1)) << 31) / (unsigned int)rp.nc);
+    c.qy = (unsigned int)((((unsigned long long)(2 * cc.y + 1)) << 31) / (unsigned int)rp.nc);
+    c.qz = (unsigned int)((((unsigned long long)(2 * cc.z + 1)) << 31) / (unsigned int)rp.nc);
+    return c;
+}
+
+template <int P>
+__device__ __forceinline__ float3 nb_rel(const KArgs &a, const Rep &rp, const NbCentre &c, int pn, int j, int &sp)
+{
+    if constexpr (P == MIXED) {
         const int4 q = q_of(a, pn)[j];
-        return make_float4(__int_as_float(q.x), __int_as_float(q.y), __int_as_float(q.z), __int_as_float(q.w));
+        sp = q.w;
+        return make_float3(sep_q((unsigned int)q.x, c.qx, rp.qunit), sep_q((unsigned int)q.y, c.qy, rp.qunit),
+                           sep_q((unsigned int)q.z, c.qz, rp.qunit));
     } else if constexpr (P == FP64) {
         const d4 x = ((const d4 *)pos_a(a, pn))[j];
-        return make_float4(__double2float_rn(x.x), __double2float_rn(x.y), __double2float_rn(x.z),
-                           __int_as_float(species_of(x.w)));
+        sp = species_of(x.w);
+        return make_float3(sep_f(__double2float_rn(x.x), c.x, rp.Lhi, rp.invLf),
+                           sep_f(__double2float_rn(x.y), c.y, rp.Lhi, rp.invLf),
+                           sep_f(__double2float_rn(x.z), c.z, rp.Lhi, rp.invLf));
     } else {
-        return ((const float4 *)pos_a(a, pn))[j];
+        const float4 x = ((const float4 *)pos_a(a, pn))[j];
+        sp = species_of(x.w);
+        return make_float3(sep_f(x.x, c.x, rp.Lhi, rp.invLf), sep_f(x.y, c.y, rp.Lhi, rp.invLf),
+                           sep_f(x.z, c.z, rp.Lhi, rp.invLf));
     }
 }
 
-template <int P>
-__device__ __forceinline__ int nb_species(float4 w)
+// Particle range of the lane's stencil cell (lanes beyond the stencil: empty).
+__device__ __forceinline__ void nb_stencil(const KArgs &a, const Rep &rp, const int4 &cc, int nst, int &s0, int &s1)
 {
-    if constexpr (P == MIXED && kNbFixed)
-        return __float_as_int(w.w);
-    else
-        return species_of(w.w);
-}
-
-// approximate coordinates of a staged word (for the candidate filter)
-template <int P>
-__device__ __forceinline__ float3 nb_coords(float4 w, const Rep &rp)
-{
-    if constexpr (P == MIXED && kNbFixed)
-        return make_float3(__uint2float_rn(__float_as_uint(w.x)) * rp.qunit,
-                           __uint2float_rn(__float_as_uint(w.y)) * rp.qunit,
-                           __uint2float_rn(__float_as_uint(w.z)) * rp.qunit);
-    else
-        return make_float3(w.x, w.y, w.z);
-}
-
-// squared minimum-image distance of two staged words; for the fixed-point
-// words in units of the grid (qunit^2), which the caller's radii are scaled to
-template <int P>
-__device__ __forceinline__ float nb_r2(float4 u, float4 w, const Rep &rp)
-{
-    float ex, ey, ez;
-    if constexpr (P == MIXED && kNbFixed) {
-        ex = __int2float_rn((int)(__float_as_uint(u.x) - __float_as_uint(w.x)));
-        ey = __int2float_rn((int)(__float_as_uint(u.y) - __float_as_uint(w.y)));
-        ez = __int2float_rn((int)(__float_as_uint(u.z) - __float_as_uint(w.z)));
-    } else {
-        ex = sep_f(u.x, w.x, rp.Lhi, rp.invLf);
-        ey = sep_f(u.y, w.y, rp.Lhi, rp.invLf);
-        ez = sep_f(u.z, w.z, rp.Lhi, rp.invLf);
-    }
-    return fmaf(ex, ex, fmaf(ey, ey, ez * ez));
-}
-
-// distance of x from the interval [c - h, c + h] on a periodic axis
-__device__ __forceinline__ float box_gap(float x, float c, float h, float L, float invL)
-{
-    return fmaxf(fabsf(sep_f(x, c, L, invL)) - h, 0.0f);
-}
-
-// Warp per cell: the lists of the particles of cell c, from the positions in
-// buffer pn (the permuted copy being built), by one warp: row i starts at nbr[i * Kstride]
-// (the cap) and holds at most K entries (the capacity in use).  Every
-// particle's full count is recorded in max_nbr; entries beyond K are dropped
-// (the build's last block then grows K and the build is redone).
-template <int P>
-__device__ __forceinline__ void nbuild_cell_warp(const KArgs &a, int pn, int c, int K, NbWarp &S)
-{
-    constexpr unsigned FULL = 0xffffffffu;
-    Ctl *ctl = a.ctl;
-    const int lane = threadIdx.x & 31;
-    const int4 cc = a.cxyz[c];
-    const Rep rp = a.rep[cc.w];
-    const int nc = rp.nc;
-    const int nst = nc >= 3 ? 27 : 1;
-    const int c0 = a.cstart[c], c1 = a.cstart[c + 1];
-    if (c0 == c1)
-        return;
+    const int lane = threadIdx.x & 31, nc = rp.nc;
+    s0 = s1 = 0;
     if (lane < nst) {
         int x = cc.x, y = cc.y, z = cc.z;
         if (nst == 27) {
-            x = (x + lane % 3 - 1 + nc) % nc;
-            y = (y + (lane / 3) % 3 - 1 + nc) % nc;
-            z = (z + lane / 9 - 1 + nc) % nc;
+            x += lane % 3 - 1;
+            y += (lane / 3) % 3 - 1;
+            z += lane / 9 - 1;
+            x += x < 0 ? nc : (x >= nc ? -nc : 0);
+            y += y < 0 ? nc : (y >= nc ? -nc : 0);
+            z += z < 0 ? nc : (z >= nc ? -nc : 0);
         }
-        S.cell[lane] = a.crank[rp.cell0 + (z * nc + y) * nc + x];
+        const int k = a.crank[rp.cell0 + (z * nc + y) * nc + x];
+        s0 = a.cstart[k];
+        s1 = a.cstart[k + 1];
     }
-    __syncwarp();
+}
 
-    // own cell box (centre, half edge) for the candidate filter
-    const float edge = rp.Lhi / (float)nc;
-    const float hx = 0.5f * edge + 1e-3f;
-    const float ccx = ((float)cc.x + 0.5f) * edge, ccy = ((float)cc.y + 0.5f) * edge,
-                ccz = ((float)cc.z + 0.5f) * edge;
+// Test of the staged candidates against the batch's particles.  WRAP: fewer
+// than three cells along the edge, where the nearest image relative to the
+// centre need not be the nearest image relative to a particle (from three cells
+// on, a pair within the list radius lies less than half a box from the centre).
+template <int P, bool WRAP>
+__device__ __forceinline__ void nbuild_scan(const KArgs &a, const Grp &g, const Rep &rp, const NbCentre &ctr, int pn, int ob, int nown,
+                                            int staged, int K, NbBlock &S)
+{
+    constexpr int NW = kForceBlock / 32;
+    const int lane = threadIdx.x & 31;
+    const unsigned lt_mask = (1u << lane) - 1u;
+    for (int o0 = (g.tid() >> 5) * kNbPass; o0 < nown; o0 += NW * kNbPass) {
+        float2 hx[kNbPass], hy[kNbPass], hz[kNbPass];
+        float rl0[kNbPass], rl1[kNbPass];
+        int cnt[kNbPass], wi[kNbPass];
+        int *row[kNbPass];
+#pragma unroll
+        for (int p = 0; p < kNbPass; ++p) {
+            const bool ok = o0 + p < nown;
+            const int i = ob + (ok ? o0 + p : o0);
+            int sp;
+            const float3 r = nb_rel<P>(a, rp, ctr, pn, i, sp);
+            hx[p] = make_float2(-r.x, -r.x);
+            hy[p] = make_float2(-r.y, -r.y);
+            hz[p] = make_float2(-r.z, -r.z);
+            rl0[p] = ok ? a.tab.rl2[sp * 2] : -1.0f;              // -1: nothing passes
+            rl1[p] = ok ? a.tab.rl2[sp * 2 + 1] : -1.0f;
+            cnt[p] = S.cnt[ok ? o0 + p : o0];
+            wi[p] = i | (sp << 31);
+            row[p] = a.nbr + (size_t)i * (size_t)a.Kstride;
+        }
+        for (int s = lane; s < staged / 2; s += 32) {             // (staged is a multiple of 64 here)
+            const float2 X = S.x[s], Y = S.y[s], Z = S.z[s];
+            const int2 W = S.w[s];
+#pragma unroll
+            for (int p = 0; p < kNbPass; ++p) {
+                float2 dx = __fadd2_rn(X, hx[p]), dy = __fadd2_rn(Y, hy[p]), dz = __fadd2_rn(Z, hz[p]);
+                if (WRAP) {
+                    dx.x = fmaf(-rintf(dx.x * rp.invLf), rp.Lhi, dx.x);
+                    dx.y = fmaf(-rintf(dx.y * rp.invLf), rp.Lhi, dx.y);
+                    dy.x = fmaf(-rintf(dy.x * rp.invLf), rp.Lhi, dy.x);
+                    dy.y = fmaf(-rintf(dy.y * rp.invLf), rp.Lhi, dy.y);
+                    dz.x = fmaf(-rintf(dz.x * rp.invLf), rp.Lhi, dz.x);
+                    dz.y = fmaf(-rintf(dz.y * rp.invLf), rp.Lhi, dz.y);
+                }
+                const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+                const bool in0 = r2.x < (W.x < 0 ? rl1[p] : rl0[p]) && W.x != wi[p];
+                const bool in1 = r2.y < (W.y < 0 ? rl1[p] : rl0[p]) && W.y != wi[p];
+                const unsigned m0 = __ballot_sync(0xffffffffu, in0), m1 = __ballot_sync(0xffffffffu, in1);
+                const int at0 = cnt[p] + __popc(m0 & lt_mask);
+                const int at1 = cnt[p] + __popc(m0) + __popc(m1 & lt_mask);
+                if (in0 && at0 < K)
+                    row[p][at0] = W.x & 0x7fffffff;
+                if (in1 && at1 < K)
+                    row[p][at1] = W.y & 0x7fffffff;
+                cnt[p] += __popc(m0) + __popc(m1);
+            }
+        }
+        if (lane == 0)
+#pragma unroll
+            for (int p = 0; p < kNbPass; ++p)
+                if (o0 + p < nown)
+                    S.cnt[o0 + p] = cnt[p];
+    }
+}
+
+// Lists of the share [part, part + 1) / nparts of the particles of cell c, from
+// the positions in buffer pn (the permuted copy being built): row i holds at
+// most K entries (the capacity in use).  The longest full count is recorded in
+// max_nbr; entries beyond K are dropped (K then grows and the build is redone).
+template <int P>
+__device__ __forceinline__ void nbuild_cell(const KArgs &a, const Grp &g, int pn, int c, int part, int nparts, int K, NbBlock &S)
+{
+    const int tid = g.tid(), lane = tid & 31, warp = tid >> 5;
+    constexpr int NW = kForceBlock / 32;
+    const int4 cc = a.cxyz[c];
+    const int first = a.cstart[c], ncell = a.cstart[c + 1] - first;
+    const int lo = first + (int)((long long)ncell * part / nparts);
+    const int hi = first + (int)((long long)ncell * (part + 1) / nparts);
+    if (lo == hi)
+        return;
+    const Rep rp = a.rep[cc.w];
+    const int nc = rp.nc;
+    const int nst = nc >= 3 ? 27 : 1;
+    const NbCentre ctr = nb_centre<P>(rp, cc);
+    const float hx = 0.5f * rp.Lhi / (float)nc + 1e-3f;           // half edge of the cell's box
     const float rlmax2 = fmaxf(fmaxf(a.tab.rl2[0], a.tab.rl2[1]), fmaxf(a.tab.rl2[2], a.tab.rl2[3]));
     const unsigned lt_mask = (1u << lane) - 1u;
-    // nb_r2 of the fixed-point words is in units of qunit^2: the list radii follow
-    const float r2unit = (P == MIXED && kNbFixed) ? 1.0f / (rp.qunit * rp.qunit) : 1.0f;
+
+    int s0, s1;
+    nb_stencil(a, rp, cc, nst, s0, s1);
+
+    for (int ob = lo; ob < hi; ob += kNbOwn) {
+        const int nown = min(kNbOwn, hi - ob);
+        for (int t = tid; t < nown; t += kForceBlock)
+            S.cnt[t] = 0;
+        if (tid == 0)
+            S.max_nbr = 0;
+        int staged = 0;
+        // groups of up to 32 particles of one stencil cell, in stencil order; the table
+        // holds kNbChunks of them at a time (a cell of more than 32 kNbChunks / 27
+        // particles is taken in several rounds)
+        int at = s0;                                              // next particle of the lane's cell
+        bool more = true;
+        while (more) {
+            const int want = min((s1 - at + 31) / 32, kNbChunks / 32);
+            // in order: a lane's cell is complete before a later one's begins
+            const unsigned left = __ballot_sync(0xffffffffu, (s1 - at + 31) / 32 > want);
+            const int stop = left ? __ffs(left) - 1 : 31;         // lanes up to this one take part
+            const int mine = lane <= stop ? want : 0;
+            int incl = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o)
+                    incl += y;
+            }
+            const int nchunk = __shfl_sync(0xffffffffu, incl, 31);
+            if (warp == 0)
+                for (int k = 0; k < mine; ++k) {
+                    S.c0[incl - mine + k] = at + 32 * k;
+                    S.c1[incl - mine + k] = min(at + 32 * k + 32, s1);
+                }
+            at += 32 * mine;
+            at = min(at, s1);
+            more = left != 0u;
+            g.sync();
+            // the block's warps take kNbGrp consecutive groups each, all loads in flight, and
+            // write what they keep behind what the warps before them keep
+            for (int m0 = 0; m0 < nchunk; m0 += NW * kNbGrp) {
+                float3 r[kNbGrp];
+                int wj[kNbGrp];
+                unsigned keep[kNbGrp];
+                int n = 0;
+#pragma unroll
+                for (int u = 0; u < kNbGrp; ++u) {
+                    const int m = m0 + warp * kNbGrp + u;
+                    bool ok = false;
+                    wj[u] = 0;
+                    if (m < nchunk) {
+                        const int j = S.c0[m] + lane;
+                        if (j < S.c1[m]) {
+                            int sp;
+                            r[u] = nb_rel<P>(a, rp, ctr, pn, checked(a, j, a.n, 0), sp);
+                            wj[u] = j | (sp << 31);
+                            ok = true;
+                        }
+                    }
+                    if (!ok)
+                        r[u] = make_float3(1e9f, 0.f, 0.f);       // (never kept)
+                }
+#pragma unroll
+                for (int u = 0; u < kNbGrp; ++u) {
+                    bool ok = r[u].x < 1e8f;
+                    if (nst == 27) {
+                        const float gx = fmaxf(fabsf(r[u].x) - hx, 0.f), gy = fmaxf(fabsf(r[u].y) - hx, 0.f),
+                                    gz = fmaxf(fabsf(r[u].z) - hx, 0.f);
+                        ok = fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < rlmax2;
+                    }
+                    keep[u] = __ballot_sync(0xffffffffu, ok);
+                    n += __popc(keep[u]);
+                }
+                if (lane == 0)
+                    S.wsum[warp] = n;
+                g.sync();
+                int off = staged, add = 0;
+#pragma unroll
+                for (int w = 0; w < NW; ++w) {
+                    off += w < warp ? S.wsum[w] : 0;
+                    add += S.wsum[w];
+                }
+#pragma unroll
+                for (int u = 0; u < kNbGrp; ++u) {
+                    if (keep[u] >> lane & 1u) {
+                        const int s = off + __popc(keep[u] & lt_mask);
+                        const int t = (s >> 6) * 32 + (s & 31), h = (s >> 5) & 1;
+                        (&S.x[t].x)[h] = r[u].x;
+                        (&S.y[t].x)[h] = r[u].y;
+                        (&S.z[t].x)[h] = r[u].z;
+                        (&S.w[t].x)[h] = wj[u];
+                    }
+                    off += __popc(keep[u]);
+                }
+                staged += add;
+                if (staged <= kNbCap - 32 * NW * kNbGrp && (more || m0 + NW * kNbGrp < nchunk)) {
+                    g.sync();
+                    continue;
+                }
+                // fill up to a multiple of 64 with candidates that fail every test
+                const int full = (staged + 63) / 64 * 64;
+                for (int s = staged + tid; s < full; s += kForceBlock) {
+                    const int t = (s >> 6) * 32 + (s & 31), h = (s >> 5) & 1;
+                    (&S.x[t].x)[h] = (&S.y[t].x)[h] = (&S.z[t].x)[h] = __int_as_float(0x7fc00000);   // NaN
+                    (&S.w[t].x)[h] = 0;
+                }
+                g.sync();
+                if (nst == 27)
+                    nbuild_scan<P, false>(a, g, rp, ctr, pn, ob, nown, full, K, S);
+                else
+                    nbuild_scan<P, true>(a, g, rp, ctr, pn, ob, nown, full, K, S);
+                staged = 0;
+                g.sync();
+            }
+            g.sync();                                      // (the table is written again)
+        }
+        for (int o = tid; o < nown; o += kForceBlock) {
+            const int cnt = S.cnt[o], kept = cnt < K ? cnt : K;
+            a.nnbr[ob + o] = kept;
+            // pad the row with the particle itself to a multiple of kUnr entries, so the
+            // pair loop reads whole groups without masking (K is a multiple of 8)
+            for (int k = kept; k < (kept + kUnr - 1) / kUnr * kUnr && k < K; ++k)
+                a.nbr[(size_t)(ob + o) * (size_t)a.Kstride + k] = ob + o;
+            atomicMax(&S.max_nbr, cnt);
+        }
+        g.sync();
+        if (tid == 0)
+            atomicMax(&a.ctl->max_nbr, S.max_nbr);
+        g.sync();
+    }
+}
+
+// ---------------------------------------------------------------------------
+// The same lists in the same order by one warp per cell, its lanes the cell's
+// particles (batches of 32), where there are cells enough to give every warp
+// one: each lane tests the staged candidates one after the other (every read a
+// broadcast of two candidates), and stores the ones kept straight into its row.
+// About ten instructions per candidate and warp, whatever number of lanes is in
+// use, against about two per candidate and particle of the form above: fewer
+// from ~6 particles a cell on, and no barrier; but a cell's time is a serial
+// chain of its ~400 candidates, so few cells are better shared out as above.
+// ---------------------------------------------------------------------------
+constexpr int kNbStage = 224;    // staged candidates per round and warp (a multiple of 32)
+constexpr int kNbBatch = 4;      // stencil cells whose particles are loaded at once
+
+struct NbWarp {
+    float4 a[kNbStage / 2], b[kNbStage / 2];   // two candidates: (x, x', y, y'), (z, z', w, w')
+};
+
+// Tests of the staged candidates [0, n): lane's particle at (hx, hy, hz) negated;
+// the entries kept go to `row` (bytes) + off, cnt counts them.  Blocks of 32
+// candidates that cannot overflow a row take the loop without that test.
+template <bool WRAP>
+__device__ __forceinline__ void nbuild_scan_warp(const NbWarp &S, int n, const Rep &rp, float2 hx, float2 hy, float2 hz,
+                                                 float rl0, float rl1, int wi, int K, char *row, int &cnt)
+{
+    for (int p0 = 0; p0 < n / 2; p0 += 16) {
+        const int p1 = min(p0 + 16, n / 2);
+        if (!WRAP && (int)__reduce_max_sync(0xffffffffu, (unsigned)cnt) + 32 <= K) {
+            unsigned off = 4u * (unsigned)cnt;
+#pragma unroll 4
+            for (int p = p0; p < p1; ++p) {
+                const float4 A = S.a[p], B = S.b[p];
+                const float2 dx = __fadd2_rn(make_float2(A.x, A.y), hx), dy = __fadd2_rn(make_float2(A.z, A.w), hy),
+                             dz = __fadd2_rn(make_float2(B.x, B.y), hz);
+                const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+                const int w0 = __float_as_int(B.z), w1 = __float_as_int(B.w);
+                if (r2.x < (w0 < 0 ? rl1 : rl0) && w0 != wi) {
+                    *(int *)(row + off) = w0 & 0x7fffffff;
+                    off += 4u;
+                }
+                if (r2.y < (w1 < 0 ? rl1 : rl0) && w1 != wi) {
+                    *(int *)(row + off) = w1 & 0x7fffffff;
+                    off += 4u;
+                }
+            }
+            cnt = (int)(off >> 2);
+        } else {
+            for (int p = p0; p < p1; ++p) {
+                const float4 A = S.a[p], B = S.b[p];
+                float2 dx = __fadd2_rn(make_float2(A.x, A.y), hx), dy = __fadd2_rn(make_float2(A.z, A.w), hy),
+                       dz = __fadd2_rn(make_float2(B.x, B.y), hz);
+                if (WRAP) {
+                    dx.x = fmaf(-rintf(dx.x * rp.invLf), rp.Lhi, dx.x);
+                    dx.y = fmaf(-rintf(dx.y * rp.invLf), rp.Lhi, dx.y);
+                    dy.x = fmaf(-rintf(dy.x * rp.invLf), rp.Lhi, dy.x);
+                    dy.y = fmaf(-rintf(dy.y * rp.invLf), rp.Lhi, dy.y);
+                    dz.x = fmaf(-rintf(dz.x * rp.invLf), rp.Lhi, dz.x);
+                    dz.y = fmaf(-rintf(dz.y * rp.invLf), rp.Lhi, dz.y);
+                }
+                const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+                const int w0 = __float_as_int(B.z), w1 = __float_as_int(B.w);
+                if (r2.x < (w0 < 0 ? rl1 : rl0) && w0 != wi) {
+                    if (cnt < K)
+                        *(int *)(row + 4u * (unsigned)cnt) = w0 & 0x7fffffff;
+                    ++cnt;
+                }
+                if (r2.y < (w1 < 0 ? rl1 : rl0) && w1 != wi) {
+                    if (cnt < K)
+                        *(int *)(row + 4u * (unsigned)cnt) = w1 & 0x7fffffff;
+                    ++cnt;
+                }
+            }
+        }
+    }
+}
+
+template <int P>
+__device__ __forceinline__ void nbuild_cell_warp(const KArgs &a, int pn, int c, int K, NbWarp &S, int &longest)
+{
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int c0 = a.cstart[c], c1 = a.cstart[c + 1];
+    const int4 cc = a.cxyz[c];
+    if (c0 == c1)
+        return;
+    const Rep &rp = a.rep[cc.w];
+    const int nst = rp.nc >= 3 ? 27 : 1;
+    const NbCentre ctr = nb_centre<P>(rp, cc);
+    const float hx = 0.5f * rp.Lhi / (float)rp.nc + 1e-3f;        // half edge of the cell's box
+    const float rlmax2 = fmaxf(fmaxf(a.tab.rl2[0], a.tab.rl2[1]), fmaxf(a.tab.rl2[2], a.tab.rl2[3]));
+    const unsigned lt_mask = (1u << lane) - 1u;
+    int s0, s1;
+    nb_stencil(a, rp, cc, nst, s0, s1);
 
     for (int ob = c0; ob < c1; ob += 32) {
-        const int i = ob + lane;
-        const bool own = i < c1;
-        const float4 H = nb_word<P>(a, pn, own ? i : ob);
-        const int ti = nb_species<P>(H);
-        const float rl0 = own ? a.tab.rl2[ti * 2] * r2unit : -1.0f;      // -1: nothing passes
-        const float rl1 = own ? a.tab.rl2[ti * 2 + 1] * r2unit : -1.0f;
-        int *row = a.nbr + (size_t)(own ? i : ob) * (size_t)a.Kstride;
-        int cnt = 0;          // neighbours found
-        int staged = 0;
+        const bool own = ob + lane < c1;
+        const int i = own ? ob + lane : ob;
+        int sp;
+        const float3 h = nb_rel<P>(a, rp, ctr, pn, i, sp);
+        const float rl0 = own ? a.tab.rl2[sp * 2] : -1.0f;        // -1: nothing passes
+        const float rl1 = own ? a.tab.rl2[sp * 2 + 1] : -1.0f;
+        char *row = (char *)(a.nbr + (size_t)i * (size_t)a.Kstride);
+        int cnt = 0, staged = 0;
 
-        // test the staged candidates against the lane's particle, in order; each
-        // entry kept goes straight to the lane's row (the L2 merges a row's writes)
-        auto scan = [&]() {
-            __syncwarp();
-#pragma unroll 4
-            for (int s = 0; s < staged; ++s) {
-                const float4 y = S.pos[s];
-                const int jj = S.idx[s];
-                const float r2 = nb_r2<P>(H, y, rp);
-                const bool in = r2 < (nb_species<P>(y) != 0 ? rl1 : rl0) && jj != i;
-                if (in && cnt < K)
-                    row[cnt] = jj;
-                cnt += in ? 1 : 0;
+        const auto scan = [&]() {
+            if (staged & 1) {                                     // (a candidate that fails every test)
+                if (lane == 0) {
+                    float *f = (float *)&S.a[staged >> 1], *e = (float *)&S.b[staged >> 1];
+                    f[1] = f[3] = e[1] = __int_as_float(0x7fc00000);
+                    e[3] = 0.f;
+                }
+                ++staged;
             }
+            __syncwarp();
+            if (nst == 27)
+                nbuild_scan_warp<false>(S, staged, rp, make_float2(-h.x, -h.x), make_float2(-h.y, -h.y),
+                                        make_float2(-h.z, -h.z), rl0, rl1, i | (sp << 31), K, row, cnt);
+            else
+                nbuild_scan_warp<true>(S, staged, rp, make_float2(-h.x, -h.x), make_float2(-h.y, -h.y),
+                                       make_float2(-h.z, -h.z), rl0, rl1, i | (sp << 31), K, row, cnt);
             __syncwarp();
             staged = 0;
         };
-
-        for (int k = 0; k < nst; ++k) {
-            const int cs = a.cstart[S.cell[k]], ce = a.cstart[S.cell[k] + 1];
-            for (int t0 = cs; t0 < ce; t0 += 32) {
-                if (staged > kNbStage - 32)
-                    scan();
-                const int t = t0 + lane;
-                bool keep = false;
-                float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (t < ce) {
-                    q = nb_word<P>(a, pn, checked(a, t, a.n, 0));
-                    keep = true;
-                    if (nst == 27) {
-                        const float3 x = nb_coords<P>(q, rp);
-                        const float gx = box_gap(x.x, ccx, hx, rp.Lhi, rp.invLf);
-                        const float gy = box_gap(x.y, ccy, hx, rp.Lhi, rp.invLf);
-                        const float gz = box_gap(x.z, ccz, hx, rp.Lhi, rp.invLf);
-                        keep = fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < rlmax2;
-                    }
+        // stage the lanes' particles r (index and species in w), in lane order
+        const auto stage = [&](const float3 &r, int w, bool ok) {
+            if (nst == 27) {
+                const float gx = fmaxf(fabsf(r.x) - hx, 0.f), gy = fmaxf(fabsf(r.y) - hx, 0.f),
+                            gz = fmaxf(fabsf(r.z) - hx, 0.f);
+                ok = ok && fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < rlmax2;
+            }
+            const unsigned m = __ballot_sync(FULL, ok);
+            if (staged + 32 > kNbStage)
+                scan();
+            if (ok) {
+                const int s = staged + __popc(m & lt_mask);
+                float *f = (float *)&S.a[s >> 1] + (s & 1), *e = (float *)&S.b[s >> 1] + (s & 1);
+                f[0] = r.x;
+                f[2] = r.y;
+                e[0] = r.z;
+                e[2] = __int_as_float(w);
+            }
+            staged += __popc(m);
+        };
+        for (int k0 = 0; k0 < nst; k0 += kNbBatch) {
+            float3 r[kNbBatch];
+            int w[kNbBatch];
+#pragma unroll
+            for (int u = 0; u < kNbBatch; ++u) {
+                const int k = min(k0 + u, 31);
+                const int t = __shfl_sync(FULL, s0, k) + lane, e = __shfl_sync(FULL, s1, k);
+                int tsp = 0;
+                w[u] = -1;
+                r[u] = make_float3(0.f, 0.f, 0.f);
+                if (t < e) {
+                    r[u] = nb_rel<P>(a, rp, ctr, pn, checked(a, t, a.n, 0), tsp);
+                    w[u] = t;
                 }
-                const unsigned m = __ballot_sync(FULL, keep);
-                if (keep) {
-                    const int sidx = staged + __popc(m & lt_mask);
-                    S.pos[sidx] = q;
-                    S.idx[sidx] = t;
+                if (tsp)
+                    w[u] |= 1 << 31;
+                else if (w[u] < 0)
+                    w[u] = 0x7fffffff;                            // (no particle)
+            }
+#pragma unroll
+            for (int u = 0; u < kNbBatch; ++u) {
+                const int k = min(k0 + u, 31);
+                const int t0 = __shfl_sync(FULL, s0, k), e = __shfl_sync(FULL, s1, k);
+                if (t0 < e)
+                    stage(r[u], w[u], w[u] != 0x7fffffff);
+                for (int t = t0 + 32; t < e; t += 32) {           // (a cell of more than 32 particles)
+                    float3 q = make_float3(0.f, 0.f, 0.f);
+                    int tsp = 0;
+                    if (t + lane < e)
+                        q = nb_rel<P>(a, rp, ctr, pn, checked(a, t + lane, a.n, 0), tsp);
+                    stage(q, (t + lane) | (tsp << 31), t + lane < e);
                 }
-                staged += __popc(m);
             }
         }
         scan();
@@ -1684,175 +2026,11 @@ __device__ __forceinline__ void nbuild_cell_warp(const KArgs &a, int pn, int c, 
             // loop reads whole groups without masking
             const int kept = cnt < K ? cnt : K;
             for (int k = kept; k < (kept + kUnr - 1) / kUnr * kUnr && k < K; ++k)
-                row[k] = i;
+                ((int *)row)[k] = i;
             a.nnbr[i] = kept;
-            atomicMax(&ctl->max_nbr, cnt);
+            longest = max(longest, cnt);
         }
         __syncwarp();
-    }
-}
-
-// Block per cell, for handles with too few cells to occupy the GPU with one
-// warp each: the block stages the candidates (kNbCap per round, the same
-// order and filter as above), and each of its warps takes kNbPass particles
-// of the cell at a time, testing 32 staged candidates per ballot; the list
-// rows come out the same as with a warp per cell.
-constexpr int kNbCap = 512;      // staged candidates per round
-constexpr int kNbOwn = 256;      // own-cell particles per batch
-constexpr int kNbPass = 2;       // own-cell particles tested per warp pass over the candidates
-
-struct NbBlock {
-    float4 pos[kNbCap];
-    int idx[kNbCap];
-    int cnt[kNbOwn];
-    int pref[28];
-    int cell[27];
-    int wsum[kNbBlockB / 32];
-};
-
-template <int P>
-__device__ __forceinline__ void nbuild_cell_block(const KArgs &a, int pn, int c, int K, NbBlock &S)
-{
-    Ctl *ctl = a.ctl;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int NW = kNbBlockB / 32;
-    const int4 cc = a.cxyz[c];
-    const Rep rp = a.rep[cc.w];
-    const int nc = rp.nc;
-    const int nst = nc >= 3 ? 27 : 1;
-    const int c0 = a.cstart[c], c1 = a.cstart[c + 1];
-    if (c0 == c1)
-        return;
-
-    if (tid < nst) {
-        int x = cc.x, y = cc.y, z = cc.z;
-        if (nst == 27) {
-            x = (x + tid % 3 - 1 + nc) % nc;
-            y = (y + (tid / 3) % 3 - 1 + nc) % nc;
-            z = (z + tid / 9 - 1 + nc) % nc;
-        }
-        S.cell[tid] = a.crank[rp.cell0 + (z * nc + y) * nc + x];
-    }
-    __syncthreads();
-    if (tid == 0) {
-        int s = 0;
-        for (int k = 0; k < nst; ++k) {
-            S.pref[k] = s;
-            s += a.cstart[S.cell[k] + 1] - a.cstart[S.cell[k]];
-        }
-        S.pref[nst] = s;
-    }
-    __syncthreads();
-    const int total = S.pref[nst];
-
-    // own cell box (centre, half edge) for the candidate filter
-    const float edge = rp.Lhi / (float)nc;
-    const float hx = 0.5f * edge + 1e-3f;
-    const float ccx = ((float)cc.x + 0.5f) * edge, ccy = ((float)cc.y + 0.5f) * edge,
-                ccz = ((float)cc.z + 0.5f) * edge;
-    const float rlmax2 = fmaxf(fmaxf(a.tab.rl2[0], a.tab.rl2[1]), fmaxf(a.tab.rl2[2], a.tab.rl2[3]));
-    const unsigned lt_mask = (1u << lane) - 1u;
-    // nb_r2 of the fixed-point words is in units of qunit^2: the list radii follow
-    const float r2unit = (P == MIXED && kNbFixed) ? 1.0f / (rp.qunit * rp.qunit) : 1.0f;
-
-    for (int ob = c0; ob < c1; ob += kNbOwn) {
-        const int nown = min(kNbOwn, c1 - ob);
-        for (int t = tid; t < nown; t += kNbBlockB)
-            S.cnt[t] = 0;
-        int staged = 0;
-        for (int base = 0; base < total; base += kNbBlockB) {
-            // stage candidates base .. base + kNbBlockB - 1, order-preserving compaction
-            const int t = base + tid;
-            bool keep = false;
-            float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
-            int j = 0;
-            if (t < total) {
-                int k = 0;
-                while (k + 1 < nst && S.pref[k + 1] <= t)
-                    ++k;
-                j = checked(a, a.cstart[S.cell[k]] + (t - S.pref[k]), a.n, 0);
-                q = nb_word<P>(a, pn, j);
-                keep = true;
-                if (nst == 27) {
-                    const float3 x = nb_coords<P>(q, rp);
-                    const float gx = box_gap(x.x, ccx, hx, rp.Lhi, rp.invLf);
-                    const float gy = box_gap(x.y, ccy, hx, rp.Lhi, rp.invLf);
-                    const float gz = box_gap(x.z, ccz, hx, rp.Lhi, rp.invLf);
-                    keep = fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < rlmax2;
-                }
-            }
-            const unsigned m = __ballot_sync(0xffffffffu, keep);
-            if (lane == 0)
-                S.wsum[warp] = __popc(m);
-            __syncthreads();
-            int off = staged, add = 0;
-#pragma unroll
-            for (int w = 0; w < NW; ++w) {
-                off += (w < warp) ? S.wsum[w] : 0;
-                add += S.wsum[w];
-            }
-            if (keep) {
-                const int s = off + __popc(m & lt_mask);
-                S.pos[s] = q;
-                S.idx[s] = j;
-            }
-            staged += add;
-            __syncthreads();
-            if (staged <= kNbCap - kNbBlockB && base + kNbBlockB < total)
-                continue;
-
-            // scan the staged candidates: each warp pass takes kNbPass particles of
-            // the batch, so that every staged candidate read serves kNbPass tests
-            for (int o0 = warp * kNbPass; o0 < nown; o0 += NW * kNbPass) {
-                float4 H[kNbPass];
-                float rl0[kNbPass], rl1[kNbPass];
-                int cnt[kNbPass];
-#pragma unroll
-                for (int p = 0; p < kNbPass; ++p) {
-                    const bool ok = o0 + p < nown;
-                    H[p] = nb_word<P>(a, pn, ob + (ok ? o0 + p : 0));
-                    const int ti = nb_species<P>(H[p]);
-                    rl0[p] = ok ? a.tab.rl2[ti * 2] * r2unit : -1.0f;       // -1: nothing passes
-                    rl1[p] = ok ? a.tab.rl2[ti * 2 + 1] * r2unit : -1.0f;
-                    cnt[p] = ok ? S.cnt[o0 + p] : 0;
-                }
-                for (int s0 = 0; s0 < staged; s0 += 32) {
-                    const int s = s0 + lane;
-                    const bool sv = s < staged;
-                    const float4 y = sv ? S.pos[s] : make_float4(0.f, 0.f, 0.f, 0.f);
-                    const int jj = sv ? S.idx[s] : -1;
-                    const bool tj = nb_species<P>(y) != 0;
-#pragma unroll
-                    for (int p = 0; p < kNbPass; ++p) {
-                        const int i = ob + o0 + p;
-                        const float r2 = nb_r2<P>(H[p], y, rp);
-                        const bool in = sv && jj != i && r2 < (tj ? rl1[p] : rl0[p]);
-                        const unsigned mm = __ballot_sync(0xffffffffu, in);
-                        const int at = cnt[p] + __popc(mm & lt_mask);
-                        if (in && at < K)
-                            a.nbr[(size_t)i * (size_t)a.Kstride + at] = jj;
-                        cnt[p] += __popc(mm);
-                    }
-                }
-                if (lane == 0)
-#pragma unroll
-                    for (int p = 0; p < kNbPass; ++p)
-                        if (o0 + p < nown)
-                            S.cnt[o0 + p] = cnt[p];
-            }
-            staged = 0;
-            __syncthreads();
-        }
-        for (int o = tid; o < nown; o += kNbBlockB) {
-            const int cnt = S.cnt[o];
-            a.nnbr[ob + o] = cnt < K ? cnt : K;
-            // pad the row with the particle itself to a multiple of kUnr entries, so the
-            // pair loop reads whole groups without masking (K is a multiple of 8)
-            for (int k = cnt; k < (cnt + kUnr - 1) / kUnr * kUnr && k < K; ++k)
-                a.nbr[(size_t)(ob + o) * (size_t)a.Kstride + k] = ob + o;
-            atomicMax(&ctl->max_nbr, cnt);
-        }
-        __syncthreads();
     }
 }
 
@@ -1901,52 +2079,62 @@ struct RunState {
     long long pend_obs, pend_rebuilds;
     unsigned long long t0, ns;
     int pp, spar, K, pos;
-    float md2, pend_md2;           // largest squared displacement since the build: now, of `pend`
     int pend_sample;
-    int last, sample;              // of the running step
+    int last, sample, check, track; // of the running step: ends md_step, is a sample, is checked, needs maxima
+    int to_sample;                 // steps until the next sample step
+    int unit;                      // next unit (cell or share of one) of the block's in the build
+
+    Rep rep;                       // of a handle of one replica
     long long done;
     unsigned int count, flags;     // barriers passed (thread 0), flags of the last one
 };
 
-// shared scratch of the phases, one at a time
-union RunScratch {
-    NbWarp warp[kNbCells];
-    NbBlock block;
-    int scan[32];
-};
-
-// ... and of a step: block reductions, and what a thread keeps between its
-// chunks (registers are scarce in the pair loop)
+// Shared scratch of a group.  Of a step: sums, and what a thread keeps between
+// its chunks (registers are scarce in the pair loop).
 struct RunSums {
-    double sh[32 * kPartF];
+    double sh[kGrpWarps * kPartF];
     double tot[kPartF];                              // sums of a one-replica sample
     double e[kForceBlock];                           // energy (ET) and maxima so far, per thread
     float d2[kForceBlock], v2[kForceBlock], a2[kForceBlock];
 };
 
+struct RunGroup {
+    union {
+        NbBlock nb;
+        NbWarp nbw[kGrpWarps];
+        RunSums step;
+        int scan[kGrpWarps];
+    };
+    int4 row;                                        // the group's first chunk
+    __align__(16) float es[4 * kGrpWarps];
+    float mx[3 * kGrpWarps];
+    int unit;                                        // the group's unit of the build
+};
+
 // Every block arrives; `decide` runs in thread 0 of the last one, sees the
-// writes of all blocks and returns the flags that every block gets.
-template <class F>
-__device__ __forceinline__ unsigned int grid_barrier(const KArgs &a, RunState &S, F &&decide)
+// writes of all blocks and returns the flags that every block gets; `after` runs
+// in thread 0 of every block with these flags.
+template <class F, class G>
+__device__ __forceinline__ unsigned int grid_barrier(const KArgs &a, RunState &S, F &&decide, G &&after)
 {
     __syncthreads();
     if (threadIdx.x == 0) {
         RunSync *rs = a.rs;
-        __threadfence();
-        const unsigned int t = atomicAdd(&rs->arrive, 1u);
         const unsigned int next = (S.count + 1u) & 0x0fffffffu;
-        unsigned int w;
+        unsigned int t, w;
+        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(t) : "l"(&rs->arrive) : "memory");
         if (t == gridDim.x - 1) {
-            __threadfence();
             rs->arrive = 0u;
             w = (next << 4) | decide();
-            __threadfence();
             asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&rs->word), "r"(w) : "memory");
         } else {
             unsigned int n = 0;
+            // (polls without acquire: an acquire empties the SM's L1, which its other
+            // blocks still use)
             do {
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(w) : "l"(&rs->word) : "memory");
+                asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(w) : "l"(&rs->word) : "memory");
             } while ((w >> 4) != next && ++n < kSpinMax);
+            asm volatile("fence.acq_rel.gpu;" ::: "memory");
             if ((w >> 4) != next) {
                 atomicOr(&a.ctl->status, ST_TIMEOUT);
                 w = RF_STOP | RF_BAD | RF_ABORT;
@@ -1954,13 +2142,19 @@ __device__ __forceinline__ unsigned int grid_barrier(const KArgs &a, RunState &S
         }
         S.count = next;
         S.flags = w & 15u;
+        after(w & 15u);
     }
     __syncthreads();
     return S.flags;
 }
 
-// Maxima of this block's displacements, speeds and accelerations into the
-// step's, thread 0.
+__device__ __forceinline__ unsigned int grid_barrier(const KArgs &a, RunState &S)
+{
+    return grid_barrier(a, S, []() -> unsigned int { return 0u; }, [](unsigned int) {});
+}
+
+// Maxima of this block's displacements, speeds and accelerations, and what went
+// wrong, into the step's, thread 0.
 __device__ __forceinline__ void put_maxima(const KArgs &a, long long step, float d2, float v2, float a2)
 {
     unsigned int *m = a.rs->m[step & 1];
@@ -1972,56 +2166,109 @@ __device__ __forceinline__ void put_maxima(const KArgs &a, long long step, float
         atomicMax(&m[2], __float_as_uint(a2));
 }
 
-// The whole grid's maxima (cleared for the step after the next): does a drift
-// call for a rebuild?  md2 gets the largest squared displacement.
-__device__ __forceinline__ bool take_maxima(const KArgs &a, long long step, int lookahead, float &md2)
+__device__ __forceinline__ void put_bad(const KArgs &a, long long step, unsigned int bad)
 {
-    unsigned int *m = a.rs->m[step & 1];
-    md2 = __uint_as_float(atomicExch(&m[0], 0u));
-    const float mv2 = __uint_as_float(atomicExch(&m[1], 0u));
-    const float ma2 = __uint_as_float(atomicExch(&m[2], 0u));
-    return need_rebuild(a, lookahead, md2, mv2, ma2);
+    atomicOr(&a.ctl->status, bad);
+    atomicOr(&a.rs->m[step & 1][3], bad);
+}
+
+// The whole grid's maxima, cleared for the step after the next (last arriver of
+// the step's barrier).  The displacement is kept by the parity of the step it
+// leads to (of the positions it belongs to).
+struct Maxima { float d2, v2, a2; unsigned int bad; };
+
+__device__ __forceinline__ Maxima take_maxima(const KArgs &a, long long step)
+{
+    uint4 *m = reinterpret_cast<uint4 *>(a.rs->m[step & 1]);
+    uint4 v;
+    asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(m) : "memory");
+    *m = make_uint4(0u, 0u, 0u, 0u);
+    a.rs->md2[(step + 1) & 1] = __uint_as_float(v.x);
+    Maxima r;
+    r.d2 = __uint_as_float(v.x);
+    r.v2 = __uint_as_float(v.y);
+    r.a2 = __uint_as_float(v.z);
+    r.bad = v.w;
+    return r;
 }
 
 // Rebuild of the lists; returns the flags of its last barrier (the state's
 // parities and capacity are those of the new lists unless RF_BAD).
 template <int P>
-__device__ __forceinline__ unsigned int run_rebuild(const KArgs &a, RunState &S, RunScratch &X)
+__device__ __forceinline__ unsigned int run_rebuild(const KArgs &a, const Grp &g, RunState &S, RunGroup &X)
 {
     Ctl *ctl = a.ctl;
-    const auto nothing = []() -> unsigned int { return 0u; };
-    const int slice_cells = (a.ncell + (int)gridDim.x - 1) / (int)gridDim.x;
     if (blockIdx.x == 0 && threadIdx.x == 0)
         ctl->max_nbr = 0;
-    rebuild_bin<P>(a, S.pp, slice_cells);
-    if (grid_barrier(a, S, nothing) & RF_ABORT)
+    rebuild_bin<P>(a, g, S.pp);
+    if (grid_barrier(a, S) & RF_ABORT)
         return S.flags;
-    rebuild_scan(a, slice_cells, X.scan);
-    if (grid_barrier(a, S, nothing) & RF_ABORT)
+    // cells per block of the scan; few cells: every block adds up the counts before its own
+    const int slice_cells = (a.ncell + g.nvb - 1) / g.nvb;
+    if (a.ncell > kScanDirect) {
+        rebuild_slices(a, g, slice_cells, X.scan);
+        if (grid_barrier(a, S) & RF_ABORT)
+            return S.flags;
+    }
+    rebuild_scan(a, g, slice_cells, X.scan);
+    if (grid_barrier(a, S) & RF_ABORT)
         return S.flags;
-    rebuild_scatter(a);
-    if (grid_barrier(a, S, nothing) & RF_ABORT)
+    rebuild_scatter(a, g);
+    if (grid_barrier(a, S) & RF_ABORT)
         return S.flags;
-    rebuild_permute<P>(a, S.pp, S.spar);
-    if (grid_barrier(a, S, nothing) & RF_ABORT)
+    rebuild_permute<P>(a, g, S.pp, S.spar);
+    const auto reset_units = [&]() -> unsigned int {
+        a.rs->unit = g.nvb;
+        return 0u;
+    };
+    if (grid_barrier(a, S, reset_units, [&](unsigned int) { S.unit = 0; }) & RF_ABORT)
         return S.flags;
     for (int retry = 0;; ++retry) {
-        // the lists: at most K entries a row; the longest list decides
+        // the lists: at most K entries a row; the longest list decides.  Every SM has a run of
+        // neighbouring cells, whose particles its L1 then holds; its warps or groups take them
+        // in turns (the time per cell differs)
         const int pn = S.pp ^ 1, K = S.K;
-        if (a.nb_block) {
-            for (int c = blockIdx.x; c < a.ncell; c += gridDim.x)
-                nbuild_cell_block<P>(a, pn, c, K, X.block);
+        if (a.nb_warp) {
+            const int u0 = (int)((long long)a.ncell * blockIdx.x / gridDim.x),
+                      u1 = (int)((long long)a.ncell * (blockIdx.x + 1) / gridDim.x);
+            int longest = 0;
+            for (;;) {
+                int u = 0;
+                if ((threadIdx.x & 31) == 0)
+                    u = u0 + atomicAdd(&S.unit, 1);
+                u = __shfl_sync(0xffffffffu, u, 0);
+                if (u >= u1)
+                    break;
+                nbuild_cell_warp<P>(a, pn, u, K, X.nbw[g.tid() >> 5], longest);
+            }
+            longest = (int)__reduce_max_sync(0xffffffffu, (unsigned)longest);
+            if ((threadIdx.x & 31) == 0 && longest > 0)
+                atomicMax(&ctl->max_nbr, longest);
         } else {
-            const int w = threadIdx.x >> 5;
-            for (int c = blockIdx.x * kNbCells + w; c < a.ncell; c += gridDim.x * kNbCells)
-                nbuild_cell_warp<P>(a, pn, c, K, X.warp[w]);
+            // (ensembles have few, uneven cells: one counter for the whole grid, read ahead)
+            const int nparts = a.nb_parts, nunit = a.ncell * nparts;
+            for (int u = g.vb; u < nunit;) {
+                unsigned int nu = 0;
+                if (g.tid() == 0)
+                    nu = atomicAdd(&a.rs->unit, 1u);
+                nbuild_cell<P>(a, g, pn, u / nparts, u % nparts, nparts, K, X.nb);
+                if (g.tid() == 0)
+                    X.unit = (int)nu;
+                g.sync();
+                u = X.unit;
+                g.sync();
+            }
         }
         const unsigned int f = grid_barrier(a, S, [&]() -> unsigned int {
+            a.rs->unit = g.nvb;
             if (atomicOr(&ctl->status, 0u))
                 return RF_STOP | RF_BAD;
             const int mx = atomicMax(&ctl->max_nbr, 0);
-            if (mx <= K)
+            if (mx <= K) {
+                a.rs->md2[S.step & 1] = 0.f;         // the lists start from these positions
                 return 0u;
+            }
             if (mx <= ctl->Kmax && retry == 0) {
                 // grow the capacity and redo the build: same positions, so the
                 // same counts, and they fit
@@ -2030,20 +2277,18 @@ __device__ __forceinline__ unsigned int run_rebuild(const KArgs &a, RunState &S,
             }
             atomicOr(&ctl->status, ST_OVERFLOW);
             return RF_STOP | RF_BAD;
-        });
-        if (threadIdx.x == 0) {
+        }, [&](unsigned int flags) {
             if (retry == 0)
                 S.rebuilds += 1;
-            if (f & RF_REBUILD) {
+            S.unit = 0;
+            if (flags & RF_REBUILD) {
                 S.K = ctl->K;
                 S.regrows += 1;
-            } else if (!(f & RF_BAD)) {
+            } else if (!(flags & RF_BAD)) {
                 S.pp ^= 1;
                 S.spar ^= 1;
-                S.md2 = 0.f;                         // the lists start from these positions
             }
-        }
-        __syncthreads();
+        });
         if (!(f & RF_REBUILD))
             return f;
     }
@@ -2051,15 +2296,15 @@ __device__ __forceinline__ unsigned int run_rebuild(const KArgs &a, RunState &S,
 
 // The half kick and drift that open md_step.
 template <int P>
-__device__ __forceinline__ void run_first(const KArgs &a, RunState &S, float *shf)
+__device__ __forceinline__ void run_first(const KArgs &a, const Grp &g, RunState &S, RunGroup &X)
 {
     const int pp = S.pp, spar = S.spar;
     float d2 = 0.f, v2 = 0.f, a2 = 0.f;
     unsigned int bad = 0u;
-    for (int row = blockIdx.x; row < a.nblk_i; row += gridDim.x) {
+    for (int row = g.vb; row < a.nblk_i; row += g.nvb) {
         const int4 b = a.blk_i[row];
         const Rep rp = a.rep[b.z];
-        for (int i = b.x + threadIdx.x; i < b.y; i += blockDim.x) {
+        for (int i = b.x + g.tid(); i < b.y; i += kForceBlock) {
             PState<P> s;
             load_pos<P>(a, pp, i, s);
             load_vel<P>(a, spar, i, s);
@@ -2072,7 +2317,7 @@ __device__ __forceinline__ void run_first(const KArgs &a, RunState &S, float *sh
                 f[0] = q.x; f[1] = q.y; f[2] = q.z;
             }
             half_kick<P>(a, s, f[0], f[1], f[2]);
-            d2 = fmaxf(d2, drift<P>(a, rp, s, pp ^ 1, spar, i, bad));
+            d2 = fmaxf(d2, drift<P>(a, rp, s, pp ^ 1, spar, i, true, bad));
             v2 = fmaxf(v2, speed2(s));
             const float im = a.inv_mass[s.sp];
             a2 = fmaxf(a2, __fmul_rn(__fmul_rn(norm2(f[0], f[1], f[2]), im), im));
@@ -2080,42 +2325,43 @@ __device__ __forceinline__ void run_first(const KArgs &a, RunState &S, float *sh
         }
     }
     if (bad)
-        atomicOr(&a.ctl->status, bad);
-    block_max3(d2, v2, a2, shf);
-    if (threadIdx.x == 0)
+        put_bad(a, S.step, bad);
+    grp_max3(g, d2, v2, a2, X.mx);
+    if (g.tid() == 0)
         put_maxima(a, S.step, d2, v2, a2);
 }
 
-// One sweep over the block's chunks: forces, the particles' update, and the
+// One sweep over the group's chunks: forces, the particles' update, and the
 // partial sums and maxima.
 template <int P, int TPP, bool SM, bool SAMPLE>
-__device__ __forceinline__ void run_chunks(const KArgs &a, RunState &S, RunSums &X, float *shf)
+__device__ __forceinline__ void run_chunks(const KArgs &a, const Grp &g, RunState &S, RunGroup &G)
 {
-    X.d2[threadIdx.x] = X.v2[threadIdx.x] = X.a2[threadIdx.x] = 0.f;
+    RunSums &X = G.step;
+    X.d2[g.tid()] = X.v2[g.tid()] = X.a2[g.tid()] = 0.f;
     ET<P> *xe = reinterpret_cast<ET<P> *>(X.e);
-    xe[threadIdx.x] = e_zero<P>();
-    if (SAMPLE && threadIdx.x < kPartF)
-        X.tot[threadIdx.x] = 0.0;
-    if ((int)blockIdx.x * a.cpb >= a.nrow)
-        return;                                      // (a block without chunks)
+    xe[g.tid()] = e_zero<P>();
+    if (SAMPLE && g.tid() < kPartF)
+        X.tot[g.tid()] = 0.0;
+    if (g.vb * a.cpb >= a.nrow)
+        return;                                      // (a group without chunks)
     for (int q = 0; q < a.cpb; ++q) {
-        const int4 b = a.blk_r[blockIdx.x * a.cpb + q];
-        if (b.w < 0)                                 // (padding rows: the same for the whole block)
+        const int4 b = q == 0 ? G.row : a.blk_r[g.vb * a.cpb + q];
+        if (b.w < 0)                                 // (padding rows: the same for the whole group)
             break;
         double part[kPartF];
         ET<P> eo;
         float d2 = 0.f, v2 = 0.f, a2 = 0.f;
         unsigned int bad = 0u;
-        step_body<P, TPP, SAMPLE, SM>(a, b, (a.what & RUN_STEPS) != 0, S.last != 0, S.pp, S.spar, part, eo, d2, v2, a2,
-                                      bad);
+        step_body<P, TPP, SAMPLE, SM>(a, a.nrep == 1 ? S.rep : a.rep[b.z], b, (a.what & RUN_STEPS) != 0, S.last != 0,
+                                      S.track != 0, S.pp, S.spar, part, eo, d2, v2, a2, bad);
         if (bad)
-            atomicOr(&a.ctl->status, bad);
-        X.d2[threadIdx.x] = fmaxf(X.d2[threadIdx.x], d2);
-        X.v2[threadIdx.x] = fmaxf(X.v2[threadIdx.x], v2);
-        X.a2[threadIdx.x] = fmaxf(X.a2[threadIdx.x], a2);
+            put_bad(a, S.step, bad);
+        X.d2[g.tid()] = fmaxf(X.d2[g.tid()], d2);
+        X.v2[g.tid()] = fmaxf(X.v2[g.tid()], v2);
+        X.a2[g.tid()] = fmaxf(X.a2[g.tid()], a2);
         if (SAMPLE) {
-            block_sum<kPartF>(part, X.sh);
-            if (threadIdx.x == 0) {
+            grp_sum<kPartF>(g, part, X.sh);
+            if (g.tid() == 0) {
                 double *p = a.nrep == 1 ? X.tot : a.part_f + part_index(a, S.step, b.w) * kPartF;
 #pragma unroll
                 for (int k = 1; k < kPartF; ++k)
@@ -2123,23 +2369,28 @@ __device__ __forceinline__ void run_chunks(const KArgs &a, RunState &S, RunSums 
             }
         }
         if (a.nrep == 1) {
-            xe[threadIdx.x] = e_add(xe[threadIdx.x], eo);
+            xe[g.tid()] = e_add(xe[g.tid()], eo);
         } else {
-            float z0 = 0.f, z1 = 0.f, z2 = 0.f;
-            block_max3_sum1(z0, z1, z2, eo, shf, X.sh);
-            if (threadIdx.x == 0)
+            grp_esum(g, eo, G.es);
+            if (g.tid() == 0)
                 put_epart<P>(a, part_index(a, S.step, b.w), eo);
+            g.sync();                                // (G.es is written again)
         }
     }
-    float d2 = X.d2[threadIdx.x], v2 = X.v2[threadIdx.x], a2 = X.a2[threadIdx.x];
-    ET<P> e = xe[threadIdx.x];
-    block_max3_sum1(d2, v2, a2, e, shf, X.sh);
-    if (threadIdx.x == 0) {
-        put_maxima(a, S.step, d2, v2, a2);
+    if (S.track) {
+        float d2 = X.d2[g.tid()], v2 = X.v2[g.tid()], a2 = X.a2[g.tid()];
+        grp_max3(g, d2, v2, a2, G.mx);
+        if (g.tid() == 0)
+            put_maxima(a, S.step, d2, v2, a2);
+    }
+    ET<P> e = xe[g.tid()];
+    if (a.nrep == 1)
+        grp_esum(g, e, G.es);
+    if (g.tid() == 0) {
         if (a.nrep == 1) {
-            put_epart<P>(a, part_index(a, S.step, blockIdx.x), e);
+            put_epart<P>(a, part_index(a, S.step, g.vb), e);
             if (SAMPLE) {
-                double *p = a.part_f + part_index(a, S.step, blockIdx.x) * kPartF;
+                double *p = a.part_f + part_index(a, S.step, g.vb) * kPartF;
 #pragma unroll
                 for (int k = 1; k < kPartF; ++k)
                     p[k] = X.tot[k];
@@ -2148,38 +2399,54 @@ __device__ __forceinline__ void run_chunks(const KArgs &a, RunState &S, RunSums 
     }
 }
 
-// Sums of the step that awaits them, one block per replica, the last blocks of
-// the grid first: they have the fewest chunks (none, where blocks are to spare).
+// Sums of the step that awaits them, one group per replica, the last groups of
+// the grid first: they have the fewest chunks (none, where groups are to spare).
 template <int P>
-__device__ __forceinline__ void run_service(const KArgs &a, RunState &S, bool totals, double *sh, float *shf)
+__device__ __forceinline__ void run_service(const KArgs &a, const Grp &g, RunState &S, bool totals, RunGroup &X)
 {
     if (S.pend < 0)
         return;
-    for (int r = (int)gridDim.x - 1 - (int)blockIdx.x; r < a.nrep; r += gridDim.x) {
-        finish_replica<P>(a, r, S.pend, S.pend_sample != 0, totals, S.pend_obs % (long long)a.obs_cap, S.pend_md2,
-                          S.pend_rebuilds, sh, shf);
-        if (r == 0 && threadIdx.x == 0 && !totals)
+    for (int r = g.nvb - 1 - g.vb; r < a.nrep; r += g.nvb) {
+        finish_replica<P>(a, g, r, S.pend, S.pend_sample != 0, totals, S.pend_obs % (long long)a.obs_cap,
+                          a.rs->md2[S.pend & 1], S.pend_rebuilds, X.step.sh, X.es);
+        if (r == 0 && g.tid() == 0 && !totals)
             a.epot_step[S.pend % a.epot_cap] = S.pend;
     }
 }
 
-// Blocks of 128 threads per SM the unsmoothed single-precision kernels are
-// compiled for: 7 at <= 72 registers, so that 1024 chunks (KA N=65536 at 2 lanes
-// per particle) are one per block on 152 SMs.  FP64 and the smoothed kernels
-// keep the compiler's own register choice (they would spill).
-template <int P, bool SM> constexpr int run_min_blocks() { return P == FP64 ? 0 : SM ? 5 : 7; }
+// Groups per SM: 7 at <= 72 registers a thread for the unsmoothed single-precision
+// kernels, so that 1024 chunks (KA N=65536 at 2 lanes per particle) are one per
+// group on 152 SMs; 5 at <= 96 for FP64 and the smoothed kernels (they would spill).
+template <int P, bool SM> constexpr int run_groups() { return P == FP64 || SM ? 5 : 7; }
+
+// What the step at S.step, position S.pos between checks, has to do (thread 0).
+// The maxima are needed where a check follows and where the positions that the
+// drift leads to are sampled.
+__device__ __forceinline__ void run_plan(const KArgs &a, RunState &S)
+{
+    const bool steps = (a.what & RUN_STEPS) != 0;
+    S.last = !steps || (S.left == 1 && a.last);
+    S.sample = steps ? S.to_sample == 0 : (a.what & RUN_FORCES) == 0;
+    S.check = !S.last && S.pos == a.check - 1;
+    S.track = S.check || (!S.last && (S.to_sample == 1 || a.si == 1));
+}
 
 template <int P, int TPP, bool SM>
-__global__ void __launch_bounds__(kForceBlock, run_min_blocks<P, SM>()) k_run(KArgs a)
+__global__ void __launch_bounds__(kForceBlock * run_groups<P, SM>(), 1) k_run(KArgs a)
 {
-    __shared__ union {
-        RunScratch nb;
-        RunSums step;
-    } X;
-    __shared__ float shf[160];
+    extern __shared__ __align__(16) unsigned char smem[];
     __shared__ RunState S;
-    double *sh = X.step.sh;
+    Grp g;
+    g.id = threadIdx.x / kForceBlock;
+    g.vb = blockIdx.x + g.id * gridDim.x;            // (groups p, p + gridDim, ... share an SM)
+    g.nvb = gridDim.x * (blockDim.x / kForceBlock);
+    RunGroup &X = reinterpret_cast<RunGroup *>(smem)[g.id];
     Ctl *ctl = a.ctl;
+    if (a.nrep == 1)
+        for (int k = threadIdx.x; k < (int)(sizeof(Rep) / 4); k += blockDim.x)
+            reinterpret_cast<int *>(&S.rep)[k] = reinterpret_cast<const int *>(a.rep)[k];
+    if (g.tid() == 0)
+        X.row = g.vb * a.cpb < a.nrow ? a.blk_r[g.vb * a.cpb] : make_int4(0, 0, 0, -1);
     if (threadIdx.x == 0) {
         S.step = ctl->step;
         S.left = a.nsteps;
@@ -2192,11 +2459,12 @@ __global__ void __launch_bounds__(kForceBlock, run_min_blocks<P, SM>()) k_run(KA
         S.spar = ctl->state_par;
         S.K = ctl->K;
         S.pos = a.pos0;
-        S.md2 = ctl->last_maxdisp2;
+        S.to_sample = (int)((a.si - S.step % a.si) % a.si);
         S.count = a.rs->word >> 4;
         S.ns = 0ull;
         S.done = 0;
         S.flags = ctl->status ? RF_STOP | RF_BAD : 0u;
+        run_plan(a, S);
     }
     __syncthreads();
     // A status pending from before: no phase does work, but every block goes to
@@ -2206,107 +2474,97 @@ __global__ void __launch_bounds__(kForceBlock, run_min_blocks<P, SM>()) k_run(KA
     const bool halted = S.flags != 0u;
     unsigned int f = 0u;
     if (a.what & RUN_REBUILD)
-        f = run_rebuild<P>(a, S, X.nb);
+        f = run_rebuild<P>(a, g, S, X);
     if (!(f & RF_STOP) && (a.what & RUN_FIRST)) {
         if (!halted)
-            run_first<P>(a, S, shf);
+            run_first<P>(a, g, S, X);
         f = grid_barrier(a, S, [&]() -> unsigned int {
-            float md2;
-            const bool reb = take_maxima(a, S.step, a.check - 1, md2);
-            if (atomicOr(&ctl->status, 0u))
+            const Maxima m = take_maxima(a, S.step);
+            if (m.bad || halted)
                 return RF_STOP | RF_BAD;
-            ctl->last_maxdisp2 = md2;
-            return reb ? RF_REBUILD : 0u;
-        });
-        if (!(f & RF_BAD)) {
-            if (threadIdx.x == 0) {
+            return need_rebuild(a, a.check - 1, m.d2, m.v2, m.a2) ? RF_REBUILD : 0u;
+        }, [&](unsigned int flags) {
+            if (!(flags & RF_BAD)) {
                 S.step += 1;
+                S.to_sample = S.to_sample == 0 ? a.si - 1 : S.to_sample - 1;
                 S.pp ^= 1;
-                S.md2 = ctl->last_maxdisp2;
+                run_plan(a, S);
             }
-            __syncthreads();
-            if ((f & RF_REBUILD) && !(a.what & RUN_DEFER))
-                f = run_rebuild<P>(a, S, X.nb);
-        }
+        });
+        if ((f & RF_REBUILD) && !(a.what & RUN_DEFER))
+            f = run_rebuild<P>(a, g, S, X);
     }
-    const bool steps = (a.what & RUN_STEPS) != 0, record = (a.what & (RUN_STEPS | RUN_SAMPLE | RUN_TOTALS)) != 0;
+    const bool steps = (a.what & RUN_STEPS) != 0;
     if (!(f & RF_STOP) && (a.what & (RUN_STEPS | RUN_SAMPLE | RUN_TOTALS | RUN_FORCES))) {
+        if (threadIdx.x == 0)
+            S.t0 = global_ns();
         for (;;) {
-            if (threadIdx.x == 0) {
-                S.last = !steps || (S.left == 1 && a.last);
-                S.sample = steps ? S.step % a.si == 0 : record;
-                if (blockIdx.x == 0)
-                    S.t0 = global_ns();
-            }
-            __syncthreads();
             // the previous step's sums (its partials were complete at the last barrier)
-            run_service<P>(a, S, false, sh, shf);
+            run_service<P>(a, g, S, false, X);
             if (halted) {
                 // (only the launch's first phase: its barrier ends the launch)
             } else if (S.sample) {
-                run_chunks<P, TPP, SM, true>(a, S, X.step, shf);
+                run_chunks<P, TPP, SM, true>(a, g, S, X);
             } else {
-                run_chunks<P, TPP, SM, false>(a, S, X.step, shf);
+                run_chunks<P, TPP, SM, false>(a, g, S, X);
             }
             f = grid_barrier(a, S, [&]() -> unsigned int {
-                float md2;
-                const int ci = a.check;
-                const bool check = steps && S.pos == ci - 1;
-                const bool reb = take_maxima(a, S.step, ci - 1, md2) && check && !S.last;
-                if (atomicOr(&ctl->status, 0u))
+                const Maxima m = take_maxima(a, S.step);
+                if (m.bad || halted)
                     return RF_STOP | RF_BAD;
-                if (!S.last)
-                    ctl->last_maxdisp2 = md2;
-                unsigned int g = reb ? RF_REBUILD : 0u;
+                unsigned int fl = 0u;
+                if (S.check && need_rebuild(a, a.check - 1, m.d2, m.v2, m.a2))
+                    fl |= RF_REBUILD;
                 if (!S.last && S.budget == 1) {
                     atomicOr(&ctl->status, ST_TIMEOUT);
-                    g |= RF_STOP;
+                    fl |= RF_STOP;
                 }
                 if (!steps || S.left == 1)
-                    g |= RF_STOP;
-                return g;
-            });
-            if (f & RF_ABORT)
-                return;
-            if (threadIdx.x == 0) {
+                    fl |= RF_STOP;
+                return fl;
+            }, [&](unsigned int flags) {
                 S.pend = -1;
-                if (!(f & RF_BAD)) {
+                if (!(flags & RF_BAD)) {
                     // this step's sums: by the service blocks during the next one
-                    S.pend = record ? S.step : -1;
+                    S.pend = (a.what & RUN_FORCES) ? -1 : S.step;
                     S.pend_sample = S.sample;
                     S.pend_obs = S.obs;
                     S.pend_rebuilds = S.rebuilds;
-                    S.pend_md2 = S.md2;
                     if (S.sample && !(a.what & RUN_TOTALS))
                         S.obs += 1;
                     if (!S.last) {
                         S.step += 1;
+                        S.to_sample = S.to_sample == 0 ? a.si - 1 : S.to_sample - 1;
                         S.pp ^= 1;
-                        S.md2 = ctl->last_maxdisp2;
                     }
                     S.left -= 1;
                     S.budget -= 1;
                     S.pos = S.pos == a.check - 1 ? 0 : S.pos + 1;
+                    run_plan(a, S);
                 }
+                S.done += 1;
                 if (blockIdx.x == 0) {
                     const unsigned long long t = global_ns();
                     S.ns += t > S.t0 ? t - S.t0 : 0ull;
+                    S.t0 = t;
                 }
-                S.done += 1;
-            }
-            __syncthreads();
+            });
+            if (f & RF_ABORT)
+                return;
             if (f & RF_STOP) {
-                run_service<P>(a, S, (a.what & RUN_TOTALS) != 0, sh, shf);
+                run_service<P>(a, g, S, (a.what & RUN_TOTALS) != 0, X);
                 break;
             }
             if (f & RF_REBUILD) {
-                f = run_rebuild<P>(a, S, X.nb);
+                f = run_rebuild<P>(a, g, S, X);
                 if (f & RF_ABORT)
                     return;
                 if (f & RF_STOP) {
-                    run_service<P>(a, S, false, sh, shf);
+                    run_service<P>(a, g, S, false, X);
                     break;
                 }
+                if (threadIdx.x == 0)
+                    S.t0 = global_ns();
             }
         }
     }
@@ -2320,7 +2578,6 @@ __global__ void __launch_bounds__(kForceBlock, run_min_blocks<P, SM>()) k_run(KA
         ctl->regrows = S.regrows;
         ctl->pos_par = S.pp;
         ctl->state_par = S.spar;
-        ctl->last_maxdisp2 = S.md2;
         ctl->rebuild = (f & (RF_REBUILD | RF_BAD)) == RF_REBUILD;
         ctl->n_kernels += 1;
         if (steps) {
@@ -2730,6 +2987,9 @@ KernelSet make_kernel_set()
 {
     KernelSet k;
     k.kinetic = (const void *)k_kinetic<P>;
+    k.groups[0] = run_groups<P, false>();
+    k.groups[1] = run_groups<P, true>();
+    k.group_smem = (int)sizeof(RunGroup);
     k.run[0][0] = (const void *)k_run<P, 1, false>;
     k.run[0][1] = (const void *)k_run<P, 2, false>;
     k.run[0][2] = (const void *)k_run<P, 4, false>;
