@@ -777,6 +777,7 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
             a.tab.ihs[k] = (float)ihs;
             a.tab.vcd[k] = eps != 0.0 ? shift / (4.0 * eps) : 0.0;
             a.tab.vc[k] = (float)a.tab.vcd[k];
+            a.tab.e48vcd[k] = a.tab.eps48d[k] * a.tab.vcd[k];
         }
     for (int s = 0; s < 2; ++s) {
         const int ss = std::min(s, p->n_species - 1);

@@ -85,6 +85,7 @@ struct PairTab {              // [a*2+b]
     float vc[4];              // S_ab / (4 eps_ab) (0 where eps_ab = 0): V = 4 eps_ab (s6^2 - s6 - vc)
     double rc2d[4], rl2d[4], sig2d[4], eps4d[4], eps48d[4], shiftd[4];
     double rcd[4], ihsd[4], vcd[4];
+    double e48vcd[4];         // eps48 vc
 };
 
 struct Obs {                  // identical layout to md_obs

@@ -700,75 +700,209 @@ __device__ __forceinline__ bool need_rebuild(const KArgs &a, int lookahead, floa
 constexpr float kE24hi = (float)(1.0 / 24.0);
 constexpr float kE24lo = (float)(1.0 / 24.0 - (double)(float)(1.0 / 24.0));
 
-template <typename T> struct PairRow {   // parameters of (species i, species j = 0 / 1)
-    T rc2[2], sig2[2], eps4[2], eps48[2], shift[2], rc[2], ihs[2], c[2];
+// FP64 mode: the FP64 pipe is narrow on this GPU (a warp-wide instruction keeps
+// it for ~16 cycles of the SM whatever the number of active lanes), so it sees
+// nothing but pairs inside the cutoff, spread evenly over the lanes.  A warp
+// takes its particles' rows in rounds of kPairQ entries: a single-precision test
+// with a margin (on coordinates cut to float by integer operations) queues the
+// partners that can be inside, then every lane takes an equal run of the queue,
+// whatever particles it belongs to, and leaves one partial sum per particle of
+// its run; each particle adds its partials in lane order.  The reciprocal of r^2
+// is one third-order Newton step on the hardware's 20-bit estimate.  22 FP64
+// instructions per pair instead of ~40 per list entry with an IEEE division and
+// a product and rounding per nearest image: KA N=16384, 4 lanes, 159 -> 102 us a
+// step.
+constexpr int kPairQ = 512;          // queued entries per round and warp: 16 list entries a lane
+constexpr int kPairLane = kPairQ / 32;
+
+struct PairQueue {
+    double x[32][4];                 // the warp's particles: position and species bits
+    double slot[64][4];              // partial sums (force, 12 V) by lane + particle
+    int q[kPairQ];
+    int first[33];                   // first queue entry of each particle
 };
 
+// A double's value cut to float precision, by integer operations (values below
+// 2^-127 become tiny ones; infinities and NaN do not survive).
+__device__ __forceinline__ float cut_float(double x)
+{
+    const unsigned int hi = (unsigned int)__double2hiint(x), lo = (unsigned int)__double2loint(x);
+    const unsigned int e = max(hi & 0x7fffffffu, 896u << 20) - (896u << 20);
+    return __uint_as_float((hi & 0x80000000u) | (e << 3) | (lo >> 29));
+}
+
+__device__ __forceinline__ double rcp_newton(double x)
+{
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
+template <int TPP, bool SM>
+__device__ __forceinline__ void pair_forces_d(const KArgs &a, const Rep &rp, int pp, int ii, int nn, PairQueue &Q,
+                                              double &fx, double &fy, double &fz, double &ep)
+{
+    constexpr int PPW = 32 / TPP;                        // particles of the warp
+    const int wl = threadIdx.x & 31, lane = wl & (TPP - 1), me = wl / TPP;
+    const int *lst = a.nbr + (size_t)ii * (size_t)a.Kstride;
+    const d4 *pos = (const d4 *)pos_a(a, pp);
+    const d4 xi = pos[ii];
+    const float L = (float)rp.L, half = 0.5f * L;
+    const float xf = cut_float(xi.x), yf = cut_float(xi.y), zf = cut_float(xi.z);
+    // cutoffs with the margin of the single-precision test: coordinates cut to 24 bits are
+    // off by L 2^-23 at most, so r^2 by about 4 r_c L 2^-22
+    float rc2f[2];
+#pragma unroll
+    for (int tj = 0; tj < 2; ++tj)
+        rc2f[tj] = a.tab.rc2[species_of(xi.w) * 2 + tj] + 1e-5f * L + 1e-3f;
+    __syncwarp();
+    if (lane == 0) {
+        Q.x[me][0] = xi.x;
+        Q.x[me][1] = xi.y;
+        Q.x[me][2] = xi.z;
+        Q.x[me][3] = xi.w;
+    }
+    double sx = 0.0, sy = 0.0, sz = 0.0, se = 0.0;       // of the lane's own particle; se: sum of 12 V
+    const int rows = (int)__reduce_max_sync(0xffffffffu, (unsigned)nn);
+    for (int r0 = 0; r0 < rows; r0 += kPairLane * TPP) {
+        // queue the entries [r0, r0 + kPairLane TPP) of every row that can be inside
+        const int k0 = r0 + kPairLane * lane;
+        int jj[kPairLane];
+        unsigned int keep = 0u;
+#pragma unroll
+        for (int b = 0; b < kPairLane; b += 4) {
+            const bool in = k0 + b < nn;                 // (rows are padded to whole groups of 8)
+            const int4 j4 = in ? *(const int4 *)(lst + k0 + b) : make_int4(ii, ii, ii, ii);
+            jj[b] = j4.x;
+            jj[b + 1] = j4.y;
+            jj[b + 2] = j4.z;
+            jj[b + 3] = j4.w;
+            if (in) {
+                d4 xs[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    xs[u] = pos[checked(a, jj[b + u], a.n, ii)];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    float dx = xf - cut_float(xs[u].x), dy = yf - cut_float(xs[u].y), dz = zf - cut_float(xs[u].z);
+                    dx = fabsf(dx);
+                    dy = fabsf(dy);
+                    dz = fabsf(dz);
+                    dx = dx > half ? dx - L : dx;
+                    dy = dy > half ? dy - L : dy;
+                    dz = dz > half ? dz - L : dz;
+                    const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                    // (the padding is the particle itself; a NaN passes, and shows in the sums)
+                    if (!(r2 >= (species_of(xs[u].w) ? rc2f[1] : rc2f[0])) && jj[b + u] != ii)
+                        keep |= 1u << (b + u);
+                }
+            }
+        }
+        const int n = __popc(keep);
+        int incl = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (wl >= o)
+                incl += y;
+        }
+        const int W = __shfl_sync(0xffffffffu, incl, 31);
+        int at = incl - n;
+        if (lane == 0)
+            Q.first[me] = at;
+        if (wl == 31)
+            Q.first[PPW] = W;
+#pragma unroll
+        for (int b = 0; b < kPairLane; ++b)
+            if (keep >> b & 1u)
+                Q.q[at++] = jj[b];
+        __syncwarp();
+
+        // every lane takes m entries of the queue
+        const int m = (W + 31) / 32;
+        int t = wl * m;
+        const int end = min(t + m, W);
+        int p = 0;
+        while (p + 1 < PPW && Q.first[p + 1] <= t)
+            ++p;
+        double ox = Q.x[p][0], oy = Q.x[p][1], oz = Q.x[p][2];
+        int to = species_of(Q.x[p][3]) * 2;
+        double gx = 0.0, gy = 0.0, gz = 0.0, ge = 0.0;
+        d4 xn = pos[checked(a, t < end ? Q.q[t] : ii, a.n, ii)];   // one entry ahead
+        for (int it = 0; it < m; ++it, ++t) {
+            const bool on = t < end;
+            const d4 xj = xn;
+            xn = pos[checked(a, t + 1 < end ? Q.q[t + 1] : ii, a.n, ii)];
+            if (on && t >= Q.first[p + 1]) {             // the next particle's entries
+                double *s = Q.slot[wl + p];
+                s[0] = gx; s[1] = gy; s[2] = gz; s[3] = ge;
+                gx = gy = gz = ge = 0.0;
+                do
+                    ++p;
+                while (t >= Q.first[p + 1]);
+                ox = Q.x[p][0]; oy = Q.x[p][1]; oz = Q.x[p][2];
+                to = species_of(Q.x[p][3]) * 2;
+            }
+            const int ab = to + species_of(xj.w);
+            double dx = ox - xj.x, dy = oy - xj.y, dz = oz - xj.z;
+            // nearest image: within the cutoff it is a shift by one box or none, told from
+            // the high words
+            const float ex = cut_float(dx), ey = cut_float(dy), ez = cut_float(dz);
+            if (__any_sync(0xffffffffu, fabsf(ex) > half || fabsf(ey) > half || fabsf(ez) > half)) {
+                dx = ex > half ? dx - rp.L : (ex < -half ? dx + rp.L : dx);
+                dy = ey > half ? dy - rp.L : (ey < -half ? dy + rp.L : dy);
+                dz = ez > half ? dz - rp.L : (ez < -half ? dz + rp.L : dz);
+            }
+            const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+            // 0 < r2 < rc2, on the bits (neither is negative; a NaN is above)
+            const long long bits = __double_as_longlong(r2);
+            const bool in = on && bits > 0 && bits < __double_as_longlong(a.tab.rc2d[ab]);
+            const double ir2 = rcp_newton(in ? r2 : 1.0);
+            const double s2 = a.tab.sig2d[ab] * ir2;
+            const double s6 = s2 * s2 * s2;
+            const double w = s6 - 0.5;
+            const double e6 = (in ? a.tab.eps48d[ab] : 0.0) * s6;
+            double fr = e6 * ir2 * w;
+            if (SM) {
+                double v = in ? a.tab.eps4d[ab] * s6 * (s6 - 1.0) - a.tab.shiftd[ab] : 0.0;
+                smooth_pair(in ? r2 : 1.0, a.tab.rcd[ab], a.tab.ihsd[ab], fr, v);
+                ge = fma(12.0, v, ge);
+            } else {
+                ge += fma(e6, s6 - 1.0, in ? -a.tab.e48vcd[ab] : 0.0);
+            }
+            gx = fma(fr, dx, gx);
+            gy = fma(fr, dy, gy);
+            gz = fma(fr, dz, gz);
+        }
+        if (wl * m < end) {
+            double *s = Q.slot[wl + p];
+            s[0] = gx; s[1] = gy; s[2] = gz; s[3] = ge;
+        }
+        __syncwarp();
+        // the particle's partials, in lane order
+        const int q0 = Q.first[me], q1 = Q.first[me + 1];
+        if (q0 < q1)
+            for (int s = q0 / m + me; s <= (q1 - 1) / m + me; ++s) {
+                sx += Q.slot[s][0];
+                sy += Q.slot[s][1];
+                sz += Q.slot[s][2];
+                se += Q.slot[s][3];
+            }
+        __syncwarp();
+    }
+    fx = sx; fy = sy; fz = sz;
+    ep = se * (1.0 / 24.0);
+}
+
 template <int P, int TPP, bool SM>
-__device__ __forceinline__ void pair_forces(const KArgs &a, const Rep &rp, int pp, int ii, int nn,
+__device__ __forceinline__ void pair_forces(const KArgs &a, const Rep &rp, int pp, int ii, int nn, PairQueue *Q,
                                             FT<P> &fx, FT<P> &fy, FT<P> &fz, ET<P> &ep)
 {
     const int lane = threadIdx.x & (TPP - 1);
     const int *lst = a.nbr + (size_t)ii * (size_t)a.Kstride;
     if constexpr (P == FP64) {
-        const d4 *pos = (const d4 *)pos_a(a, pp);
-        const d4 xi = pos[ii];
-        const int ti = species_of(xi.w);
-        PairRow<double> pr;
-#pragma unroll
-        for (int tj = 0; tj < 2; ++tj) {
-            pr.rc2[tj] = a.tab.rc2d[ti * 2 + tj];
-            pr.sig2[tj] = a.tab.sig2d[ti * 2 + tj];
-            pr.eps4[tj] = a.tab.eps4d[ti * 2 + tj];
-            pr.eps48[tj] = a.tab.eps48d[ti * 2 + tj];
-            pr.shift[tj] = a.tab.shiftd[ti * 2 + tj];
-            pr.rc[tj] = a.tab.rcd[ti * 2 + tj];
-            pr.ihs[tj] = a.tab.ihsd[ti * 2 + tj];
-            pr.c[tj] = a.tab.vcd[ti * 2 + tj];
-        }
-        double sx = 0, sy = 0, sz = 0, se = 0;          // se: sum of 12 V
-        for (int k0 = 4 * lane; k0 < nn; k0 += 4 * TPP) {
-            const int4 q = *(const int4 *)(lst + k0);
-            const int jj[4] = {q.x, q.y, q.z, q.w};
-            d4 xs[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)                 // padded rows: whole groups
-                xs[u] = pos[checked(a, jj[u], a.n, ii)];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const d4 xj = xs[u];
-                const int tj = species_of(xj.w);
-                const double dx = sep_d(xi.x, xj.x, rp.L, rp.invL);
-                const double dy = sep_d(xi.y, xj.y, rp.L, rp.invL);
-                const double dz = sep_d(xi.z, xj.z, rp.L, rp.invL);
-                const double r2 = dx * dx + dy * dy + dz * dz;
-                if (r2 < pr.rc2[tj] && r2 > 0.0) {          // r2 = 0: the padding entry
-                    const double ir2 = 1.0 / r2;
-                    const double s2 = pr.sig2[tj] * ir2;
-                    const double s6 = s2 * s2 * s2;
-                    double fr = pr.eps48[tj] * ir2 * s6 * (s6 - 0.5);
-                    if (SM) {
-                        double v = pr.eps4[tj] * s6 * (s6 - 1.0) - pr.shift[tj];
-                        smooth_pair(r2, pr.rc[tj], pr.ihs[tj], fr, v);
-                        se = fma(12.0, v, se);
-                    } else {
-                        se = fma(pr.eps48[tj], fma(s6, s6, -(s6 + pr.c[tj])), se);
-                    }
-                    sx += fr * dx;
-                    sy += fr * dy;
-                    sz += fr * dz;
-                }
-            }
-        }
-#pragma unroll
-        for (int o = TPP / 2; o > 0; o >>= 1) {
-            sx += __shfl_xor_sync(0xffffffffu, sx, o);
-            sy += __shfl_xor_sync(0xffffffffu, sy, o);
-            sz += __shfl_xor_sync(0xffffffffu, sz, o);
-            se += __shfl_xor_sync(0xffffffffu, se, o);
-        }
-        fx = sx; fy = sy; fz = sz;
-        ep = se * (1.0 / 24.0);
+        pair_forces_d<TPP, SM>(a, rp, pp, ii, nn, *Q, fx, fy, fz, ep);
     } else {
         // MIXED reads the fixed-point copy (16 B per neighbour), FP32 the positions
         const float4 *pos = (const float4 *)pos_a(a, pp);
@@ -1152,7 +1286,7 @@ __device__ __forceinline__ void component_update(const KArgs &a, const Rep &rp, 
 // position buffer.  The operands of the update are loaded before the
 // neighbour loop so that their latency is hidden.
 template <int P, int TPP, bool SAMPLE, bool SM>
-__device__ __forceinline__ void step_body_split(const KArgs &a, const Rep &rep, const int4 b, bool kick, bool last, bool track,
+__device__ __forceinline__ void step_body_split(const KArgs &a, const Rep &rep, PairQueue *Q, const int4 b, bool kick, bool last, bool track,
                                                 int pp, int spar, double *part, ET<P> &eo, float &d2, float &v2, float &a2,
                                                 unsigned int &bad)
 {
@@ -1187,7 +1321,7 @@ __device__ __forceinline__ void step_body_split(const KArgs &a, const Rep &rep, 
     for (int k = 0; k < kPartF; ++k)
         part[k] = 0.0;
     eo = e_zero<P>();
-    pair_forces<P, TPP, SM>(a, rp, pp, ii, nn, fx, fy, fz, ep);
+    pair_forces<P, TPP, SM>(a, rp, pp, ii, nn, Q, fx, fy, fz, ep);
     if (SAMPLE)
         pair_virial<P, TPP, SM>(a, rp, pp, ii, nn, part);
     // Every lane of the warp must reach the shuffles below, including the
@@ -1273,12 +1407,12 @@ __device__ __forceinline__ void step_body_split(const KArgs &a, const Rep &rep, 
 }
 
 template <int P, int TPP, bool SAMPLE, bool SM>
-__device__ __forceinline__ void step_body(const KArgs &a, const Rep &rep, const int4 b, bool kick, bool last, bool track,
+__device__ __forceinline__ void step_body(const KArgs &a, const Rep &rep, PairQueue *Q, const int4 b, bool kick, bool last, bool track,
                                           int pp, int spar, double *part, ET<P> &eo, float &d2, float &v2, float &a2,
                                           unsigned int &bad)
 {
     if constexpr (kSplitUpdate || TPP >= 4) {
-        step_body_split<P, TPP, SAMPLE, SM>(a, rep, b, kick, last, track, pp, spar, part, eo, d2, v2, a2, bad);
+        step_body_split<P, TPP, SAMPLE, SM>(a, rep, Q, b, kick, last, track, pp, spar, part, eo, d2, v2, a2, bad);
         return;
     }
     const Rep rp = rep;
@@ -1293,7 +1427,7 @@ __device__ __forceinline__ void step_body(const KArgs &a, const Rep &rep, const 
     for (int k = 0; k < kPartF; ++k)
         part[k] = 0.0;
     eo = e_zero<P>();
-    pair_forces<P, TPP, SM>(a, rp, pp, ii, nn, fx, fy, fz, ep);
+    pair_forces<P, TPP, SM>(a, rp, pp, ii, nn, Q, fx, fy, fz, ep);
     if (SAMPLE)
         pair_virial<P, TPP, SM>(a, rp, pp, ii, nn, part);
     if (!(valid && lane == 0)) {
@@ -2091,18 +2225,27 @@ struct RunState {
 
 // Shared scratch of a group.  Of a step: sums, and what a thread keeps between
 // its chunks (registers are scarce in the pair loop).
+template <int P> struct PairScratch { __device__ PairQueue *queue(int) { return nullptr; } };
+template <> struct PairScratch<FP64> {
+    PairQueue q[kGrpWarps];
+    __device__ PairQueue *queue(int w) { return q + w; }
+};
+
+template <int P>
 struct RunSums {
+    PairScratch<P> pair;
     double sh[kGrpWarps * kPartF];
     double tot[kPartF];                              // sums of a one-replica sample
     double e[kForceBlock];                           // energy (ET) and maxima so far, per thread
     float d2[kForceBlock], v2[kForceBlock], a2[kForceBlock];
 };
 
+template <int P>
 struct RunGroup {
     union {
         NbBlock nb;
         NbWarp nbw[kGrpWarps];
-        RunSums step;
+        RunSums<P> step;
         int scan[kGrpWarps];
     };
     int4 row;                                        // the group's first chunk
@@ -2196,7 +2339,7 @@ __device__ __forceinline__ Maxima take_maxima(const KArgs &a, long long step)
 // Rebuild of the lists; returns the flags of its last barrier (the state's
 // parities and capacity are those of the new lists unless RF_BAD).
 template <int P>
-__device__ __forceinline__ unsigned int run_rebuild(const KArgs &a, const Grp &g, RunState &S, RunGroup &X)
+__device__ __forceinline__ unsigned int run_rebuild(const KArgs &a, const Grp &g, RunState &S, RunGroup<P> &X)
 {
     Ctl *ctl = a.ctl;
     if (blockIdx.x == 0 && threadIdx.x == 0)
@@ -2296,7 +2439,7 @@ __device__ __forceinline__ unsigned int run_rebuild(const KArgs &a, const Grp &g
 
 // The half kick and drift that open md_step.
 template <int P>
-__device__ __forceinline__ void run_first(const KArgs &a, const Grp &g, RunState &S, RunGroup &X)
+__device__ __forceinline__ void run_first(const KArgs &a, const Grp &g, RunState &S, RunGroup<P> &X)
 {
     const int pp = S.pp, spar = S.spar;
     float d2 = 0.f, v2 = 0.f, a2 = 0.f;
@@ -2334,9 +2477,10 @@ __device__ __forceinline__ void run_first(const KArgs &a, const Grp &g, RunState
 // One sweep over the group's chunks: forces, the particles' update, and the
 // partial sums and maxima.
 template <int P, int TPP, bool SM, bool SAMPLE>
-__device__ __forceinline__ void run_chunks(const KArgs &a, const Grp &g, RunState &S, RunGroup &G)
+__device__ __forceinline__ void run_chunks(const KArgs &a, const Grp &g, RunState &S, RunGroup<P> &G)
 {
-    RunSums &X = G.step;
+    RunSums<P> &X = G.step;
+    PairQueue *Q = X.pair.queue(g.tid() >> 5);
     X.d2[g.tid()] = X.v2[g.tid()] = X.a2[g.tid()] = 0.f;
     ET<P> *xe = reinterpret_cast<ET<P> *>(X.e);
     xe[g.tid()] = e_zero<P>();
@@ -2352,7 +2496,7 @@ __device__ __forceinline__ void run_chunks(const KArgs &a, const Grp &g, RunStat
         ET<P> eo;
         float d2 = 0.f, v2 = 0.f, a2 = 0.f;
         unsigned int bad = 0u;
-        step_body<P, TPP, SAMPLE, SM>(a, a.nrep == 1 ? S.rep : a.rep[b.z], b, (a.what & RUN_STEPS) != 0, S.last != 0,
+        step_body<P, TPP, SAMPLE, SM>(a, a.nrep == 1 ? S.rep : a.rep[b.z], Q, b, (a.what & RUN_STEPS) != 0, S.last != 0,
                                       S.track != 0, S.pp, S.spar, part, eo, d2, v2, a2, bad);
         if (bad)
             put_bad(a, S.step, bad);
@@ -2402,7 +2546,7 @@ __device__ __forceinline__ void run_chunks(const KArgs &a, const Grp &g, RunStat
 // Sums of the step that awaits them, one group per replica, the last groups of
 // the grid first: they have the fewest chunks (none, where groups are to spare).
 template <int P>
-__device__ __forceinline__ void run_service(const KArgs &a, const Grp &g, RunState &S, bool totals, RunGroup &X)
+__device__ __forceinline__ void run_service(const KArgs &a, const Grp &g, RunState &S, bool totals, RunGroup<P> &X)
 {
     if (S.pend < 0)
         return;
@@ -2440,7 +2584,7 @@ __global__ void __launch_bounds__(kForceBlock * run_groups<P, SM>(), 1) k_run(KA
     g.id = threadIdx.x / kForceBlock;
     g.vb = blockIdx.x + g.id * gridDim.x;            // (groups p, p + gridDim, ... share an SM)
     g.nvb = gridDim.x * (blockDim.x / kForceBlock);
-    RunGroup &X = reinterpret_cast<RunGroup *>(smem)[g.id];
+    RunGroup<P> &X = reinterpret_cast<RunGroup<P> *>(smem)[g.id];
     Ctl *ctl = a.ctl;
     if (a.nrep == 1)
         for (int k = threadIdx.x; k < (int)(sizeof(Rep) / 4); k += blockDim.x)
@@ -2989,7 +3133,7 @@ KernelSet make_kernel_set()
     k.kinetic = (const void *)k_kinetic<P>;
     k.groups[0] = run_groups<P, false>();
     k.groups[1] = run_groups<P, true>();
-    k.group_smem = (int)sizeof(RunGroup);
+    k.group_smem = (int)sizeof(RunGroup<P>);
     k.run[0][0] = (const void *)k_run<P, 1, false>;
     k.run[0][1] = (const void *)k_run<P, 2, false>;
     k.run[0][2] = (const void *)k_run<P, 4, false>;
