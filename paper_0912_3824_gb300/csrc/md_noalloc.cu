@@ -16,6 +16,7 @@
 // device address is looked up once per device with cudaGetSymbolAddress().
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <cstddef>
 #include <cstdio>
 #include <mutex>
@@ -24,12 +25,12 @@
 
 namespace {
 
-constexpr int kBlock = 128;
-constexpr int kMaxBlocks = 8192;   // n <= kMaxBlocks * kBlock = MD_NOALLOC_MAX_N
+constexpr int kMaxBlocks = 8192;   // blocks of a call: the scratch holds a partial sum of each
+constexpr int kRows = 4;           // particles per warp at a time
+constexpr int kTile = 512;         // partners staged at a time
 constexpr int kPart = 8;           // e_pot, virial, w_xx, w_yy, w_zz, w_xy, w_xz, w_yz
 constexpr int kMaxDevices = 64;
 
-static_assert((long long)kMaxBlocks * kBlock == MD_NOALLOC_MAX_N, "scratch sized for MD_NOALLOC_MAX_N");
 
 // Per-block partial sums, the ticket that elects the block finishing the
 // totals, and a flag raised by any block that met a species outside
@@ -45,12 +46,8 @@ static __device__ __align__(256) Scratch g_noalloc_scratch;
 
 struct Pot {
     double rc2[4], sig2[4], eps4[4], eps48[4], shift[4];
+    float rc2u[4];                 // (r_c + margin)^2 in units of (L / 2^32)^2
 };
-
-__device__ __forceinline__ double min_image(double d, double L, double invL)
-{
-    return d - L * rint(d * invL);
-}
 
 // Species code of a particle, clamped into [0, nsp) so that it always indexes
 // the pair table; an out-of-range code raises the call's bad flag.
@@ -63,91 +60,186 @@ __device__ __forceinline__ int species_in_range(int t, int nsp, Scratch *s)
     return t;
 }
 
-// One thread per particle i, looping over every j through shared-memory tiles
-// of positions; pair arithmetic in double (FP64 mode) or single precision on
-// separations formed in double (the other modes).
-template <bool FP64MATH>
-__global__ void __launch_bounds__(kBlock) k_forces_allpairs(Pot pot, int n, int nsp, double L, const int *species,
-                                                            const double *pos, double *force, double *energy,
-                                                            double *totals, Scratch *s)
+// Number of boxes nearest to d / L, as a double: adding 1.5 2^52 rounds.
+__device__ __forceinline__ double boxes(double d, double invL)
 {
-    __shared__ double tx[kBlock], ty[kBlock], tz[kBlock];
-    __shared__ int tt[kBlock];
-    __shared__ double red[kBlock / 32][kPart];
-    __shared__ int is_last;
-    const int i = blockIdx.x * kBlock + threadIdx.x;
-    const double invL = 1.0 / L;
-    double xi = 0.0, yi = 0.0, zi = 0.0;
-    int ti = 0;
-    bool ti_bad = false;
-    if (i < n) {
-        xi = pos[3 * (size_t)i];
-        yi = pos[3 * (size_t)i + 1];
-        zi = pos[3 * (size_t)i + 2];
-        ti_bad = species[i] < 0 || species[i] >= nsp;
-        ti = species_in_range(species[i], nsp, s);
-    }
-    double fx = 0.0, fy = 0.0, fz = 0.0, acc[kPart] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int j0 = 0; j0 < n; j0 += kBlock) {
-        const int j = j0 + threadIdx.x;
-        if (j < n) {
-            tx[threadIdx.x] = pos[3 * (size_t)j];
-            ty[threadIdx.x] = pos[3 * (size_t)j + 1];
-            tz[threadIdx.x] = pos[3 * (size_t)j + 2];
-            tt[threadIdx.x] = species_in_range(species[j], nsp, s);
+    constexpr double big = 6755399441055744.0;
+    return fma(d, invL, big) - big;
+}
+
+// x / L modulo 1 in units of 2^-32: the low word of x 2^32 / L + 1.5 2^52.  Off
+// by less than 1 1/4 units for |x| < 2^18 L; beyond (or not finite), `far` is set.
+__device__ __forceinline__ int circle(double x, double scale, unsigned int far_hi, bool &far)
+{
+    far |= (unsigned int)(__double2hiint(x) & 0x7fffffff) >= far_hi;
+    return __double2loint(fma(x, scale, 6755399441055744.0));
+}
+
+// Direct sum over all pairs.  A warp takes kRows particles, its lanes the
+// partners, staged by the block as 32-bit fractions of the box: their wrapped
+// differences are the nearest images, so the test that lets a pair through (with
+// a margin for the rounding) is single precision and integers only.  The FP64
+// pipe, narrow on this GPU, sees only the pairs let through: they wait in a
+// queue per particle and are evaluated 32 at a time, one per lane, from the
+// caller's coordinates, in double (FP64 mode) or in single precision on
+// separations formed in double (the other modes).  Coordinates so far from the
+// box that the fractions are not safe let every pair through.
+//
+// Bound by the tests for large n (about 13 instructions per 32 partners and
+// particle) and by the FP64 sums for small n.  KA mixture, mixed: 0.14 ms at
+// n = 6000, 0.55 at 16,384, 5.5 at 65,536; one thread per particle doing every test
+// in FP64 took 4.5, 10.3 and 154 ms.
+template <bool FP64MATH, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS) k_forces_allpairs(Pot pot, int n, int nsp, double L, const int *species,
+                                                                const double *pos, double *force, double *energy,
+                                                                double *totals, Scratch *s)
+{
+    __shared__ int4 tile[kTile];
+    __shared__ int queue[WARPS][kRows][64];
+    __shared__ double red[WARPS][kPart];
+    __shared__ double tot[32][kPart];
+    __shared__ int is_last, tile_far;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned lt_mask = (1u << lane) - 1u;
+    const double invL = 1.0 / L, scale = 4294967296.0 / L;
+    const unsigned int far_hi = (unsigned int)__double2hiint(262144.0 * L);
+    double acc[kPart] = {0, 0, 0, 0, 0, 0, 0, 0};         // totals of the lane's pairs, each seen from both sides
+
+    for (long long base = (long long)blockIdx.x * WARPS * kRows; base < n; base += (long long)gridDim.x * WARPS * kRows) {
+        const int i0 = (int)base + w * kRows;             // the warp's particles i0 .. i0 + kRows - 1
+        int4 qi[kRows];
+        float lim[kRows][2];
+        double f[kRows][4];                               // force, energy
+        int cnt[kRows];
+        bool own_far = false;
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) {
+            const size_t i = (size_t)min(i0 + r, n - 1);
+            qi[r].x = circle(pos[3 * i], scale, far_hi, own_far);
+            qi[r].y = circle(pos[3 * i + 1], scale, far_hi, own_far);
+            qi[r].z = circle(pos[3 * i + 2], scale, far_hi, own_far);
+            qi[r].w = species_in_range(species[i], nsp, s);
+            lim[r][0] = i0 + r < n ? pot.rc2u[qi[r].w * 2] : 0.0f;
+            lim[r][1] = i0 + r < n ? pot.rc2u[qi[r].w * 2 + 1] : 0.0f;
+            f[r][0] = f[r][1] = f[r][2] = f[r][3] = 0.0;
+            cnt[r] = 0;
         }
-        __syncthreads();
-        const int m = min(kBlock, n - j0);
-        if (i < n) {
-            for (int k = 0; k < m; ++k) {
-                if (j0 + k == i)
-                    continue;
-                const double dx = min_image(xi - tx[k], L, invL);
-                const double dy = min_image(yi - ty[k], L, invL);
-                const double dz = min_image(zi - tz[k], L, invL);
+        // evaluates the first m (up to 32) queued partners of particle i0 + r
+        const auto flush = [&](int r, int m) {
+            const int i = i0 + r, j = lane < m ? queue[w][r][lane] : i;
+            if (j != i) {
+                double dx = pos[3 * (size_t)i] - pos[3 * (size_t)j];
+                double dy = pos[3 * (size_t)i + 1] - pos[3 * (size_t)j + 1];
+                double dz = pos[3 * (size_t)i + 2] - pos[3 * (size_t)j + 2];
+                dx = fma(-L, boxes(dx, invL), dx);
+                dy = fma(-L, boxes(dy, invL), dy);
+                dz = fma(-L, boxes(dz, invL), dz);
                 const double r2 = dx * dx + dy * dy + dz * dz;
-                const int ab = ti * 2 + tt[k];
-                if (!(r2 < pot.rc2[ab]))
-                    continue;
-                double fr, v;
-                if (FP64MATH) {
-                    const double ir2 = 1.0 / r2;
-                    const double s2 = pot.sig2[ab] * ir2;
-                    const double s6 = s2 * s2 * s2;
-                    fr = pot.eps48[ab] * ir2 * s6 * (s6 - 0.5);
-                    v = pot.eps4[ab] * s6 * (s6 - 1.0) - pot.shift[ab];
-                } else {
-                    const float ir2 = 1.0f / (float)r2;
-                    const float s2 = (float)pot.sig2[ab] * ir2;
-                    const float s6 = s2 * s2 * s2;
-                    fr = (double)((float)pot.eps48[ab] * ir2 * s6 * (s6 - 0.5f));
-                    v = (double)((float)pot.eps4[ab] * s6 * (s6 - 1.0f) - (float)pot.shift[ab]);
+                const int tj = species[j];
+                const int ab = qi[r].w * 2 + (tj < 0 ? 0 : (tj >= nsp ? nsp - 1 : tj));
+                if (r2 < pot.rc2[ab]) {
+                    double fr, v;
+                    if (FP64MATH) {
+                        const double ir2 = 1.0 / r2;
+                        const double s2 = pot.sig2[ab] * ir2;
+                        const double s6 = s2 * s2 * s2;
+                        fr = pot.eps48[ab] * ir2 * s6 * (s6 - 0.5);
+                        v = pot.eps4[ab] * s6 * (s6 - 1.0) - pot.shift[ab];
+                    } else {
+                        const float ir2 = 1.0f / (float)r2;
+                        const float s2 = (float)pot.sig2[ab] * ir2;
+                        const float s6 = s2 * s2 * s2;
+                        fr = (double)((float)pot.eps48[ab] * ir2 * s6 * (s6 - 0.5f));
+                        v = (double)((float)pot.eps4[ab] * s6 * (s6 - 1.0f) - (float)pot.shift[ab]);
+                    }
+                    const double px = fr * dx, py = fr * dy, pz = fr * dz;
+                    f[r][0] += px;
+                    f[r][1] += py;
+                    f[r][2] += pz;
+                    f[r][3] += v;
+                    acc[1] += fr * r2;
+                    acc[2] += px * dx;
+                    acc[3] += py * dy;
+                    acc[4] += pz * dz;
+                    acc[5] += px * dy;
+                    acc[6] += px * dz;
+                    acc[7] += py * dz;
                 }
-                fx += fr * dx;
-                fy += fr * dy;
-                fz += fr * dz;
-                acc[0] += v;
-                acc[1] += fr * r2;
-                acc[2] += fr * dx * dx;
-                acc[3] += fr * dy * dy;
-                acc[4] += fr * dz * dz;
-                acc[5] += fr * dx * dy;
-                acc[6] += fr * dx * dz;
-                acc[7] += fr * dy * dz;
+            }
+        };
+
+        for (int j0 = 0; j0 < n; j0 += kTile) {
+            __syncthreads();
+            if (threadIdx.x == 0)
+                tile_far = 0;
+            __syncthreads();
+            for (int t = threadIdx.x; t < kTile && j0 + t < n; t += 32 * WARPS) {
+                const size_t j = (size_t)(j0 + t);
+                bool far = own_far;
+                int4 q;
+                q.x = circle(pos[3 * j], scale, far_hi, far);
+                q.y = circle(pos[3 * j + 1], scale, far_hi, far);
+                q.z = circle(pos[3 * j + 2], scale, far_hi, far);
+                q.w = species_in_range(species[j], nsp, s);
+                tile[t] = q;
+                if (far)
+                    tile_far = 1;
+            }
+            __syncthreads();
+            const int m = min(kTile, n - j0);
+            const bool all = tile_far != 0 || own_far;
+            for (int t0 = 0; t0 < m; t0 += 32) {
+                const int t = t0 + lane;
+                const bool ok = t < m;
+                const int4 q = tile[ok ? t : 0];
+#pragma unroll
+                for (int r = 0; r < kRows; ++r) {
+                    const float x = __int2float_rn((int)((unsigned)qi[r].x - (unsigned)q.x));
+                    const float y = __int2float_rn((int)((unsigned)qi[r].y - (unsigned)q.y));
+                    const float z = __int2float_rn((int)((unsigned)qi[r].z - (unsigned)q.z));
+                    const float r2 = fmaf(x, x, fmaf(y, y, z * z));
+                    const unsigned b =
+                        __ballot_sync(0xffffffffu, ok && (r2 < (q.w ? lim[r][1] : lim[r][0]) || all) && i0 + r < n);
+                    if (b == 0u)
+                        continue;
+                    if (b >> lane & 1u)
+                        queue[w][r][cnt[r] + __popc(b & lt_mask)] = j0 + t;
+                    cnt[r] += __popc(b);
+                    if (cnt[r] >= 32) {
+                        __syncwarp();
+                        flush(r, 32);
+                        __syncwarp();
+                        const int next = lane < cnt[r] - 32 ? queue[w][r][32 + lane] : 0;
+                        __syncwarp();
+                        queue[w][r][lane] = next;
+                        cnt[r] -= 32;
+                    }
+                }
             }
         }
-        __syncthreads();
-    }
-    if (i < n) {
-        const double poison = ti_bad ? __longlong_as_double(0x7ff8000000000000ll) : 0.0;   // NaN
-        force[3 * (size_t)i] = fx + poison;
-        force[3 * (size_t)i + 1] = fy + poison;
-        force[3 * (size_t)i + 2] = fz + poison;
-        if (energy)
-            energy[i] = 0.5 * acc[0] + poison;
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < kRows; ++r) {
+            flush(r, cnt[r]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                for (int o = 16; o > 0; o >>= 1)
+                    f[r][k] += __shfl_xor_sync(0xffffffffu, f[r][k], o);
+            const int i = i0 + r;
+            if (lane == 0 && i < n) {
+                // a species code out of range: NaN
+                const bool bad = species[i] < 0 || species[i] >= nsp;
+                const double poison = bad ? __longlong_as_double(0x7ff8000000000000ll) : 0.0;
+                force[3 * (size_t)i] = f[r][0] + poison;
+                force[3 * (size_t)i + 1] = f[r][1] + poison;
+                force[3 * (size_t)i + 2] = f[r][2] + poison;
+                if (energy)
+                    energy[i] = 0.5 * f[r][3] + poison;
+                acc[0] += f[r][3];
+            }
+        }
     }
     // block sums in a fixed order, then the last block adds the blocks' sums
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
     for (int k = 0; k < kPart; ++k) {
         double v = 0.5 * acc[k];
@@ -160,7 +252,7 @@ __global__ void __launch_bounds__(kBlock) k_forces_allpairs(Pot pot, int n, int 
     if (threadIdx.x == 0) {
         for (int k = 0; k < kPart; ++k) {
             double v = 0.0;
-            for (int q = 0; q < kBlock / 32; ++q)
+            for (int q = 0; q < WARPS; ++q)
                 v += red[q][k];
             s->part[(size_t)blockIdx.x * kPart + k] = v;
         }
@@ -171,15 +263,35 @@ __global__ void __launch_bounds__(kBlock) k_forces_allpairs(Pot pot, int n, int 
     if (!is_last)
         return;
     __threadfence();
+    // (a slice of the blocks per 8 threads, then the slices in order)
+    constexpr int kSlices = 32 * WARPS / kPart;
+    const int c = threadIdx.x % kPart, sl = threadIdx.x / kPart;
+    double v = 0.0;
+#pragma unroll 4
+    for (unsigned int b = sl; b < gridDim.x; b += kSlices)
+        v += __ldcg(&s->part[(size_t)b * kPart + c]);
+    tot[sl][c] = v;
+    __syncthreads();
     if (threadIdx.x < kPart) {
-        double v = 0.0;
-        for (unsigned int b = 0; b < gridDim.x; ++b)
-            v += ((volatile double *)s->part)[(size_t)b * kPart + threadIdx.x];
+        v = 0.0;
+        for (int q = 0; q < kSlices; ++q)
+            v += tot[q][threadIdx.x];
         // a species code out of range makes every total NaN
         if (atomicOr(&s->bad, 0u) != 0u)
             v = __longlong_as_double(0x7ff8000000000000ll);
         totals[threadIdx.x] = v;
     }
+}
+
+template <int WARPS>
+void launch(bool fp64, cudaStream_t st, const Pot &pot, int n, int nsp, double box, const int *species, const double *pos,
+            double *force, double *energy, double *totals, Scratch *s)
+{
+    const int per = WARPS * kRows, need = (n + per - 1) / per, grid = need < kMaxBlocks ? need : kMaxBlocks;
+    if (fp64)
+        k_forces_allpairs<true, WARPS><<<grid, 32 * WARPS, 0, st>>>(pot, n, nsp, box, species, pos, force, energy, totals, s);
+    else
+        k_forces_allpairs<false, WARPS><<<grid, 32 * WARPS, 0, st>>>(pot, n, nsp, box, species, pos, force, energy, totals, s);
 }
 
 std::mutex g_lock;
@@ -259,14 +371,20 @@ extern "C" int md_forces_noalloc(const md_params *p, int64_t n, double box, cons
     static_assert(offsetof(Scratch, bad) == offsetof(Scratch, ticket) + sizeof(unsigned int), "adjacent words");
     if (cudaMemsetAsync(&s->ticket, 0, 2 * sizeof(unsigned int), st) != cudaSuccess)
         return fail(MD_E_CUDA, "md_forces_noalloc: clearing the scratch ticket failed");
-    const int grid = (int)((n + kBlock - 1) / kBlock);
+    // margin of the single-precision test: the fractions are off by 2.5 units in a difference,
+    // its conversion and the sum of squares by a few 2^-24 of it
+    const double unit = box / 4294967296.0;
+    for (int k = 0; k < 4; ++k) {
+        const double rc = sqrt(pot.rc2[k]) * (1.0 + 1e-6) / unit + 8.0;
+        pot.rc2u[k] = (float)(rc * rc * (1.0 + 1e-6));
+    }
+    // few particles: smaller blocks, to spread over the SMs
     const int nsp = p->n_species;
-    if (p->precision == MD_PREC_FP64)
-        k_forces_allpairs<true><<<grid, kBlock, 0, st>>>(pot, (int)n, nsp, box, species, pos, force, energy, totals,
-                                                          s);
+    const bool fp64 = p->precision == MD_PREC_FP64;
+    if (n <= 16384)
+        launch<4>(fp64, st, pot, (int)n, nsp, box, species, pos, force, energy, totals, s);
     else
-        k_forces_allpairs<false><<<grid, kBlock, 0, st>>>(pot, (int)n, nsp, box, species, pos, force, energy, totals,
-                                                           s);
+        launch<8>(fp64, st, pot, (int)n, nsp, box, species, pos, force, energy, totals, s);
     if (cudaGetLastError() != cudaSuccess)
         return fail(MD_E_CUDA, "md_forces_noalloc: kernel launch failed");
     return MD_OK;
