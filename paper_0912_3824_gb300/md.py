@@ -226,11 +226,12 @@ def md_compute_forces(h, n_total: int, n_replicas: int):
 
 
 def md_observables(h, n_replicas: int, max_samples: int = 1 << 16):
-    buf = (md_obs * (max_samples * n_replicas))()
+    # (np.empty: only the records written are ever touched; a zeroed buffer for 65536 samples
+    # of 64 replicas is 537 MB, 21 ms a call)
+    buf = np.empty(max_samples * n_replicas, dtype=OBS_DTYPE)
     n = C.c_int32()
-    _check(_lib.md_observables(h, buf, max_samples, C.byref(n)), h)
-    arr = np.frombuffer(buf, dtype=OBS_DTYPE)[: n.value * n_replicas].copy()
-    return arr.reshape(n.value, n_replicas)
+    _check(_lib.md_observables(h, buf.ctypes.data_as(C.POINTER(md_obs)), max_samples, C.byref(n)), h)
+    return buf[: n.value * n_replicas].copy().reshape(n.value, n_replicas)
 
 
 def md_epot_series(h, n_replicas: int, max_steps: int = 1 << 16):
