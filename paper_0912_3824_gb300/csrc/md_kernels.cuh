@@ -125,31 +125,45 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double *sh)
     __syncthreads();
 }
 
-// Sum of NV doubles over a group in a fixed order; valid in its thread 0.
-// sh: kGrpWarps*NV doubles.  Every thread of the group must call it.
+// Sums of 12 doubles over a group in a fixed order; valid in its thread 0.  Each
+// butterfly step halves the values a lane still holds, so a warp takes 16 FP64
+// additions, where 12 butterflies take 60: on this GPU a warp-wide FP64 addition
+// keeps its pipe for ~18 cycles of the SM (the reductions of a sample step at KA
+// N=65536 took 15 us that way).  sh: kGrpWarps*kPartF doubles.  Every thread of
+// the group must call it.
 constexpr int kGrpWarps = kForceBlock / 32;
 
-template <int NV>
-__device__ __forceinline__ void grp_sum(const Grp &g, double (&v)[NV], double *sh)
+__device__ __forceinline__ void grp_sum(const Grp &g, double (&v)[kPartF], double *sh)
 {
     const int lane = threadIdx.x & 31, w = g.tid() >> 5;
+    double x[8];
 #pragma unroll
-    for (int k = 0; k < NV; ++k)
-        v[k] = warp_sum(v[k]);
-    if (lane == 0) {
-#pragma unroll
-        for (int k = 0; k < NV; ++k)
-            sh[w * NV + k] = v[k];
+    for (int k = 0; k < 8; ++k) {                        // lanes 16..31 go on with values 8..15 (12..15: 0)
+        const double up = k + 8 < kPartF ? v[k + 8] : 0.0;
+        const double give = lane & 16 ? v[k] : up, keep = lane & 16 ? up : v[k];
+        x[k] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
     }
+#pragma unroll
+    for (int o = 8, n = 4; n >= 1; o >>= 1, n >>= 1)
+#pragma unroll
+        for (int k = 0; k < n; ++k) {
+            const double give = lane & o ? x[k] : x[k + n], keep = lane & o ? x[k + n] : x[k];
+            x[k] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    x[0] += __shfl_xor_sync(0xffffffffu, x[0], 1);
+    // value of the lane: bit 16 -> 8, 8 -> 4, 4 -> 2, 2 -> 1
+    const int k = (lane >> 1) & 15;
+    if (!(lane & 1) && k < kPartF)
+        sh[w * kPartF + k] = x[0];
     g.sync();
     if (g.tid() == 0) {
 #pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            double x = sh[k];
+        for (int q = 0; q < kPartF; ++q) {
+            double y = sh[q];
 #pragma unroll
             for (int u = 1; u < kGrpWarps; ++u)
-                x += sh[u * NV + k];
-            v[k] = x;
+                y += sh[u * kPartF + q];
+            v[q] = y;
         }
     }
     g.sync();
@@ -648,7 +662,7 @@ __device__ void finish_replica(const KArgs &a, const Grp &g, int r, long long st
         for (int k = 1; k < kPartF; ++k)
             v[k] += p[k];
     }
-    grp_sum<kPartF>(g, v, sh);
+    grp_sum(g, v, sh);
     if (g.tid() == 0) {
         Obs o;
         o.step = step;
@@ -931,20 +945,21 @@ __device__ __forceinline__ void pair_forces(const KArgs &a, const Rep &rp, int p
         // list indices are loaded kPfDepth iterations ahead, so that only the
         // position gathers remain on each iteration's critical path
         // (K is a multiple of 8: every 16-byte index load is in bounds and aligned)
-        constexpr int kStride = kUnr * TPP;
-        int4 pf[kPfDepth][kUnr / 4];
+        // (8 or more lanes: groups of 4, so that a row of ~80 entries fills the lanes evenly)
+        constexpr int U = TPP >= 8 ? 4 : kUnr, kStride = U * TPP;
+        int4 pf[kPfDepth][U / 4];
 #pragma unroll
         for (int d = 0; d < kPfDepth; ++d)
 #pragma unroll
-            for (int w = 0; w < kUnr / 4; ++w) {
-                const int k = kUnr * lane + d * kStride;
+            for (int w = 0; w < U / 4; ++w) {
+                const int k = U * lane + d * kStride;
                 // (the first ones without waiting for the row's length)
                 pf[d][w] = k < (d == 0 ? a.Kstride : nn) ? *(const int4 *)(lst + k + 4 * w) : make_int4(0, 0, 0, 0);
             }
-        for (int k0 = kUnr * lane; k0 < nn; k0 += kStride) {
-            int jj[kUnr];
+        for (int k0 = U * lane; k0 < nn; k0 += kStride) {
+            int jj[U];
 #pragma unroll
-            for (int w = 0; w < kUnr / 4; ++w) {
+            for (int w = 0; w < U / 4; ++w) {
                 const int4 q = pf[0][w];
                 jj[4 * w] = q.x;
                 jj[4 * w + 1] = q.y;
@@ -954,16 +969,16 @@ __device__ __forceinline__ void pair_forces(const KArgs &a, const Rep &rp, int p
 #pragma unroll
             for (int d = 0; d + 1 < kPfDepth; ++d)
 #pragma unroll
-                for (int w = 0; w < kUnr / 4; ++w)
+                for (int w = 0; w < U / 4; ++w)
                     pf[d][w] = pf[d + 1][w];
             if (k0 + kPfDepth * kStride < nn)
 #pragma unroll
-                for (int w = 0; w < kUnr / 4; ++w)
+                for (int w = 0; w < U / 4; ++w)
                     pf[kPfDepth - 1][w] = *(const int4 *)(lst + k0 + kPfDepth * kStride + 4 * w);
-            float4 Hs[kUnr];
-            int4 Qs[kUnr];
+            float4 Hs[U];
+            int4 Qs[U];
 #pragma unroll
-            for (int u = 0; u < kUnr; ++u) {
+            for (int u = 0; u < U; ++u) {
                 // rows are padded with the particle itself up to a multiple of kUnr
                 const int j = checked(a, jj[u], a.n, ii);
                 if constexpr (P == MIXED)
@@ -975,7 +990,7 @@ __device__ __forceinline__ void pair_forces(const KArgs &a, const Rep &rp, int p
             // entries is one packed instruction each
             float gx = 0.f, gy = 0.f, gz = 0.f, gv = 0.f;
 #pragma unroll
-            for (int u = 0; u < kUnr; u += 2) {
+            for (int u = 0; u < U; u += 2) {
                 float2 dx, dy, dz;
                 bool bj[2];
                 if constexpr (P == MIXED) {
@@ -1116,36 +1131,50 @@ __device__ __forceinline__ void pair_virial(const KArgs &a, const Rep &rp, int p
             Hi = pos[ii];
             ti = species_of(Hi.w);
         }
-        for (int k = lane; k < nn; k += TPP) {
-            const int j = checked(a, lst[k], a.n, ii);
-            float dx, dy, dz;
-            int ab;
-            if constexpr (P == MIXED) {
-                const int4 Qj = qp[j];
-                ab = ti * 2 + Qj.w;
-                dx = sep_q(Qi.x, Qj.x, rp.qunit);
-                dy = sep_q(Qi.y, Qj.y, rp.qunit);
-                dz = sep_q(Qi.z, Qj.z, rp.qunit);
-            } else {
-                const float4 Hj = pos[j];
-                ab = ti * 2 + species_of(Hj.w);
-                dx = sep_f(Hi.x, Hj.x, rp.Lhi, rp.invLf);
-                dy = sep_f(Hi.y, Hj.y, rp.Lhi, rp.invLf);
-                dz = sep_f(Hi.z, Hj.z, rp.Lhi, rp.invLf);
+        // groups of 4 entries, their gathers in flight together (rows are padded with the
+        // particle itself, r2 = 0, to whole groups)
+        for (int k0 = 4 * lane; k0 < nn; k0 += 4 * TPP) {
+            const int4 j4 = *(const int4 *)(lst + k0);
+            const int jj[4] = {j4.x, j4.y, j4.z, j4.w};
+            int4 Qs[4];
+            float4 Hs[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int j = checked(a, jj[u], a.n, ii);
+                if constexpr (P == MIXED)
+                    Qs[u] = qp[j];
+                else
+                    Hs[u] = pos[j];
             }
-            const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-            if (r2 < a.tab.rc2[ab] && r2 > 0.0f) {
-                const float ir2 = __fdividef(1.0f, r2);
-                const float s2 = a.tab.sig2[ab] * ir2;
-                const float s6 = s2 * s2 * s2;
-                float fr = a.tab.eps48[ab] * ir2 * s6 * (s6 - 0.5f);
-                if (SM) {
-                    float v = a.tab.eps4[ab] * s6 * (s6 - 1.0f) - a.tab.shift[ab];
-                    smooth_pair(r2, a.tab.rc[ab], a.tab.ihs[ab], fr, v);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                float dx, dy, dz;
+                int ab;
+                if constexpr (P == MIXED) {
+                    ab = ti * 2 + Qs[u].w;
+                    dx = sep_q(Qi.x, Qs[u].x, rp.qunit);
+                    dy = sep_q(Qi.y, Qs[u].y, rp.qunit);
+                    dz = sep_q(Qi.z, Qs[u].z, rp.qunit);
+                } else {
+                    ab = ti * 2 + species_of(Hs[u].w);
+                    dx = sep_f(Hi.x, Hs[u].x, rp.Lhi, rp.invLf);
+                    dy = sep_f(Hi.y, Hs[u].y, rp.Lhi, rp.invLf);
+                    dz = sep_f(Hi.z, Hs[u].z, rp.Lhi, rp.invLf);
                 }
-                d7[0] += fr * r2;
-                d7[1] += fr * dx * dx; d7[2] += fr * dy * dy; d7[3] += fr * dz * dz;
-                d7[4] += fr * dx * dy; d7[5] += fr * dx * dz; d7[6] += fr * dy * dz;
+                const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                if (r2 < a.tab.rc2[ab] && r2 > 0.0f) {
+                    const float ir2 = __fdividef(1.0f, r2);
+                    const float s2 = a.tab.sig2[ab] * ir2;
+                    const float s6 = s2 * s2 * s2;
+                    float fr = a.tab.eps48[ab] * ir2 * s6 * (s6 - 0.5f);
+                    if (SM) {
+                        float v = a.tab.eps4[ab] * s6 * (s6 - 1.0f) - a.tab.shift[ab];
+                        smooth_pair(r2, a.tab.rc[ab], a.tab.ihs[ab], fr, v);
+                    }
+                    d7[0] += fr * r2;
+                    d7[1] += fr * dx * dx; d7[2] += fr * dy * dy; d7[3] += fr * dz * dz;
+                    d7[4] += fr * dx * dy; d7[5] += fr * dx * dz; d7[6] += fr * dy * dz;
+                }
             }
         }
     }
@@ -2216,6 +2245,7 @@ struct RunState {
     int pend_sample;
     int last, sample, check, track; // of the running step: ends md_step, is a sample, is checked, needs maxima
     int to_sample;                 // steps until the next sample step
+    int bad;                       // something went wrong in this block
     int unit;                      // next unit (cell or share of one) of the block's in the build
 
     Rep rep;                       // of a handle of one replica
@@ -2265,10 +2295,14 @@ __device__ __forceinline__ unsigned int grid_barrier(const KArgs &a, RunState &S
         RunSync *rs = a.rs;
         const unsigned int next = (S.count + 1u) & 0x0fffffffu;
         unsigned int t, w;
-        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(t) : "l"(&rs->arrive) : "memory");
-        if (t == gridDim.x - 1) {
+        // (the high half counts the blocks with something wrong)
+        const unsigned int add = S.bad ? 0x10001u : 1u;
+        asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], %2;"
+                     : "=r"(t) : "l"(&rs->arrive), "r"(add) : "memory");
+        t += add;
+        if ((t & 0xffffu) == gridDim.x) {
             rs->arrive = 0u;
-            w = (next << 4) | decide();
+            w = (next << 4) | decide((t >> 16) != 0u);
             asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&rs->word), "r"(w) : "memory");
         } else {
             unsigned int n = 0;
@@ -2293,11 +2327,11 @@ __device__ __forceinline__ unsigned int grid_barrier(const KArgs &a, RunState &S
 
 __device__ __forceinline__ unsigned int grid_barrier(const KArgs &a, RunState &S)
 {
-    return grid_barrier(a, S, []() -> unsigned int { return 0u; }, [](unsigned int) {});
+    return grid_barrier(a, S, [](bool) -> unsigned int { return 0u; }, [](unsigned int) {});
 }
 
-// Maxima of this block's displacements, speeds and accelerations, and what went
-// wrong, into the step's, thread 0.
+// Maxima of this group's displacements, speeds and accelerations into the step's,
+// thread 0.
 __device__ __forceinline__ void put_maxima(const KArgs &a, long long step, float d2, float v2, float a2)
 {
     unsigned int *m = a.rs->m[step & 1];
@@ -2309,16 +2343,16 @@ __device__ __forceinline__ void put_maxima(const KArgs &a, long long step, float
         atomicMax(&m[2], __float_as_uint(a2));
 }
 
-__device__ __forceinline__ void put_bad(const KArgs &a, long long step, unsigned int bad)
+__device__ __forceinline__ void put_bad(const KArgs &a, RunState &S, unsigned int bad)
 {
     atomicOr(&a.ctl->status, bad);
-    atomicOr(&a.rs->m[step & 1][3], bad);
+    S.bad = 1;
 }
 
 // The whole grid's maxima, cleared for the step after the next (last arriver of
 // the step's barrier).  The displacement is kept by the parity of the step it
 // leads to (of the positions it belongs to).
-struct Maxima { float d2, v2, a2; unsigned int bad; };
+struct Maxima { float d2, v2, a2; };
 
 __device__ __forceinline__ Maxima take_maxima(const KArgs &a, long long step)
 {
@@ -2332,7 +2366,6 @@ __device__ __forceinline__ Maxima take_maxima(const KArgs &a, long long step)
     r.d2 = __uint_as_float(v.x);
     r.v2 = __uint_as_float(v.y);
     r.a2 = __uint_as_float(v.z);
-    r.bad = v.w;
     return r;
 }
 
@@ -2361,7 +2394,7 @@ __device__ __forceinline__ unsigned int run_rebuild(const KArgs &a, const Grp &g
     if (grid_barrier(a, S) & RF_ABORT)
         return S.flags;
     rebuild_permute<P>(a, g, S.pp, S.spar);
-    const auto reset_units = [&]() -> unsigned int {
+    const auto reset_units = [&](bool) -> unsigned int {
         a.rs->unit = g.nvb;
         return 0u;
     };
@@ -2403,7 +2436,7 @@ __device__ __forceinline__ unsigned int run_rebuild(const KArgs &a, const Grp &g
                 g.sync();
             }
         }
-        const unsigned int f = grid_barrier(a, S, [&]() -> unsigned int {
+        const unsigned int f = grid_barrier(a, S, [&](bool) -> unsigned int {
             a.rs->unit = g.nvb;
             if (atomicOr(&ctl->status, 0u))
                 return RF_STOP | RF_BAD;
@@ -2468,7 +2501,7 @@ __device__ __forceinline__ void run_first(const KArgs &a, const Grp &g, RunState
         }
     }
     if (bad)
-        put_bad(a, S.step, bad);
+        put_bad(a, S, bad);
     grp_max3(g, d2, v2, a2, X.mx);
     if (g.tid() == 0)
         put_maxima(a, S.step, d2, v2, a2);
@@ -2499,12 +2532,12 @@ __device__ __forceinline__ void run_chunks(const KArgs &a, const Grp &g, RunStat
         step_body<P, TPP, SAMPLE, SM>(a, a.nrep == 1 ? S.rep : a.rep[b.z], Q, b, (a.what & RUN_STEPS) != 0, S.last != 0,
                                       S.track != 0, S.pp, S.spar, part, eo, d2, v2, a2, bad);
         if (bad)
-            put_bad(a, S.step, bad);
+            put_bad(a, S, bad);
         X.d2[g.tid()] = fmaxf(X.d2[g.tid()], d2);
         X.v2[g.tid()] = fmaxf(X.v2[g.tid()], v2);
         X.a2[g.tid()] = fmaxf(X.a2[g.tid()], a2);
         if (SAMPLE) {
-            grp_sum<kPartF>(g, part, X.sh);
+            grp_sum(g, part, X.sh);
             if (g.tid() == 0) {
                 double *p = a.nrep == 1 ? X.tot : a.part_f + part_index(a, S.step, b.w) * kPartF;
 #pragma unroll
@@ -2607,6 +2640,7 @@ __global__ void __launch_bounds__(kForceBlock * run_groups<P, SM>(), 1) k_run(KA
         S.count = a.rs->word >> 4;
         S.ns = 0ull;
         S.done = 0;
+        S.bad = 0;
         S.flags = ctl->status ? RF_STOP | RF_BAD : 0u;
         run_plan(a, S);
     }
@@ -2622,9 +2656,9 @@ __global__ void __launch_bounds__(kForceBlock * run_groups<P, SM>(), 1) k_run(KA
     if (!(f & RF_STOP) && (a.what & RUN_FIRST)) {
         if (!halted)
             run_first<P>(a, g, S, X);
-        f = grid_barrier(a, S, [&]() -> unsigned int {
+        f = grid_barrier(a, S, [&](bool bad) -> unsigned int {
             const Maxima m = take_maxima(a, S.step);
-            if (m.bad || halted)
+            if (bad || halted)
                 return RF_STOP | RF_BAD;
             return need_rebuild(a, a.check - 1, m.d2, m.v2, m.a2) ? RF_REBUILD : 0u;
         }, [&](unsigned int flags) {
@@ -2652,9 +2686,11 @@ __global__ void __launch_bounds__(kForceBlock * run_groups<P, SM>(), 1) k_run(KA
             } else {
                 run_chunks<P, TPP, SM, false>(a, g, S, X);
             }
-            f = grid_barrier(a, S, [&]() -> unsigned int {
-                const Maxima m = take_maxima(a, S.step);
-                if (m.bad || halted)
+            f = grid_barrier(a, S, [&](bool bad) -> unsigned int {
+                Maxima m = {0.f, 0.f, 0.f};
+                if (S.track)
+                    m = take_maxima(a, S.step);
+                if (bad || halted)
                     return RF_STOP | RF_BAD;
                 unsigned int fl = 0u;
                 if (S.check && need_rebuild(a, a.check - 1, m.d2, m.v2, m.a2))
