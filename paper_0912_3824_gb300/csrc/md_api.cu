@@ -1209,7 +1209,7 @@ int md_corr_sample(md_corr *c)
         ca.acc = c->acc + (size_t)b * (c->l - 1) * 4;
         ca.nblocks = c->nblocks;
         mdk::k_corr<<<c->nblocks, mdk::kCorrBlock, 0, h->s>>>(ca);
-        mdk::k_corr_reduce<<<1, 128, 0, h->s>>>(ca);
+        mdk::k_corr_reduce<<<1, mdk::kCorrReduce, 0, h->s>>>(ca);
         CK(h, cudaGetLastError());
         for (int j = 0; j < c->l - 1; ++j)
             c->origins[(size_t)b * (c->l - 1) + j] += 1;

@@ -6,9 +6,13 @@
 // Snapshots hold unwrapped positions in FP64 by original particle index.
 // Per particle i of species a and per later snapshot j: d = r_j - r_0 (FP64),
 // |d|^2 (FP64) and the average over the n_q wavevectors of cos(q . d) (phase in
-// FP64, cosine in FP32).  Sums per block of 256 particles go to a partial array;
-// k_corr_reduce adds the partials in block order into the accumulator of the
+// FP64, cosine in FP32).  Sums per block of 64 particles go to a partial array;
+// k_corr_reduce adds the partials in a fixed order into the accumulator of the
 // block level (deterministic).
+//
+// k_corr is bound by the FP64 pipe (four instructions per phase), so what counts
+// is that every SM has its share: with blocks of 256, N = 20,011 used 79 of 152
+// SMs.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -17,7 +21,7 @@ namespace mdk {
 
 constexpr int kCorrMaxJ = 31;      // at most 32 entries per block level
 constexpr int kCorrMaxQ = 64;
-constexpr int kCorrBlock = 256;
+constexpr int kCorrBlock = 64;
 
 struct CorrArgs {
     const double *s0;               // origin snapshot [n][3]
@@ -83,13 +87,22 @@ __global__ void __launch_bounds__(kCorrBlock) k_corr(CorrArgs c)
     }
 }
 
-__global__ void k_corr_reduce(CorrArgs c)
+// One warp per sum: lane l adds partials l, l + 32, ..., then a butterfly.
+constexpr int kCorrReduce = 1024;
+
+__global__ void __launch_bounds__(kCorrReduce) k_corr_reduce(CorrArgs c)
 {
-    for (int t = threadIdx.x; t < 4 * c.nj; t += blockDim.x) {
+    const int lane = threadIdx.x & 31;
+    for (int t = threadIdx.x >> 5; t < 4 * c.nj; t += kCorrReduce / 32) {
         double s = 0.0;
-        for (int b = 0; b < c.nblocks; ++b)
+#pragma unroll 8
+        for (int b = lane; b < c.nblocks; b += 32)
             s += c.part[(size_t)b * c.nj * 4 + t];
-        c.acc[t] += s;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0)
+            c.acc[t] += s;
     }
 }
 
