@@ -96,8 +96,9 @@ typedef struct {
     int32_t obs_capacity;     /* ring-buffer samples kept on the device (0 = 4096); also the
                                  number of newest steps the per-step potential-energy series
                                  keeps (md_epot_series)                                         */
-    int32_t threads_per_particle; /* force-kernel lanes per particle: 0 = automatic (2 for MIXED
-                                     and FP32, 4 for FP64), else a power of two in 1..32 (1..8
+    int32_t threads_per_particle; /* force-kernel lanes per particle: 0 = automatic (2 for MIXED and
+                                     FP32, 4 for FP64; more below ~12,000 (FP64: ~6,500) particles
+                                     with long enough lists), else a power of two in 1..32 (1..8
                                      with smooth_h > 0)                                          */
     int32_t use_graph;        /* 1 = md_step is one launch with the rebuild branch and the step
                                  loop decided on the device (default); 0 = a launch for every

@@ -142,6 +142,33 @@ int auto_capacity(const md_params *p, const Geometry &g, const std::vector<doubl
     return std::max(k, 32);
 }
 
+// Automatic lanes per particle.  From ~12,000 particles on (FP64: ~6,500) the
+// work fills the GPU and 2 lanes (4) lose least to combining them; fewer particles
+// leave it idle, and more lanes shorten the chain of a row's entries, as long as
+// rows are long enough to share.  Measured on GB300, us per MD step:
+//   KA mixed, N = 1000: 9.57 (2 lanes) 8.60 (4) 7.30 (8) 7.28 (16); 6000: 10.48 10.56
+//     8.81 9.26; 12,000: 11.44 11.35 10.62 14.03; 24,000: 13.28 14.88 - -
+//   LJ 0.8442 mixed, N = 2000: 9.51 9.49 9.13 9.06; 8000: 11.21 11.30 11.12 12.00
+//   LJ 0.3 mixed (~28 entries a row), N = 2000: 7.98 8.65 8.56 8.38
+//   KA smoothed, N = 1000: 12.90 9.89 7.68 (8); 12,000: 14.88 12.47 12.04; 24,000: 17.26 16.52 -
+//   KA FP64, N = 1000: 68.8 36.5 23.5 18.5; 4000: 69.4 37.4 33.6 43.5; 8000: 69.8 54.6 59.1 70.8
+int auto_lanes(const md_params *p, int R, const int64_t *nrep, const double *box, double rl)
+{
+    double n = 0.0, vol = 0.0;
+    for (int r = 0; r < R; ++r) {
+        n += (double)nrep[r];
+        vol += box[r] * box[r] * box[r];
+    }
+    const bool longrow = 4.18879020478639 * rl * rl * rl * n > 48.0 * vol;   // entries a row on average
+    if (p->precision == MD_PREC_FP64)
+        return p->smooth_h > 0.0 || !longrow || n > 6500 ? 4 : n > 1200 ? 8 : 16;
+    if (p->step_form == 2 || !longrow)
+        return 2;
+    if (p->smooth_h > 0.0)
+        return n > 24000 ? 2 : n > 12000 ? 4 : 8;
+    return n > 12000 ? 2 : n > 2048 ? 8 : 16;
+}
+
 // Returns MD_OK or MD_E_INVAL with *msg set.
 int make_geometry(const md_params *p, int R, const int64_t *nrep, const double *box, Geometry &g,
                   std::string &msg)
@@ -211,9 +238,7 @@ int make_geometry(const md_params *p, int R, const int64_t *nrep, const double *
     }
     g.R = R;
     g.rl_max = rcmax + p->skin + (double)mdk::kListMargin;
-    // lanes per particle: 2 for the FP32 pair loops (4096 warps at KA N=65536 fit one wave at
-    // 64 registers), 4 for FP64 (measured on GB300)
-    g.tpp = tpp ? tpp : (p->precision == MD_PREC_FP64 ? 4 : 2);
+    g.tpp = tpp ? tpp : auto_lanes(p, R, nrep, box, g.rl_max);
     g.ppb_f = kForceBlock / g.tpp;
     if (p->step_form == 2 && (p->precision == MD_PREC_FP64 || g.tpp > 2)) {
         msg = "step_form 2 needs MIXED or FP32 and 1 or 2 threads per particle";
