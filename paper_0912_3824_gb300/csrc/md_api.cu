@@ -1441,7 +1441,7 @@ int md_get_neighbours(md_handle *h, int32_t *counts, int32_t *lists, int32_t kma
     if ((rc = read_ctl(h, &c)))
         return rc;
     const size_t K = (size_t)h->g.Kmax;                  // row stride of the lists (the cap)
-    if ((rc = ensure_pinned(h, 4 * n * K + 4 * n + 16 * n + 256)) || (rc = stage_wait(h)))
+    if ((rc = ensure_pinned(h, align_up(4 * n) + align_up(16 * n) + 4 * n * K)) || (rc = stage_wait(h)))
         return rc;
     char *q = h->pin;
     int *nn = (int *)q;
