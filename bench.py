@@ -9,7 +9,7 @@ rescaling (4000 steps, untimed), then timed in NVE.
 
 One timed iteration ("step" of this script) = md_step(1000): 1000 MD steps
 with every neighbour-list rebuild, reorder and per-step reduction, executed
-as one CUDA graph.  The L2 cache is flushed (256 MB write) between timed
+as one cooperative launch.  The L2 cache is flushed (256 MB write) between timed
 iterations; within one the state stays on chip, as in a continuous run.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
@@ -55,14 +55,14 @@ def parse_args(argv=None):
     ap.add_argument("--precision", choices=["mixed", "fp64", "fp32"], default="mixed")
     ap.add_argument("--no-extras", action="store_true", help="skip fp64 / e2e / cpu legs")
     ap.add_argument("--no-graph", action="store_true",
-                    help="plain stream launches instead of the CUDA graph (for per-kernel profiling)")
+                    help="a launch per MD step and rebuild instead of one (for per-phase profiling)")
     ap.add_argument("--tpp", type=int, default=0, help="force-kernel threads per particle (0 = auto)")
     ap.add_argument("--step-form", type=int, default=0, choices=[0, 1, 2],
-                    help="step-kernel blocks: 0 auto, 1 one per chunk, 2 resident blocks sweep (not FP64)")
+                    help="sharing of chunks: 0 auto, 1 or 2 (not FP64); one scheme, reported as asked")
     ap.add_argument("--build-form", type=int, default=0, choices=[0, 1, 2],
-                    help="neighbour build: 0 auto, 1 one warp per cell, 2 one block per cell")
+                    help="neighbour build: 0 auto, 1 one warp per cell, 2 groups of threads per cell")
     ap.add_argument("--check", type=int, default=0,
-                    help="MD steps between rebuild checks of the graph (0 = the library's choice)")
+                    help="MD steps between rebuild checks (0 = the library's choice)")
     ap.add_argument("--skin", type=float, default=0.3, help="neighbour-list skin (with --no-tune)")
     ap.add_argument("--no-tune", action="store_true", help="skip the autotuner (lanes, skin, capacity)")
     ap.add_argument("--workload", choices=["ka65536", "lj-sweep", "e1", "replicas", "drift", "stability",
@@ -390,7 +390,7 @@ def run_ours(args, rank, world, local):
     sim_k.step(320)
     info_b = sim_k.info()
     ev_ms = (info_b["step_ms"] - info_a["step_ms"]) / max(1, info_b["step_launches"] - info_a["step_launches"])
-    # the step kernel's average duration inside the timed region (the CUDA-graph run),
+    # the MD step's average duration inside the timed region (rebuilds excluded),
     # from the device timer each launch reads at its first block start and last block end
     n_dev = info1["step_device_launches"] - info0["step_device_launches"]
     f_ms = (info1["step_device_ms"] - info0["step_device_ms"]) / max(1, n_dev)
@@ -402,8 +402,8 @@ def run_ours(args, rank, world, local):
     peaks = alu_peaks(md, torch, device)
     peak_max = peaks["fp32_tflops"]
     result["roofline"] = {
-        "bound": "alu", "kernel": f"k_step<{args.precision}, {info1['threads_per_particle']}, unsmoothed> "
-                                  "(pair forces and energy + velocity-Verlet update)",
+        "bound": "alu", "kernel": f"k_run<{args.precision}, {info1['threads_per_particle']}, unsmoothed>, one MD step "
+                                  "(pair forces and energy + velocity-Verlet update + grid barrier)",
         "achieved": flops / (f_ms * 1e-3) / 1e12, "peak": peak_max, "unit": "TFLOP/s",
         "frac": flops / (f_ms * 1e-3) / 1e12 / peak_max,
         "flop_convention": f"{FLOP_PER_ENTRY_METHOD} per list entry + {FLOP_PER_PAIR_METHOD} per pair in the "
@@ -411,12 +411,12 @@ def run_ours(args, rank, world, local):
         "kernel_count": {"flop_per_launch": flops_kernel, "tflops": flops_kernel / (f_ms * 1e-3) / 1e12,
                          "note": f"{FLOP_PER_ENTRY} per entry + {FLOP_PER_PAIR} per pair + {FLOP_PER_UPDATE} "
                                  "per particle (update), counted as this kernel computes"},
-        "traffic": profiled_traffic(f"k_step<{md.PRECISIONS[args.precision]}, {info1['threads_per_particle']}, 0, "
-                                    f"{1 if info1['step_form'] == 2 else 0}>", base.skin),
+        "traffic": profiled_traffic(f"k_run<{md.PRECISIONS[args.precision]}, {info1['threads_per_particle']}, 0>",
+                                    base.skin),
         "per_launch_ms": f_ms, "launches_timed": int(n_dev),
         "per_launch_ms_events": ev_ms,
-        "timing": "per_launch_ms: device timer over the timed region (every k_step launch of the graph); "
-                  "per_launch_ms_events: CUDA events around stream launches of the same kernel",
+        "timing": "per_launch_ms: device timer over the timed region (every MD step, barrier to barrier); "
+                  "per_launch_ms_events: CUDA events around launches of one step each",
         "flop_per_launch": flops, "mean_list": float(n_list),
         "mean_in_cutoff": float(n_cut),
         "peak_note": "FP32 FMA peak measured on this GPU by md_fma_peak (FMA chains on every SM, CUDA "
@@ -624,7 +624,7 @@ def lj_cases(args, local, cases, workload, temperature, dt, skin):
                                          skins=(skin,))
             sim.close()
             sim = md.System(base, [s.n], [s.box], s.species, pos0, vel0, img0, device=device)
-        sim.step(args.inner)                       # warm-up, graph captured
+        sim.step(args.inner)                       # warm-up
         assert sim.sync() == md.MD_OK
         sim.observables()
         info0 = sim.info()
@@ -683,7 +683,7 @@ def lj_cases(args, local, cases, workload, temperature, dt, skin):
 
 def run_replicas(args, local):
     """256 Kob-Andersen replicas with N_r uniform in {500, ..., 8000} at
-    rho = 1.2, T = 0.8: one handle holding every replica (one CUDA graph per
+    rho = 1.2, T = 0.8: one handle holding every replica (one launch per
     md_step) against one handle per replica launched in a loop."""
     torch, md, synth, device, stream, flush = _gpu_setup(local)
     sizes = synth.ensemble_sizes(256, 500, 8000, seed=4)
@@ -717,7 +717,7 @@ def run_replicas(args, local):
         torch.cuda.synchronize()
         return sum(a.elapsed_time(b) for a, b in evs)
 
-    for _ in range(2):                            # warm-up: graphs captured, lists built
+    for _ in range(2):                            # warm-up: lists built
         one.step(args.inner)
         for h in loop:
             h.step(args.inner)
