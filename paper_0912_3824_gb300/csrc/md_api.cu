@@ -75,7 +75,7 @@ struct Geometry {
 };
 
 struct Layout {
-    size_t off_ctl, off_rep, off_blk_i, off_blk_f, off_blk_r, off_crank, off_cxyz;
+    size_t off_ctl, off_rep, off_blk_i, off_blk_r, off_crank, off_cxyz;
     size_t off_pa, off_pb, off_va, off_vb, off_pa2, off_pb2, off_va2, off_vb2, off_qa, off_qb, off_force;
     size_t off_rref, off_image, off_image2, off_key, off_tmpidx;
     size_t off_ccount, off_ccursor, off_cstart, off_nbr, off_nnbr, off_part_f, off_part_i, off_part_e;
@@ -361,7 +361,6 @@ Layout make_layout(const md_params *p, const Geometry &g)
     L.off_ctl = take(sizeof(mdk::Ctl));
     L.off_rep = take(sizeof(mdk::Rep) * g.R);
     L.off_blk_i = take(sizeof(int4) * g.nblk_i);
-    L.off_blk_f = take(sizeof(int4) * g.nblk_f);
     L.off_blk_r = take(sizeof(int4) * 2 * (size_t)g.nblk_f);   // < nblk_f + resident blocks rows
     L.off_rs = take(sizeof(mdk::RunSync));
     L.off_slice = take(sizeof(int) * kMaxRunGroups);
@@ -774,7 +773,6 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
     a.nrep = g.R;
     a.ncell = g.ncell;
     a.Kstride = g.Kmax;
-    a.tpp = g.tpp;
     a.si = p->sample_interval;
     a.obs_cap = h->cap;
     a.epot_cap = h->cap;
@@ -797,7 +795,6 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
     a.nbr = (int *)(w + L.off_nbr);
     a.nnbr = (int *)(w + L.off_nnbr);
     a.blk_i = (const int4 *)(w + L.off_blk_i);
-    a.blk_f = (const int4 *)(w + L.off_blk_f);
     a.blk_r = (const int4 *)(w + L.off_blk_r);
     a.rs = (mdk::RunSync *)(w + L.off_rs);
     a.slice = (int *)(w + L.off_slice);
@@ -862,7 +859,6 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
     a.dt_hi = (float)p->dt;
     a.dt_lo = (float)(p->dt - (double)(float)p->dt);
     const double thr = std::max(0.5 * p->skin - (double)mdk::kDispMargin, 0.0);
-    a.disp_thr2 = (float)(thr * thr);
     a.disp_thr = (float)thr;
     for (int s = 0; s < 2; ++s)
         a.inv_mass[s] = (float)(1.0 / a.mass[s]);
@@ -928,7 +924,6 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
         h->a.nb_parts = std::max(1, std::min(8, nsm * h->g.groups / g.ncell));
         if ((rc = put(L.off_rep, g.rep.data(), sizeof(mdk::Rep) * g.R)) ||
             (rc = put(L.off_blk_i, g.blk_i.data(), sizeof(int4) * g.nblk_i)) ||
-            (rc = put(L.off_blk_f, bf.data(), sizeof(int4) * g.nblk_f)) ||
             (rc = put(L.off_blk_r, br.data(), sizeof(int4) * br.size())) ||
             (rc = put(L.off_crank, g.crank.data(), sizeof(int) * g.ncell)) ||
             (rc = put(L.off_cxyz, g.cxyz.data(), sizeof(int4) * g.ncell)))

@@ -98,7 +98,7 @@ struct __align__(32) d4 { double x, y, z, w; };
 
 // Every kernel takes this one struct by value.
 struct KArgs {
-    int n, nrep, ncell, tpp, si, obs_cap, epot_cap, imode, what;
+    int n, nrep, ncell, si, obs_cap, epot_cap, imode, what;
     int Kstride;                      // list row stride: the capacity cap (Ctl::Kmax); the rows hold
                                       // at most Ctl::K entries, so K can grow without a new layout
     int nblk_i, nblk_f;
@@ -120,12 +120,11 @@ struct KArgs {
     const int *crank;                 // [global linear cell] -> global sorted cell id
     const int4 *cxyz;                 // [global sorted cell id] -> cx, cy, cz, replica
     int *nbr, *nnbr;
-    const int4 *blk_i, *blk_f;        // per block: first particle, end, replica (blk_f: + its
-                                      // chunk index, the slot of its partial sums)
-    const int4 *blk_r;                // run kernel: rows of blk_f in the order its blocks take them,
-                                      // cpb per block (w = -1: padding)
-    int cpb;                          // run kernel: chunks per block
-    int *slice;                       // run kernel: particles in each block's slice of the cells
+    const int4 *blk_i;                // per block of 256 particles: first particle, end, replica
+    const int4 *blk_r;                // run kernel: chunks (first particle, end, replica, chunk index) in
+                                      // the order its groups take them, cpb per group (w = -1: padding)
+    int cpb;                          // run kernel: chunks per group
+    int *slice;                       // run kernel: particles in each group's slice of the cells
     double *part_f, *part_i;          // partial sums [2][nslot][12], [nblk_i][4]
     void *part_e;                     // potential energy [2][nslot]: double (FP64 mode) or float2
                                       // double-single (MIXED, FP32)
@@ -147,7 +146,7 @@ struct KArgs {
     double hdtm[2], dt, mass[2];      // dt / (2 m_a), dt, m_a
     long long nsteps;                 // run kernel: MD steps of this launch
     float hdtm_hi[2], hdtm_lo[2], dt_hi, dt_lo, inv_mass[2];
-    float disp_thr2, disp_thr;        // (skin/2 - margin)^2 and skin/2 - margin
+    float disp_thr;                   // skin/2 - margin
     long long budget;                 // run kernel: bound on the steps of this launch
 };
 

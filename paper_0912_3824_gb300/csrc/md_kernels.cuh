@@ -34,7 +34,7 @@ namespace mdk {
 
 constexpr int kIntBlock = 256;   // per-particle kernels: one thread per particle
 constexpr int kForceBlock = 128; // run kernel: threads of a group (tpp threads per particle)
-constexpr int kPartF = 12;       // doubles per block partial of the force / step kernels
+constexpr int kPartF = 12;       // doubles per partial sum of a sample step
 constexpr int kUnr = 8;          // list entries per lane and iteration of the FP32 pair loops
                                  // (a multiple of 4, at most 8: lists are padded to 8)
 constexpr int kPfDepth = 1;      // iterations ahead at which the list indices are loaded
