@@ -764,12 +764,18 @@ __device__ __forceinline__ void pair_forces_d(const KArgs &a, const Rep &rp, int
     const d4 xi = pos[ii];
     const float L = (float)rp.L, half = 0.5f * L;
     const float xf = cut_float(xi.x), yf = cut_float(xi.y), zf = cut_float(xi.z);
-    // cutoffs with the margin of the single-precision test: coordinates cut to 24 bits are
-    // off by L 2^-23 at most, so r^2 by about 4 r_c L 2^-22
+    // cutoffs with the margin of the single-precision test.  A coordinate cut to 24 bits
+    // is off by less than L 2^-23, always downwards, so a difference by as much; its
+    // rounding, L in single precision and a shift on the wrong side of half a box add at
+    // most twice that again: d = 3 L 2^-23 per component, 2 sqrt(3) r_c d + 3 d^2 in r^2,
+    // and four roundings of r_c^2.  Taken: (16 r_c L + 4 r_c^2) 2^-23 + (8 L 2^-23)^2.
     float rc2f[2];
 #pragma unroll
-    for (int tj = 0; tj < 2; ++tj)
-        rc2f[tj] = a.tab.rc2[species_of(xi.w) * 2 + tj] + 1e-5f * L + 1e-3f;
+    for (int tj = 0; tj < 2; ++tj) {
+        const int ab = species_of(xi.w) * 2 + tj;
+        const float dl = L * 0x1p-20f;
+        rc2f[tj] = a.tab.rc2[ab] + (fmaf(a.tab.rc[ab], 2.0f * dl, a.tab.rc2[ab] * 0x1p-21f) + dl * dl);
+    }
     __syncwarp();
     if (lane == 0) {
         Q.x[me][0] = xi.x;
@@ -807,7 +813,7 @@ __device__ __forceinline__ void pair_forces_d(const KArgs &a, const Rep &rp, int
                     dy = dy > half ? dy - L : dy;
                     dz = dz > half ? dz - L : dz;
                     const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                    // (the padding is the particle itself; a NaN passes, and shows in the sums)
+                    // (the padding is the particle itself)
                     if (!(r2 >= (species_of(xs[u].w) ? rc2f[1] : rc2f[0])) && jj[b + u] != ii)
                         keep |= 1u << (b + u);
                 }
