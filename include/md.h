@@ -44,7 +44,13 @@
  *     neigh_capacity_max, a non-finite value, a particle moving more than a
  *     quarter box in one step, an exhausted step-loop bound) stop the step
  *     loop at the end of the offending step, leave the positions at that
- *     step, and are reported by the next md_sync / md_observables / md_step.
+ *     step, and are reported once, by the next call that returns a status
+ *     (md_sync, md_observables, md_epot_series, md_compute_forces).  Until then
+ *     md_step does nothing and leaves the state and the lists as they are;
+ *     a state given to md_set_state meanwhile is kept, and its lists and forces
+ *     are made by the first call after the report that needs them.  After
+ *     MD_E_CAPACITY every md_step asks for the same build and fails alike until
+ *     the state changes.
  *     A list longer than the current capacity but within the cap is not a
  *     failure: the capacity grows on the device and the build is redone.
  */

@@ -446,6 +446,7 @@ struct md_handle {
     int64_t obs_read = 0;
     int64_t epot_read = -1;          // newest step returned by md_epot_series
     int64_t n_species[2] = {0, 0};   // particles per species over all replicas
+    bool stale = false;              // reported with a status: Ctl::stale, not mended yet
     std::string err;
 };
 
@@ -597,9 +598,20 @@ int check_device(md_handle *h)
         if ((rc = launch(h, h->ks->reset, 1, 1, a)))
             return rc;
         CK(h, cudaStreamSynchronize(h->s));
+        h->stale = c.stale != 0;
         return fail(h, code, status_message(code));
     }
     return MD_OK;
+}
+
+// After a failure that left lists of another order or a state loaded while the
+// failure was pending: lists and forces of the current state.
+int refresh(md_handle *h)
+{
+    if (!h->stale)
+        return MD_OK;
+    h->stale = false;
+    return launch_run(h, mdk::RUN_REBUILD | mdk::RUN_FORCES);
 }
 
 // Copies between the caller's arrays and the pinned staging area, shared out
@@ -982,6 +994,8 @@ int md_step(md_handle *h, int64_t nsteps)
     if (nsteps < 1)
         return fail(h, MD_E_INVAL, "nsteps must be >= 1");
     int rc;
+    if ((rc = refresh(h)))
+        return rc;
     // bound on the steps executed (a device loop that could not end would hold the GPU)
     const int64_t budget = h->p.step_budget > 0 ? h->p.step_budget : nsteps + 64;
     if (h->p.use_graph)
@@ -1284,6 +1298,7 @@ int md_compute_forces(md_handle *h, double *f, double *e, md_obs *totals)
         return MD_E_INVAL;
     int rc;
     const size_t n = (size_t)h->g.n;
+    h->stale = false;
     if ((rc = launch_run(h, mdk::RUN_REBUILD | mdk::RUN_TOTALS)) ||
         (rc = launch(h, h->ks->expforce, grid_n(h->g.n, kIntBlock), kIntBlock, h->a)))
         return rc;
@@ -1420,6 +1435,7 @@ int md_set_state(md_handle *h, const double *pos, const double *vel, const int32
     CK(h, cudaMemcpyAsync(h->a.st_vel, q + 24 * n, 24 * n, cudaMemcpyHostToDevice, h->s));
     CK(h, cudaMemcpyAsync(h->a.st_img, q + 48 * n, 12 * n, cudaMemcpyHostToDevice, h->s));
     CK(h, cudaEventRecord(h->ev_stage, h->s));
+    h->stale = false;
     if ((rc = launch(h, h->ks->load, h->g.nblk_i, kIntBlock, h->a)))
         return rc;
     return launch_run(h, mdk::RUN_REBUILD | mdk::RUN_FORCES);
@@ -1433,7 +1449,7 @@ int md_get_neighbours(md_handle *h, int32_t *counts, int32_t *lists, int32_t kma
     const size_t n = (size_t)h->g.n;
     int rc;
     mdk::Ctl c;
-    if ((rc = read_ctl(h, &c)))
+    if ((rc = refresh(h)) || (rc = read_ctl(h, &c)))
         return rc;
     const size_t K = (size_t)h->g.Kmax;                  // row stride of the lists (the cap)
     if ((rc = ensure_pinned(h, align_up(4 * n) + align_up(16 * n) + 4 * n * K)) || (rc = stage_wait(h)))

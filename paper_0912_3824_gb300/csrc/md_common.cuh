@@ -53,6 +53,9 @@ struct Ctl {
     unsigned long long dev_ns;        // summed device duration of the MD steps of the run kernel
     long long dev_launches;           // MD steps summed into dev_ns
     long long regrows;        // builds redone with a larger K since md_create
+    unsigned int halted;      // 1: a run ended with a status that has not been reported yet; runs do
+                              // nothing until it has (status itself can change while blocks start)
+    unsigned int stale;       // 1: lists and forces are not those of the current state and order
 };
 
 // Grid barrier and shared decisions of the run kernel, each on a cache line of its own.
@@ -60,7 +63,7 @@ struct RunSync {
     unsigned int arrive, pad0[31];   // blocks that have reached the running barrier
     unsigned int word, pad1[31];     // (barriers passed << 4) | what the last one decided (RunFlag)
     unsigned int m[2][4], pad2[24];  // float bits of the largest squared displacement, speed and
-                                     // acceleration of a step, and its ST_* bits, by the parity of the step
+                                     // acceleration of a step, by the parity of the step (m[][3]: unused)
     float md2[2];                    // largest squared displacement since the build, by the parity of
     unsigned int unit, pad3[29];     //   the positions' step; next unit of the build
 };

@@ -2320,6 +2320,7 @@ __device__ __forceinline__ unsigned int grid_barrier(const KArgs &a, RunState &S
             asm volatile("fence.acq_rel.gpu;" ::: "memory");
             if ((w >> 4) != next) {
                 atomicOr(&a.ctl->status, ST_TIMEOUT);
+                a.ctl->halted = 1u;
                 w = RF_STOP | RF_BAD | RF_ABORT;
             }
         }
@@ -2444,11 +2445,13 @@ __device__ __forceinline__ unsigned int run_rebuild(const KArgs &a, const Grp &g
         }
         const unsigned int f = grid_barrier(a, S, [&](bool) -> unsigned int {
             a.rs->unit = g.nvb;
+            ctl->stale = 1u;                         // (rref and the rows are those of the new order)
             if (atomicOr(&ctl->status, 0u))
                 return RF_STOP | RF_BAD;
             const int mx = atomicMax(&ctl->max_nbr, 0);
             if (mx <= K) {
                 a.rs->md2[S.step & 1] = 0.f;         // the lists start from these positions
+                ctl->stale = 0u;
                 return 0u;
             }
             if (mx <= ctl->Kmax && retry == 0) {
@@ -2647,24 +2650,26 @@ __global__ void __launch_bounds__(kForceBlock * run_groups<P, SM>(), 1) k_run(KA
         S.ns = 0ull;
         S.done = 0;
         S.bad = 0;
-        S.flags = ctl->status ? RF_STOP | RF_BAD : 0u;
+        S.flags = ctl->halted;
         run_plan(a, S);
     }
     __syncthreads();
-    // A status pending from before: no phase does work, but every block goes to
-    // the first barrier, which ends the launch.  (A block that comes late may see
-    // a status set by another one's first phase: that phase has failed, so its
-    // own share of it is not wanted either.)
-    const bool halted = S.flags != 0u;
+    // A status pending from before: nothing is done until it has been reported.  (Every
+    // block sees the same word: a launch writes it after its last barrier, or when a
+    // barrier gave up, and then a block that starts late has nothing to add.)
+    if (S.flags) {
+        if (blockIdx.x == 0 && threadIdx.x == 0)
+            ctl->n_kernels += 1;
+        return;
+    }
     unsigned int f = 0u;
     if (a.what & RUN_REBUILD)
         f = run_rebuild<P>(a, g, S, X);
     if (!(f & RF_STOP) && (a.what & RUN_FIRST)) {
-        if (!halted)
-            run_first<P>(a, g, S, X);
+        run_first<P>(a, g, S, X);
         f = grid_barrier(a, S, [&](bool bad) -> unsigned int {
             const Maxima m = take_maxima(a, S.step);
-            if (bad || halted)
+            if (bad)
                 return RF_STOP | RF_BAD;
             return need_rebuild(a, a.check - 1, m.d2, m.v2, m.a2) ? RF_REBUILD : 0u;
         }, [&](unsigned int flags) {
@@ -2685,18 +2690,15 @@ __global__ void __launch_bounds__(kForceBlock * run_groups<P, SM>(), 1) k_run(KA
         for (;;) {
             // the previous step's sums (its partials were complete at the last barrier)
             run_service<P>(a, g, S, false, X);
-            if (halted) {
-                // (only the launch's first phase: its barrier ends the launch)
-            } else if (S.sample) {
+            if (S.sample)
                 run_chunks<P, TPP, SM, true>(a, g, S, X);
-            } else {
+            else
                 run_chunks<P, TPP, SM, false>(a, g, S, X);
-            }
             f = grid_barrier(a, S, [&](bool bad) -> unsigned int {
                 Maxima m = {0.f, 0.f, 0.f};
                 if (S.track)
                     m = take_maxima(a, S.step);
-                if (bad || halted)
+                if (bad)
                     return RF_STOP | RF_BAD;
                 unsigned int fl = 0u;
                 if (S.check && need_rebuild(a, a.check - 1, m.d2, m.v2, m.a2))
@@ -2765,6 +2767,8 @@ __global__ void __launch_bounds__(kForceBlock * run_groups<P, SM>(), 1) k_run(KA
         ctl->pos_par = S.pp;
         ctl->state_par = S.spar;
         ctl->rebuild = (f & (RF_REBUILD | RF_BAD)) == RF_REBUILD;
+        if (atomicOr(&ctl->status, 0u))
+            ctl->halted = 1u;
         ctl->n_kernels += 1;
         if (steps) {
             ctl->dev_ns += S.ns;
@@ -2857,8 +2861,10 @@ template <int P>
 __global__ void __launch_bounds__(kIntBlock) k_load(KArgs a)
 {
     Ctl *ctl = a.ctl;
-    if (blockIdx.x == 0 && threadIdx.x == 0)
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
         atomicAdd((unsigned long long *)&ctl->n_kernels, 1ull);
+        ctl->stale = 1u;
+    }
     const int4 b = a.blk_i[blockIdx.x];
     const int i = b.x + threadIdx.x;
     if (i >= b.y)
@@ -3013,6 +3019,7 @@ template <int P>
 __global__ void k_reset(KArgs a)
 {
     a.ctl->status = 0u;
+    a.ctl->halted = 0u;
     a.ctl->ticket = 0u;
     a.rs->arrive = 0u;
     for (int k = 0; k < 8; ++k)
