@@ -71,7 +71,12 @@ extern "C" {
 #define MD_E_CUDA       3  /* a CUDA runtime call failed                                      */
 #define MD_E_NONFINITE  4  /* a position became NaN or infinite                               */
 #define MD_E_UNSTABLE   5  /* a particle moved more than a quarter box length in one step     */
-#define MD_E_TIMEOUT    6  /* the device-side step loop exceeded its iteration bound          */
+#define MD_E_TIMEOUT    6  /* the device-side step loop exceeded its iteration bound, or a wait
+                              of the step kernel for its own blocks gave up after about ten
+                              seconds.  In the second case (md_last_error tells) the state is
+                              lost: until md_set_state has loaded one, the calls that advance or
+                              read it return this code; samples and correlations recorded since
+                              the last good status are not valid                            */
 #define MD_E_CAPACITY   7  /* a neighbour list needed more than neigh_capacity_max entries    */
 #define MD_E_BOUNDS     8  /* only in a library built with MD_CHECK_BOUNDS: a kernel index
                               left its array (the access was redirected to a valid one)     */

@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "md.h"
+#include "md_bench.h"
 #include "md_tables.h"
 #include "md_common.cuh"
 #include "md_corr.cuh"
@@ -397,7 +398,7 @@ Layout make_layout(const md_params *p, const Geometry &g)
     L.off_scale = take(8 * (size_t)g.R);
     L.off_st_pos = take(24 * n);
     L.off_st_vel = take(24 * n);
-    L.off_st_img = take(12 * n);
+    L.off_st_img = take(12 * n + 4);                // (and a word: is the state lost)
     L.off_st_code = take(4 * n);
     L.off_st_f = take(24 * n);
     L.off_st_e = take(8 * n);
@@ -446,7 +447,7 @@ struct md_handle {
     int64_t obs_read = 0;
     int64_t epot_read = -1;          // newest step returned by md_epot_series
     int64_t n_species[2] = {0, 0};   // particles per species over all replicas
-    bool stale = false;              // reported with a status: Ctl::stale, not mended yet
+    bool stale = false, lost = false;   // reported with a status and not mended yet: Ctl::stale
     std::string err;
 };
 
@@ -585,7 +586,11 @@ const char *status_message(int code)
     }
 }
 
-// Synchronise, report (once) and clear a device status.
+constexpr const char *kLostMessage = "a wait of the step kernel for its other blocks gave up: the state is lost "
+                                     "until md_set_state";
+
+// Synchronise, report (once) and clear a device status.  (A launch that gave up
+// may have left counts of a binning that never ended.)
 int check_device(md_handle *h)
 {
     mdk::Ctl c;
@@ -597,12 +602,16 @@ int check_device(md_handle *h)
         KArgs a = h->a;
         if ((rc = launch(h, h->ks->reset, 1, 1, a)))
             return rc;
+        CK(h, cudaMemsetAsync(h->a.ccount, 0, 4 * (size_t)h->g.ncell, h->s));
         CK(h, cudaStreamSynchronize(h->s));
-        h->stale = c.stale != 0;
-        return fail(h, code, status_message(code));
+        h->stale = (c.stale & mdk::STALE_LISTS) != 0;
+        h->lost = (c.stale & mdk::STALE_STATE) != 0;
+        return fail(h, code, h->lost ? kLostMessage : status_message(code));
     }
     return MD_OK;
 }
+
+int lost(md_handle *h) { return h->lost ? fail(h, MD_E_TIMEOUT, kLostMessage) : MD_OK; }
 
 // After a failure that left lists of another order or a state loaded while the
 // failure was pending: lists and forces of the current state.
@@ -872,6 +881,7 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
     a.dt_lo = (float)(p->dt - (double)(float)p->dt);
     const double thr = std::max(0.5 * p->skin - (double)mdk::kDispMargin, 0.0);
     a.disp_thr = (float)thr;
+    a.spin_max = mdk::kSpinMax;
     for (int s = 0; s < 2; ++s)
         a.inv_mass[s] = (float)(1.0 / a.mass[s]);
     if (a.hdtm_hi[0] == 0.0f)
@@ -994,7 +1004,7 @@ int md_step(md_handle *h, int64_t nsteps)
     if (nsteps < 1)
         return fail(h, MD_E_INVAL, "nsteps must be >= 1");
     int rc;
-    if ((rc = refresh(h)))
+    if ((rc = lost(h)) || (rc = refresh(h)))
         return rc;
     // bound on the steps executed (a device loop that could not end would hold the GPU)
     const int64_t budget = h->p.step_budget > 0 ? h->p.step_budget : nsteps + 64;
@@ -1035,7 +1045,7 @@ int md_rescale_velocities(md_handle *h, const double *T_target)
     for (int r = 0; r < h->g.R; ++r)
         if (!(T_target[r] >= 0.0))
             return fail(h, MD_E_INVAL, "target temperatures must be >= 0");
-    if ((rc = stage_wait(h)))
+    if ((rc = lost(h)) || (rc = stage_wait(h)))
         return rc;
     memcpy(h->pin, T_target, 8 * (size_t)h->g.R);
     CK(h, cudaMemcpyAsync(h->a.scale, h->pin, 8 * (size_t)h->g.R, cudaMemcpyHostToDevice, h->s));
@@ -1060,7 +1070,7 @@ int md_andersen(md_handle *h, const double *T_target, uint64_t seed, int64_t eve
     for (int r = 0; r < h->g.R; ++r)
         if (!(T_target[r] >= 0.0) || !std::isfinite(T_target[r]))
             return fail(h, MD_E_INVAL, "target temperatures must be finite and >= 0");
-    if ((rc = stage_wait(h)))
+    if ((rc = lost(h)) || (rc = stage_wait(h)))
         return rc;
     memcpy(h->pin, T_target, 8 * (size_t)h->g.R);
     CK(h, cudaMemcpyAsync(h->a.scale, h->pin, 8 * (size_t)h->g.R, cudaMemcpyHostToDevice, h->s));
@@ -1204,6 +1214,8 @@ int md_corr_sample(md_corr *c)
     if (!c)
         return MD_E_INVAL;
     md_handle *h = c->h;
+    if (const int rl = lost(h))
+        return rl;
     int slot = -1;
     for (size_t s = 0; s < c->refs.size(); ++s)
         if (c->refs[s] == 0) {
@@ -1298,6 +1310,8 @@ int md_compute_forces(md_handle *h, double *f, double *e, md_obs *totals)
         return MD_E_INVAL;
     int rc;
     const size_t n = (size_t)h->g.n;
+    if ((rc = lost(h)))
+        return rc;
     h->stale = false;
     if ((rc = launch_run(h, mdk::RUN_REBUILD | mdk::RUN_TOTALS)) ||
         (rc = launch(h, h->ks->expforce, grid_n(h->g.n, kIntBlock), kIntBlock, h->a)))
@@ -1399,15 +1413,19 @@ int md_get_state(md_handle *h, double *pos, double *vel, int32_t *image)
         return MD_E_INVAL;
     int rc;
     const size_t n = (size_t)h->g.n;
-    if ((rc = launch(h, h->ks->getstate, grid_n(h->g.n, kIntBlock), kIntBlock, h->a)))
+    if ((rc = lost(h)) || (rc = launch(h, h->ks->getstate, grid_n(h->g.n, kIntBlock), kIntBlock, h->a)))
         return rc;
-    if ((rc = ensure_pinned(h, 60 * n)) || (rc = stage_wait(h)))
+    if ((rc = ensure_pinned(h, 60 * n + 4)) || (rc = stage_wait(h)))
         return rc;
     char *q = h->pin;
     CK(h, cudaMemcpyAsync(q, h->a.st_pos, 24 * n, cudaMemcpyDeviceToHost, h->s));
     CK(h, cudaMemcpyAsync(q + 24 * n, h->a.st_vel, 24 * n, cudaMemcpyDeviceToHost, h->s));
-    CK(h, cudaMemcpyAsync(q + 48 * n, h->a.st_img, 12 * n, cudaMemcpyDeviceToHost, h->s));
+    CK(h, cudaMemcpyAsync(q + 48 * n, h->a.st_img, 12 * n + 4, cudaMemcpyDeviceToHost, h->s));
     CK(h, cudaStreamSynchronize(h->s));
+    int32_t gone;
+    memcpy(&gone, q + 60 * n, 4);
+    if (gone)                                            // (not reported yet)
+        return check_device(h);
     const CopyJob out[3] = {{pos, q, pos ? 24 * n : 0},
                             {vel, q + 24 * n, vel ? 24 * n : 0},
                             {image, q + 48 * n, image ? 12 * n : 0}};
@@ -1435,7 +1453,7 @@ int md_set_state(md_handle *h, const double *pos, const double *vel, const int32
     CK(h, cudaMemcpyAsync(h->a.st_vel, q + 24 * n, 24 * n, cudaMemcpyHostToDevice, h->s));
     CK(h, cudaMemcpyAsync(h->a.st_img, q + 48 * n, 12 * n, cudaMemcpyHostToDevice, h->s));
     CK(h, cudaEventRecord(h->ev_stage, h->s));
-    h->stale = false;
+    h->stale = h->lost = false;
     if ((rc = launch(h, h->ks->load, h->g.nblk_i, kIntBlock, h->a)))
         return rc;
     return launch_run(h, mdk::RUN_REBUILD | mdk::RUN_FORCES);
@@ -1449,8 +1467,10 @@ int md_get_neighbours(md_handle *h, int32_t *counts, int32_t *lists, int32_t kma
     const size_t n = (size_t)h->g.n;
     int rc;
     mdk::Ctl c;
-    if ((rc = refresh(h)) || (rc = read_ctl(h, &c)))
+    if ((rc = lost(h)) || (rc = refresh(h)) || (rc = read_ctl(h, &c)))
         return rc;
+    if (c.stale & mdk::STALE_STATE)                      // (not reported yet)
+        return check_device(h);
     const size_t K = (size_t)h->g.Kmax;                  // row stride of the lists (the cap)
     if ((rc = ensure_pinned(h, align_up(4 * n) + align_up(16 * n) + 4 * n * K)) || (rc = stage_wait(h)))
         return rc;
@@ -1513,6 +1533,14 @@ int md_sync(md_handle *h)
     if (!h)
         return MD_E_INVAL;
     return check_device(h);
+}
+
+int md_set_wait_limit(md_handle *h, uint32_t polls)
+{
+    if (!h)
+        return MD_E_INVAL;
+    h->a.spin_max = polls ? polls : mdk::kSpinMax;
+    return MD_OK;
 }
 
 int md_destroy(md_handle *h)

@@ -35,6 +35,16 @@ enum {
 constexpr float kListMargin = 1e-4f;
 constexpr float kDispMargin = 1e-4f;
 
+// Polls before a barrier of the run kernel gives up (about ten seconds of polling; the
+// count does not advance while the kernel is preempted).
+constexpr unsigned int kSpinMax = 1u << 24;
+
+// Ctl::stale
+enum {
+    STALE_LISTS = 1u,         // lists and forces are not those of the current state and order
+    STALE_STATE = 2u          // a barrier gave up: parities and step are not those of the buffers
+};
+
 // Control block in device memory, written by the kernels.
 struct Ctl {
     unsigned int status;      // ST_* bits
@@ -55,7 +65,7 @@ struct Ctl {
     long long regrows;        // builds redone with a larger K since md_create
     unsigned int halted;      // 1: a run ended with a status that has not been reported yet; runs do
                               // nothing until it has (status itself can change while blocks start)
-    unsigned int stale;       // 1: lists and forces are not those of the current state and order
+    unsigned int stale;       // STALE_* bits
 };
 
 // Grid barrier and shared decisions of the run kernel, each on a cache line of its own.
@@ -151,6 +161,7 @@ struct KArgs {
     float hdtm_hi[2], hdtm_lo[2], dt_hi, dt_lo, inv_mass[2];
     float disp_thr;                   // skin/2 - margin
     long long budget;                 // run kernel: bound on the steps of this launch
+    unsigned int spin_max;            // run kernel: polls before a barrier gives up
 };
 
 // ---------------------------------------------------------------------------

@@ -2238,10 +2238,6 @@ enum RunFlag : unsigned int {
     RF_ABORT = 8u      // a barrier gave up waiting: leave at once
 };
 
-// Polls before a barrier gives up (about ten seconds of polling; the count does
-// not advance while the kernel is preempted).
-constexpr unsigned int kSpinMax = 1u << 24;
-
 struct RunState {
     long long step, left, obs, rebuilds, regrows, budget;
     long long pend;                // step whose partial sums await their sum (-1: none)
@@ -2316,9 +2312,10 @@ __device__ __forceinline__ unsigned int grid_barrier(const KArgs &a, RunState &S
             // blocks still use)
             do {
                 asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(w) : "l"(&rs->word) : "memory");
-            } while ((w >> 4) != next && ++n < kSpinMax);
+            } while ((w >> 4) != next && ++n < a.spin_max);
             asm volatile("fence.acq_rel.gpu;" ::: "memory");
             if ((w >> 4) != next) {
+                atomicOr(&a.ctl->stale, STALE_LISTS | STALE_STATE);
                 atomicOr(&a.ctl->status, ST_TIMEOUT);
                 a.ctl->halted = 1u;
                 w = RF_STOP | RF_BAD | RF_ABORT;
@@ -2445,13 +2442,13 @@ __device__ __forceinline__ unsigned int run_rebuild(const KArgs &a, const Grp &g
         }
         const unsigned int f = grid_barrier(a, S, [&](bool) -> unsigned int {
             a.rs->unit = g.nvb;
-            ctl->stale = 1u;                         // (rref and the rows are those of the new order)
+            atomicOr(&ctl->stale, STALE_LISTS);      // (rref and the rows are those of the new order)
             if (atomicOr(&ctl->status, 0u))
                 return RF_STOP | RF_BAD;
             const int mx = atomicMax(&ctl->max_nbr, 0);
             if (mx <= K) {
                 a.rs->md2[S.step & 1] = 0.f;         // the lists start from these positions
-                ctl->stale = 0u;
+                atomicAnd(&ctl->stale, ~(unsigned int)STALE_LISTS);
                 return 0u;
             }
             if (mx <= ctl->Kmax && retry == 0) {
@@ -2863,7 +2860,7 @@ __global__ void __launch_bounds__(kIntBlock) k_load(KArgs a)
     Ctl *ctl = a.ctl;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         atomicAdd((unsigned long long *)&ctl->n_kernels, 1ull);
-        ctl->stale = 1u;
+        ctl->stale = STALE_LISTS;
     }
     const int4 b = a.blk_i[blockIdx.x];
     const int i = b.x + threadIdx.x;
@@ -2925,8 +2922,10 @@ __global__ void __launch_bounds__(kIntBlock) k_getstate(KArgs a)
 {
     const Ctl *ctl = a.ctl;
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (blockIdx.x == 0 && threadIdx.x == 0)
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
         atomicAdd((unsigned long long *)&a.ctl->n_kernels, 1ull);
+        a.st_img[3 * (size_t)a.n] = (int)(ctl->stale & STALE_STATE);   // (read back with the images)
+    }
     if (s >= a.n)
         return;
     const int pp = ctl->pos_par, spar = ctl->state_par;

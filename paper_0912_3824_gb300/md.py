@@ -107,8 +107,9 @@ def _load() -> C.CDLL:
         "md_status_string": ([C.c_int], C.c_char_p),
         "md_forces_noalloc": ([P, C.c_int64, C.c_double, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p,
                                C.c_void_p, C.c_void_p], C.c_int),
-        # measurement helper (include/md_bench.h)
+        # measurement and test helpers (include/md_bench.h)
         "md_fma_peak": ([C.c_int32, C.c_int64, d, d], C.c_int),
+        "md_set_wait_limit": ([H, C.c_uint32], C.c_int),
     }
     for name, (args, res) in sig.items():
         fn = getattr(lib, name)
@@ -125,7 +126,7 @@ EXPORTED = ("md_params_default", "md_workspace_size", "md_create", "md_step",
             "md_corr_workspace_size", "md_corr_create", "md_corr_sample", "md_corr_result",
             "md_corr_destroy", "md_cell_order", "md_epot_series")
 MD_NOALLOC_MAX_N = 1048576
-EXPORTED_BENCH = ("md_fma_peak",)
+EXPORTED_BENCH = ("md_fma_peak", "md_set_wait_limit")
 
 
 def _status_name(code: int) -> str:
@@ -295,6 +296,11 @@ def md_fma_peak(precision: int, iters: int = 2000) -> tuple[float, float]:
     if rc != 0:
         raise MDError(rc, "md_fma_peak failed")
     return t.value, ms.value
+
+
+def md_set_wait_limit(h, polls: int):
+    """Bound on the waits of the handle's later launches (md_bench.h; 0: the library's own)."""
+    _check(_lib.md_set_wait_limit(h, int(polls)), h)
 
 
 def md_forces_noalloc(p: md_params, n: int, box: float, species_ptr: int, pos_ptr: int, force_ptr: int,

@@ -1,5 +1,5 @@
 """What a handle does after a failure has been reported: its lists belong to its
-state again."""
+state again, and a state that was lost is asked for."""
 import numpy as np
 import pytest
 
@@ -101,4 +101,49 @@ def test_a_list_past_the_cap_fails_again_until_the_state_changes(md):
     assert np.abs(f - fr).max() <= 1e-5 * np.sqrt((fr ** 2).sum(axis=1).mean())
     sim.step(20)
     assert sim.sync() == md.MD_OK and sim.info()["step"] == 20
+    sim.close()
+
+
+@pytest.mark.parametrize("prec", ["mixed", "fp64", "fp32"])
+@pytest.mark.parametrize("where", ["step", "rebuild"])
+def test_a_wait_that_ran_out_is_reported_and_a_new_state_mends_it(md, prec, where):
+    """The barriers' limit set to one poll: a launch ends with MD_E_TIMEOUT inside a
+    step or inside a rebuild (after its binning has counted the particles).  The
+    handle then refuses what needs the state it lost, and goes on bit for bit like
+    a fresh one once a state has been loaded."""
+    s = synth.perturb(synth.ka_mixture(n=2000, temperature=1.0, seed=3), 0.05, 103)
+    sim = _sim(md, s, precision=md.PRECISIONS[prec])
+    sim.step(20)
+    assert sim.sync() == md.MD_OK
+    for reported in (True, False):
+        md.md_set_wait_limit(sim.h, 1)
+        if where == "step":
+            sim.step(20)
+            sim.step(20)
+        else:
+            sim.set_state(s.pos, s.vel)
+        md.md_set_wait_limit(sim.h, 0)
+        if reported:
+            assert sim.sync() == md.MD_E_TIMEOUT
+            assert sim.sync() == md.MD_OK
+            for call in (lambda: sim.step(1), sim.get_state, sim.forces, sim.neighbours, lambda: sim.rescale(1.0),
+                         lambda: sim.andersen(1.0, 1, 0)):
+                with pytest.raises(md.MDError) as ei:
+                    call()
+                assert ei.value.code == md.MD_E_TIMEOUT and "md_set_state" in str(ei.value)
+        else:
+            with pytest.raises(md.MDError) as ei:            # (the read-back reports it)
+                sim.get_state()
+            assert ei.value.code == md.MD_E_TIMEOUT
+        sim.set_state(s.pos, s.vel)
+        f, _, _ = sim.forces()
+        ref = _sim(md, s, precision=md.PRECISIONS[prec])
+        fr, _, _ = ref.forces()
+        assert np.array_equal(f, fr)
+        sim.step(40)
+        ref.step(40)
+        assert sim.sync() == md.MD_OK and ref.sync() == md.MD_OK
+        for x, y in zip(sim.get_state(), ref.get_state()):
+            assert np.array_equal(x, y)
+        ref.close()
     sim.close()
