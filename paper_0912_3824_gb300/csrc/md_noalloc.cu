@@ -209,9 +209,14 @@ __global__ void __launch_bounds__(32 * WARPS) k_forces_allpairs(Pot pot, int n, 
                         __syncwarp();
                         flush(r, 32);
                         __syncwarp();
-                        const int next = lane < cnt[r] - 32 ? queue[w][r][32 + lane] : 0;
+                        // the rest moves to the front: by its own lanes only, and ordered before the
+                        // next partners, which other lanes add behind it
+                        const bool rest = lane < cnt[r] - 32;
+                        const int next = rest ? queue[w][r][32 + lane] : 0;
                         __syncwarp();
-                        queue[w][r][lane] = next;
+                        if (rest)
+                            queue[w][r][lane] = next;
+                        __syncwarp();
                         cnt[r] -= 32;
                     }
                 }

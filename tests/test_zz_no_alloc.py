@@ -111,3 +111,22 @@ def test_noalloc_rejects_sizes_beyond_its_scratch(md):
                              buf.data_ptr(), 0, buf.data_ptr(), torch.cuda.current_stream(dev).cuda_stream)
     assert ei.value.code == md.MD_E_INVAL
     assert "MD_NOALLOC_MAX_N" in str(ei.value)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("n,rc", [(4001, 5.0), (1500, 4.2)])
+def test_noalloc_rows_of_many_partners(md, prec, n, rc):
+    """Cutoffs that hold ~370 to ~630 partners, so that a particle's queue of partners is
+    emptied and its rest moved to the front a dozen times: the oracle's sums, and
+    the same bits from every call."""
+    s = synth.perturb(synth.ka_mixture(n=n, temperature=0.7, seed=9), 0.05, 19)
+    s.params["rcut"] = [[rc, rc], [rc, rc]]
+    fr, er, _ = oracle.forces_brute(s.params, s.box, s.species, s.pos)
+    d = _device_arrays(s)
+    p = md.make_params(s.params, 0.001, precision=md.PRECISIONS[prec])
+    first = _call(md, p, s, d)
+    assert np.abs(first[0] - fr).max() <= TOL_F[prec] * np.sqrt((fr ** 2).sum(axis=1).mean())
+    assert np.abs(first[1] - er).max() <= TOL_F[prec] * np.sqrt((er ** 2).mean())
+    for _ in range(5):
+        for x, y in zip(first, _call(md, p, s, d)):
+            assert np.array_equal(x, y)
