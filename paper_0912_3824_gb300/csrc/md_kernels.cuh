@@ -1730,8 +1730,26 @@ struct NbBlock {
 };
 
 // Word of particle j for the build: coordinates relative to `ctr` (nearest
-// image) and index with the species in the sign bit.
-struct NbCentre { float x, y, z; unsigned int qx, qy, qz; };
+// image) and index with the species in the sign bit.  The rounding is that of the
+// small difference: MIXED and FP64 subtract on the fixed-point circle, to which
+// one FP64 instruction takes a coordinate (as the conversion to single precision
+// would; subtracting in double cost 1.3 % of a step at KA N=16384), FP32 shifts by
+// the box where that is exact (nb_sep).
+struct NbCentre { float x, y, z; unsigned int qx, qy, qz; double qscale; };
+
+// x / L in units of 2^-32 modulo 2^32, to the nearest, for |x| <= 2^18 L
+__device__ __forceinline__ unsigned int circle_d(double x, double qscale)
+{
+    return (unsigned int)__double2loint(fma(x, qscale, 6755399441055744.0));   // 1.5 2^52
+}
+
+// Nearest image of x - c: x - L is exact for x in [L/2, L], and so is c - L.
+__device__ __forceinline__ float nb_sep(float x, float c, float L, float invL)
+{
+    const float k = rintf((x - c) * invL);
+    const float t = k > 0.f ? x - L : x, u = k < 0.f ? c - L : c;
+    return t - u;
+}
 
 template <int P>
 __device__ __forceinline__ NbCentre nb_centre(const Rep &rp, const int4 &cc)
@@ -1741,6 +1759,7 @@ __device__ __forceinline__ NbCentre nb_centre(const Rep &rp, const int4 &cc)
     c.x = ((float)cc.x + 0.5f) * edge;
     c.y = ((float)cc.y + 0.5f) * edge;
     c.z = ((float)cc.z + 0.5f) * edge;
+    c.qscale = rp.invL * 4294967296.0;
     // the same on the fixed-point circle
     c.qx = (unsigned int)((((unsigned long long)(2 * cc.x + 1)) << 31) / (unsigned int)rp.nc);
     c.qy = (unsigned int)((((unsigned long long)(2 * cc.y + 1)) << 31) / (unsigned int)rp.nc);
@@ -1759,14 +1778,13 @@ __device__ __forceinline__ float3 nb_rel(const KArgs &a, const Rep &rp, const Nb
     } else if constexpr (P == FP64) {
         const d4 x = ((const d4 *)pos_a(a, pn))[j];
         sp = species_of(x.w);
-        return make_float3(sep_f(__double2float_rn(x.x), c.x, rp.Lhi, rp.invLf),
-                           sep_f(__double2float_rn(x.y), c.y, rp.Lhi, rp.invLf),
-                           sep_f(__double2float_rn(x.z), c.z, rp.Lhi, rp.invLf));
+        return make_float3(sep_q(circle_d(x.x, c.qscale), c.qx, rp.qunit), sep_q(circle_d(x.y, c.qscale), c.qy, rp.qunit),
+                           sep_q(circle_d(x.z, c.qscale), c.qz, rp.qunit));
     } else {
         const float4 x = ((const float4 *)pos_a(a, pn))[j];
         sp = species_of(x.w);
-        return make_float3(sep_f(x.x, c.x, rp.Lhi, rp.invLf), sep_f(x.y, c.y, rp.Lhi, rp.invLf),
-                           sep_f(x.z, c.z, rp.Lhi, rp.invLf));
+        return make_float3(nb_sep(x.x, c.x, rp.Lhi, rp.invLf), nb_sep(x.y, c.y, rp.Lhi, rp.invLf),
+                           nb_sep(x.z, c.z, rp.Lhi, rp.invLf));
     }
 }
 

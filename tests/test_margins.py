@@ -1,6 +1,6 @@
 """Margins of the single-precision tests that precede exact work: the FP64 pair
-loop's cutoff test, in boxes and with cutoffs large enough for its rounding to
-count.  Lengths are in whatever unit the caller
+loop's cutoff test and the list distances, in boxes and with cutoffs large
+enough for their rounding to count.  Lengths are in whatever unit the caller
 takes: argon in picometres has sigma = 340 and r_c = 850."""
 import numpy as np
 import pytest
@@ -70,3 +70,30 @@ def test_fp64_finds_pairs_just_inside_a_large_cutoff(md, sigma, L, tpp, h):
         sim.close()
         assert np.abs(f - fr).max() <= tol
         assert np.abs(e - er).max() <= 1e-13 * max(np.abs(er).max(), 1.0)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed", "fp32"])
+@pytest.mark.parametrize("form", [1, 2])
+def test_lists_hold_every_pair_within_the_list_radius_of_a_large_box(md, prec, form):
+    """r_c 50, skin 0.3, L 1500, where a single-precision coordinate is good to
+    6e-5: isolated pairs up to 2e-5 inside the list radius, at and away from the
+    box faces, are all listed (the margin of 1e-4 is there for the rounding of
+    the distances alone), and pairs 1e-3 outside it are not."""
+    sigma, L, rl = 20.0, 1500.0, 50.3
+    p = _params(sigma)
+    for seed in range(3):
+        rng = np.random.default_rng(seed)
+        sep = lambda k: np.where(np.arange(k) % 8 == 7, rl + 1e-3, rl - rng.uniform(1e-8, 2e-5, k))
+        pos = _pairs(L, 8, sep, rng.uniform(-40.0, 40.0, 3), rng)
+        n = len(pos)
+        q = md.make_params(p, 0.001, precision=md.PRECISIONS[prec], build_form=form)
+        sim = md.System(q, [n], [L], np.zeros(n, dtype=np.int32), pos, np.zeros((n, 3)))
+        held, _, _ = sim.get_state()
+        counts, lists = sim.neighbours()
+        sim.close()
+        d = held[0::2] - held[1::2]
+        d -= L * np.round(d / L)
+        r = np.repeat(np.sqrt((d ** 2).sum(1)), 2)           # distances of the positions held
+        listed = np.array([counts[i] == 1 and lists[i, 0] == (i ^ 1) for i in range(n)])
+        assert listed[r < rl].all()
+        assert not listed[r > rl + 4e-4].any()
