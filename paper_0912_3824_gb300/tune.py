@@ -2,8 +2,8 @@
 parameters.
 
 The throughput of the step depends on how many lanes share a particle (the
-shape of the step kernel's blocks: 1, 2, 4 or 8 lanes, 128 threads per
-block), on the skin (a longer list against rarer rebuilds; the result of the
+shape of the step kernel's groups: 1 to 16 lanes, 128 threads per group), on
+the skin (a longer list against rarer rebuilds; the result of the
 method does not depend on it, Sec. 2.2) and, through memory, on the list
 capacity.  `autotune` times short runs of the caller's own configuration for
 every candidate and returns the fastest parameters, with the list capacity
@@ -47,16 +47,23 @@ def autotune(base: md.md_params, n_per_replica, box, species, pos, vel, image=No
     """Returns (best md_params, table of trials).  The state (pos, vel, image,
     original order) is the starting point of every trial; each trial warms up
     for `steps` MD steps (several list rebuilds) and is then timed `repeats`
-    times over `steps` steps with CUDA events (median)."""
+    times over `steps` steps with CUDA events (median).  Without `lanes` the
+    library's automatic number of lanes (which goes by the size of the system and
+    its lists) is among the candidates, so the result is never slower than the
+    default by more than the timing's noise."""
     import torch
-    if lanes is None:
+    auto = lanes is None
+    if auto:
         lanes = (2, 4, 8) if base.precision == md.MD_PREC_FP64 else (1, 2, 4)
     if base.smooth_h > 0:
         lanes = tuple(t for t in lanes if t <= 8)
     trials = []
     best = None
     for skin in skins:
-        for tpp in lanes:
+        tried = set()
+        for tpp in ((0,) if auto else ()) + tuple(lanes):
+            if tpp in tried:
+                continue
             p = _clone(base)
             p.skin = float(skin)
             p.threads_per_particle = int(tpp)
@@ -67,7 +74,10 @@ def autotune(base: md.md_params, n_per_replica, box, species, pos, vel, image=No
             ms = _time(torch, sim, steps, repeats) if status == md.MD_OK else math.inf
             info = sim.info()
             sim.close()
-            trials.append({"skin": float(skin), "threads_per_particle": int(tpp), "ms_per_step": ms,
+            tpp = int(info["threads_per_particle"])          # (0: as resolved)
+            p.threads_per_particle = tpp
+            tried.add(tpp)
+            trials.append({"skin": float(skin), "threads_per_particle": tpp, "ms_per_step": ms,
                            "max_neighbours": int(info["max_neighbours"]),
                            "neigh_capacity": int(info["neigh_capacity"]), "status": md._status_name(status)})
             if best is None or ms < best[0]:
