@@ -40,6 +40,15 @@
  *     md_step() returns without waiting for the GPU; the calls that return
  *     data (md_compute_forces, md_observables, md_get_state,
  *     md_get_neighbours, md_info, md_sync) wait for the stream.
+ *   - The step kernel is a cooperative launch of one block per SM whose blocks
+ *     wait for one another, so it starts when every SM has room for its block,
+ *     and holds that room until md_step's last step.  Handles on streams of their
+ *     own run side by side as long as their blocks fit an SM together: three up
+ *     to ~4,800 particles (automatic lanes, MIXED or FP32, not smoothed), two up
+ *     to ~7,200, and above that one after the other (fewer
+ *     threads_per_particle make a block smaller).  Systems that share the
+ *     potential and dt advance fastest together as replicas of one handle.  A
+ *     kernel of the caller's that fills an SM delays md_step until it ends.
  *   - Device-side failures (a neighbour list longer than the cap
  *     neigh_capacity_max, a non-finite value, a particle moving more than a
  *     quarter box in one step, an exhausted step-loop bound) stop the step

@@ -939,9 +939,18 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
         h->a.nslot = g.R == 1 ? h->g.nwork : g.nblk_f;
         // groups without chunks, where the GPU holds more than there are chunks, add up the
         // steps' partial sums, a replica each; in a rebuild a group takes a cell (or a share of
-        // one where cells are few)
-        const int parts = std::max(1, std::min(8, 4 * nsm / g.ncell));
-        const int want = std::max(h->g.nwork + std::min(g.R, nsm), g.ncell < kMaxRunGroups ? g.ncell * parts : kMaxRunGroups);
+        // one where cells are few).  Where the chunks' groups outnumber the cells, shares ask for
+        // 2 groups per SM at most: the launch occupies every SM, and up to 3 groups (2 of the
+        // kernels that hold 5) leave room for another handle's on another stream.  us per MD
+        // step and handle, 1 / 2 / 4 / 8 handles, with up to 4 groups for shares and with 2:
+        // KA N = 2000 8.4 8.5 8.4 8.4 and 8.4 4.6 4.6 3.6; 4000 9.5 9.5 9.5 9.4 and 9.5 5.2 5.1
+        // 4.1; FP64 N = 4000 33.9 33.7 33.7 - and 33.9 29.2 29.0 -.  (Cells that outnumber the
+        // chunks do need groups: N = 16,384, 512 cells, 13.1 with 4 and 14.2 with 3, which
+        // would let two handles take 8.7 each.  One group at N = 864 would let seven handles in,
+        // 2.2 for 3.1 of eight, but costs a single one 1 to 3 %.)
+        const int base = h->g.nwork + std::min(g.R, nsm), parts = std::max(1, std::min(8, 4 * nsm / g.ncell));
+        const int cells = g.ncell < kMaxRunGroups ? g.ncell * parts : kMaxRunGroups;
+        const int want = std::max(base, g.ncell <= base ? std::min(cells, 2 * nsm) : cells);
         h->g.groups = std::min(per_sm, (want + nsm - 1) / nsm);
         h->a.nb_parts = std::max(1, std::min(8, nsm * h->g.groups / g.ncell));
         if ((rc = put(L.off_rep, g.rep.data(), sizeof(mdk::Rep) * g.R)) ||
