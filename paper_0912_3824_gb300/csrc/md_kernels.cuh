@@ -1744,11 +1744,9 @@ __device__ __forceinline__ unsigned int circle_d(double x, double qscale)
 }
 
 // Nearest image of x - c: x - L is exact for x in [L/2, L], and so is c - L.
-__device__ __forceinline__ float nb_sep(float x, float c, float L, float invL)
+__device__ __forceinline__ float nb_sep(float x, float c, float d, float L)
 {
-    const float k = rintf((x - c) * invL);
-    const float t = k > 0.f ? x - L : x, u = k < 0.f ? c - L : c;
-    return t - u;
+    return d > 0.5f * L ? (x - L) - c : d < -0.5f * L ? x - (c - L) : d;
 }
 
 template <int P>
@@ -1783,8 +1781,13 @@ __device__ __forceinline__ float3 nb_rel(const KArgs &a, const Rep &rp, const Nb
     } else {
         const float4 x = ((const float4 *)pos_a(a, pn))[j];
         sp = species_of(x.w);
-        return make_float3(nb_sep(x.x, c.x, rp.Lhi, rp.invLf), nb_sep(x.y, c.y, rp.Lhi, rp.invLf),
-                           nb_sep(x.z, c.z, rp.Lhi, rp.invLf));
+        float3 d = make_float3(x.x - c.x, x.y - c.y, x.z - c.z);
+        if (fmaxf(fmaxf(fabsf(d.x), fabsf(d.y)), fabsf(d.z)) > 0.5f * rp.Lhi) {   // (cells at the faces)
+            d.x = nb_sep(x.x, c.x, d.x, rp.Lhi);
+            d.y = nb_sep(x.y, c.y, d.y, rp.Lhi);
+            d.z = nb_sep(x.z, c.z, d.z, rp.Lhi);
+        }
+        return d;
     }
 }
 
