@@ -40,8 +40,8 @@
  *     md_step() returns without waiting for the GPU; the calls that return
  *     data (md_compute_forces, md_observables, md_get_state,
  *     md_get_neighbours, md_info, md_sync) wait for the stream.
- *   - The step kernel is a cooperative launch of one block per SM whose blocks
- *     wait for one another, so it starts when every SM has room for its block,
+ *   - The step kernel is a cooperative launch of one block per SM (of the SMs of
+ *     the stream's green context, where it has one) whose blocks wait for one another, so it starts when every SM has room for its block,
  *     and holds that room until md_step's last step.  Handles on streams of their
  *     own run side by side as long as their blocks fit an SM together: three up
  *     to ~4,800 particles (automatic lanes, MIXED or FP32, not smoothed), two up

@@ -8,6 +8,7 @@
 // n steps needs no host round trip.  With use_graph = 0 the same kernel is
 // launched once per phase (each step, each rebuild) with its time taken (the
 // results are bitwise identical).
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
@@ -433,7 +434,7 @@ struct md_handle {
     char *ws = nullptr;
     KArgs a;
     const KernelSet *ks = nullptr;
-    int nsm = 0;                     // blocks of the run kernel: one per SM
+    int nsm = 0;                     // blocks of the run kernel: one per SM that the stream can have
     const void *runk = nullptr;      // the run kernel in use: precision, lanes per particle, smoothing
     int cap = 4096;
     // pinned host staging
@@ -480,6 +481,42 @@ int launch(md_handle *h, const void *f, int grid, int block, const KArgs &a)
     void *pp[1] = {(void *)&a};
     CK(h, cudaLaunchKernel(f, dim3((unsigned)grid), dim3((unsigned)block), pp, 0, h->s));
     return MD_OK;
+}
+
+// SMs that launches on stream s can have: all of the device's, or those of the
+// green context that the stream (or, for a default stream, the current context)
+// belongs to.  The run kernel's blocks must all be resident, one per SM.
+int stream_sms(cudaStream_t s, int device_sms)
+{
+    const auto entry = [](const char *name) {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion(name, &fn, 12040, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            fn = nullptr;
+        }
+        return fn;
+    };
+    CUdevResource r;
+    memset(&r, 0, sizeof r);
+    CUgreenCtx green = nullptr;
+    CUcontext ctx = nullptr;
+    bool known = false;
+    if (s && s != cudaStreamLegacy && s != cudaStreamPerThread) {
+        const auto of_stream = (CUresult(*)(CUstream, CUgreenCtx *))entry("cuStreamGetGreenCtx");
+        const auto of_green = (CUresult(*)(CUgreenCtx, CUdevResource *, CUdevResourceType))entry("cuGreenCtxGetDevResource");
+        if (of_stream && of_green && of_stream(s, &green) == CUDA_SUCCESS && green)
+            known = of_green(green, &r, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS;
+    }
+    if (!green) {
+        const auto current = (CUresult(*)(CUcontext *))entry("cuCtxGetCurrent");
+        const auto of_ctx = (CUresult(*)(CUcontext, CUdevResource *, CUdevResourceType))entry("cuCtxGetDevResource");
+        known = current && of_ctx && current(&ctx) == CUDA_SUCCESS && ctx &&
+                of_ctx(ctx, &r, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS;
+    }
+    const int n = known ? (int)r.sm.smCount : 0;
+    return n > 0 && n < device_sms ? n : device_sms;
 }
 
 int grid_n(int64_t n, int per) { return (int)((n + per - 1) / per); }
@@ -890,6 +927,7 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
     int dev = 0, nsm = 0, per_sm = 0, resident = 0;
     CK(h, cudaGetDevice(&dev));
     CK(h, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    nsm = stream_sms(h->s, nsm);
     h->runk = h->ks->run[h->p.smooth_h > 0.0][force_index(g.tpp)];
     const int most = std::min(h->ks->groups[h->p.smooth_h > 0.0], kMaxRunGroups / std::max(nsm, 1));
     if (most < 1)
