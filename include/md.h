@@ -116,7 +116,7 @@ typedef struct {
     int32_t obs_capacity;     /* ring-buffer samples kept on the device (0 = 4096); also the
                                  number of newest steps the per-step potential-energy series
                                  keeps (md_epot_series)                                         */
-    int32_t threads_per_particle; /* force-kernel lanes per particle: 0 = automatic (2 for MIXED and
+    int32_t threads_per_particle; /* lanes (threads) per particle: 0 = automatic (2 for MIXED and
                                      FP32, 4 for FP64; more below ~12,000 (FP64: ~6,500) particles
                                      with long enough lists), else a power of two in 1..32 (1..8
                                      with smooth_h > 0)                                          */

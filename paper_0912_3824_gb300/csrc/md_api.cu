@@ -65,9 +65,9 @@ struct Geometry {
     int64_t n = 0;
     int K = 0, Kmax = 0, tpp = 8, ppb_f = 32;   // starting list capacity, its cap
     int check = kCheck;                 // MD steps between rebuild checks
-    bool nb_block = false;              // neighbour build with one block per cell
+    bool nb_block = false;              // neighbour build by groups of threads
     int nblk_i = 0, nblk_f = 0, ncell = 0;
-    bool sweep = false;                 // step_form as reported: more chunks than resident blocks
+    bool sweep = false;                 // step_form as reported: more chunks than groups
     int groups = 1, nwork = 0, cpb = 1; // run kernel: groups per block, groups with chunks, chunks per group
     double rl_max = 0.0;
     std::vector<mdk::Rep> rep;
@@ -149,11 +149,15 @@ int auto_capacity(const md_params *p, const Geometry &g, const std::vector<doubl
 // leave it idle, and more lanes shorten the chain of a row's entries, as long as
 // rows are long enough to share.  Measured on GB300, us per MD step:
 //   KA mixed, N = 1000: 9.57 (2 lanes) 8.60 (4) 7.30 (8) 7.28 (16); 6000: 10.48 10.56
-//     8.81 9.26; 12,000: 11.44 11.35 10.62 14.03; 24,000: 13.28 14.88 - -
+//     8.81 9.26; 10,000: 11.25 11.20 9.93 -; 12,000: 11.15 11.83 10.78 -; 14,000: 11.30
+//     11.78 11.54 -; 16,384: 11.43 11.67 11.92 -; 20,000: 13.19 13.35 16.18 -
+//     (so the lines of 2 and 8 lanes cross between 12,000 and 14,000)
 //   LJ 0.8442 mixed, N = 2000: 9.51 9.49 9.13 9.06; 8000: 11.21 11.30 11.12 12.00
 //   LJ 0.3 mixed (~28 entries a row), N = 2000: 7.98 8.65 8.56 8.38
 //   KA smoothed, N = 1000: 12.90 9.89 7.68 (8); 12,000: 14.88 12.47 12.04; 24,000: 17.26 16.52 -
 //   KA FP64, N = 1000: 68.8 36.5 23.5 18.5; 4000: 69.4 37.4 33.6 43.5; 8000: 69.8 54.6 59.1 70.8
+//   KA FP64 smoothed, N = 1000: 138 74.8 43.0 (8); 4000: 138 74.8 63.8; 8000: 140 115 115
+//     (4 lanes at every size: 8 would be faster below ~6,000)
 int auto_lanes(const md_params *p, int R, const int64_t *nrep, const double *box, double rl)
 {
     double n = 0.0, vol = 0.0;
@@ -190,11 +194,11 @@ int make_geometry(const md_params *p, int R, const int64_t *nrep, const double *
         return MD_E_INVAL;
     }
     if (p->step_form < 0 || p->step_form > 2) {
-        msg = "step_form must be 0 (automatic), 1 (one block per chunk) or 2 (resident blocks sweep)";
+        msg = "step_form must be 0 (automatic), 1 or 2";
         return MD_E_INVAL;
     }
     if (p->build_form < 0 || p->build_form > 2) {
-        msg = "build_form must be 0 (automatic), 1 (warp per cell) or 2 (block per cell)";
+        msg = "build_form must be 0 (automatic), 1 (warp per cell) or 2 (groups of threads per cell)";
         return MD_E_INVAL;
     }
     if (p->neigh_capacity < 0 || p->neigh_capacity_max < 0) {
@@ -363,7 +367,7 @@ Layout make_layout(const md_params *p, const Geometry &g)
     L.off_ctl = take(sizeof(mdk::Ctl));
     L.off_rep = take(sizeof(mdk::Rep) * g.R);
     L.off_blk_i = take(sizeof(int4) * g.nblk_i);
-    L.off_blk_r = take(sizeof(int4) * 2 * (size_t)g.nblk_f);   // < nblk_f + resident blocks rows
+    L.off_blk_r = take(sizeof(int4) * 2 * (size_t)g.nblk_f);   // < nblk_f + groups rows
     L.off_rs = take(sizeof(mdk::RunSync));
     L.off_slice = take(sizeof(int) * kMaxRunGroups);
     L.off_crank = take(sizeof(int) * g.ncell);
@@ -835,7 +839,6 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
     a.obs_cap = h->cap;
     a.epot_cap = h->cap;
     a.nblk_i = g.nblk_i;
-    a.nblk_f = g.nblk_f;
     a.pa = w + L.off_pa; a.pb = w + L.off_pb; a.va = w + L.off_va; a.vb = w + L.off_vb;
     a.pa2 = w + L.off_pa2; a.pb2 = w + L.off_pb2; a.va2 = w + L.off_va2; a.vb2 = w + L.off_vb2;
     a.qa = (int4 *)(w + L.off_qa); a.qb = (int4 *)(w + L.off_qb);
@@ -883,7 +886,6 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
             const double shift = p->shift ? 4.0 * eps * (sr6 * sr6 - sr6) : 0.0;
             const double rl = rc + p->skin + (double)mdk::kListMargin;
             a.tab.rc2d[k] = rc * rc;
-            a.tab.rl2d[k] = rl * rl;
             a.tab.sig2d[k] = sig * sig;
             a.tab.eps4d[k] = 4.0 * eps;
             a.tab.eps48d[k] = 48.0 * eps;
@@ -939,12 +941,12 @@ static int create_impl(md_handle *h, const md_params *p, const int32_t *species,
         return fail(h, MD_E_CUDA, "the run kernel does not fit the device");
     per_sm = most;
     h->nsm = nsm;
-    const bool one_each = g.nblk_f <= nsm * per_sm;   // a block for every chunk
+    const bool one_each = g.nblk_f <= nsm * per_sm;   // a group for every chunk
     h->g.sweep = p->step_form == 2 || (p->step_form == 0 && !one_each && p->precision != MD_PREC_FP64 && g.tpp <= 2);
     // the build takes a warp per cell when there are at least kNbWarpCellsPerSm cells per SM
-    // and a cell's particles fit one batch of lanes on average; a block per cell otherwise
-    // (measured on GB300: LJ at 729 cells or fewer and dense cells of ~40 are faster with a
-    // block per cell, LJ from 1331 cells and KA N=65,536 with a warp per cell)
+    // and a cell's particles fit one batch of lanes on average; groups of threads otherwise
+    // (measured on GB300: LJ at 729 cells or fewer and dense cells of ~40 are faster with
+    // groups, LJ from 1331 cells and KA N=65,536 with a warp per cell)
     h->g.nb_block = p->build_form == 2 ||
                     (p->build_form == 0 && ((int64_t)g.ncell < (int64_t)kNbWarpCellsPerSm * nsm ||
                                             (double)g.n > 32.0 * (double)g.ncell));

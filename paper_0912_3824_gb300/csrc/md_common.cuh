@@ -81,8 +81,8 @@ struct RunSync {
 struct Rep {                  // one independent system
     int start, n;             // particle range (sorted order keeps replicas contiguous)
     int cell0, nc;            // first global cell id, cells per edge (1 if fewer than 3 fit)
-    int bi0, bi1;             // integrate-kernel block range
-    int bf0, bf1;             // force-kernel block range
+    int bi0, bi1;             // range of the blocks of 256 particles (KArgs::blk_i)
+    int bf0, bf1;             // range of the chunks
     double L, invL, cscale;   // box edge, 1/L, nc/L
     float Lhi, Llo, invLf, cscalef;
     float grid, inv_grid;     // anchoring grid of MIXED positions (powers of two)
@@ -96,7 +96,7 @@ struct PairTab {              // [a*2+b]
     float rc2[4], rl2[4], sig2[4], eps4[4], eps48[4], shift[4];
     float rc[4], ihs[4];      // r_c and 1 / (h sigma) of the smoothing (Sec. 4)
     float vc[4];              // S_ab / (4 eps_ab) (0 where eps_ab = 0): V = 4 eps_ab (s6^2 - s6 - vc)
-    double rc2d[4], rl2d[4], sig2d[4], eps4d[4], eps48d[4], shiftd[4];
+    double rc2d[4], sig2d[4], eps4d[4], eps48d[4], shiftd[4];
     double rcd[4], ihsd[4], vcd[4];
     double e48vcd[4];         // eps48 vc
 };
@@ -114,7 +114,7 @@ struct KArgs {
     int n, nrep, ncell, si, obs_cap, epot_cap, imode, what;
     int Kstride;                      // list row stride: the capacity cap (Ctl::Kmax); the rows hold
                                       // at most Ctl::K entries, so K can grow without a new layout
-    int nblk_i, nblk_f;
+    int nblk_i;
     int check;                        // MD steps between rebuild checks
     int pos0;                         // position of the first step of this launch in its md_step
     int last;                         // this launch ends its md_step

@@ -38,7 +38,6 @@ constexpr int kPartF = 12;       // doubles per partial sum of a sample step
 constexpr int kUnr = 8;          // list entries per lane and iteration of the FP32 pair loops
                                  // (a multiple of 4, at most 8: lists are padded to 8)
 constexpr int kPfDepth = 1;      // iterations ahead at which the list indices are loaded
-constexpr bool kSplitUpdate = false; // below 4 lanes: one lane updates (measured faster than sharing)
 
 // Bounds-checked build (compile with -DMD_CHECK_BOUNDS=1; off in the product
 // library): every index read from device memory (list entries, cell keys,
@@ -715,7 +714,7 @@ constexpr float kE24hi = (float)(1.0 / 24.0);
 constexpr float kE24lo = (float)(1.0 / 24.0 - (double)(float)(1.0 / 24.0));
 
 // FP64 mode: the FP64 pipe is narrow on this GPU (a warp-wide instruction keeps
-// it for ~16 cycles of the SM whatever the number of active lanes), so it sees
+// it for ~18 cycles of the SM whatever the number of active lanes), so it sees
 // nothing but pairs inside the cutoff, spread evenly over the lanes.  A warp
 // takes its particles' rows in rounds of kPairQ entries: a single-precision test
 // with a margin (on coordinates cut to float by integer operations) queues the
@@ -737,7 +736,9 @@ struct PairQueue {
 };
 
 // A double's value cut to float precision, by integer operations (values below
-// 2^-127 become tiny ones; infinities and NaN do not survive).
+// 2^-127 become tiny ones; infinities and NaN become ordinary numbers: a particle
+// with such a coordinate is in nobody's list or fails the FP64 test, and its next
+// drift reports it).
 __device__ __forceinline__ float cut_float(double x)
 {
     const unsigned int hi = (unsigned int)__double2hiint(x), lo = (unsigned int)__double2loint(x);
@@ -745,6 +746,9 @@ __device__ __forceinline__ float cut_float(double x)
     return __uint_as_float((hi & 0x80000000u) | (e << 3) | (lo >> 29));
 }
 
+// 1/x of a normal number: y (1 + e + e^2) with e = 1 - x y, from the hardware's estimate
+// y, whose relative error is below 2^-19.  The terms left out are below 2^-57, so
+// the error is that of the last rounding, at most 2^-53 (1 + 2^-4).
 __device__ __forceinline__ double rcp_newton(double x)
 {
     double y;
@@ -1314,41 +1318,34 @@ __device__ __forceinline__ void component_update(const KArgs &a, const Rep &rp, 
     }
 }
 
-// Step body: after the pair loop the lanes of a particle's group share its
-// update.  Lane l owns the components c = l*NC .. l*NC + NC - 1 (NC = 1 for 4
-// or more lanes, 4 / TPP below): c = 0..2 are the Cartesian components of the
-// double-single kick-drift-kick, c = 3 carries the species word to the new
-// position buffer.  The operands of the update are loaded before the
-// neighbour loop so that their latency is hidden.
+// Step body from 4 lanes per particle on: after the pair loop its lanes share the
+// update.  Lanes c = 0..2 do one Cartesian component each of the double-single
+// kick-drift-kick, lane 3 carries the species word to the new position buffer.
+// The operands of the update are loaded before the neighbour loop so that their
+// latency is hidden.
 template <int P, int TPP, bool SAMPLE, bool SM>
-__device__ __forceinline__ void step_body_split(const KArgs &a, const Rep &rep, PairQueue *Q, const int4 b, bool kick, bool last, bool track,
+__device__ __forceinline__ void step_body_split(const KArgs &a, const Rep &rep, PairQueue *Q, const int4 b, bool kick, bool last,
                                                 int pp, int spar, double *part, ET<P> &eo, float &d2, float &v2, float &a2,
                                                 unsigned int &bad)
 {
-    constexpr int NC = TPP >= 4 ? 1 : 4 / TPP;
     const Rep rp = rep;
     const int lane = threadIdx.x & (TPP - 1);
     const int i = b.x + Grp::tid() / TPP;
     const bool valid = i < b.y;
     const int ii = valid ? i : b.x;
     const int nn = valid ? a.nnbr[ii] : 0;
-    float vh[NC], vl[NC], rr[NC];
-    double vd[NC];
-#pragma unroll
-    for (int u = 0; u < NC; ++u) {
-        const int c = lane * NC + u;
-        const size_t e = 4 * (size_t)ii + (c < 3 ? c : 0);
-        vh[u] = 0.f; vl[u] = 0.f; rr[u] = 0.f; vd[u] = 0.0;
-        if (valid && c < 3) {
-            if constexpr (P == FP64) {
-                vd[u] = ((const double *)vel_a(a, spar))[e];
-            } else {
-                vh[u] = ((const float *)vel_a(a, spar))[e];
-                if constexpr (P == MIXED)
-                    vl[u] = ((const float *)vel_b(a, spar))[e];
-            }
-            rr[u] = ((const float *)a.rref)[e];
+    float vh = 0.f, vl = 0.f, rr = 0.f;
+    double vd = 0.0;
+    if (valid && lane < 3) {
+        const size_t e = 4 * (size_t)ii + lane;
+        if constexpr (P == FP64) {
+            vd = ((const double *)vel_a(a, spar))[e];
+        } else {
+            vh = ((const float *)vel_a(a, spar))[e];
+            if constexpr (P == MIXED)
+                vl = ((const float *)vel_b(a, spar))[e];
         }
+        rr = ((const float *)a.rref)[e];
     }
     FT<P> fx = 0, fy = 0, fz = 0;
     ET<P> ep = e_zero<P>();
@@ -1373,44 +1370,36 @@ __device__ __forceinline__ void step_body_split(const KArgs &a, const Rep &rep, 
         store_force<P>(a, i, fx, fy, fz, ep);
     double ke = 0.0, p3[3] = {0.0, 0.0, 0.0};
     float dd = 0.f, vv = 0.f;
-#pragma unroll
-    for (int u = 0; u < NC; ++u) {
-        const int c = lane * NC + u;
-        if (!valid) {
-            // no update
-        } else if (c < 3) {
-            const size_t e = 4 * (size_t)i + c;
-            const FT<P> f_c = c == 0 ? fx : (c == 1 ? fy : fz);
-            double kc = 0.0, pc = 0.0;
-            float dc = 0.f, wc = 0.f;
-            component_update<P>(a, rp, pp, spar, i, c, sp, (float)f_c, (double)f_c, SAMPLE, kick, last, vh[u], vl[u],
-                                vd[u], rr[u], kc, pc, dc, wc, bad);
-            ke += kc;
-            dd += dc;
-            vv += wc;
-            p3[0] += c == 0 ? pc : 0.0;
-            p3[1] += c == 1 ? pc : 0.0;
-            p3[2] += c == 2 ? pc : 0.0;
-            if constexpr (P == FP64) {
-                ((double *)vel_a(a, spar))[e] = vd[u];
-            } else {
-                ((float *)vel_a(a, spar))[e] = vh[u];
-                if constexpr (P == MIXED)
-                    ((float *)vel_b(a, spar))[e] = vl[u];
-            }
-        } else if (c == 3 && !last) {
-            // the species word travels with the position
-            if constexpr (P == FP64)
-                ((double *)pos_a(a, pp ^ 1))[4 * (size_t)i + 3] = ((const double *)pos_a(a, pp))[4 * (size_t)i + 3];
-            else
-                ((float *)pos_a(a, pp ^ 1))[4 * (size_t)i + 3] = ((const float *)pos_a(a, pp))[4 * (size_t)i + 3];
+    if (!valid) {
+        // no update
+    } else if (lane < 3) {
+        const size_t e = 4 * (size_t)i + lane;
+        const FT<P> f_c = lane == 0 ? fx : (lane == 1 ? fy : fz);
+        double pc = 0.0;
+        component_update<P>(a, rp, pp, spar, i, lane, sp, (float)f_c, (double)f_c, SAMPLE, kick, last, vh, vl, vd, rr, ke, pc,
+                            dd, vv, bad);
+        p3[0] = lane == 0 ? pc : 0.0;
+        p3[1] = lane == 1 ? pc : 0.0;
+        p3[2] = lane == 2 ? pc : 0.0;
+        if constexpr (P == FP64) {
+            ((double *)vel_a(a, spar))[e] = vd;
+        } else {
+            ((float *)vel_a(a, spar))[e] = vh;
             if constexpr (P == MIXED)
-                ((int *)q_of(a, pp ^ 1))[4 * (size_t)i + 3] = sp;
+                ((float *)vel_b(a, spar))[e] = vl;
         }
+    } else if (lane == 3 && !last) {
+        // the species word travels with the position
+        if constexpr (P == FP64)
+            ((double *)pos_a(a, pp ^ 1))[4 * (size_t)i + 3] = ((const double *)pos_a(a, pp))[4 * (size_t)i + 3];
+        else
+            ((float *)pos_a(a, pp ^ 1))[4 * (size_t)i + 3] = ((const float *)pos_a(a, pp))[4 * (size_t)i + 3];
+        if constexpr (P == MIXED)
+            ((int *)q_of(a, pp ^ 1))[4 * (size_t)i + 3] = sp;
     }
-    // combine the component lanes (the first min(TPP, 4) lanes of the group)
+    // combine the component lanes (the first 4 of the particle)
 #pragma unroll
-    for (int o = (TPP < 4 ? TPP : 4) / 2; o > 0; o >>= 1) {
+    for (int o = 2; o > 0; o >>= 1) {
         dd += __shfl_xor_sync(0xffffffffu, dd, o);
         vv += __shfl_xor_sync(0xffffffffu, vv, o);
         if (SAMPLE) {
@@ -1446,8 +1435,8 @@ __device__ __forceinline__ void step_body(const KArgs &a, const Rep &rep, PairQu
                                           int pp, int spar, double *part, ET<P> &eo, float &d2, float &v2, float &a2,
                                           unsigned int &bad)
 {
-    if constexpr (kSplitUpdate || TPP >= 4) {
-        step_body_split<P, TPP, SAMPLE, SM>(a, rep, Q, b, kick, last, track, pp, spar, part, eo, d2, v2, a2, bad);
+    if constexpr (TPP >= 4) {                        // (below 4 lanes one lane updates: measured faster)
+        step_body_split<P, TPP, SAMPLE, SM>(a, rep, Q, b, kick, last, pp, spar, part, eo, d2, v2, a2, bad);
         return;
     }
     const Rep rp = rep;
@@ -2620,7 +2609,11 @@ __device__ __forceinline__ void run_service(const KArgs &a, const Grp &g, RunSta
 
 // Groups per SM: 7 at <= 72 registers a thread for the unsmoothed single-precision
 // kernels, so that 1024 chunks (KA N=65536 at 2 lanes per particle) are one per
-// group on 152 SMs; 5 at <= 96 for FP64 and the smoothed kernels (they would spill).
+// group on 152 SMs (1064 blocks of 128 threads took 26.5 us a step there, 7 groups
+// 23.3); 5 at <= 96 for FP64 and the smoothed kernels.  The kernels of 7 groups spill
+// (`-Xptxas -v`, bytes stored at 1 / 2 / 4 / 8 or more lanes: mixed 276 / 232 / 304 / 128,
+// FP32 192 / 208 / 200 / 136), FP64 smoothed 180 to 192, the others 40 at most.  6 or 8
+// groups were not measured at other sizes.
 template <int P, bool SM> constexpr int run_groups() { return P == FP64 || SM ? 5 : 7; }
 
 // What the step at S.step, position S.pos between checks, has to do (thread 0).

@@ -1,4 +1,4 @@
-// md_tables.h -- host-side chunk tables of the force and step kernels.
+// md_tables.h -- host-side chunk tables of the run kernel.
 //
 // Plain C++ over CUDA's int4 (x = first particle, y = end, z = replica,
 // w = chunk index): no device code, so the tables can be checked on the CPU
@@ -23,16 +23,14 @@ inline int4 mk4(int x, int y, int z, int w)
     return v;
 }
 
-// Launch order of the force-kernel chunks.  A launch that fits in one wave
-// (at most `resident` blocks) hands its blocks to the SMs in turns: the first
-// nsm blocks go one to each SM (in an order of the GPU's own, not p -> SM p),
-// and the next nsm in the same order, so blocks p, p + nsm, p + 2 nsm, ...
-// share an SM (per-block SM ids read on GB300); giving them consecutive chunks
-// (neighbouring cells along the cell curve) lets one SM's blocks share the
-// neighbour positions they gather in its L1.  A longer launch keeps the chunk
-// order, so that the blocks resident at any time cover one compact region.
-// Block p carries its chunk index in w, where its partial sums go, so the
-// per-replica sums keep their order.
+// Order of the run kernel's chunks over its groups of threads, where there is a
+// group for every chunk.  Group p works on SM p mod nsm (block p mod nsm of one
+// block per SM), so groups p, p + nsm, p + 2 nsm, ... share an SM; giving them
+// consecutive chunks (neighbouring cells along the cell curve) lets one SM's groups
+// share the neighbour positions they gather in its L1.  With more chunks than
+// `resident` groups the chunk order is kept (step_table then shares them out).
+// Row p carries its chunk index in w, where its partial sums go with several
+// replicas, so the per-replica sums keep their order.
 inline std::vector<int4> sm_block_order(const std::vector<int4> &chunks, int nsm, int resident)
 {
     const int nb = (int)chunks.size();
@@ -50,18 +48,15 @@ inline std::vector<int4> sm_block_order(const std::vector<int4> &chunks, int nsm
     return out;
 }
 
-// Rows of the step kernel's table (see KArgs::blk_s).  With one block per
-// chunk they are the force kernel's rows.  The sweeping form launches only the
-// resident blocks (nsm * per_sm) and gives each group of blocks that share an
-// SM (blocks s, s + nsm, s + 2 nsm, ...) one run of consecutive chunks along
-// the cell curve: the per_sm blocks of group s take neighbouring chunks of its
-// run side by side (block s + k nsm: chunks base_s + k, base_s + k + per_sm,
-// ...), so that at any time they work on one compact region and share the
-// neighbour positions they gather in the SM's L1
-// (with one block per chunk, a launch longer than one wave hands each freed
-// slot the next chunk, so an SM's blocks lie anywhere in the resident region).
-// Each row carries its chunk index in w; a block's rows end in padding
-// (w = -1).  Returns the rows, cpb per block.
+// Rows of the run kernel's table (KArgs::blk_r), cpb per group.  With a group for
+// every chunk (`sweep` false) they are the rows of sm_block_order.  With more chunks
+// than groups (nsm * per_sm) the groups that share an SM (s, s + nsm, s + 2 nsm,
+// ...) get one run of consecutive chunks along the cell curve and take neighbouring
+// chunks of it side by side (group s + k nsm: chunks base_s + k, base_s + k +
+// per_sm, ...), so that at any time they work on one compact region and share
+// the neighbour positions they gather in the SM's L1.  Each row carries its chunk
+// index in w; a group's rows end in padding (w = -1).  Returns the rows; nblk_s is
+// the number of groups with chunks.
 inline std::vector<int4> step_table(const std::vector<int4> &order, const std::vector<int4> &chunks, bool sweep,
                                     int nsm, int per_sm, int &nblk_s, int &cpb)
 {
@@ -71,7 +66,7 @@ inline std::vector<int4> step_table(const std::vector<int4> &order, const std::v
         cpb = 1;
         return order;
     }
-    if ((int64_t)nsm * per_sm > nb) {           // fewer chunks than resident blocks: at most nb blocks
+    if ((int64_t)nsm * per_sm > nb) {           // fewer chunks than groups: at most nb groups
         if (nb < nsm) {
             nsm = nb;
             per_sm = 1;

@@ -346,8 +346,8 @@ def make_params(pot: dict, dt: float, skin: float = 0.3, precision: int = MD_PRE
     p.check_interval = int(check_interval)   # 0 automatic, else 1, 2, 4, 8, 16
     p.neigh_capacity_max = int(neigh_capacity_max)   # 0: twice the starting capacity
     p.step_budget = int(step_budget)         # 0: automatic bound of md_step's device loop
-    p.build_form = int(build_form)           # 0 automatic, 1 warp per cell, 2 block per cell
-    p.step_form = int(step_form)             # 0 automatic, 1 block per chunk, 2 resident blocks sweep
+    p.build_form = int(build_form)           # 0 automatic, 1 warp per cell, 2 groups of threads
+    p.step_form = int(step_form)             # 0 automatic, 1 or 2: one scheme, reported as asked
     return p
 
 
