@@ -56,7 +56,7 @@ def parse_args(argv=None):
     ap.add_argument("--no-extras", action="store_true", help="skip fp64 / e2e / cpu legs")
     ap.add_argument("--no-graph", action="store_true",
                     help="a launch per MD step and rebuild instead of one (for per-phase profiling)")
-    ap.add_argument("--tpp", type=int, default=0, help="force-kernel threads per particle (0 = auto)")
+    ap.add_argument("--tpp", type=int, default=0, help="threads per particle (0 = auto)")
     ap.add_argument("--step-form", type=int, default=0, choices=[0, 1, 2],
                     help="sharing of chunks: 0 auto, 1 or 2 (not FP64); one scheme, reported as asked")
     ap.add_argument("--build-form", type=int, default=0, choices=[0, 1, 2],
@@ -379,7 +379,7 @@ def run_ours(args, rank, world, local):
     if args.no_extras or rank != 0:
         return result
 
-    # ---- force kernel: live per-launch duration (stream launches + CUDA events) ----
+    # ---- MD step: live duration (a launch per step + CUDA events) ----
     pos, vel, img = sim.get_state()
     p_nog = md.make_params(s.params, 0.001, skin=base.skin, precision=md.PRECISIONS[args.precision],
                            sample_interval=100, use_graph=False, threads_per_particle=base.threads_per_particle,
@@ -391,7 +391,7 @@ def run_ours(args, rank, world, local):
     info_b = sim_k.info()
     ev_ms = (info_b["step_ms"] - info_a["step_ms"]) / max(1, info_b["step_launches"] - info_a["step_launches"])
     # the MD step's average duration inside the timed region (rebuilds excluded),
-    # from the device timer each launch reads at its first block start and last block end
+    # from the device timer read at each grid barrier
     n_dev = info1["step_device_launches"] - info0["step_device_launches"]
     f_ms = (info1["step_device_ms"] - info0["step_device_ms"]) / max(1, n_dev)
     n_list, n_cut = list_statistics(sim_k, s.params)

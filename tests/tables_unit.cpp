@@ -1,8 +1,8 @@
-// Host-side checks of the chunk tables of the force and step kernels
-// (paper_0912_3824_gb300/csrc/md_tables.h): the launch orders are
-// permutations of the chunks, blocks that share an SM get neighbouring
-// chunks, and the step kernel's sweeping table covers every chunk once with
-// padding only at the end of a block's rows.  Prints "ok" or the first
+// Host-side checks of the chunk tables of the run kernel
+// (paper_0912_3824_gb300/csrc/md_tables.h): the orders are permutations of the
+// chunks, groups that share an SM get neighbouring chunks, and the table for
+// more chunks than groups covers every chunk once with padding only at the end
+// of a group's rows.  Prints "ok" or the first
 // failure; exit status 0 on success.
 #include <cstdio>
 #include <cstdlib>

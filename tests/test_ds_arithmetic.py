@@ -2,7 +2,8 @@
 on the GPU against exact rational arithmetic: sums and products to the
 paper's 44-bit effective precision, normalised results, and exact two-sum /
 two-product error terms (which any contraction of the error-free
-transformations into fused operations would break)."""
+transformations into fused operations would break); and the helpers of the FP64
+pair loop against their bounds."""
 import os
 import subprocess
 from fractions import Fraction as Fr
@@ -16,14 +17,14 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 
 
-def _program(tmp_path):
+def _program(tmp_path, name="ds_unit"):
     import shutil
     if shutil.which("nvcc") is None:
         pytest.skip("nvcc not available")
-    exe = tmp_path / "ds_unit"
+    exe = tmp_path / name
     subprocess.run(["nvcc", "-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-std=c++17",
                     "-I", os.path.join(ROOT, "paper_0912_3824_gb300", "csrc"), "-o", str(exe),
-                    os.path.join(HERE, "ds_unit.cu")], check=True)
+                    os.path.join(HERE, name + ".cu")], check=True)
     return exe
 
 
@@ -72,3 +73,27 @@ def test_ds_add_mul_against_exact_rationals(tmp_path):
         if al == 0 and bl == 0:         # two-sum and two-product are exact
             assert s == a + b
             assert p == a * b and q == a * b
+
+
+def test_fp64_reciprocal_and_cut_against_exact_rationals(tmp_path):
+    """The FP64 pair loop's reciprocal: one Newton step of third order on an estimate
+    good to 2^-19 leaves 2^-57, and the last rounding 2^-53 (relative, of a result
+    just above a power of two): at most 2^-53 (1 + 2^-4), here over squared
+    distances and the range of exponents.  Its cut to single precision keeps 24
+    bits, towards zero."""
+    exe = _program(tmp_path, "fp64_unit")
+    rng = np.random.default_rng(11)
+    x = np.concatenate([rng.uniform(0.3, 40.0, 20000), 2.0 ** rng.uniform(-120, 120, 20000),
+                        np.nextafter(2.0 ** np.arange(-40, 40), 0), 2.0 ** np.arange(-40.0, 40.0),
+                        1.0 + np.arange(64) * 2.0 ** -52])
+    inp, outp = tmp_path / "in.bin", tmp_path / "out.bin"
+    with open(inp, "wb") as f:
+        f.write(np.int32(len(x)).tobytes())
+        f.write(x.tobytes())
+    subprocess.run([str(exe), str(inp), str(outp)], check=True)
+    res = np.fromfile(outp, dtype=np.float64).reshape(-1, 2)
+    bound = Fr(1, 2 ** 53) * (1 + Fr(1, 16))
+    worst = max(abs(Fr(float(y)) * Fr(float(v)) - 1) for v, (y, _) in zip(x, res))
+    assert worst <= bound, float(worst) * 2 ** 53
+    mant, ex = np.frexp(x)
+    assert np.array_equal(res[:, 1], np.ldexp(np.floor(mant * 2.0 ** 24), ex - 24))

@@ -270,7 +270,7 @@ def test_e1_sparse_corner_trajectory(md):
 @pytest.mark.parametrize("prec", ["fp64", "mixed", "fp32"])
 @pytest.mark.parametrize("kind,n,skin", [("ka", 4000, 0.3), ("lj", 2048, 0.3), ("ka", 6000, 0.9)])
 def test_build_forms_give_the_same_lists_and_trajectory(md, prec, kind, n, skin):
-    """The neighbour build with one warp per cell and with one block per cell
+    """The neighbour build with one warp per cell and with groups of threads per cell
     (the handle picks by the cell count) write the same rows in the same
     order: equal lists at creation and equal positions after 200 steps with
     several rebuilds, bit for bit.  Skin 0.9 makes cells of ~45 particles, so
@@ -297,13 +297,12 @@ def test_build_forms_give_the_same_lists_and_trajectory(md, prec, kind, n, skin)
 @pytest.mark.parametrize("kind,n,tpp,smooth", [("lj", 262144, 1, 0.0), ("ka", 4000, 2, 0.0), ("ka", 4000, 2, 0.005),
                                                ("lj", 300, 1, 0.0)])
 def test_step_forms_give_the_same_trajectory(md, prec, kind, n, tpp, smooth):
-    """The step kernel with one block per chunk and with the resident blocks
-    sweeping runs of chunks compute every particle and every chunk's partial
-    sums the same way: equal positions, velocities, images, samples and
-    per-step energies after 150 steps with rebuilds, bit for bit.  LJ at
-    N = 262,144 and 1 lane needs more blocks than are resident (the automatic
-    choice is the sweep); the small systems force it on fewer chunks than
-    resident blocks (N = 300: fewer chunks than SMs)."""
+    """step_form 1 and 2 are accepted and reported as asked and take one scheme
+    (chunks shared out in runs wherever there are more of them than groups of
+    threads): the same positions, velocities, images, samples and per-step energies
+    after 150 steps with rebuilds.  LJ at N = 262,144 and 1 lane has more chunks than
+    groups (reported as form 2 by default).  (Distributions that really differ:
+    test_chunks_shared_out_over_one_and_over_many_sweeps.)"""
     s = _system(kind, n, amp=0.02)
     if smooth:
         s.params["smooth"] = smooth
@@ -332,7 +331,7 @@ def test_step_forms_give_the_same_trajectory(md, prec, kind, n, tpp, smooth):
 
 def test_automatic_build_form_follows_cells_per_sm_and_cell_occupancy(md):
     """The automatic neighbour build takes a warp per cell from 8 cells per SM
-    with at most 32 particles per cell on average, a block per cell otherwise."""
+    with at most 32 particles per cell on average, groups of threads otherwise."""
     import torch
     nsm = torch.cuda.get_device_properties(0).multi_processor_count
     for kind, n in (("lj", 4096), ("lj", 32768), ("ka", 65536)):
@@ -625,8 +624,7 @@ def _heated_run(md, s, nsteps, use_graph, **kw):
 def test_capacity_grows_during_a_run(md, use_graph):
     """A capacity that fits the start but not the heated liquid, with a cap to
     grow into: the run finishes with MD_OK, the capacity has grown in place
-    (a redone build inside the CUDA graph's rebuild branch, or in the stream
-    launches), and the trajectory equals that of a run with room to spare from
+    (a build redone inside the one launch, or in a launch of its own), and the trajectory equals that of a run with room to spare from
     the start, bit for bit (the list contents and their order do not depend on
     the capacity)."""
     s = _melted(synth.ka_params(), 2000, 1.2, 1.0)     # longest list 112 at the start, on a
@@ -656,8 +654,8 @@ def test_capacity_grows_during_a_run(md, use_graph):
 def test_overflow_past_the_cap_keeps_the_last_consistent_state(md, use_graph):
     """The same heated run with the capacity fixed (cap = start): the step loop
     stops at the rebuild whose list exceeds the cap, MD_E_CAPACITY is reported,
-    and the buffers stay those of the last completed step (the build's last
-    block does not make the half-written permutation current), so the
+    and the buffers stay those of the last completed step (the permutation written
+    by the build is not made current), so the
     positions equal those of an unconstrained run after the same number of
     steps."""
     s = _melted(synth.ka_params(), 2000, 1.2, 1.0)
@@ -691,8 +689,8 @@ def test_instability_is_reported_and_state_kept(md):
 
 @pytest.mark.parametrize("use_graph", [True, False])
 def test_exhausted_step_budget_is_reported_and_state_kept(md, use_graph):
-    """md_step's device loop is bounded.  With the bound lowered to 40 step-
-    kernel executions (step_budget), md_step(100) stops inside the loop with
+    """md_step's device loop is bounded.  With the bound lowered to 40 steps
+    (step_budget), md_step(100) stops inside the loop with
     MD_E_TIMEOUT, reported once, and the positions are those of an
     unconstrained run of the same number of steps."""
     s = _system("ka", 1000)
@@ -750,7 +748,7 @@ def test_overlapping_particles_are_reported(md, prec):
 
 def test_full_size_sampled_parity_ka65536(md):
     """The benchmark's system (KA, N = 65536, mixed, default launch shape):
-    after 200 graph-driven steps, forces on 256 sampled particles equal the
+    after 200 steps, forces on 256 sampled particles equal the
     oracle's one-by-one brute-force sums; Newton's third law holds for the
     total; E_pot equals the oracle cell-list sum."""
     s = synth.ka_mixture(n=65536, temperature=0.7, seed=5)
@@ -799,8 +797,8 @@ def test_correlator_matches_blocking_oracle(md, prec):
 
 @pytest.mark.parametrize("use_graph", [True, False])
 def test_step_kernel_device_timer(md, use_graph):
-    """Every step-kernel launch adds its device duration (first block start to
-    last block end) to md_info: one launch per MD step, graph or not."""
+    """Every MD step adds its device duration (from one grid barrier to the next) to
+    md_info, in one launch or in a launch each."""
     s = _system("ka", 4000, amp=0.05)
     sim = _sim(md, s, "mixed", use_graph=use_graph)
     sim.step(10)

@@ -133,6 +133,36 @@ def test_more_replicas_than_groups(md):
         assert (obs[k] == obs[k][:, :1]).all()
 
 
+@pytest.mark.parametrize("prec,tpp", [("mixed", 1), ("mixed", 8), ("fp64", 4), ("fp32", 2)])
+def test_chunks_shared_out_over_one_and_over_many_sweeps(md, prec, tpp):
+    """One system alone (a chunk per group at most, sums per group) and as one of
+    enough copies that every group sweeps several chunks (sums per chunk): equal
+    states of every copy after 60 steps with rebuilds, bit for bit, and the same
+    energies up to the order of their sums."""
+    n, steps = 2000, 60
+    s = synth.perturb(synth.ka_mixture(n=n, temperature=1.5, seed=5), 0.05, 105)
+    r = 3 * 1064 * 128 // tpp // n + 1                         # > 3 chunks per group of a GB300
+    # (the maxima behind the rebuild decision are those of all replicas, here the same)
+    p = md.make_params(s.params, 0.002, precision=md.PRECISIONS[prec], threads_per_particle=tpp, check_interval=4,
+                       sample_interval=20, obs_capacity=128)
+    one = md.System(p, [n], [s.box], s.species, s.pos, s.vel)
+    all_ = md.System(p, [n] * r, [s.box] * r, np.tile(s.species, r), np.tile(s.pos, (r, 1)), np.tile(s.vel, (r, 1)))
+    for sim in (one, all_):
+        sim.step(steps)
+        assert sim.sync() == md.MD_OK and sim.info()["rebuilds"] >= 3
+    for a, b in zip(one.get_state(), all_.get_state()):
+        assert np.array_equal(np.tile(a, (r, 1)), b)
+    o1, o2 = one.observables(), all_.observables()
+    e1, e2 = one.epot_series()[1], all_.epot_series()[1]
+    one.close()
+    all_.close()
+    assert np.array_equal(o1["step"], o2["step"][:, :1])
+    # sums of 2000 terms in double, or energies in double-single (2^-44 a sum)
+    for k in ("e_pot", "e_kin", "virial"):
+        assert np.abs(o2[k] / o1[k] - 1.0).max() <= 1e-10
+    assert np.abs(e2 / e1 - 1.0).max() <= 1e-10
+
+
 @pytest.mark.parametrize("n", [2, 31, 33, 513, 1030])
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
 @pytest.mark.parametrize("far", [0.0, 2.0e3, 1.0e6])

@@ -1,4 +1,4 @@
-"""The chunk tables of the force and step kernels (host logic of
+"""The chunk tables of the run kernel (host logic of
 csrc/md_tables.h), checked on the CPU by a small C++ program."""
 import os
 import shutil
