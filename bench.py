@@ -191,15 +191,16 @@ FLOP_PER_UPDATE = 210
 
 
 KERNEL_SOURCES = ("paper_0912_3824_gb300/csrc/md_kernels.cuh", "paper_0912_3824_gb300/csrc/md_common.cuh")
+TRAFFIC_PROFILE = os.path.join("profiles", "k_run_ka65536_lj1048576_mixed.md")
 
 
 def profiled_traffic(kernel, skin):
-    """DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum)
-    of `kernel` from the committed ncu summary, or None when no summary
-    covers it, its sources changed since the capture, or the capture ran with
-    another skin (another list length)."""
+    """DRAM bytes of a launch of one MD step with cold caches
+    (dram__bytes_read.sum + dram__bytes_write.sum) of `kernel` from the committed
+    ncu summary, or None when no summary covers it, its sources changed since the
+    capture, or the capture ran with another skin (another list length)."""
     import hashlib
-    path = os.path.join(ROOT, "profiles", "k_step_ka65536_mixed.md")
+    path = os.path.join(ROOT, TRAFFIC_PROFILE)
     if not os.path.exists(path):
         return None
     fields = {}

@@ -40,7 +40,7 @@ def test_profiled_traffic_only_for_the_captured_kernel_and_skin():
     that kernel, skin and source state, None otherwise."""
     import hashlib
     fields = {}
-    for line in open(os.path.join(ROOT, "profiles", "k_step_ka65536_mixed.md")):
+    for line in open(os.path.join(ROOT, bench.TRAFFIC_PROFILE)):
         k, sep, v = line.partition(":")
         if sep and k in ("traffic_bytes_per_launch", "kernel", "skin", "source_sha256"):
             fields[k] = v.strip()
@@ -53,7 +53,8 @@ def test_profiled_traffic_only_for_the_captured_kernel_and_skin():
         assert 20e6 < got < 40e6                  # one cold launch at KA N=65536: list + state
     else:
         assert got is None                        # sources changed since the capture
-    assert bench.profiled_traffic("k_step<0, 4, 0, 0>", skin) is None
+    assert kernel == "k_run<1, 2, 0>"             # what the bench asks for at KA N=65536, mixed, 2 lanes
+    assert bench.profiled_traffic("k_run<0, 4, 0>", skin) is None
     assert bench.profiled_traffic(kernel, skin + 0.1) is None
 
 
