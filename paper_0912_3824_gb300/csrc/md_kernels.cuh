@@ -1722,20 +1722,15 @@ struct NbBlock {
 // image) and index with the species in the sign bit.  The rounding is that of the
 // small difference: MIXED and FP64 subtract on the fixed-point circle, to which
 // one FP64 instruction takes a coordinate (as the conversion to single precision
-// would; subtracting in double cost 1.3 % of a step at KA N=16384), FP32 shifts by
-// the box where that is exact (nb_sep).
+// would; subtracting in double cost 1.3 % of a step at KA N=16384).  FP32 rounds once
+// more where it shifts by the box, by half an ulp of L for each of a pair: 8.9e-5 at
+// L = 1500, within the list margin (an exact shift cost 1 to 2 % of a step).
 struct NbCentre { float x, y, z; unsigned int qx, qy, qz; double qscale; };
 
 // x / L in units of 2^-32 modulo 2^32, to the nearest, for |x| <= 2^18 L
 __device__ __forceinline__ unsigned int circle_d(double x, double qscale)
 {
     return (unsigned int)__double2loint(fma(x, qscale, 6755399441055744.0));   // 1.5 2^52
-}
-
-// Nearest image of x - c: x - L is exact for x in [L/2, L], and so is c - L.
-__device__ __forceinline__ float nb_sep(float x, float c, float d, float L)
-{
-    return d > 0.5f * L ? (x - L) - c : d < -0.5f * L ? x - (c - L) : d;
 }
 
 template <int P>
@@ -1770,13 +1765,8 @@ __device__ __forceinline__ float3 nb_rel(const KArgs &a, const Rep &rp, const Nb
     } else {
         const float4 x = ((const float4 *)pos_a(a, pn))[j];
         sp = species_of(x.w);
-        float3 d = make_float3(x.x - c.x, x.y - c.y, x.z - c.z);
-        if (fmaxf(fmaxf(fabsf(d.x), fabsf(d.y)), fabsf(d.z)) > 0.5f * rp.Lhi) {   // (cells at the faces)
-            d.x = nb_sep(x.x, c.x, d.x, rp.Lhi);
-            d.y = nb_sep(x.y, c.y, d.y, rp.Lhi);
-            d.z = nb_sep(x.z, c.z, d.z, rp.Lhi);
-        }
-        return d;
+        return make_float3(sep_f(x.x, c.x, rp.Lhi, rp.invLf), sep_f(x.y, c.y, rp.Lhi, rp.invLf),
+                           sep_f(x.z, c.z, rp.Lhi, rp.invLf));
     }
 }
 
@@ -2612,7 +2602,7 @@ __device__ __forceinline__ void run_service(const KArgs &a, const Grp &g, RunSta
 // group on 152 SMs (1064 blocks of 128 threads took 26.5 us a step there, 7 groups
 // 23.3); 5 at <= 96 for FP64 and the smoothed kernels.  The kernels of 7 groups spill
 // (`-Xptxas -v`, bytes stored at 1 / 2 / 4 / 8 or more lanes: mixed 276 / 232 / 304 / 128,
-// FP32 192 / 208 / 200 / 136), FP64 smoothed 180 to 192, the others 40 at most.  6 or 8
+// FP32 184 / 200 / 184 / 120), FP64 smoothed 180 to 192, the others 40 at most.  6 or 8
 // groups were not measured at other sizes.
 template <int P, bool SM> constexpr int run_groups() { return P == FP64 || SM ? 5 : 7; }
 
